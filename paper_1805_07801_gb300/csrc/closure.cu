@@ -16,6 +16,7 @@
 
 #include "fft_engine.cuh"
 #include "internal.h"
+#include "mlp_train.cuh"
 #include "tcgen05.cuh"
 
 namespace fftk {
@@ -271,178 +272,6 @@ __global__ void k_closure_features(const float* __restrict__ A9, const float* __
       for (int i = 0; i < 6; ++i) taup6[i * Mc + c] = t6[i];
     }
   }
-}
-
-// ------------------------------------------------------------------- MLP ---
-// 5 -> 64 -> 64 -> 64 -> 6, tanh on the hidden layers; parameters (FP32):
-// W1[64][5] b1 W2[64][64] b2 W3[64][64] b3 W4[6][64] b4 (9094 values).
-// Each layer's input (x, h1, h2, h3) is rounded to bfloat16; products and
-// sums are FP32.
-constexpr int kNP = 9094;
-constexpr int kChunk = 128;   // samples per CTA
-constexpr int kAStride = kChunk + 1;
-__device__ __constant__ int kDims[5] = {5, 64, 64, 64, 6};
-__device__ __constant__ int kWOff[4] = {0, 384, 4544, 8704};
-__device__ __constant__ int kBOff[4] = {320, 4480, 8640, 9088};
-
-__device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-// a layer input as the network defines it (BF16), or unrounded in the FP32
-// test mode that isolates the kernels' arithmetic from the BF16 rounding
-template <bool BF16>
-__device__ __forceinline__ float act_round(float x) {
-  return BF16 ? bf16r(x) : x;
-}
-
-struct MLPSmem {
-  float w[kNP];
-  float act0[5 * kAStride];        // input of layer 0, [feature][sample]
-  float act123[3][64 * kAStride];  // inputs of layers 1..3
-  float d0[64 * kAStride];         // deltas
-  float d1[64 * kAStride];
-  __device__ __forceinline__ float* act(int l) { return l == 0 ? act0 : act123[l - 1]; }
-};
-
-// forward of the chunk; y written for samples < nb; returns nothing
-template <bool BF16>
-__device__ void mlp_chunk_forward(MLPSmem& s, const float* __restrict__ x, int nb, int base, float* y6) {
-  const int b = threadIdx.x;
-  if (b < kChunk) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-      s.act(0)[i * kAStride + b] = b < nb ? act_round<BF16>(x[(long long)(base + b) * 5 + i]) : 0.f;
-  }
-  __syncthreads();
-  for (int l = 0; l < 4; ++l) {
-    const int din = kDims[l], dout = kDims[l + 1];
-    const float* W = s.w + kWOff[l];
-    const float* bias = s.w + kBOff[l];
-    for (int o = 0; o < dout; ++o) {
-      float z = bias[o];
-      for (int i = 0; i < din; ++i) z = fmaf(W[o * din + i], s.act(l)[i * kAStride + b], z);
-      if (l < 3)
-        s.act(l + 1)[o * kAStride + b] = act_round<BF16>(tanhf(z));
-      else
-        y6[o] = z;
-    }
-    __syncthreads();
-  }
-}
-
-// one CTA: forward + backward of 128 samples; writes its gradient partial and
-// its loss partial (sum of squared errors).  BF16: layer inputs rounded to
-// bfloat16 (the network's definition); false in the FP32 test mode.
-template <bool BF16>
-__global__ void __launch_bounds__(kChunk) k_mlp_grad(const float* __restrict__ params, const float* __restrict__ x,
-                                                     const float* __restrict__ t, int B, float* __restrict__ part,
-                                                     double* __restrict__ loss_part) {
-  extern __shared__ float smem_mlp[];
-  MLPSmem& s = *reinterpret_cast<MLPSmem*>(smem_mlp);
-  const int b = threadIdx.x;
-  const int base = blockIdx.x * kChunk;
-  const int nb = min(kChunk, B - base);
-  for (int i = b; i < kNP; i += kChunk) s.w[i] = params[i];
-  __syncthreads();
-  float y[6];
-  mlp_chunk_forward<BF16>(s, x, nb, base, y);
-  // output error: dL/dz4 = 2 (y - t) / (6 B)
-  __shared__ double lsum[kChunk];
-  double l2 = 0.0;
-  const float g = 2.f / (6.f * (float)B);
-#pragma unroll
-  for (int o = 0; o < 6; ++o) {
-    float e = 0.f;
-    if (b < nb) e = y[o] - t[(long long)(base + b) * 6 + o];
-    l2 += (double)e * e;
-    s.d0[o * kAStride + b] = e * g;
-  }
-  lsum[b] = l2;
-  __syncthreads();
-  float* dcur = s.d0;
-  float* dnext = s.d1;
-  float* out = part + (long long)blockIdx.x * kNP;
-  for (int l = 3; l >= 0; --l) {
-    const int din = kDims[l], dout = kDims[l + 1];
-    // weight and bias gradients of layer l: sums over the chunk's samples
-    for (int pr = b; pr < dout * din; pr += kChunk) {
-      const int o = pr / din, i = pr % din;
-      float acc = 0.f;
-      for (int k = 0; k < kChunk; ++k) acc = fmaf(dcur[o * kAStride + k], s.act(l)[i * kAStride + k], acc);
-      out[kWOff[l] + pr] = acc;
-    }
-    for (int o = b; o < dout; o += kChunk) {
-      float acc = 0.f;
-      for (int k = 0; k < kChunk; ++k) acc += dcur[o * kAStride + k];
-      out[kBOff[l] + o] = acc;
-    }
-    if (l > 0) {
-      const float* W = s.w + kWOff[l];
-      for (int i = 0; i < din; ++i) {
-        float acc = 0.f;
-        for (int o = 0; o < dout; ++o) acc = fmaf(W[o * din + i], dcur[o * kAStride + b], acc);
-        const float a = s.act(l)[i * kAStride + b];
-        dnext[i * kAStride + b] = acc * (1.f - a * a);
-      }
-    }
-    __syncthreads();
-    float* t2 = dcur;
-    dcur = dnext;
-    dnext = t2;
-  }
-  if (b == 0) {
-    double acc = 0.0;
-    for (int k = 0; k < kChunk; ++k) acc += lsum[k];
-    loss_part[blockIdx.x] = acc;
-  }
-}
-
-// the forward pass alone on the CUDA cores (128 samples per CTA), the
-// arithmetic of k_mlp_grad's forward: y[B][6]
-template <bool BF16>
-__global__ void __launch_bounds__(kChunk) k_mlp_forward_cc(const float* __restrict__ params,
-                                                           const float* __restrict__ x, float* __restrict__ y, int B) {
-  extern __shared__ float smem_mlp[];
-  MLPSmem& s = *reinterpret_cast<MLPSmem*>(smem_mlp);
-  const int b = threadIdx.x;
-  const int base = blockIdx.x * kChunk;
-  const int nb = min(kChunk, B - base);
-  for (int i = b; i < kNP; i += kChunk) s.w[i] = params[i];
-  __syncthreads();
-  float y6[6];
-  mlp_chunk_forward<BF16>(s, x, nb, base, y6);
-  if (b < nb) {
-#pragma unroll
-    for (int o = 0; o < 6; ++o) y[(long long)(base + b) * 6 + o] = y6[o];
-  }
-}
-
-// fixed-order sums of the per-CTA partials
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nblk, float* __restrict__ grad,
-                             const double* __restrict__ loss_part, double* __restrict__ loss, double inv_count) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < kNP) {
-    double acc = 0.0;
-    for (int k = 0; k < nblk; ++k) acc += part[(long long)k * kNP + i];
-    grad[i] = (float)acc;
-  }
-  if (i == 0 && loss) {
-    double acc = 0.0;
-    for (int k = 0; k < nblk; ++k) acc += loss_part[k];
-    *loss = acc * inv_count;
-  }
-}
-
-// Adam (Kingma and Ba 2015) with bias corrections; step counted from 1
-__global__ void k_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                       const float* __restrict__ g, int n, float lr, float b1, float b2, float eps, float c1,
-                       float c2) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
 // Constants of the learned model (normalisation of inputs and outputs).
@@ -759,23 +588,11 @@ static int grid_for(long long work, int threads) {
   return (int)(b < 152 * 16 ? b : 152 * 16);
 }
 
-static size_t mlp_smem() { return sizeof(MLPSmem); }
-
 static cudaError_t mlp_attrs() {
   static PerDevice once;
   return once.run([](int) {
-    cudaError_t err = cudaFuncSetAttribute(k_mlp_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)mlp_smem());
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_mlp_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mlp_smem());
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_mlp_forward_cc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mlp_smem());
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_mlp_forward_cc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mlp_smem());
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mlptc::kSmem);
+    cudaError_t err =
+        cudaFuncSetAttribute(k_mlp_forward_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mlptc::kSmem);
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_sgs_pointwise_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, mlptc::kSmem);
     return err;
@@ -943,7 +760,7 @@ extern "C" fftk_status tarang_mlp_create(int max_batch, tarang_mlp* out) {
   tarang_mlp m = new (std::nothrow) tarang_mlp_s;
   if (!m) return FFTK_ERR_OOM;
   m->max_batch = max_batch;
-  const int nblk = (max_batch + kChunk - 1) / kChunk;
+  const int nblk = mlp_grad_blocks(max_batch);
   cudaError_t e = cudaMalloc(&m->part, sizeof(float) * (size_t)nblk * kNP);
   if (e == cudaSuccess) e = cudaMalloc(&m->loss_part, sizeof(double) * (size_t)nblk);
   if (e == cudaSuccess) e = cudaMalloc(&m->grad, sizeof(float) * kNP);
@@ -997,19 +814,26 @@ extern "C" fftk_status tarang_mlp_sync(tarang_mlp m, void* cuda_stream) {
   return FFTK_OK;
 }
 
+// gradient and loss into grad and loss, then with `adam` the update from them
+static cudaError_t mlp_gradient(tarang_mlp m, const float* params, const float* x, const float* t, int B, float* grad,
+                                double* loss, bool bf16, const AdamStep* adam, cudaStream_t st) {
+  const cudaError_t e = launch_mlp_grad(bf16, params, x, t, B, m->part, m->loss_part, st);
+  return e == cudaSuccess ? launch_mlp_reduce(B, m->part, m->loss_part, grad, loss, adam, st) : e;
+}
+
+static AdamStep adam_step(float* params, float* mom, float* var, int step, float lr, float beta1, float beta2,
+                          float eps) {
+  const float c1 = (float)(1.0 - std::pow((double)beta1, step));
+  const float c2 = (float)(1.0 - std::pow((double)beta2, step));
+  return AdamStep{params, mom, var, lr, beta1, beta2, eps, c1, c2};
+}
+
 extern "C" fftk_status tarang_mlp_loss_grad_mode(tarang_mlp m, const float* params, const float* x, const float* t,
                                                  int B, float* grad, double* loss, int act_mode, void* cuda_stream) {
   if (!m || !params || !x || !t || !grad || B < 1 || B > m->max_batch) return FFTK_ERR_INVALID_ARG;
   if (act_mode != TARANG_ACT_BF16 && act_mode != TARANG_ACT_FP32) return FFTK_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int nblk = (B + kChunk - 1) / kChunk;
-  if (act_mode == TARANG_ACT_BF16)
-    k_mlp_grad<true><<<nblk, kChunk, mlp_smem(), st>>>(params, x, t, B, m->part, m->loss_part);
-  else
-    k_mlp_grad<false><<<nblk, kChunk, mlp_smem(), st>>>(params, x, t, B, m->part, m->loss_part);
-  k_mlp_reduce<<<(kNP + 255) / 256, 256, 0, st>>>(m->part, nblk, grad, m->loss_part, loss,
-                                                 1.0 / (6.0 * (double)B));
-  return from_cuda(cudaGetLastError());
+  return from_cuda(mlp_gradient(m, params, x, t, B, grad, loss, act_mode == TARANG_ACT_BF16, nullptr, st));
 }
 
 extern "C" fftk_status tarang_mlp_loss_grad(tarang_mlp m, const float* params, const float* x, const float* t,
@@ -1022,30 +846,27 @@ extern "C" fftk_status tarang_mlp_forward_mode(tarang_mlp m, const float* params
   if (!m || !params || !x || !y || B < 1) return FFTK_ERR_INVALID_ARG;
   if (act_mode != TARANG_ACT_BF16 && act_mode != TARANG_ACT_FP32) return FFTK_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const int nblk = (B + kChunk - 1) / kChunk;
-  if (act_mode == TARANG_ACT_BF16)
-    k_mlp_forward_cc<true><<<nblk, kChunk, mlp_smem(), st>>>(params, x, y, B);
-  else
-    k_mlp_forward_cc<false><<<nblk, kChunk, mlp_smem(), st>>>(params, x, y, B);
-  return from_cuda(cudaGetLastError());
+  return from_cuda(launch_mlp_forward_cc(act_mode == TARANG_ACT_BF16, params, x, y, B, st));
 }
 
 extern "C" fftk_status tarang_mlp_adam(float* params, float* mom, float* var, const float* grad, int step,
                                        float lr, float beta1, float beta2, float eps, void* cuda_stream) {
   if (!params || !mom || !var || !grad || step < 1) return FFTK_ERR_INVALID_ARG;
-  const float c1 = (float)(1.0 - std::pow((double)beta1, step));
-  const float c2 = (float)(1.0 - std::pow((double)beta2, step));
-  k_adam<<<(kNP + 255) / 256, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(params, mom, var, grad, kNP, lr,
-                                                                                beta1, beta2, eps, c1, c2);
-  return from_cuda(cudaGetLastError());
+  return from_cuda(launch_adam(adam_step(params, mom, var, step, lr, beta1, beta2, eps), grad,
+                               static_cast<cudaStream_t>(cuda_stream)));
 }
 
 extern "C" fftk_status tarang_mlp_train_step(tarang_mlp m, float* params, float* mom, float* var, int step,
                                              const float* x, const float* t, int B, float lr, double* loss,
                                              void* cuda_stream) {
-  fftk_status s = tarang_mlp_loss_grad(m, params, x, t, B, m ? m->grad : nullptr, loss, cuda_stream);
-  if (s != FFTK_OK) return s;
-  return tarang_mlp_adam(params, mom, var, m->grad, step, lr, 0.9f, 0.999f, 1e-8f, cuda_stream);
+  if (!m || !params || !x || !t || B < 1 || B > m->max_batch) return FFTK_ERR_INVALID_ARG;
+  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  if (!mom || !var || step < 1) {  // the gradient and the loss are formed all the same
+    const fftk_status s = from_cuda(mlp_gradient(m, params, x, t, B, m->grad, loss, true, nullptr, st));
+    return s != FFTK_OK ? s : FFTK_ERR_INVALID_ARG;
+  }
+  const AdamStep a = adam_step(params, mom, var, step, lr, 0.9f, 0.999f, 1e-8f);
+  return from_cuda(mlp_gradient(m, params, x, t, B, m->grad, loss, true, &a, st));
 }
 
 // SplitMix64 (Steele, Lea & Flood 2014): output number c of the stream that
