@@ -71,7 +71,8 @@ def ns_kernel_bytes(n):
 
 
 def ns_rhs_bytes_unfused(n):
-    """Bytes one right-hand side moves on a 3 * 2^m grid (no fused passes): the
+    """Bytes one right-hand side would move through full transforms (no fused
+    passes), the yardstick that the fused passes are held against: the
     six spectra cleared and filled with (u, i k x u) on the kept modes, their
     inverse x and y passes (out of place through a second workspace, the same
     bytes) and the z pass to six real fields, u x omega
@@ -107,7 +108,7 @@ def fft_pass_bytes(n):
 
 # --------------------------------------------------- measured DRAM traffic ---
 KERNEL_SOURCES = {
-    "ns": ["ns.cu", "ns_common.cuh", "fft_engine.cuh", "internal.h", "tcgen05.cuh"],
+    "ns": ["ns.cu", "ns_passes.cuh", "ns_radix3.cu", "ns_common.cuh", "fft_engine.cuh", "internal.h", "tcgen05.cuh"],
     "fft": ["fft_passes.cu", "fft_engine.cuh", "internal.h", "abi.cu"],
     "fft16": ["fft_tc.cu", "tcgen05.cuh", "fft_passes.cu", "fft_engine.cuh", "internal.h", "abi.cu"],
 }
@@ -837,10 +838,8 @@ def run_schemes(n: int, steps: int):
     u0 = torch.empty((3, n, n, n // 2 + 1, 2), dtype=torch.float32, device=dev)
     fk.tarang_ic_random(plan, nr.data_ptr(), u0.data_ptr(), K0, E0, st)
     del nr
-    fused = n & (n - 1) == 0
-    pruned = ns_step_bytes(n)[0] if fused else 2 * ns_rhs_bytes_unfused(n)
-    out = {"path": "fused passes restricted to the 2/3 set" if fused else
-           "unfused: the plan's radix-3 transforms, u x omega in real space, the fused path's update"}
+    pruned = ns_step_bytes(n)[0]
+    out = {"path": "fused passes restricted to the 2/3 set"}
     for name, scheme in (("rk2", fk.TARANG_RK2), ("rk4", fk.TARANG_RK4)):
         u = u0.clone()
         prm = fk.make_params(NU, DT, scheme=scheme)

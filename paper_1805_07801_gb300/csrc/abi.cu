@@ -184,20 +184,31 @@ extern "C" fftk_status fftk_plan_create(int nx, int ny, int nz, fftk_dtype dtype
     p->d_tw = p->d_tw_alloc + fftk::kStageTwiddles;
     e = cudaMemcpy(p->d_tw_alloc, h.data(), sizeof(float2) * h.size(), cudaMemcpyHostToDevice);
   }
-  // tables of size 3 * 2^j for the radix-3 lines, at offset L (2 L3 values)
+  // tables of size 3 * 2^j for the lines with a factor 3, at offset L (2 L3
+  // values), and below them the r-major tables of their last stages
   int lt3 = 0;
   for (int d : {nx, ny, nz})
     if (!is_pow2(d) && d > lt3) lt3 = d;
   if (e == cudaSuccess && lt3 > 0) {
-    std::vector<float2> h3(2 * (size_t)lt3, make_float2(1.f, 0.f));
-    for (int L = 3; L <= lt3; L *= 2)
+    std::vector<float2> h3((size_t)fftk::kStage3Twiddles + 2 * (size_t)lt3, make_float2(1.f, 0.f));
+    float2* pyr3 = h3.data() + fftk::kStage3Twiddles;
+    for (int L = 3; L <= lt3; L *= 2) {
       for (int m = 0; m < L; ++m) {
         const double ang = two_pi * (double)m / (double)L;
-        h3[(size_t)L + m] = make_float2((float)std::cos(ang), (float)(-std::sin(ang)));
+        pyr3[(size_t)L + m] = make_float2((float)std::cos(ang), (float)(-std::sin(ang)));
       }
-    e = cudaMalloc(&p->d_tw3, sizeof(float2) * h3.size());
-    if (e == cudaSuccess)
-      e = cudaMemcpy(p->d_tw3, h3.data(), sizeof(float2) * h3.size(), cudaMemcpyHostToDevice);
+      for (int R = 3; R <= 24 && R <= L / 2; R *= 2) {
+        const int ns = L / R;
+        float2* ts = h3.data() + fftk::stage3_tw_offset(L, R);
+        for (int r = 0; r < R; ++r)
+          for (int k = 0; k < ns; ++k) ts[(size_t)r * ns + k] = pyr3[(size_t)L + (size_t)r * k];
+      }
+    }
+    e = cudaMalloc(&p->d_tw3_alloc, sizeof(float2) * h3.size());
+    if (e == cudaSuccess) {
+      p->d_tw3 = p->d_tw3_alloc + fftk::kStage3Twiddles;
+      e = cudaMemcpy(p->d_tw3_alloc, h3.data(), sizeof(float2) * h3.size(), cudaMemcpyHostToDevice);
+    }
   }
   if (e == cudaSuccess) e = cudaMalloc(&p->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
@@ -206,7 +217,7 @@ extern "C" fftk_status fftk_plan_create(int nx, int ny, int nz, fftk_dtype dtype
     fftk_status s = from_cuda(e);
     cudaGetLastError();
     if (p->d_tw_alloc) cudaFree(p->d_tw_alloc);
-    if (p->d_tw3) cudaFree(p->d_tw3);
+    if (p->d_tw3_alloc) cudaFree(p->d_tw3_alloc);
     if (p->d_err) cudaFree(p->d_err);
     if (p->d_dft16) cudaFree(p->d_dft16);
     delete p;
@@ -223,7 +234,7 @@ extern "C" fftk_status fftk_plan_destroy(fftk_plan p) {
   cudaDeviceSynchronize();
   ns_free(p);
   if (p->d_tw_alloc) cudaFree(p->d_tw_alloc);
-  if (p->d_tw3) cudaFree(p->d_tw3);
+  if (p->d_tw3_alloc) cudaFree(p->d_tw3_alloc);
   if (p->d_err) cudaFree(p->d_err);
   if (p->d_dft16) cudaFree(p->d_dft16);
   if (p->ws && p->ws_owned) cudaFree(p->ws);

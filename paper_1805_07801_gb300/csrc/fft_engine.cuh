@@ -1,16 +1,18 @@
 // Device-side 1D FFT engine shared by every pass kernel.
 //
-// A line of length L (power of two) is held by S = L/G threads, G complex
-// values per thread in the "natural" pattern v[m] = x[j + m*S] (j = thread
-// index within the line).  The transform is a sequence of self-sorting
-// (Stockham) radix-R stages, R = min(16, G, remaining length): every thread
-// runs G/R radix-R butterflies in registers, and consecutive stages exchange
-// data through a shared-memory buffer.  After the last stage the output is
+// A line of length L (a power of two, or three times one) is held by S = L/G
+// threads, G complex values per thread in the "natural" pattern
+// v[m] = x[j + m*S] (j = thread index within the line).  The transform is a
+// sequence of self-sorting (Stockham) radix-R stages (stage_radix): every
+// thread runs G/R radix-R butterflies in registers, and consecutive stages
+// exchange data through a shared-memory buffer.  Lines of 3 * 2^m points take
+// their factor 3 in the last stage, as a radix-3, 6, 12 or 24 butterfly, so
+// every stage before it spans a power of two.  After the last stage the output is
 // again in the natural pattern, so a pass can load and store global memory
 // directly from registers with the same coalesced pattern.
 //
 // This replaces the FFTW 1D line transforms used by FFTK (paper Sec. 3);
-// the radix-16/8/4/2 factorisation is fixed at compile time by Stage below.
+// the factorisation is fixed at compile time by Stage below.
 //
 // Sign convention: SIGN = -1 computes X[k] = sum_n x[n] exp(-2 pi i n k / L)
 // (forward), SIGN = +1 the unnormalised inverse.
@@ -112,6 +114,53 @@ __device__ __forceinline__ float2 mul_root32(float2 a, int q) {
   return (q & 16) ? make_float2(-r.x, -r.y) : r;
 }
 
+// cos and sin of pi/24, 2 pi/24 and 5 pi/24
+#define FFTK_C48A 0.99144486137381041114f
+#define FFTK_S48A 0.13052619222005159155f
+#define FFTK_C48B 0.96592582628906828675f
+#define FFTK_S48B 0.25881904510252076235f
+#define FFTK_C48E 0.79335334029123516458f
+#define FFTK_S48E 0.60876142900872063942f
+#define FFTK_C6 0.86602540378443864676f  // cos(pi/6) = sin(pi/3)
+
+// a * exp(-2 pi i m / NR) for m in [0, NR/2) known at compile time, NR a power
+// of two up to 32 (mul_root32), 12, 24 or 48 (the same split for lines of
+// 3 * 2^m values: steps of pi/24 by their constants, the quarter turn exactly)
+template <int NR>
+__device__ __forceinline__ float2 mul_root(float2 a, int m) {
+  if constexpr (NR % 3 != 0) {
+    return mul_root32(a, m * (32 / NR));
+  } else {
+    const int q = m * (48 / NR);
+    float2 r;
+    switch (q % 12) {
+      case 0: r = a; break;
+      case 1: r = rot<-1>(a, FFTK_C48A, FFTK_S48A); break;
+      case 2: r = rot<-1>(a, FFTK_C48B, FFTK_S48B); break;
+      case 3: r = rot<-1>(a, FFTK_C16, FFTK_S16); break;
+      case 4: r = rot<-1>(a, FFTK_C6, 0.5f); break;
+      case 5: r = rot<-1>(a, FFTK_C48E, FFTK_S48E); break;
+      case 6: r = rot<-1>(a, FFTK_C8, FFTK_C8); break;
+      case 7: r = rot<-1>(a, FFTK_S48E, FFTK_C48E); break;
+      case 8: r = rot<-1>(a, 0.5f, FFTK_C6); break;
+      case 9: r = rot<-1>(a, FFTK_S16, FFTK_C16); break;
+      case 10: r = rot<-1>(a, FFTK_S48B, FFTK_C48B); break;
+      default: r = rot<-1>(a, FFTK_S48A, FFTK_C48A); break;
+    }
+    return q >= 12 ? mul_si<-1>(r) : r;
+  }
+}
+
+// index of the mirror H - k of entry k of a packed line of H values (k = 0: itself)
+template <int H>
+__device__ __forceinline__ int mirror(int k) {
+  if constexpr ((H & (H - 1)) == 0) {
+    return (H - k) & (H - 1);
+  } else {
+    return k == 0 ? 0 : H - k;
+  }
+}
+
 // --------------------------------------------------------------- codelets --
 // In-place DFT of R values held in registers, natural order in and out.
 template <int SIGN>
@@ -177,9 +226,39 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
     for (int k2 = 0; k2 < 4; ++k2) x[k1 + 4 * k2] = t[4 * k1 + k2];
 }
 
+// X1,2 = a - (b + c)/2 +- SIGN i sin(pi/3) (b - c)
+template <int SIGN>
+__device__ __forceinline__ void dft3(float2& a, float2& b, float2& c) {
+  const float2 s = cadd(b, c), d = cscale(mul_si<SIGN>(csub(b, c)), FFTK_C6);
+  const float2 t = make_float2(fmaf(-0.5f, s.x, a.x), fmaf(-0.5f, s.y, a.y));
+  a = cadd(a, s);
+  b = cadd(t, d);
+  c = csub(t, d);
+}
+
 template <int R, int SIGN>
 __device__ __forceinline__ void dftR(float2 (&a)[R]) {
-  if constexpr (R == 2) {
+  if constexpr (R % 3 == 0) {
+    // R = 3 P, P = 1, 2, 4 or 8: 3 and P have no common factor, so the DFT is
+    // the two-dimensional 3 x P one without twiddles (Good's mapping):
+    // n = P n1 + 3 n2, k = k1 (mod 3) = k2 (mod P)
+    constexpr int P = R / 3;
+    constexpr int E1 = P == 1 ? 1 : (P == 8 ? 16 : 4), E2 = P == 1 ? 0 : (P == 2 ? 3 : 9);
+#pragma unroll
+    for (int n2 = 0; n2 < P; ++n2) dft3<SIGN>(a[3 * n2], a[(P + 3 * n2) % R], a[(2 * P + 3 * n2) % R]);
+    float2 o[R];
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) {
+      float2 t[P];
+#pragma unroll
+      for (int n2 = 0; n2 < P; ++n2) t[n2] = a[(P * k1 + 3 * n2) % R];
+      if constexpr (P > 1) dftR<P, SIGN>(t);
+#pragma unroll
+      for (int k2 = 0; k2 < P; ++k2) o[(E1 * k1 + E2 * k2) % R] = t[k2];
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) a[k] = o[k];
+  } else if constexpr (R == 2) {
     dft2<SIGN>(a[0], a[1]);
   } else if constexpr (R == 4) {
     dft4<SIGN>(a[0], a[1], a[2], a[3]);
@@ -271,29 +350,40 @@ __host__ __device__ constexpr int stage_tw_offset(int M, int R) {
   return 4 * M + (R == 2 ? 0 : (R == 4 ? 1 : (R == 8 ? 2 : 3))) * M;
 }
 
-template <int L, int G>
-struct Shape {
-  static_assert(L >= 1 && (L & (L - 1)) == 0, "L must be a power of two");
-  static constexpr int g = G;
-  static constexpr int S = L / G;  // threads per line
-};
+// The last stage of a line of M = 3 * 2^j points has radix R in {3, 6, 12, 24}.
+// The plan holds exp(-2 pi i m / M), m < M, for every M = 3 * 2^j up to its
+// longest such axis at offset M of one array, and below that array the r-major
+// tables of the pairs (M, R) for contiguous lines, laid out as above.
+constexpr int kStage3Twiddles = 24576;
+__host__ __device__ constexpr int stage3_tw_offset(int M, int R) {
+  return 4 * M + (R == 3 ? 0 : (R == 6 ? 1 : (R == 12 ? 2 : 3))) * M;
+}
 
 __host__ __device__ constexpr int fftk_min3(int a, int b, int c) {
   return a < b ? (a < c ? a : c) : (b < c ? b : c);
 }
 
+// Radix of the stage that takes up `rem` remaining points at g values per
+// thread: min(16, g, rem) for powers of two; while the factor 3 remains, all
+// of rem if one butterfly can hold it, else the largest power of two in g.
+__host__ __device__ constexpr int stage_radix(int rem, int g) {
+  if (rem % 3 != 0) return fftk_min3(16, g, rem);
+  if (rem <= g && g % rem == 0) return rem;
+  return fftk_min3(16, g & -g, rem / 3);
+}
+
 template <int L, int G, int SIGN, int NS, int TL>
 struct Stage {
   template <class X>
-  __device__ __forceinline__ static void run(float2 (&v)[G], int j, const X& xc,
-                                             const float2* __restrict__ tw) {
+  __device__ __forceinline__ static void run(float2 (&v)[G], int j, const X& xc, const float2* __restrict__ tw,
+                                             const float2* __restrict__ t3) {
     if constexpr (NS < L) {
       constexpr int REM = L / NS;
-      constexpr int R = fftk_min3(16, G, REM);
+      constexpr int R = stage_radix(REM, G);
       constexpr int B = G / R;   // butterflies per thread
       constexpr int S = L / G;   // threads per line
+      static_assert(B * R == G && REM % R == 0, "radix");
       constexpr bool LAST = (NS * R == L);
-      constexpr int LOG_NSR = Log2<NS * R>::value;
 #pragma unroll
       for (int t = 0; t < B; ++t) {
         const int b = j + t * S;   // butterfly index in [0, L/R)
@@ -301,10 +391,20 @@ struct Stage {
         float2 a[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) a[r] = v[t + r * B];
-        if constexpr (NS > 1) {
+        if constexpr (NS > 1 && R % 3 == 0) {
+          // exp(SIGN 2 pi i r k / L) of the last stage, L = NS R = 3 * 2^m
+          const float2* ts = t3 - kStage3Twiddles + stage3_tw_offset(L, R);
+          const float2* tg = t3 + L;
+#pragma unroll
+          for (int r = 1; r < R; ++r) {
+            const float2 w = X::kStageTables ? __ldg(&ts[r * NS + k]) : __ldg(&tg[r * k]);
+            a[r] = SIGN < 0 ? cmul(a[r], w) : cmulc(a[r], w);
+          }
+        } else if constexpr (NS > 1) {
           // exp(SIGN 2 pi i r k / (NS R)): from this stage's r-major table for
           // contiguous lines, else from the size-2^TL table (tw, at offset 2^TL
           // of the pyramid) at index r k 2^TL / (NS R)
+          constexpr int LOG_NSR = Log2<NS * R>::value;
           const float2* ts = tw - (1 << TL) - kStageTwiddles + stage_tw_offset(NS * R, R);
 #pragma unroll
           for (int r = 1; r < R; ++r) {
@@ -327,7 +427,7 @@ struct Stage {
 #pragma unroll
         for (int m = 0; m < G; ++m) v[m] = xc.ld(j + m * S);
         xc.sync();
-        Stage<L, G, SIGN, NS * R, TL>::run(v, j, xc, tw);
+        Stage<L, G, SIGN, NS * R, TL>::run(v, j, xc, tw, t3);
       }
     }
   }
@@ -335,15 +435,25 @@ struct Stage {
 
 // Full L-point transform of the line held in v (natural pattern in and out).
 // The exchange buffer must be free on entry; it is free again on exit.
-// tw: the twiddle table of size 2^TL (TL >= log2 L; by default the size-L one).
+// tw: the power-of-two twiddle table of size 2^TL (by default the largest one
+// not longer than L); t3: the plan's 3 * 2^m tables (such lines only).
 template <int L, int G, int SIGN, int TL = Log2<L>::value, class X>
-__device__ __forceinline__ void fft_line(float2 (&v)[G], int j, const X& xc, const float2* __restrict__ tw) {
-  static_assert((1 << TL) >= L, "twiddle table too short");
-  Stage<L, G, SIGN, 1, TL>::run(v, j, xc, tw);
+__device__ __forceinline__ void fft_line(float2 (&v)[G], int j, const X& xc, const float2* __restrict__ tw,
+                                         const float2* __restrict__ t3 = nullptr) {
+  static_assert((1 << TL) >= (L % 3 == 0 ? L / 3 : L), "twiddle table too short");
+  Stage<L, G, SIGN, 1, TL>::run(v, j, xc, tw, t3);
 }
 
-// Elements per thread used by the passes for a line of length L.
-__host__ __device__ constexpr int elems_per_thread(int L) { return L < 16 ? L : 16; }
+// Elements per thread used by the strided passes for a line of length L: 16,
+// and 24 (radices 8, 8, 12 at 768) for lines of 3 * 2^m points that are long
+// enough to spread over several threads.
+__host__ __device__ constexpr int elems_per_thread(int L) {
+  if (L % 3 == 0) return L >= 96 ? 24 : (L >= 12 ? 12 : L);
+  return L < 16 ? L : 16;
+}
+// slots of the exchange buffer of one contiguous line of H values (swz_line
+// permutes within blocks of 16)
+__host__ __device__ constexpr int line_slots(int H) { return H % 3 == 0 ? (H + 15) / 16 * 16 : H; }
 
 }  // inline namespace
 }  // namespace fftk

@@ -1,0 +1,672 @@
+// The fused passes of the Navier-Stokes right-hand side (ns.cu describes the
+// method), as templates on the grid size: instantiated for powers of two in
+// ns.cu and for 3 * 2^m in ns_radix3.cu.
+#pragma once
+
+#include "fft_engine.cuh"
+#include "internal.h"
+#include "ns_common.cuh"
+#include "tcgen05.cuh"
+
+namespace fftk {
+// ---------------------------------------------------- padded workspace ---
+// Row length of the fused passes' six-field workspace: n/2 + 1 rounded up to
+// a multiple of 16 complex values (272 at n = 512, 528 at n = 1024), so that
+// every (x, y) row starts on a 128-byte line and a tile of 16 (or 8) k_z
+// columns covers whole lines.  With rows of n/2 + 1 values each 128-byte row
+// segment straddles two lines: measured on the access patterns alone, the
+// inverse x pass's writes ran at 2.5 TB/s against 4.3 TB/s on lines, the y
+// passes' at 5.2 against 6.4 TB/s.  The caller's spectra keep n/2 + 1.
+__host__ __device__ constexpr long long ns_row(int n) { return ((long long)(n / 2 + 1) + 15) / 16 * 16; }
+
+// ------------------------------------------------------------ x/y config ---
+// Single-field passes (both y passes): the strided FFT pass configuration,
+// 16 k_z columns per tile (128-byte row segments); powers of two: 16 values
+// per thread, 32 warps per SM at <= 64 registers; 3 * 2^m: 24 values, 128
+// registers.
+template <int N>
+struct NXCfg {
+  static constexpr int G = elems_per_thread(N);
+  static constexpr int S = N / G;
+  static constexpr int T = S <= 16 ? 16 : (S <= 64 ? 16 : 1024 / S);
+  static constexpr int THREADS = T * S;
+  static constexpr int MINB = N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
+                                         : (THREADS <= 512 ? (THREADS <= 256 ? 4 : 2) : 1);
+  static constexpr size_t SMEM = sizeof(float2) * (size_t)N * T;
+};
+
+// 2./4. y pass, columns (x, k_z < kc), blockIdx -> (field, x, k_z tile).
+//    SIGN=+1: only kept k_y rows are read, every y row is written;
+//    SIGN=-1: every y row is read, only kept k_y rows are written.
+template <int N, int SIGN>
+__global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
+    k_ns_ypass(const float2* w, float2* wo, int ktiles, const float2* __restrict__ tw,
+               const float2* __restrict__ t3) {  // wo may be w
+  constexpr long long H1 = ns_row(N), MM = (long long)N * N * H1;  // the padded workspace
+  constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
+  using C = NXCfg<N>;
+  constexpr int G = C::G, S = C::S, T = C::T;
+  extern __shared__ float2 smn[];
+  const int c = threadIdx.x % T, j = threadIdx.x / T;
+  const int kt = blockIdx.x % ktiles;
+  const int rest = blockIdx.x / ktiles;
+  const int x = rest % N;
+  const int f = rest / N;
+  const int kz = kt * T + c;
+  const bool valid = kz < (KD + 1);
+  const long long off = f * MM + (long long)x * N * H1 + kz;
+  float2 v[G];
+#pragma unroll
+  for (int m = 0; m < G; ++m) {
+    const int pos = j + m * S;
+    const bool rd = valid && (SIGN < 0 || kept_xy(pos, N, KD));
+    v[m] = rd ? (SIGN < 0 ? wo[off + (long long)pos * H1] : __ldg(&w[off + (long long)pos * H1]))
+              : make_float2(0.f, 0.f);
+  }
+  fft_line<N, G, SIGN>(v, j, ColX<T>{smn, c}, tw, t3);
+  if (valid) {
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int pos = j + m * S;
+      if (SIGN > 0 || kept_xy(pos, N, KD)) wo[off + (long long)pos * H1] = v[m];
+    }
+  }
+}
+
+// Base shape of the x passes of powers of two: 8 values per thread.
+template <int N>
+struct NFCfg {
+  static constexpr int G = N < 8 ? N : 8;
+  static constexpr int S = N / G;
+  static constexpr int T = S >= 32 ? (S == 32 ? 16 : (S == 64 ? 8 : 4)) : 16;
+};
+
+// Inverse x pass.  Powers of two hold two fields at once, 16 values per thread
+// for n >= 512 with 16 columns per tile (128-byte row segments) at n = 512 and
+// 8 at n = 1024.  3 * 2^m lines (24 values per thread, 16 columns) hold one
+// and park the other in shared memory.
+template <int N>
+struct NICfg {
+  static constexpr bool PARK = N % 3 == 0;
+  static constexpr int G = PARK ? elems_per_thread(N) : (N >= 512 ? 16 : NFCfg<N>::G);
+  static constexpr int S = N / G;
+  static constexpr int T = PARK || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
+  static constexpr int THREADS = T * S;
+  static constexpr int MINB = PARK ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1)) : (THREADS <= 256 ? 2 : 1);
+  static constexpr size_t SMEM = sizeof(float2) * (size_t)N * T * (PARK ? 2 : 1);
+};
+
+// Forward x pass (one field in registers, two parked): 1024 threads, 8 values
+// per thread, 16 columns per tile at n = 512 and 8 at n = 1024; 3 * 2^m: 24
+// values per thread, 16 columns; there only the slots m whose rows j + m S can
+// be kept by the 2/3 rule are parked, the first LOW and those from HIGH on
+// (all slots would not fit beside the exchange buffer at n = 768).
+template <int N>
+struct NUCfg {
+  static constexpr int G = N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G;
+  static constexpr int S = N / G;
+  static constexpr int T = N % 3 == 0 || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
+  static constexpr int THREADS = T * S;
+  static constexpr int KD = (N - 1) / 3;
+  static constexpr int LOW = N % 3 != 0 ? G : KD / S + 1;
+  static constexpr int HIGH = (N - KD) / S > LOW ? (N - KD) / S : LOW;
+  static constexpr int SLOTS = LOW + G - HIGH;
+  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N * T + 2 * (size_t)SLOTS * THREADS);
+  static constexpr int MINB = N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
+                                         : (1024 / THREADS < 16 ? 1024 / THREADS : 16);  // 64 registers
+  __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
+  __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
+};
+
+// 1. inverse x pass with the curl.  Columns: kept (k_y, k_z); rows: k_x.
+//    U_c = F^-1_x(u_c), D_c = F^-1_x(i k_x u_c), then
+//    omega_x = i (k_y U_z - k_z U_y), omega_y = i k_z U_x - D_z,
+//    omega_z = D_y - i k_y U_x   (five transforms instead of six).
+//    Output field order: u_x, u_y, u_z, omega_x, omega_y, omega_z.
+template <int N>
+__global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
+    k_ns_invx(const float2* __restrict__ u, float2* __restrict__ w, int ktiles, const float2* __restrict__ tw,
+              const float2* __restrict__ t3) {
+  constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
+  constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace
+  constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
+  using C = NICfg<N>;
+  constexpr int G = C::G, S = C::S, T = C::T;
+  extern __shared__ float2 smn[];
+  const int c = threadIdx.x % T, j = threadIdx.x / T;
+  const int dky = blockIdx.x / ktiles;
+  const int ay = dense_to_a(dky, N, KD);
+  const int kz = (blockIdx.x - dky * ktiles) * T + c;
+  const bool valid = kz < (KD + 1);
+  const long long q = (long long)ay * H1 + kz;
+  const long long rs = (long long)N * H1;
+  const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
+  const float ky = (float)kwav(ay, N), kzf = (float)kz;
+  const ColX<T> xc{smn, c};
+  auto load = [&](int f, float2(&v)[G], bool ikx) {
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int pos = j + m * S;
+      float2 a = make_float2(0.f, 0.f);
+      if (valid && kept_xy(pos, N, KD)) a = u[f * MM + pos * rs + q];
+      v[m] = ikx ? mul_i(a, (float)kwav(pos, N)) : a;
+    }
+  };
+  auto store = [&](int f, const float2(&v)[G]) {
+    if (valid) {
+#pragma unroll
+      for (int m = 0; m < G; ++m) w[f * MW + (j + m * S) * rw + qw] = v[m];
+    }
+  };
+  if constexpr (C::PARK) {
+    float2* park = smn + (size_t)N * T + threadIdx.x;  // this thread's slots
+    float2 a[G];
+    load(0, a, false);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_x
+    store(0, a);
+#pragma unroll
+    for (int m = 0; m < G; ++m) park[m * C::THREADS] = a[m];
+    load(1, a, true);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_y
+#pragma unroll
+    for (int m = 0; m < G; ++m) a[m] = csub(a[m], mul_i(park[m * C::THREADS], ky));  // omega_z
+    store(5, a);
+    load(2, a, true);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_z
+#pragma unroll
+    for (int m = 0; m < G; ++m) a[m] = csub(mul_i(park[m * C::THREADS], kzf), a[m]);  // omega_y
+    store(4, a);
+    load(1, a, false);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_y
+    store(1, a);
+#pragma unroll
+    for (int m = 0; m < G; ++m) park[m * C::THREADS] = a[m];
+    load(2, a, false);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_z
+    store(2, a);
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const float2 y = park[m * C::THREADS];
+      a[m] = make_float2(-(ky * a[m].y - kzf * y.y), ky * a[m].x - kzf * y.x);  // omega_x
+    }
+    store(3, a);
+  } else {
+    float2 a[G], b[G];
+    load(1, a, true);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_y
+    load(0, b, false);
+    fft_line<N, G, +1>(b, j, xc, tw, t3);  // U_x
+    store(0, b);
+  #pragma unroll
+    for (int m = 0; m < G; ++m) a[m] = csub(a[m], mul_i(b[m], ky));  // omega_z
+    store(5, a);
+    load(2, a, true);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_z
+  #pragma unroll
+    for (int m = 0; m < G; ++m) a[m] = csub(mul_i(b[m], kzf), a[m]);  // omega_y
+    store(4, a);
+    load(1, a, false);
+    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_y
+    store(1, a);
+    load(2, b, false);
+    fft_line<N, G, +1>(b, j, xc, tw, t3);  // U_z
+    store(2, b);
+  #pragma unroll
+    for (int m = 0; m < G; ++m)
+      b[m] = make_float2(-(ky * b[m].y - kzf * a[m].y), ky * b[m].x - kzf * a[m].x);  // omega_x
+    store(3, b);
+  }
+}
+
+// ------------------------------------------------------------- z product ---
+// The z kernel holds a 256-point line (n = 512) as 16 values per thread on 16
+// threads, two lines per warp: each transform is two radix-16 stages with one
+// exchange through shared memory (8 values per thread would need three stages
+// and two exchanges, and the exchanges dominated the L1 traffic).  A thread
+// holds up to four such arrays (u x omega accumulators and a vorticity
+// component), 230 registers at n = 512: two CTAs of 128 threads per SM.
+// Measured and dropped: three CTAs per SM with one staging buffer (168
+// registers, 1.120 against 1.126 ms), CTAs of 64 or 32 threads with five or
+// ten per SM (spills; 1.20 ms), the velocity parked in TMEM (slower).
+template <int N>
+struct NZCfg {
+  static constexpr int H = N / 2;
+  static constexpr int HB = line_slots(H);        // exchange slots per line
+  static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (H < 16 ? H : 16);
+  static constexpr int S = H / G;
+  static constexpr int LPC = S >= 128 ? 1 : 128 / S;
+  static constexpr int NBUF = 2;                  // staging buffers per line
+  static constexpr int THREADS = LPC * S;
+  static constexpr bool WARP = S <= 32;
+  static constexpr int KC = (N - 1) / 3 + 1;      // kept k_z count (2/3 rule)
+  static constexpr int KCP = (KC + 2) & ~1;       // staged values per line and buffer (KC + alignment slack)
+  static constexpr size_t FIELDS = sizeof(float2) * (size_t)LPC * (HB + 3 * H);  // exchange + 3 parked fields
+  static constexpr size_t STAGE = sizeof(float2) * (size_t)LPC * NBUF * KCP;  // staging buffers
+  static constexpr size_t SMEM = FIELDS + STAGE + sizeof(uint64_t) * NBUF * LPC;  // + one mbarrier per buffer
+  static constexpr int MINB = G == 16 ? 2 : (G == 12 ? 3 : 4);  // CTAs per SM the registers must allow
+};
+
+// 3. per (x, y) line: the six c2r transforms, the product n = u x omega and
+//    the three r2c transforms.  Reads k_z < kc of fields 0..5 of w, writes
+//    k_z < kc of fields 0..2 of wo (wo may be w: a line is fully read before
+//    it is written).
+//    The three velocity components are parked in real space in shared memory;
+//    each vorticity component is then transformed and folded into the
+//    accumulators of n, so at most 4 fields are held in registers.
+//    A line's kept coefficients of each input field arrive by one bulk
+//    asynchronous copy into one of two staging buffers, issued two fields
+//    ahead of their use, so the global loads' latency overlaps the transforms
+//    of the field before; the c2r reads X[k] and its mirror X[H - k] from there.
+template <int N, int HW>  // HW: row length of the workspace (n/2 + 1, or the fused path's padded rows)
+__global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
+    k_ns_z(const float2* w, float2* wo, const float2* __restrict__ tw, const float2* __restrict__ t3, int* err) {
+  constexpr long long H1 = HW, MM = (long long)N * N * H1;  // geometry of the workspace
+  using C = NZCfg<N>;
+  constexpr int H = C::H, G = C::G, S = C::S;
+  constexpr int LOGN = Log2<N>::value;
+  constexpr int KC = C::KC;  // kept k_z count
+  extern __shared__ __align__(16) float2 smz[];
+  const int li = threadIdx.x / S, j = threadIdx.x % S;
+  const long long line = (long long)blockIdx.x * C::LPC + li;
+  const bool valid = line < (long long)N * N;
+  const LineX<C::WARP> xc{smz + li * C::HB};
+  float2* park = smz + C::LPC * C::HB + li * 3 * H + j;  // [3][G][S] per line, this thread's column
+  constexpr int NB = C::NBUF;
+  float2* stage = smz + C::FIELDS / sizeof(float2) + li * NB * C::KCP;  // this line's buffers
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smz + (C::FIELDS + C::STAGE) / sizeof(float2)) + NB * li;
+
+  // Field f's element k of this line sits at element f MM + line H1 + k.  MM
+  // is even; with H1 odd (rows of n/2 + 1) the line starts 16-byte aligned for
+  // even lines and 8 bytes past a 16-byte boundary for odd ones: the copy then
+  // starts `lead` elements early (the previous line's last value, k_z = n/2,
+  // which this kernel never writes) and ends at k_z <= kc, inside the line.
+  // With padded rows (H1 a multiple of 16) every line is aligned.
+  const int lead = (int)((line * H1) & 1);
+  const uint32_t bytes = (uint32_t)(sizeof(float2) * ((KC + lead + 1) & ~1));
+  auto issue = [&](int f) {  // one thread of the line; buffer f % NB was last read NB fields ago
+    uint64_t* b = bar + f % NB;
+    tcg::fence_smem_async();
+    tcg::mbar_expect(b, bytes);
+    tcg::bulk_g2s(stage + (f % NB) * C::KCP, w + f * MM + line * H1 - lead, bytes, b);
+  };
+  bool ok = true;
+  auto arrive = [&](int f) {  // wait for field f's copy (bounded; an expired wait is reported)
+    if (!valid) return;
+    const uint32_t par = (uint32_t)((f / NB) & 1);
+    if (!tcg::mbar_wait(bar + f % NB, par)) {
+      if (j == 0 && ok) atomicOr(err, 1);
+      ok = false;
+      tcg::mbar_wait(bar + f % NB, par);  // once more for the copy still in flight
+    }
+  };
+  if (j == 0 && valid) {
+    for (int b = 0; b < NB; ++b) tcg::mbar_init(bar + b);
+    for (int b = 0; b < NB; ++b) issue(b);
+  }
+  xc.sync();  // the barriers are initialised before anyone polls them
+  // exp(-2 pi i k / N) at k = j + m S is Wj exp(-2 pi i m / (2G)) (N = 2 G S):
+  // one table load per thread instead of one per value
+  // (measured against one table load per value at 16 values per thread:
+  // 1.126 against 1.190 ms per launch at 512^3)
+  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
+  auto twk = [&](int m) { return mul_root<2 * G>(Wj, m); };
+
+  // inverse z transform of field f (half-complex -> N real points, two per slot)
+  auto c2r = [&](int f, float2 (&U)[G]) {
+    const float2* src = stage + (f % NB) * C::KCP + lead;
+    arrive(f);
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int k = j + m * S;
+      float2 A = make_float2(0.f, 0.f), B = make_float2(0.f, 0.f);
+      if (k < KC) A = src[k];
+      if (H - k < KC) B = src[H - k];
+      if (k == 0) {
+        A.y = 0.f;
+        B.y = 0.f;
+      }
+      const float2 Bc = cconj(B);
+      const float2 E = cadd(A, Bc);
+      const float2 O = cmulc(csub(A, Bc), twk(m));
+      U[m] = make_float2(E.x - O.y, E.y + O.x);
+    }
+    if constexpr (S == 1) xc.sync();  // (one thread per line: the transform has no exchange)
+    fft_line<H, G, +1, LOGN>(U, j, xc, tw, t3);
+    // every thread of the line has passed an exchange barrier since it read
+    // the buffer: refill it with field f + NB
+    if (f + NB < 6 && j == 0 && valid) issue(f + NB);
+  };
+
+  {
+    float2 U[G];
+#pragma unroll 1
+    for (int f = 0; f < 3; ++f) {
+      c2r(f, U);
+#pragma unroll
+      for (int m = 0; m < G; ++m) park[(f * G + m) * S] = U[m];
+    }
+  }
+  // forward z transforms of n (N real points -> half-complex), k_z < kc written
+  auto r2c = [&](int f, float2 (&U)[G]) {
+    fft_line<H, G, -1, LOGN>(U, j, xc, tw, t3);
+#pragma unroll
+    for (int m = 0; m < G; ++m) xc.st(j + m * S, U[m]);
+    xc.sync();
+    float2* dst = wo + f * MM + line * H1;
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int k = j + m * S;
+      const float2 A = U[m];
+      const float2 Bc = cconj(xc.ld(mirror<H>(k)));
+      const float2 E = cscale(cadd(A, Bc), 0.5f);
+      const float2 D = csub(A, Bc);
+      const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);
+      if (valid && k < KC) dst[k] = cadd(E, cmul(twk(m), O));
+    }
+    xc.sync();
+  };
+  // n = u x omega at the two real points held by each slot (elementwise
+  // products of the (even, odd) point pairs, paired FP32 instructions):
+  //   n_x = u_y w_z - u_z w_y,  n_y = u_z w_x - u_x w_z,  n_z = u_x w_y - u_y w_x
+  // n_z is complete after omega_y and is transformed before omega_z is loaded.
+  auto neg = [](float2 a) { return make_float2(-a.x, -a.y); };
+  float2 Ny[G], Nx[G];
+  {
+    float2 Nz[G];
+    {
+      float2 W[G];
+      c2r(3, W);  // omega_x
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        const float2 uy = park[(1 * G + m) * S], uz = park[(2 * G + m) * S];
+        Ny[m] = __fmul2_rn(uz, W[m]);
+        Nz[m] = __fmul2_rn(neg(uy), W[m]);
+      }
+      c2r(4, W);  // omega_y
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        const float2 ux = park[(0 * G + m) * S], uz = park[(2 * G + m) * S];
+        Nx[m] = __fmul2_rn(neg(uz), W[m]);
+        Nz[m] = __ffma2_rn(ux, W[m], Nz[m]);
+      }
+    }
+    r2c(2, Nz);
+  }
+  {
+    float2 W[G];
+    c2r(5, W);  // omega_z
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const float2 ux = park[(0 * G + m) * S], uy = park[(1 * G + m) * S];
+      Nx[m] = __ffma2_rn(uy, W[m], Nx[m]);
+      Ny[m] = __ffma2_rn(neg(ux), W[m], Ny[m]);
+    }
+  }
+  r2c(0, Nx);
+  r2c(1, Ny);
+}
+
+// ----------------------------------------------------- x pass + update -----
+
+struct NSUpdate {
+  const float2* etab;  // exp(-nu k^2 dt) = hi + lo (two FP32 parts), indexed by integer k^2;
+                       // exp(-nu k^2 dt/2) follows at offset etab_len (the RK4 half steps)
+  int etab_len;
+  float2* acc;         // RK4 accumulator (3 fields)
+  const double* ef;    // forced-mode energy (device scalar)
+  double feps;         // injected power (0 = off)
+  int k2min, k2max;
+  float dt;
+  float scale;         // 1 / n^3
+};
+
+// One kept mode (k_x, k_y, k_z) at index idx of each field: N = P[n] (Eq. (8)),
+// + subgrid force, + forcing, then
+//   RHS:    out = N
+//   STAGE1: out = E (u0 + dt N)                      (out = u1)
+//   STAGE2: out = 1/2 E u0 + 1/2 (u1 + dt N)         (out = u0, in place)
+// or one stage of RK4 with H = exp(-nu k^2 dt/2), state u0, stage state u1,
+// accumulator A (N from the stage's input: u0 in RK4_1, u1 after):
+//   RK4_1:  A = E u0 + dt/6 E N,   out = H (u0 + dt/2 N)   (out = u1)
+//   RK4_2:  A += dt/3 H N,         out = H u0 + dt/2 N     (out = u1)
+//   RK4_3:  A += dt/3 H N,         out = E u0 + dt H N     (out = u1)
+//   RK4_4:  out = A + dt/6 N                                (out = u0)
+__device__ __forceinline__ void ns_mode_update(float2 nx, float2 ny, float2 nz, int kx, int ky, int kz,
+                                               long long idx, long long M, const NSUpdate& upd, int mode,
+                                               float gforce, const float2* u0, const float2* u1,
+                                               const float2* __restrict__ extra, float2* out) {
+  const int k2 = kx * kx + ky * ky + kz * kz;
+  if (k2 == 0) {
+    nx = ny = nz = make_float2(0.f, 0.f);
+  } else {
+    const float fkx = (float)kx, fky = (float)ky, fkz = (float)kz;
+    const float inv = 1.f / (float)k2;
+    const float2 kn = make_float2((fkx * nx.x + fky * ny.x + fkz * nz.x) * inv,
+                                  (fkx * nx.y + fky * ny.y + fkz * nz.y) * inv);
+    nx = csub(nx, cscale(kn, fkx));
+    ny = csub(ny, cscale(kn, fky));
+    nz = csub(nz, cscale(kn, fkz));
+  }
+  if (extra) {  // subgrid force, already dealiased and projected
+    nx = cadd(nx, extra[idx]);
+    ny = cadd(ny, extra[idx + M]);
+    nz = cadd(nz, extra[idx + 2 * M]);
+  }
+  const bool forced = gforce != 0.f && k2 >= upd.k2min && k2 <= upd.k2max;
+  const float2* ucur = (mode == NS_STAGE2 || mode >= NS_RK4_2) ? u1 : u0;
+  if (forced) {
+    nx = cadd(nx, cscale(ucur[idx], gforce));
+    ny = cadd(ny, cscale(ucur[idx + M], gforce));
+    nz = cadd(nz, cscale(ucur[idx + 2 * M], gforce));
+  }
+  if (mode == NS_RHS) {
+    out[idx] = nx;
+    out[idx + M] = ny;
+    out[idx + 2 * M] = nz;
+    return;
+  }
+  // E = hi + lo carries the factor to ~2^-48; v * E is formed as
+  // fma(v, hi, v * lo), one rounding, so repeated steps do not bias the decay.
+  const float2 E = __ldg(&upd.etab[k2]);
+  const float dt = upd.dt;
+  const float2 n3[3] = {nx, ny, nz};
+  if (mode >= NS_RK4_1) {
+    const float2 H = __ldg(&upd.etab[upd.etab_len + k2]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) {
+      const long long i = idx + f * M;
+      const float2 nv = n3[f];
+      if (mode == NS_RK4_4) {
+        const float2 a = upd.acc[i];
+        out[i] = make_float2(fmaf(dt / 6.f, nv.x, a.x), fmaf(dt / 6.f, nv.y, a.y));
+        continue;
+      }
+      const float2 a = u0[i];
+      const float2 ea = make_float2(fmaf(a.x, E.x, a.x * E.y), fmaf(a.y, E.x, a.y * E.y));  // E u0
+      const float2 ha = make_float2(fmaf(a.x, H.x, a.x * H.y), fmaf(a.y, H.x, a.y * H.y));  // H u0
+      const float2 hn = make_float2(fmaf(nv.x, H.x, nv.x * H.y), fmaf(nv.y, H.x, nv.y * H.y));  // H N
+      if (mode == NS_RK4_1) {
+        const float2 en = make_float2(fmaf(nv.x, E.x, nv.x * E.y), fmaf(nv.y, E.x, nv.y * E.y));
+        upd.acc[i] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
+        const float sx = a.x + 0.5f * dt * nv.x, sy = a.y + 0.5f * dt * nv.y;
+        out[i] = make_float2(fmaf(sx, H.x, sx * H.y), fmaf(sy, H.x, sy * H.y));
+      } else {
+        const float2 ac = upd.acc[i];
+        upd.acc[i] = make_float2(fmaf(dt / 3.f, hn.x, ac.x), fmaf(dt / 3.f, hn.y, ac.y));
+        out[i] = (mode == NS_RK4_2) ? make_float2(fmaf(0.5f * dt, nv.x, ha.x), fmaf(0.5f * dt, nv.y, ha.y))
+                                    : make_float2(fmaf(dt, hn.x, ea.x), fmaf(dt, hn.y, ea.y));
+      }
+    }
+    return;
+  }
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    const float2 a = u0[idx + f * M];
+    float2 r;
+    if (mode == NS_STAGE1) {
+      const float sx = a.x + dt * n3[f].x, sy = a.y + dt * n3[f].y;
+      r = make_float2(fmaf(sx, E.x, sx * E.y), fmaf(sy, E.x, sy * E.y));
+    } else {
+      const float2 b = u1[idx + f * M];
+      const float ex = fmaf(a.x, E.x, a.x * E.y), ey = fmaf(a.y, E.x, a.y * E.y);
+      r = make_float2(0.5f * (ex + (b.x + dt * n3[f].x)), 0.5f * (ey + (b.y + dt * n3[f].y)));
+    }
+    out[idx + f * M] = r;
+  }
+}
+
+// 5. forward x pass of the 3 nonlinear fields, then on every kept mode:
+//    N = P[n] (Eq. (8)), + forcing, and
+//    RHS:    out = N
+//    STAGE1: out = E (u0 + dt N)                      (out = u1)
+//    STAGE2: out = 1/2 E u0 + 1/2 (u1 + dt N)         (out = u0, in place)
+template <int N>
+__global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
+    k_ns_fwdx(const float2* __restrict__ nh, const float2* u0, const float2* u1, float2* out,
+              int ktiles, NSUpdate upd, int mode, const float2* __restrict__ extra, const float2* __restrict__ tw,
+              const float2* __restrict__ t3) {
+  constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
+  constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace (nh)
+  constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
+  using C = NUCfg<N>;
+  constexpr int G = C::G, S = C::S, T = C::T;
+  extern __shared__ float2 smn[];
+  const int c = threadIdx.x % T, j = threadIdx.x / T;
+  const int dky = blockIdx.x / ktiles;
+  const int ay = dense_to_a(dky, N, KD);
+  const int kz = (blockIdx.x - dky * ktiles) * T + c;
+  const bool valid = kz < (KD + 1);
+  const long long q = (long long)ay * H1 + kz;
+  const long long rs = (long long)N * H1;
+  const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
+  const ColX<T> xc{smn, c};
+  // fields 0 and 1 are parked in shared memory after their transforms (this
+  // thread's slots only), so one field at a time is held in registers
+  float2* park = smn + (size_t)N * T + threadIdx.x;
+  float2 V[G];
+#pragma unroll 1
+  for (int f = 0; f < 3; ++f) {
+#pragma unroll
+    for (int m = 0; m < G; ++m)
+      V[m] = valid ? nh[f * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
+    fft_line<N, G, -1>(V, j, xc, tw, t3);
+    if (f < 2) {
+#pragma unroll
+      for (int m = 0; m < G; ++m)
+        if (C::parked(m)) park[(f * C::SLOTS + C::slot(m)) * C::THREADS] = V[m];
+    }
+  }
+  if (!valid) return;
+  const int ky = kwav(ay, N);
+  float gforce = 0.f;
+  if (upd.feps > 0.0) {
+    const double ef = *upd.ef;
+    gforce = ef > 0.0 ? (float)(upd.feps / (2.0 * ef)) : 0.f;
+  }
+#pragma unroll
+  for (int m = 0; m < G; ++m) {
+    const int pos = j + m * S;
+    if (!C::parked(m) || !kept_xy(pos, N, KD)) continue;
+    ns_mode_update(cscale(park[C::slot(m) * C::THREADS], upd.scale),
+                   cscale(park[(C::SLOTS + C::slot(m)) * C::THREADS], upd.scale), cscale(V[m], upd.scale), kwav(pos, N), ky, kz, pos * rs + q, MM, upd, mode, gforce, u0, u1,
+                   extra, out);
+  }
+}
+
+// One right-hand side and update on a cube of 3 * 2^m points (ns_radix3.cu).
+cudaError_t ns_rhs_radix3(fftk_plan p, const float2* u, const float2* u0, const float2* u1, float2* out,
+                          const NSUpdate& upd, int mode, const float2* extra, cudaStream_t st);
+
+// --------------------------------------------------------------- launchers --
+template <int N>
+struct NSLaunch {
+  static cudaError_t attrs() {
+    static PerDevice once;
+    return once.run([](int) {
+      const int sx = (int)NXCfg<N>::SMEM;
+      cudaError_t err = cudaFuncSetAttribute(k_ns_invx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)NICfg<N>::SMEM);
+      if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(k_ns_ypass<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
+      if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(k_ns_ypass<N, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
+      if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(k_ns_fwdx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)NUCfg<N>::SMEM);
+      if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(k_ns_z<N, (int)ns_row(N)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)NZCfg<N>::SMEM);
+      if constexpr (N % 3 != 0)
+        if (err == cudaSuccess)
+          err = cudaFuncSetAttribute(k_ns_z<N, N / 2 + 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)NZCfg<N>::SMEM);
+      return err;
+    });
+  }
+
+  // The fused z pass alone (c2r of the six fields in s->w, u x omega, r2c of
+  // n into fields 0..2), for the split-precision right-hand side.
+  static cudaError_t z(fftk_plan p, cudaStream_t st) {
+    using Z = NZCfg<N>;
+    cudaError_t e = attrs();
+    if (e != cudaSuccess) return e;
+    NSWork* s = p->ns;
+    LaunchScope ls(p, KK_NS_Z, st);
+    const long long lines = (long long)N * N;
+    k_ns_z<N, N / 2 + 1><<<(unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st>>>(
+        s->w, s->w, twiddles(p, N), nullptr, p->d_err);
+    return cudaGetLastError();
+  }
+
+  // One evaluation of N(u) followed by the update selected by `mode`.
+  static cudaError_t rhs(fftk_plan p, const float2* u, const float2* u0, const float2* u1,
+                         float2* out, const NSUpdate& upd, int mode, const float2* extra,
+                         cudaStream_t st) {
+    using X = NXCfg<N>;
+    using Z = NZCfg<N>;
+    cudaError_t e = attrs();
+    if (e != cudaSuccess) return e;
+    NSWork* s = p->ns;
+    const NSGeom g = s->g;
+    const int kx = (g.kc + X::T - 1) / X::T;
+    using I = NICfg<N>;
+    const int ki = (g.kc + I::T - 1) / I::T;
+    using U = NUCfg<N>;
+    const int ku = (g.kc + U::T - 1) / U::T;
+    // invx u -> A, inverse y A -> B, z B -> A (fields 0..2), forward y A -> A,
+    // forward x A -> out.  The inverse y pass out of place measured 0.684 ->
+    // 0.647 ms at 512^3; the forward y pass, which writes only the kept rows,
+    // measured slower out of place (0.313 -> 0.331 ms), so it stays in place.
+    e = ns_second_workspace(p);
+    if (e != cudaSuccess) return e;
+    float2* A = s->w;
+    float2* Bw = s->w2;
+    const float2* tw = twiddles(p, 1 << Log2<N>::value);
+    const float2* t3 = p->d_tw3;
+    {
+      LaunchScope ls(p, KK_NS_INVX, st);
+      k_ns_invx<N><<<g.nk * ki, I::THREADS, I::SMEM, st>>>(u, A, ki, tw, t3);
+    }
+    {
+      LaunchScope ls(p, KK_NS_INVY, st);
+      k_ns_ypass<N, 1><<<6 * N * kx, X::THREADS, X::SMEM, st>>>(A, Bw, kx, tw, t3);
+    }
+    {
+      LaunchScope ls(p, KK_NS_Z, st);
+      const long long lines = (long long)N * N;
+      k_ns_z<N, (int)ns_row(N)><<<(unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st>>>(
+          Bw, A, tw, t3, p->d_err);
+    }
+    {
+      LaunchScope ls(p, KK_NS_FWDY, st);
+      k_ns_ypass<N, -1><<<3 * N * kx, X::THREADS, X::SMEM, st>>>(A, A, kx, tw, t3);
+    }
+    {
+      LaunchScope ls(p, KK_NS_FWDX, st);
+      k_ns_fwdx<N><<<g.nk * ku, U::THREADS, U::SMEM, st>>>(A, u0, u1, out, ku, upd, mode, extra, tw, t3);
+    }
+    return cudaGetLastError();
+  }
+};
+
+}  // namespace fftk
