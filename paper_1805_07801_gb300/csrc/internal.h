@@ -82,9 +82,6 @@ struct fftk_plan_s {
 
 namespace fftk {
 
-// The table of size L = 3 * 2^m (a dimension of the plan or a divisor of one).
-inline const float2* twiddles3(const fftk_plan_s* p, int L) { return p->d_tw3 + L; }
-
 // The plan's twiddle table of size L (a power of two <= 4 LT): exp(-2 pi i m / L), m < L.
 // Tables beyond LT serve the quarter-wave factors of the sine/cosine passes.
 inline const float2* twiddles(const fftk_plan_s* p, int L) { return p->d_tw + L; }
