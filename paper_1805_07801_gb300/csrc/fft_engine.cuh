@@ -329,6 +329,9 @@ struct LineX {
   }
 };
 
+// brings the line of p (a valid global address) into L2
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // ---------------------------------------------------------------- engine ---
 // Twiddle tables: the plan holds, for every power of two L' <= 4 LT, the
 // table exp(-2 pi i m / L'), m < L', at offset L' of one array (entries

@@ -188,7 +188,10 @@ __global__ void k_update_full(const float2* __restrict__ nh, const float2* u0, c
     const long long ab = it / g.kc;
     const int a = dense_to_a((int)(ab / g.nk), g.n, g.kd), b = dense_to_a((int)(ab % g.nk), g.n, g.kd);
     const long long idx = ((long long)a * g.n + b) * g.h1 + c;
-    ns_mode_update(nh[idx], nh[idx + g.M], nh[idx + 2 * g.M], kwav(a, g.n), kwav(b, g.n), c, idx, g.M, upd, mode,
+    const int kx = kwav(a, g.n), ky = kwav(b, g.n);
+    NSModeIn in;
+    ns_mode_load(in, kx * kx + ky * ky + c * c, idx, g.M, upd, mode, u0, u1);
+    ns_mode_update(in, nh[idx], nh[idx + g.M], nh[idx + 2 * g.M], kwav(a, g.n), kwav(b, g.n), c, idx, g.M, upd, mode,
                    gforce, u0, u1, extra, out);
   }
 }

@@ -6,19 +6,10 @@
 #include "fft_engine.cuh"
 #include "internal.h"
 #include "ns_common.cuh"
+#include "ns_update.cuh"
 #include "tcgen05.cuh"
 
 namespace fftk {
-// ---------------------------------------------------- padded workspace ---
-// Row length of the fused passes' six-field workspace: n/2 + 1 rounded up to
-// a multiple of 16 complex values (272 at n = 512, 528 at n = 1024), so that
-// every (x, y) row starts on a 128-byte line and a tile of 16 (or 8) k_z
-// columns covers whole lines.  With rows of n/2 + 1 values each 128-byte row
-// segment straddles two lines: measured on the access patterns alone, the
-// inverse x pass's writes ran at 2.5 TB/s against 4.3 TB/s on lines, the y
-// passes' at 5.2 against 6.4 TB/s.  The caller's spectra keep n/2 + 1.
-__host__ __device__ constexpr long long ns_row(int n) { return ((long long)(n / 2 + 1) + 15) / 16 * 16; }
-
 // ------------------------------------------------------------ x/y config ---
 // Single-field passes (both y passes): the strided FFT pass configuration,
 // 16 k_z columns per tile (128-byte row segments); powers of two: 16 values
@@ -73,14 +64,6 @@ __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
   }
 }
 
-// Base shape of the x passes of powers of two: 8 values per thread.
-template <int N>
-struct NFCfg {
-  static constexpr int G = N < 8 ? N : 8;
-  static constexpr int S = N / G;
-  static constexpr int T = S >= 32 ? (S == 32 ? 16 : (S == 64 ? 8 : 4)) : 16;
-};
-
 // Inverse x pass.  Powers of two hold two fields at once, 16 values per thread
 // for n >= 512 with 16 columns per tile (128-byte row segments) at n = 512 and
 // 8 at n = 1024.  3 * 2^m lines (24 values per thread, 16 columns) hold one
@@ -94,28 +77,6 @@ struct NICfg {
   static constexpr int THREADS = T * S;
   static constexpr int MINB = PARK ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1)) : (THREADS <= 256 ? 2 : 1);
   static constexpr size_t SMEM = sizeof(float2) * (size_t)N * T * (PARK ? 2 : 1);
-};
-
-// Forward x pass (one field in registers, two parked): 1024 threads, 8 values
-// per thread, 16 columns per tile at n = 512 and 8 at n = 1024; 3 * 2^m: 24
-// values per thread, 16 columns; there only the slots m whose rows j + m S can
-// be kept by the 2/3 rule are parked, the first LOW and those from HIGH on
-// (all slots would not fit beside the exchange buffer at n = 768).
-template <int N>
-struct NUCfg {
-  static constexpr int G = N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G;
-  static constexpr int S = N / G;
-  static constexpr int T = N % 3 == 0 || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
-  static constexpr int THREADS = T * S;
-  static constexpr int KD = (N - 1) / 3;
-  static constexpr int LOW = N % 3 != 0 ? G : KD / S + 1;
-  static constexpr int HIGH = (N - KD) / S > LOW ? (N - KD) / S : LOW;
-  static constexpr int SLOTS = LOW + G - HIGH;
-  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N * T + 2 * (size_t)SLOTS * THREADS);
-  static constexpr int MINB = N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
-                                         : (1024 / THREADS < 16 ? 1024 / THREADS : 16);  // 64 registers
-  __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
-  __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };
 
 // 1. inverse x pass with the curl.  Columns: kept (k_y, k_z); rows: k_x.
@@ -225,6 +186,7 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
 // and two exchanges, and the exchanges dominated the L1 traffic).  A thread
 // holds up to four such arrays (u x omega accumulators and a vorticity
 // component), 230 registers at n = 512: two CTAs of 128 threads per SM.
+// 3 * 2^m lines: 12 values (radices 4, 4, 4, 6 at n = 768), 32 threads a line.
 // Measured and dropped: three CTAs per SM with one staging buffer (168
 // registers, 1.120 against 1.126 ms), CTAs of 64 or 32 threads with five or
 // ten per SM (spills; 1.20 ms), the velocity parked in TMEM (slower).
@@ -232,7 +194,7 @@ template <int N>
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-  static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (H < 16 ? H : 16);
+    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (H < 16 ? H : 16);
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
   static constexpr int NBUF = 2;                  // staging buffers per line
@@ -406,173 +368,6 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
   r2c(1, Ny);
 }
 
-// ----------------------------------------------------- x pass + update -----
-
-struct NSUpdate {
-  const float2* etab;  // exp(-nu k^2 dt) = hi + lo (two FP32 parts), indexed by integer k^2;
-                       // exp(-nu k^2 dt/2) follows at offset etab_len (the RK4 half steps)
-  int etab_len;
-  float2* acc;         // RK4 accumulator (3 fields)
-  const double* ef;    // forced-mode energy (device scalar)
-  double feps;         // injected power (0 = off)
-  int k2min, k2max;
-  float dt;
-  float scale;         // 1 / n^3
-};
-
-// One kept mode (k_x, k_y, k_z) at index idx of each field: N = P[n] (Eq. (8)),
-// + subgrid force, + forcing, then
-//   RHS:    out = N
-//   STAGE1: out = E (u0 + dt N)                      (out = u1)
-//   STAGE2: out = 1/2 E u0 + 1/2 (u1 + dt N)         (out = u0, in place)
-// or one stage of RK4 with H = exp(-nu k^2 dt/2), state u0, stage state u1,
-// accumulator A (N from the stage's input: u0 in RK4_1, u1 after):
-//   RK4_1:  A = E u0 + dt/6 E N,   out = H (u0 + dt/2 N)   (out = u1)
-//   RK4_2:  A += dt/3 H N,         out = H u0 + dt/2 N     (out = u1)
-//   RK4_3:  A += dt/3 H N,         out = E u0 + dt H N     (out = u1)
-//   RK4_4:  out = A + dt/6 N                                (out = u0)
-__device__ __forceinline__ void ns_mode_update(float2 nx, float2 ny, float2 nz, int kx, int ky, int kz,
-                                               long long idx, long long M, const NSUpdate& upd, int mode,
-                                               float gforce, const float2* u0, const float2* u1,
-                                               const float2* __restrict__ extra, float2* out) {
-  const int k2 = kx * kx + ky * ky + kz * kz;
-  if (k2 == 0) {
-    nx = ny = nz = make_float2(0.f, 0.f);
-  } else {
-    const float fkx = (float)kx, fky = (float)ky, fkz = (float)kz;
-    const float inv = 1.f / (float)k2;
-    const float2 kn = make_float2((fkx * nx.x + fky * ny.x + fkz * nz.x) * inv,
-                                  (fkx * nx.y + fky * ny.y + fkz * nz.y) * inv);
-    nx = csub(nx, cscale(kn, fkx));
-    ny = csub(ny, cscale(kn, fky));
-    nz = csub(nz, cscale(kn, fkz));
-  }
-  if (extra) {  // subgrid force, already dealiased and projected
-    nx = cadd(nx, extra[idx]);
-    ny = cadd(ny, extra[idx + M]);
-    nz = cadd(nz, extra[idx + 2 * M]);
-  }
-  const bool forced = gforce != 0.f && k2 >= upd.k2min && k2 <= upd.k2max;
-  const float2* ucur = (mode == NS_STAGE2 || mode >= NS_RK4_2) ? u1 : u0;
-  if (forced) {
-    nx = cadd(nx, cscale(ucur[idx], gforce));
-    ny = cadd(ny, cscale(ucur[idx + M], gforce));
-    nz = cadd(nz, cscale(ucur[idx + 2 * M], gforce));
-  }
-  if (mode == NS_RHS) {
-    out[idx] = nx;
-    out[idx + M] = ny;
-    out[idx + 2 * M] = nz;
-    return;
-  }
-  // E = hi + lo carries the factor to ~2^-48; v * E is formed as
-  // fma(v, hi, v * lo), one rounding, so repeated steps do not bias the decay.
-  const float2 E = __ldg(&upd.etab[k2]);
-  const float dt = upd.dt;
-  const float2 n3[3] = {nx, ny, nz};
-  if (mode >= NS_RK4_1) {
-    const float2 H = __ldg(&upd.etab[upd.etab_len + k2]);
-#pragma unroll
-    for (int f = 0; f < 3; ++f) {
-      const long long i = idx + f * M;
-      const float2 nv = n3[f];
-      if (mode == NS_RK4_4) {
-        const float2 a = upd.acc[i];
-        out[i] = make_float2(fmaf(dt / 6.f, nv.x, a.x), fmaf(dt / 6.f, nv.y, a.y));
-        continue;
-      }
-      const float2 a = u0[i];
-      const float2 ea = make_float2(fmaf(a.x, E.x, a.x * E.y), fmaf(a.y, E.x, a.y * E.y));  // E u0
-      const float2 ha = make_float2(fmaf(a.x, H.x, a.x * H.y), fmaf(a.y, H.x, a.y * H.y));  // H u0
-      const float2 hn = make_float2(fmaf(nv.x, H.x, nv.x * H.y), fmaf(nv.y, H.x, nv.y * H.y));  // H N
-      if (mode == NS_RK4_1) {
-        const float2 en = make_float2(fmaf(nv.x, E.x, nv.x * E.y), fmaf(nv.y, E.x, nv.y * E.y));
-        upd.acc[i] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
-        const float sx = a.x + 0.5f * dt * nv.x, sy = a.y + 0.5f * dt * nv.y;
-        out[i] = make_float2(fmaf(sx, H.x, sx * H.y), fmaf(sy, H.x, sy * H.y));
-      } else {
-        const float2 ac = upd.acc[i];
-        upd.acc[i] = make_float2(fmaf(dt / 3.f, hn.x, ac.x), fmaf(dt / 3.f, hn.y, ac.y));
-        out[i] = (mode == NS_RK4_2) ? make_float2(fmaf(0.5f * dt, nv.x, ha.x), fmaf(0.5f * dt, nv.y, ha.y))
-                                    : make_float2(fmaf(dt, hn.x, ea.x), fmaf(dt, hn.y, ea.y));
-      }
-    }
-    return;
-  }
-#pragma unroll
-  for (int f = 0; f < 3; ++f) {
-    const float2 a = u0[idx + f * M];
-    float2 r;
-    if (mode == NS_STAGE1) {
-      const float sx = a.x + dt * n3[f].x, sy = a.y + dt * n3[f].y;
-      r = make_float2(fmaf(sx, E.x, sx * E.y), fmaf(sy, E.x, sy * E.y));
-    } else {
-      const float2 b = u1[idx + f * M];
-      const float ex = fmaf(a.x, E.x, a.x * E.y), ey = fmaf(a.y, E.x, a.y * E.y);
-      r = make_float2(0.5f * (ex + (b.x + dt * n3[f].x)), 0.5f * (ey + (b.y + dt * n3[f].y)));
-    }
-    out[idx + f * M] = r;
-  }
-}
-
-// 5. forward x pass of the 3 nonlinear fields, then on every kept mode:
-//    N = P[n] (Eq. (8)), + forcing, and
-//    RHS:    out = N
-//    STAGE1: out = E (u0 + dt N)                      (out = u1)
-//    STAGE2: out = 1/2 E u0 + 1/2 (u1 + dt N)         (out = u0, in place)
-template <int N>
-__global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
-    k_ns_fwdx(const float2* __restrict__ nh, const float2* u0, const float2* u1, float2* out,
-              int ktiles, NSUpdate upd, int mode, const float2* __restrict__ extra, const float2* __restrict__ tw,
-              const float2* __restrict__ t3) {
-  constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
-  constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace (nh)
-  constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
-  using C = NUCfg<N>;
-  constexpr int G = C::G, S = C::S, T = C::T;
-  extern __shared__ float2 smn[];
-  const int c = threadIdx.x % T, j = threadIdx.x / T;
-  const int dky = blockIdx.x / ktiles;
-  const int ay = dense_to_a(dky, N, KD);
-  const int kz = (blockIdx.x - dky * ktiles) * T + c;
-  const bool valid = kz < (KD + 1);
-  const long long q = (long long)ay * H1 + kz;
-  const long long rs = (long long)N * H1;
-  const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
-  const ColX<T> xc{smn, c};
-  // fields 0 and 1 are parked in shared memory after their transforms (this
-  // thread's slots only), so one field at a time is held in registers
-  float2* park = smn + (size_t)N * T + threadIdx.x;
-  float2 V[G];
-#pragma unroll 1
-  for (int f = 0; f < 3; ++f) {
-#pragma unroll
-    for (int m = 0; m < G; ++m)
-      V[m] = valid ? nh[f * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
-    fft_line<N, G, -1>(V, j, xc, tw, t3);
-    if (f < 2) {
-#pragma unroll
-      for (int m = 0; m < G; ++m)
-        if (C::parked(m)) park[(f * C::SLOTS + C::slot(m)) * C::THREADS] = V[m];
-    }
-  }
-  if (!valid) return;
-  const int ky = kwav(ay, N);
-  float gforce = 0.f;
-  if (upd.feps > 0.0) {
-    const double ef = *upd.ef;
-    gforce = ef > 0.0 ? (float)(upd.feps / (2.0 * ef)) : 0.f;
-  }
-#pragma unroll
-  for (int m = 0; m < G; ++m) {
-    const int pos = j + m * S;
-    if (!C::parked(m) || !kept_xy(pos, N, KD)) continue;
-    ns_mode_update(cscale(park[C::slot(m) * C::THREADS], upd.scale),
-                   cscale(park[(C::SLOTS + C::slot(m)) * C::THREADS], upd.scale), cscale(V[m], upd.scale), kwav(pos, N), ky, kz, pos * rs + q, MM, upd, mode, gforce, u0, u1,
-                   extra, out);
-  }
-}
-
 // One right-hand side and update on a cube of 3 * 2^m points (ns_radix3.cu).
 cudaError_t ns_rhs_radix3(fftk_plan p, const float2* u, const float2* u0, const float2* u1, float2* out,
                           const NSUpdate& upd, int mode, const float2* extra, cudaStream_t st);
@@ -590,9 +385,6 @@ struct NSLaunch {
         err = cudaFuncSetAttribute(k_ns_ypass<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
       if (err == cudaSuccess)
         err = cudaFuncSetAttribute(k_ns_ypass<N, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
-      if (err == cudaSuccess)
-        err = cudaFuncSetAttribute(k_ns_fwdx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)NUCfg<N>::SMEM);
       if (err == cudaSuccess)
         err = cudaFuncSetAttribute(k_ns_z<N, (int)ns_row(N)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)NZCfg<N>::SMEM);
@@ -631,8 +423,6 @@ struct NSLaunch {
     const int kx = (g.kc + X::T - 1) / X::T;
     using I = NICfg<N>;
     const int ki = (g.kc + I::T - 1) / I::T;
-    using U = NUCfg<N>;
-    const int ku = (g.kc + U::T - 1) / U::T;
     // invx u -> A, inverse y A -> B, z B -> A (fields 0..2), forward y A -> A,
     // forward x A -> out.  The inverse y pass out of place measured 0.684 ->
     // 0.647 ms at 512^3; the forward y pass, which writes only the kept rows,
@@ -661,11 +451,8 @@ struct NSLaunch {
       LaunchScope ls(p, KK_NS_FWDY, st);
       k_ns_ypass<N, -1><<<3 * N * kx, X::THREADS, X::SMEM, st>>>(A, A, kx, tw, t3);
     }
-    {
-      LaunchScope ls(p, KK_NS_FWDX, st);
-      k_ns_fwdx<N><<<g.nk * ku, U::THREADS, U::SMEM, st>>>(A, u0, u1, out, ku, upd, mode, extra, tw, t3);
-    }
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    return e == cudaSuccess ? ns_fwdx(p, A, u0, u1, out, upd, mode, extra, st) : e;
   }
 };
 
