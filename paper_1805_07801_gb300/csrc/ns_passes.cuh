@@ -186,6 +186,9 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
 // and two exchanges, and the exchanges dominated the L1 traffic).  A thread
 // holds up to four such arrays (u x omega accumulators and a vorticity
 // component), 230 registers at n = 512: two CTAs of 128 threads per SM.
+// Small grids have few lines: below n = 256 a line goes to more threads with
+// fewer values (8 at 128, 4 below), which fills the chip (per RK2 step, 16
+// values -> these: 64^3 101 -> 62 us, 32^3 82 -> 53 us, 128^3 180 -> 139 us).
 // 3 * 2^m lines: 12 values (radices 4, 4, 4, 6 at n = 768), 32 threads a line.
 // Measured and dropped: three CTAs per SM with one staging buffer (168
 // registers, 1.120 against 1.126 ms), CTAs of 64 or 32 threads with five or
@@ -194,7 +197,7 @@ template <int N>
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (H < 16 ? H : 16);
+    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (N >= 256 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
   static constexpr int NBUF = 2;                  // staging buffers per line
