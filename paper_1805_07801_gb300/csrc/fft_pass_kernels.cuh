@@ -19,12 +19,12 @@ namespace fftk {
 // least eight threads share a line of 16 or more (64-byte pieces, more threads
 // for small grids); 24 or 12 for 3 * 2^m.  Pairs with 16 values -> these:
 // 64^3 35.6 -> 24.6 us, 64 fields of 64^3 308 -> 217 us, 8 of 256 x 256 x 128
-// 818 -> 670 us, 16 of 256^3 2508 -> 2406 us, 16 of 512 x 512 x 32 2369 -> 1709 us; H = 256 is
+// 818 -> 683 us, 16 of 256^3 2508 -> 2406 us, 16 of 512 x 512 x 32 2369 -> 1709 us; H = 256 is
 // slower with 8 (two 512^3 fields 2277 against 2190 us).
 __host__ __device__ constexpr int z_elems(int H) {
   if (H % 3 == 0) return H >= 192 ? 24 : (H >= 48 ? 12 : 6);
   if (H <= 16) return H < 2 ? H : 2;
-  return H <= 32 ? 4 : (H <= 128 ? 8 : 16);
+  return H <= 64 ? 4 : (H <= 128 ? 8 : 16);
 }
 
 template <int N>
