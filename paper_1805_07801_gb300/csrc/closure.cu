@@ -318,35 +318,65 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 //   P = 34459425 + 4729725 y + 135135 y^2 + 990 y^3 + y^4,
 //   Q = 34459425 + 16216200 y + 945945 y^2 + 13860 y^3 + 45 y^4
 // (both divided by 34459425 below); relative error below 3e-7 in FP32 for
-// |x| < 3.5.  For |x| >= 3.5 the BF16 rounding of tanh x is exactly +-1.
-__device__ __forceinline__ float tanh_to_bf16(float x) {
-  const float y = x * x;
-  const float p = fmaf(fmaf(fmaf(fmaf(1.f / 34459425.f, y, 2.f / 69615.f), y, 1.f / 255.f), y, 7.f / 51.f), y, 1.f);
-  const float q = fmaf(fmaf(fmaf(fmaf(1.f / 765765.f, y, 4.f / 9945.f), y, 7.f / 255.f), y, 8.f / 17.f), y, 1.f);
-  return fabsf(x) >= 3.5f ? copysignf(1.f, x) : x * __fdividef(p, q);
+// |x| < 3.5.  From 3.5 on the BF16 rounding of tanh x is exactly +-1 and so is
+// that of the value at 3.5 (0.99818): x is clamped there (a NaN stays one).
+// Two values at a time: the polynomials take one paired multiply-add for both.
+__device__ __forceinline__ float clamp35(float x) {
+  float r;
+  asm("{\n.reg .f32 t;\nmin.NaN.f32 t, %1, 0f40600000;\nmax.NaN.f32 %0, t, 0fC0600000;\n}" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float2 tanh_to_bf16(float2 v) {
+  const float2 x = make_float2(clamp35(v.x), clamp35(v.y));
+  const float2 y = __fmul2_rn(x, x);
+  auto c = [](float k) { return make_float2(k, k); };
+  float2 p = __ffma2_rn(c(1.f / 34459425.f), y, c(2.f / 69615.f));
+  float2 q = __ffma2_rn(c(1.f / 765765.f), y, c(4.f / 9945.f));
+  p = __ffma2_rn(p, y, c(1.f / 255.f));
+  q = __ffma2_rn(q, y, c(7.f / 255.f));
+  p = __ffma2_rn(p, y, c(7.f / 51.f));
+  q = __ffma2_rn(q, y, c(8.f / 17.f));
+  p = __ffma2_rn(p, y, c(1.f));
+  q = __ffma2_rn(q, y, c(1.f));
+  return make_float2(x.x * __fdividef(p.x, q.x), x.y * __fdividef(p.y, q.y));
 }
 
-__device__ __forceinline__ void store_split(unsigned char* hi, unsigned char* lo, int off, float w) {
-  const __nv_bfloat16 h = __float2bfloat16_rn(w);
-  const __nv_bfloat16 l = __float2bfloat16_rn(w - __bfloat162float(h));
-  *reinterpret_cast<__nv_bfloat16*>(hi + off) = h;
-  *reinterpret_cast<__nv_bfloat16*>(lo + off) = l;
+// eight consecutive inputs of one output's weights as BF16 hi and lo parts
+__device__ __forceinline__ void store_split8(unsigned char* hi, unsigned char* lo, int off, const float (&w)[8]) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    h[i] = pack_bf16(w[2 * i], w[2 * i + 1]);
+    l[i] = pack_bf16(w[2 * i] - __uint_as_float(h[i] << 16), w[2 * i + 1] - __uint_as_float(h[i] & 0xffff0000u));
+  }
+  *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// weights as BF16 hi/lo B operands and biases, from the FP32 parameters
+// weights as BF16 hi/lo B operands and biases, from the FP32 parameters (any
+// 4-byte aligned address): a thread takes eight inputs at a time, whose parts
+// are one 16-byte store each
 __device__ void load_weights(unsigned char* base, const float* __restrict__ params) {
-  for (int e = threadIdx.x; e < 64 * 16; e += blockDim.x) {
-    const int o = e >> 4, i = e & 15;
-    store_split(base + oW1, base + oW1 + kW1, tcg::kmajor_off<16>(o, i), i < 5 ? params[o * 5 + i] : 0.f);
+  float w[8];
+  for (int e = threadIdx.x; e < 64 * 2; e += blockDim.x) {
+    const int o = e >> 1, i = 8 * (e & 1);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = i + k < 5 ? params[o * 5 + i + k] : 0.f;
+    store_split8(base + oW1, base + oW1 + kW1, tcg::kmajor_off<16>(o, i), w);
   }
-  for (int e = threadIdx.x; e < 64 * 64; e += blockDim.x) {
-    const int off = tcg::kmajor_off<64>(e >> 6, e & 63);
-    store_split(base + oW2, base + oW2 + kW2, off, params[384 + e]);
-    store_split(base + oW3, base + oW3 + kW2, off, params[4544 + e]);
+  for (int e = threadIdx.x; e < 2 * 64 * 8; e += blockDim.x) {
+    const int m = e >> 9, o = (e >> 3) & 63, i = 8 * (e & 7);
+    const float* src = params + (m ? 4544 : 384) + o * 64 + i;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = src[k];
+    unsigned char* dst = base + (m ? oW3 : oW2);
+    store_split8(dst, dst + kW2, tcg::kmajor_off<64>(o, i), w);
   }
-  for (int e = threadIdx.x; e < 16 * 64; e += blockDim.x) {
-    const int o = e >> 6, i = e & 63;
-    store_split(base + oW4, base + oW4 + kW4, tcg::kmajor_off<64>(o, i), o < 6 ? params[8704 + o * 64 + i] : 0.f);
+  for (int e = threadIdx.x; e < 16 * 8; e += blockDim.x) {
+    const int o = e >> 3, i = 8 * (e & 7);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w[k] = o < 6 ? params[8704 + o * 64 + i + k] : 0.f;
+    store_split8(base + oW4, base + oW4 + kW4, tcg::kmajor_off<64>(o, i), w);
   }
   float* bias = reinterpret_cast<float*>(base + oBias);
   for (int e = threadIdx.x; e < 198; e += blockDim.x)
@@ -418,8 +448,9 @@ __device__ bool forward(unsigned char* base, uint32_t tmem, uint64_t* bar, uint3
         uint32_t pk[16];
 #pragma unroll
         for (int j = 0; j < 32; j += 2) {
-          const float* bl = bias + 64 * l + 32 * hh + j;
-          pk[j / 2] = pack_bf16(tanh_to_bf16(d[j] + bl[0]), tanh_to_bf16(d[j + 1] + bl[1]));
+          const float2 bl = *reinterpret_cast<const float2*>(bias + 64 * l + 32 * hh + j);
+          const float2 th = tanh_to_bf16(__fadd2_rn(make_float2(d[j], d[j + 1]), bl));
+          pk[j / 2] = pack_bf16(th.x, th.y);
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
