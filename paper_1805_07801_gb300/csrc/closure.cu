@@ -292,15 +292,14 @@ struct SGSConst {
 namespace mlptc {
 constexpr int kThreads = 256;
 constexpr int kBlocks = 2;
+constexpr int kPerSm = 3;  // CTAs per SM (shared memory, 80 registers); 128^3 step with the model: 1445 us with 2, 1371 with 3
 constexpr int kW1 = 64 * 16 * 2;  // bytes of one BF16 part of W1 as B [64 x 16]
 constexpr int kW2 = 64 * 64 * 2;  // W2, W3 as B [64 x 64]
 constexpr int kW4 = 16 * 64 * 2;  // W4 as B [16 x 64]
-constexpr int kX = 128 * 16 * 2;  // one block of inputs as A [128 x 16]
 constexpr int kH = 128 * 64 * 2;  // one block of a hidden layer as A [128 x 64]
 constexpr int oW1 = 0, oW2 = oW1 + 2 * kW1, oW3 = oW2 + 2 * kW2, oW4 = oW3 + 2 * kW2;
 constexpr int oBias = oW4 + 2 * kW4;  // b1, b2, b3 (64 each), b4 (6): FP32
-constexpr int oX = oBias + 1024;
-constexpr int oH = oX + kBlocks * kX;
+constexpr int oH = oBias + 1024;  // a block's inputs x lie where its hidden layers come afterwards
 constexpr int oBar = oH + kBlocks * kH;
 constexpr int kSmem = 1024 + oBar + 64;
 constexpr int kCols = 128;  // TMEM: 64 FP32 columns per block
@@ -386,7 +385,7 @@ __device__ void load_weights(unsigned char* base, const float* __restrict__ para
 
 // the network input of thread t's point (row t & 127 of block t >> 7), rounded to BF16
 __device__ __forceinline__ void write_x(unsigned char* base, int t, const float x[5]) {
-  unsigned char* X = base + oX + (t >> 7) * kX;
+  unsigned char* X = base + oH + (t >> 7) * kH;
   const int r = t & 127;
   *reinterpret_cast<uint4*>(X + tcg::kmajor_off<16>(r, 0)) =
       make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], 0.f), 0u);
@@ -412,7 +411,7 @@ __device__ bool forward(unsigned char* base, uint32_t tmem, uint64_t* bar, uint3
       for (int b = 0; b < kBlocks; ++b) {
         const uint32_t d = tmem + 64u * b;
         if (l == 0) {
-          const uint32_t a = sb + oX + b * kX;
+          const uint32_t a = sb + oH + b * kH;
           tcg::mma_f16(d, tcg::desc(a, 128, 256), tcg::desc(sb + oW1, 128, 256), kIdN64, 0);
           tcg::mma_f16(d, tcg::desc(a, 128, 256), tcg::desc(sb + oW1 + kW1, 128, 256), kIdN64, 1);
         } else {
@@ -501,7 +500,7 @@ __device__ __forceinline__ void finish(unsigned char* base, uint32_t tmem, uint3
 // Fused SGS inference with the network on the tensor cores: per point the
 // gradient A -> invariants and strain eigenframe -> normalised input -> MLP
 // -> tau' -> tau = Q tau' Q^T.  Writes tau[6][n^3].
-__global__ void __launch_bounds__(mlptc::kThreads, 2)
+__global__ void __launch_bounds__(mlptc::kThreads, mlptc::kPerSm)
     k_sgs_pointwise_tc(const float* __restrict__ A9, long long R, const float* __restrict__ params, SGSConst cst,
                        float* __restrict__ tau6, int* err) {
   extern __shared__ __align__(1024) unsigned char smraw_tc[];
@@ -548,7 +547,7 @@ __global__ void __launch_bounds__(mlptc::kThreads, 2)
 }
 
 // Plain inference y[B][6] = MLP(x[B][5]) with the network on the tensor cores.
-__global__ void __launch_bounds__(mlptc::kThreads, 2)
+__global__ void __launch_bounds__(mlptc::kThreads, mlptc::kPerSm)
     k_mlp_forward_tc(const float* __restrict__ params, const float* __restrict__ x, float* __restrict__ y,
                      long long B, int* err) {
   extern __shared__ __align__(1024) unsigned char smraw_tc[];
@@ -630,13 +629,13 @@ static cudaError_t mlp_attrs() {
   });
 }
 
-// persistent grid of the tensor-core inference kernels: two CTAs per SM
+// persistent grid of the tensor-core inference kernels
 static int mlptc_grid(long long points) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const long long need = (points + mlptc::kThreads - 1) / mlptc::kThreads;
-  const long long cap = 2LL * sms;
+  const long long cap = (long long)mlptc::kPerSm * sms;
   return (int)(need < cap ? need : cap);
 }
 
