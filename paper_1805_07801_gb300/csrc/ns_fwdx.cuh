@@ -14,8 +14,8 @@ namespace fftk {
 // fields fill the shared memory) loads, transforms and updates in turn.
 // 512^3, RK2: 648 us per launch with the update's loads one mode at a time,
 // 567 us with the loads of two modes in flight (the mode a template argument,
-// so that they fit into 64 registers), 546 us with the L2 prefetch below;
-// 64^3: 12.6 -> 8.3 us.
+// so that they fit into 64 registers), 484 us with the L2 prefetches below
+// (546 us with all of them at the start); 64^3: 12.6 -> 8.3 us.
 //
 // Forward x pass (one field in registers, two parked): 1024 threads, 8 values
 // per thread, 16 columns per tile at n = 512 and 8 at n = 1024; 3 * 2^m: 24
@@ -68,32 +68,29 @@ __global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
   // fields 0 and 1 are parked in shared memory after their transforms (this
   // thread's slots only), so one field at a time is held in registers
   float2* park = smn + (size_t)N * T + threadIdx.x;
-  if constexpr (N >= 256) {
-    // What the update and the fields 1 and 2 will read goes to L2 while field 0
-    // is loaded and transformed: one CTA holds the SM, so nothing else covers
-    // those loads (512^3: 567 -> 546 us per launch).
-    constexpr bool A0 = MODE != NS_RHS && MODE != NS_RK4_4, B0 = MODE == NS_STAGE2 || MODE >= NS_RK4_2;
-    const float2* b = MODE == NS_STAGE2 ? u1 : upd.acc;
-    for (int r = threadIdx.x; r < 2 * KD + 1; r += C::THREADS) {
-      const long long o = dense_to_a(r, N, KD) * rs + q - c;
-#pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        if (A0) prefetch_l2(u0 + f * MM + o);
-        if (B0) prefetch_l2(b + f * MM + o);
-      }
-    }
-    for (int r = threadIdx.x; r < N; r += C::THREADS) {
-      const long long o = r * rw + qw - c;
-      prefetch_l2(nh + MW + o);
-      prefetch_l2(nh + 2 * MW + o);
-    }
-  }
+  const float2* bsrc = MODE == NS_STAGE2 ? u1 : upd.acc;
+  constexpr bool A0 = MODE != NS_RHS && MODE != NS_RK4_4, B0 = MODE == NS_STAGE2 || MODE >= NS_RK4_2;
   float2 V[G];
 #pragma unroll 1
   for (int f = 0; f < 3; ++f) {
 #pragma unroll
     for (int m = 0; m < G; ++m)
       V[m] = valid ? nh[f * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
+    if constexpr (N >= 256) {
+      // The next field, and with the last two the update's reads, go to L2
+      // while this field is transformed: one CTA holds the SM, so nothing else
+      // covers those loads.  (All at once at the start would fill the L2.)
+      if (f < 2)
+        for (int r = threadIdx.x; r < N; r += C::THREADS) prefetch_l2(nh + (f + 1) * MW + r * rw + qw - c);
+      if ((A0 && f == 1) || (B0 && f == 2)) {
+        const float2* src = f == 1 ? u0 : bsrc;
+        for (int r = threadIdx.x; r < 2 * KD + 1; r += C::THREADS) {
+          const long long o = dense_to_a(r, N, KD) * rs + q - c;
+#pragma unroll
+          for (int i = 0; i < 3; ++i) prefetch_l2(src + i * MM + o);
+        }
+      }
+    }
     fft_line<N, G, -1>(V, j, xc, tw, t3);
     if (f < 2) {
 #pragma unroll

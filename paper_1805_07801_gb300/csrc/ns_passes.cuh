@@ -54,6 +54,21 @@ __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
     v[m] = rd ? (SIGN < 0 ? wo[off + (long long)pos * H1] : __ldg(&w[off + (long long)pos * H1]))
               : make_float2(0.f, 0.f);
   }
+  constexpr int AHEAD = N >= 768 ? 152 : (N == 512 && SIGN > 0 ? 304 : 0);  // tiles
+  if constexpr (AHEAD > 0) {
+    // One CTA holds the SM: while it transforms, the rows of the tile that
+    // comes next on some SM (CTAs start in order) go to L2.  768^3, per launch:
+    // inverse 3.06 -> 2.43 ms, forward 1.52 -> 1.16 ms.  512^3 (two CTAs per
+    // SM): inverse in place (convection) 795 -> 747 us, out of place 646 -> 641;
+    // the forward pass, 310 against 315 us, does without.
+    const long long nb = (long long)blockIdx.x + AHEAD;
+    if (nb < gridDim.x) {
+      const long long nr = nb / ktiles;  // f N + x of that tile
+      const float2* src = (SIGN < 0 ? wo : w) + (nr / N) * MM + (nr % N) * N * H1 + (nb - nr * ktiles) * T;
+      for (int r = threadIdx.x; r < (SIGN < 0 ? N : 2 * KD + 1); r += C::THREADS)
+        prefetch_l2(src + (long long)(SIGN < 0 ? r : dense_to_a(r, N, KD)) * H1);
+    }
+  }
   fft_line<N, G, SIGN>(v, j, ColX<T>{smn, c}, tw, t3);
   if (valid) {
 #pragma unroll
@@ -84,7 +99,8 @@ struct NICfg {
 //    omega_x = i (k_y U_z - k_z U_y), omega_y = i k_z U_x - D_z,
 //    omega_z = D_y - i k_y U_x   (five transforms instead of six).
 //    Output field order: u_x, u_y, u_z, omega_x, omega_y, omega_z.
-template <int N>
+//    THETA (convection): field 3 of u, the temperature, goes to field 6 of w.
+template <int N, bool THETA = false>
 __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     k_ns_invx(const float2* __restrict__ u, float2* __restrict__ w, int ktiles, const float2* __restrict__ tw,
               const float2* __restrict__ t3) {
@@ -151,6 +167,11 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
       a[m] = make_float2(-(ky * a[m].y - kzf * y.y), ky * a[m].x - kzf * y.x);  // omega_x
     }
     store(3, a);
+    if constexpr (THETA) {
+      load(3, a, false);
+      fft_line<N, G, +1>(a, j, xc, tw, t3);
+      store(6, a);
+    }
   } else {
     float2 a[G], b[G];
     load(1, a, true);
@@ -176,6 +197,11 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     for (int m = 0; m < G; ++m)
       b[m] = make_float2(-(ky * b[m].y - kzf * a[m].y), ky * b[m].x - kzf * a[m].x);  // omega_x
     store(3, b);
+    if constexpr (THETA) {
+      load(3, a, false);
+      fft_line<N, G, +1>(a, j, xc, tw, t3);
+      store(6, a);
+    }
   }
 }
 
@@ -186,9 +212,10 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
 // and two exchanges, and the exchanges dominated the L1 traffic).  A thread
 // holds up to four such arrays (u x omega accumulators and a vorticity
 // component), 230 registers at n = 512: two CTAs of 128 threads per SM.
-// Small grids have few lines: below n = 256 a line goes to more threads with
-// fewer values (8 at 128, 4 below), which fills the chip (per RK2 step, 16
-// values -> these: 64^3 101 -> 62 us, 32^3 82 -> 53 us, 128^3 180 -> 139 us).
+// Small grids have few lines: below n = 512 a line goes to more threads with
+// fewer values (8 at 128 and 256, 4 below), which fills the chip (per RK2 step,
+// 16 values -> these: 32^3 82 -> 53 us, 64^3 101 -> 62 us, 128^3 180 -> 139 us,
+// 256^3 929 -> 843 us).
 // 3 * 2^m lines: 12 values (radices 4, 4, 4, 6 at n = 768), 32 threads a line.
 // Measured and dropped: three CTAs per SM with one staging buffer (168
 // registers, 1.120 against 1.126 ms), CTAs of 64 or 32 threads with five or
@@ -197,7 +224,7 @@ template <int N>
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (N >= 256 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
+    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
   static constexpr int NBUF = 2;                  // staging buffers per line
@@ -208,7 +235,7 @@ struct NZCfg {
   static constexpr size_t FIELDS = sizeof(float2) * (size_t)LPC * (HB + 3 * H);  // exchange + 3 parked fields
   static constexpr size_t STAGE = sizeof(float2) * (size_t)LPC * NBUF * KCP;  // staging buffers
   static constexpr size_t SMEM = FIELDS + STAGE + sizeof(uint64_t) * NBUF * LPC;  // + one mbarrier per buffer
-  static constexpr int MINB = G == 16 ? 2 : (G == 12 ? 3 : 4);  // CTAs per SM the registers must allow
+  static constexpr int MINB = G == 16 ? 2 : (G == 12 || N == 256 ? 3 : 4);  // CTAs per SM the registers must allow
 };
 
 // 3. per (x, y) line: the six c2r transforms, the product n = u x omega and

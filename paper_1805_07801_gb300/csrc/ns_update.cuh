@@ -6,16 +6,6 @@
 #include "ns_common.cuh"
 
 namespace fftk {
-// ---------------------------------------------------- padded workspace ---
-// Row length of the fused passes' six-field workspace: n/2 + 1 rounded up to
-// a multiple of 16 complex values (272 at n = 512, 528 at n = 1024), so that
-// every (x, y) row starts on a 128-byte line and a tile of 16 (or 8) k_z
-// columns covers whole lines.  With rows of n/2 + 1 values each 128-byte row
-// segment straddles two lines: measured on the access patterns alone, the
-// inverse x pass's writes ran at 2.5 TB/s against 4.3 TB/s on lines, the y
-// passes' at 5.2 against 6.4 TB/s.  The caller's spectra keep n/2 + 1.
-__host__ __device__ constexpr long long ns_row(int n) { return ((long long)(n / 2 + 1) + 15) / 16 * 16; }
-
 // Base shape of the x passes of powers of two: 8 values per thread.
 template <int N>
 struct NFCfg {
