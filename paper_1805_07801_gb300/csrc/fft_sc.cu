@@ -22,6 +22,7 @@
 
 #include "fft_engine.cuh"
 #include "internal.h"
+#include "ns_common.cuh"
 
 namespace fftk {
 
@@ -129,14 +130,14 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
 // (L = n along x): columns are the kept (k_y, k_z) only (k_y rows 0..kd and
 // n-kd..n-1, k_z < kd + 1), the inverse reads only coefficient rows with
 // 3 k_x < 2n (sine row s is k_x = s + 1, cosine row s is k_x = s) and the
-// forward writes only those; B batch elements of [n][n][n/2+1].
+// forward writes only those; B batch elements of [n][n][ns_row(n)].
 template <int L, bool SINE, int DIR>
 __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
     k_scpass_pr(const float2* in, float2* out, int ktiles, const float2* __restrict__ tw,
                 const float2* __restrict__ tq, float scale) {
   using C = SCfg<L>;
   constexpr int G = C::G, S = C::S, T = C::T;
-  constexpr long long H1 = L / 2 + 1, M = (long long)L * L * H1, Q = (long long)L * H1;
+  constexpr long long H1 = ns_row(L), M = (long long)L * L * H1, Q = (long long)L * H1;
   constexpr int KD = (L - 1) / 3, KC = KD + 1, NK = 2 * KD + 1;
   extern __shared__ float2 smc[];
   const int c = threadIdx.x % T, j = threadIdx.x / T;

@@ -1,0 +1,450 @@
+// The fused passes of the convection right-hand side (rbc.cu describes the
+// method), as templates on the grid size: instantiated for powers of two in
+// rbc_pow2.cu and for 3 * 2^m in rbc_radix3.cu.  The workspace has the fused
+// Navier-Stokes passes' padded rows (ns_row).
+#pragma once
+
+#include <mutex>
+
+#include "ns_passes.cuh"
+
+namespace fftk {
+
+struct RBCUpdate {
+  const float2* tab;  // E_nu, E_kappa, H_nu, H_kappa at offsets 0, L, 2L, 3L
+  int tab_len;
+  float dt;
+};
+
+__device__ __forceinline__ float2 mul_pair(float2 v, float2 E) {  // v * (hi + lo), one rounding
+  return make_float2(fmaf(v.x, E.x, v.x * E.y), fmaf(v.y, E.x, v.y * E.y));
+}
+
+// the update of entry i of one field in mode MODE (the modes of
+// ns_mode_update): N = n, a = u0, b = the stage state or the accumulator
+template <int MODE>
+__device__ __forceinline__ void rbc_entry_store(long long i, float2 n, float2 a, float2 b, float2 E, float2 H, float dt,
+                                                float2* acc, float2* out) {
+  if constexpr (MODE == NS_RHS) {
+    out[i] = n;
+  } else if constexpr (MODE == NS_STAGE1) {
+    out[i] = mul_pair(make_float2(a.x + dt * n.x, a.y + dt * n.y), E);
+  } else if constexpr (MODE == NS_STAGE2) {
+    const float2 ea = mul_pair(a, E);
+    out[i] = make_float2(0.5f * (ea.x + (b.x + dt * n.x)), 0.5f * (ea.y + (b.y + dt * n.y)));
+  } else if constexpr (MODE == NS_RK4_4) {
+    out[i] = make_float2(fmaf(dt / 6.f, n.x, b.x), fmaf(dt / 6.f, n.y, b.y));
+  } else if constexpr (MODE == NS_RK4_1) {
+    const float2 ea = mul_pair(a, E), en = mul_pair(n, E);
+    acc[i] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
+    out[i] = mul_pair(make_float2(a.x + 0.5f * dt * n.x, a.y + 0.5f * dt * n.y), H);
+  } else {
+    const float2 hn = mul_pair(n, H);
+    acc[i] = make_float2(fmaf(dt / 3.f, hn.x, b.x), fmaf(dt / 3.f, hn.y, b.y));
+    if constexpr (MODE == NS_RK4_2) {
+      const float2 ha = mul_pair(a, H);
+      out[i] = make_float2(fmaf(0.5f * dt, n.x, ha.x), fmaf(0.5f * dt, n.y, ha.y));
+    } else {
+      const float2 ea = mul_pair(a, E);
+      out[i] = make_float2(fmaf(dt, hn.x, ea.x), fmaf(dt, hn.y, ea.y));
+    }
+  }
+}
+
+// Slots of the workspace: in[7] = u_x, u_y, u_z, omega_x, omega_y, omega_z,
+// theta; out[6] = n_x, n_y, n_z, u_x theta, u_y theta, u_z theta.
+struct RBCSlots {
+  int in[7];
+  int out[6];
+};
+
+// What the launchers of one stage need besides the plan.
+struct RBCStage {
+  float2* w;          // 7 fields, padded rows
+  const float2* x;    // the stage's input state
+  const float2* u0;   // the step's state
+  const float2* s1;   // stage state
+  float2* acc;        // RK4 accumulator
+  float2* out;
+  RBCUpdate upd;
+  int mode;
+  float scale;        // 1 / n^3
+};
+
+// y passes (sign +1: 7 fields, -1: 6) and the fused z pass on the padded workspace
+cudaError_t rbc_y(fftk_plan p, float2* w, int sign, cudaStream_t st);
+cudaError_t rbc_y3(fftk_plan p, float2* w, int sign, cudaStream_t st);
+cudaError_t rbc_z(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
+cudaError_t rbc_z3(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
+// periodic cube: the inverse x pass with the curl (state -> 7 fields), and the
+// forward x pass with the update (6 fields -> out)
+cudaError_t rbc_invx(fftk_plan p, const float2* x, float2* w, cudaStream_t st);
+cudaError_t rbc_invx3(fftk_plan p, const float2* x, float2* w, cudaStream_t st);
+cudaError_t rbc_fwdx(fftk_plan p, const RBCStage& s, cudaStream_t st);
+cudaError_t rbc_fwdx3(fftk_plan p, const RBCStage& s, cudaStream_t st);
+
+// ---- fused z pass (both bases: z is Fourier in each) ----------------------
+// Per (x, y) line: c2r of u, theta (parked in shared memory) and of the three
+// vorticity components (folded into the accumulators of n = u x omega), then
+// r2c of n and of u theta: thirteen transforms, in place (a slot is written
+// after it has been read).  Like the Navier-Stokes z pass it is bound by its
+// instructions; it shares that pass's shape (NZCfg): few long-radix stages,
+// the inputs staged by bulk copies two fields ahead, Hermitian-split factors
+// from one table load per thread.  512^3: 2031 us per launch with 8 values per
+// thread and plain loads, 1679 us so; 256^3: 265 and 225 us.
+template <int N>
+struct RZCfg {
+  using Z = NZCfg<N>;
+  static constexpr int H = Z::H, HB = Z::HB, G = Z::G, S = Z::S, LPC = Z::LPC, NBUF = Z::NBUF, THREADS = Z::THREADS;
+  static constexpr bool WARP = Z::WARP;
+  static constexpr int KC = Z::KC, KCP = Z::KCP;
+  static constexpr size_t FIELDS = sizeof(float2) * (size_t)LPC * (HB + 4 * H);  // exchange + 4 parked fields
+  static constexpr size_t STAGE = Z::STAGE;
+  static constexpr size_t SMEM = FIELDS + STAGE + sizeof(uint64_t) * NBUF * LPC;
+  static constexpr int MINB = G == 12 ? 2 : (N == 256 ? 4 : Z::MINB);
+};
+
+template <int N>
+__global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
+    k_rbc_z(float2* w, RBCSlots sl, const float2* __restrict__ tw, const float2* __restrict__ t3, int* err) {
+  constexpr long long HW = ns_row(N), MM = (long long)N * N * HW;
+  using C = RZCfg<N>;
+  constexpr int H = C::H, G = C::G, S = C::S, KC = C::KC, NB = C::NBUF;
+  constexpr int LOGN = Log2<N>::value;
+  extern __shared__ __align__(16) float2 smz[];
+  const int li = threadIdx.x / S, j = threadIdx.x % S;
+  const long long line = (long long)blockIdx.x * C::LPC + li;
+  const bool valid = line < (long long)N * N;
+  const LineX<C::WARP> xc{smz + li * C::HB};
+  float2* park = smz + C::LPC * C::HB + li * 4 * H + j;  // [4][G][S]: u_x, u_y, u_z, theta
+  float2* stage = smz + C::FIELDS / sizeof(float2) + li * NB * C::KCP;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smz + (C::FIELDS + C::STAGE) / sizeof(float2)) + NB * li;
+
+  // the inputs in the order of their use: u, theta, omega; a line's rows start
+  // on 128-byte lines, a copy is KC values rounded up to even
+  constexpr uint32_t bytes = (uint32_t)(sizeof(float2) * ((KC + 1) & ~1));
+  auto issue = [&](int f) {  // one thread of the line; buffer f % NB was last read NB fields ago
+    const int slot = sl.in[f < 3 ? f : (f == 3 ? 6 : f - 1)];
+    uint64_t* b = bar + f % NB;
+    tcg::fence_smem_async();
+    tcg::mbar_expect(b, bytes);
+    tcg::bulk_g2s(stage + (f % NB) * C::KCP, w + slot * MM + line * HW, bytes, b);
+  };
+  bool ok = true;
+  auto arrive = [&](int f) {  // wait for input f's copy (bounded; an expired wait is reported)
+    if (!valid) return;
+    const uint32_t par = (uint32_t)((f / NB) & 1);
+    if (!tcg::mbar_wait(bar + f % NB, par)) {
+      if (j == 0 && ok) atomicOr(err, 1);
+      ok = false;
+      tcg::mbar_wait(bar + f % NB, par);  // once more for the copy still in flight
+    }
+  };
+  if (j == 0 && valid) {
+    for (int b = 0; b < NB; ++b) tcg::mbar_init(bar + b);
+    for (int b = 0; b < NB; ++b) issue(b);
+  }
+  xc.sync();  // the barriers are initialised before anyone polls them
+  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
+  auto twk = [&](int m) { return mul_root<2 * G>(Wj, m); };
+
+  auto c2r = [&](int f, float2(&U)[G]) {
+    const float2* src = stage + (f % NB) * C::KCP;
+    arrive(f);
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int k = j + m * S;
+      float2 A = make_float2(0.f, 0.f), B = make_float2(0.f, 0.f);
+      if (k < KC) A = src[k];
+      if (H - k < KC) B = src[H - k];
+      if (k == 0) {
+        A.y = 0.f;
+        B.y = 0.f;
+      }
+      const float2 Bc = cconj(B);
+      const float2 E = cadd(A, Bc);
+      const float2 O = cmulc(csub(A, Bc), twk(m));
+      U[m] = make_float2(E.x - O.y, E.y + O.x);
+    }
+    if constexpr (S == 1) xc.sync();  // (one thread per line: the transform has no exchange)
+    fft_line<H, G, +1, LOGN>(U, j, xc, tw, t3);
+    if (f + NB < 7 && j == 0 && valid) issue(f + NB);
+  };
+  auto r2c = [&](int slot, float2(&U)[G]) {
+    fft_line<H, G, -1, LOGN>(U, j, xc, tw, t3);
+#pragma unroll
+    for (int m = 0; m < G; ++m) xc.st(j + m * S, U[m]);
+    xc.sync();
+    float2* dst = w + slot * MM + line * HW;
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int k = j + m * S;
+      const float2 Bc = cconj(xc.ld(mirror<H>(k)));
+      const float2 E = cscale(cadd(U[m], Bc), 0.5f);
+      const float2 D = csub(U[m], Bc);
+      const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);
+      if (valid && k < KC) dst[k] = cadd(E, cmul(twk(m), O));
+    }
+    xc.sync();
+  };
+  auto pk = [&](int f, int m) -> float2& { return park[(f * G + m) * S]; };
+  auto neg = [](float2 a) { return make_float2(-a.x, -a.y); };
+  {
+    float2 U[G];
+#pragma unroll 1
+    for (int f = 0; f < 4; ++f) {
+      c2r(f, U);
+#pragma unroll
+      for (int m = 0; m < G; ++m) pk(f, m) = U[m];
+    }
+  }
+  // n = u x omega, two real points per slot (see k_ns_z)
+  float2 Ny[G], Nx[G];
+  {
+    float2 Nz[G];
+    {
+      float2 W[G];
+      c2r(4, W);  // omega_x
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        Ny[m] = __fmul2_rn(pk(2, m), W[m]);
+        Nz[m] = __fmul2_rn(neg(pk(1, m)), W[m]);
+      }
+      c2r(5, W);  // omega_y
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        Nx[m] = __fmul2_rn(neg(pk(2, m)), W[m]);
+        Nz[m] = __ffma2_rn(pk(0, m), W[m], Nz[m]);
+      }
+    }
+    r2c(sl.out[2], Nz);
+  }
+  {
+    float2 W[G];
+    c2r(6, W);  // omega_z
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      Nx[m] = __ffma2_rn(pk(1, m), W[m], Nx[m]);
+      Ny[m] = __ffma2_rn(neg(pk(0, m)), W[m], Ny[m]);
+    }
+  }
+  r2c(sl.out[0], Nx);
+  r2c(sl.out[1], Ny);
+#pragma unroll 1
+  for (int i = 0; i < 3; ++i) {
+    float2 P[G];
+#pragma unroll
+    for (int m = 0; m < G; ++m) P[m] = __fmul2_rn(pk(i, m), pk(3, m));
+    r2c(sl.out[3 + i], P);
+  }
+}
+
+// ---- forward x pass with the update (periodic cube) ------------------------
+// As the Navier-Stokes forward x pass (ns_fwdx.cuh), with six fields and three
+// parked arrays: the divergence k . F(u theta), summed as its three fields are
+// transformed, then n_x and n_y.  512^3, per launch: forward x pass 528 us and
+// update 922 us as kernels of their own, 1355 us fused (1607 us with all its L2
+// prefetches at the start instead of one field ahead).
+template <int N>
+struct RUCfg {
+  static constexpr int G = N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G;
+  static constexpr int S = N / G;
+  static constexpr int T = N == 512 ? 16 : (N >= 768 ? 8 : (N % 3 == 0 ? 16 : NFCfg<N>::T));
+  static constexpr int THREADS = T * S;
+  static constexpr int KD = (N - 1) / 3;
+  static constexpr int LOW = KD / S + 1;
+  static constexpr int HIGH = (N - KD) / S > LOW ? (N - KD) / S : LOW;
+  static constexpr int SLOTS = LOW + G - HIGH;
+  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N * T + 3 * (size_t)SLOTS * THREADS);
+  static constexpr int MINB = THREADS >= 512 ? 1 : (THREADS == 256 ? (N == 768 ? 1 : 2) : 4);
+  __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
+  __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
+};
+
+template <int N, int MODE>
+__global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
+    k_rbc_fwdx(const float2* __restrict__ w, const float2* x, const float2* u0, const float2* s1, float2* acc,
+               float2* out, int ktiles, RBCUpdate upd, float scale, const float2* __restrict__ tw,
+               const float2* __restrict__ t3) {
+  constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
+  constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace
+  constexpr int KD = (N - 1) / 3;
+  constexpr bool A0 = MODE != NS_RHS && MODE != NS_RK4_4;             // reads the step's state
+  constexpr bool B0 = MODE == NS_STAGE2 || MODE >= NS_RK4_2;           // reads the stage state or the accumulator
+  using C = RUCfg<N>;
+  constexpr int G = C::G, S = C::S, T = C::T;
+  extern __shared__ float2 smn[];
+  const int c = threadIdx.x % T, j = threadIdx.x / T;
+  const int dky = blockIdx.x / ktiles;
+  const int ay = dense_to_a(dky, N, KD);
+  const int kz = (blockIdx.x - dky * ktiles) * T + c;
+  const bool valid = kz < (KD + 1);
+  const long long q = (long long)ay * H1 + kz, rs = (long long)N * H1;
+  const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
+  const ColX<T> xc{smn, c};
+  float2* park = smn + (size_t)N * T + threadIdx.x;
+  const int ky = kwav(ay, N);
+  const float2* bsrc = MODE == NS_STAGE2 ? s1 : acc;
+  float2 V[G];
+#pragma unroll 1
+  for (int i = 0; i < 6; ++i) {
+    const int f = i < 3 ? 3 + i : i - 3;  // u theta first, then n
+#pragma unroll
+    for (int m = 0; m < G; ++m)
+      V[m] = valid ? w[f * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
+    if constexpr (N >= 256) {  // the next field, and at last the update's reads, go to L2 meanwhile (see k_ns_fwdx)
+      if (i < 5) {
+        const int nf = i < 2 ? 4 + i : i - 2;
+        for (int r = threadIdx.x; r < N; r += C::THREADS) prefetch_l2(w + nf * MW + r * rw + qw - c);
+      }
+      if (i == 4 || i == 5)
+        for (int r = threadIdx.x; r < 2 * KD + 1; r += C::THREADS) {
+          const long long o = dense_to_a(r, N, KD) * rs + q - c;
+          if (i == 4) {
+            prefetch_l2(x + 2 * MM + o);
+            prefetch_l2(x + 3 * MM + o);
+          }
+#pragma unroll
+          for (int f2 = 0; f2 < 4; ++f2) {
+            if (A0 && i == 4) prefetch_l2(u0 + f2 * MM + o);
+            if (B0 && i == 5) prefetch_l2(bsrc + f2 * MM + o);
+          }
+        }
+    }
+    fft_line<N, G, -1>(V, j, xc, tw, t3);
+    if (i < 3) {
+#pragma unroll
+      for (int m = 0; m < G; ++m)
+        if (C::parked(m)) {
+          const float kf = i == 0 ? (float)kwav(j + m * S, N) : (i == 1 ? (float)ky : (float)kz);
+          float2& d = park[C::slot(m) * C::THREADS];
+          const float2 v = cscale(V[m], scale);
+          d = i == 0 ? make_float2(kf * v.x, kf * v.y) : make_float2(fmaf(kf, v.x, d.x), fmaf(kf, v.y, d.y));
+        }
+    } else if (i < 5) {
+#pragma unroll
+      for (int m = 0; m < G; ++m)
+        if (C::parked(m)) park[((i - 2) * C::SLOTS + C::slot(m)) * C::THREADS] = V[m];
+    }
+  }
+  if (!valid) return;
+  const float fky = (float)ky, fkz = (float)kz, dt = upd.dt;
+#pragma unroll
+  for (int m = 0; m < G; ++m) {
+    const int pos = j + m * S;
+    if (!C::parked(m) || !kept_xy(pos, N, KD)) continue;
+    const long long idx = pos * rs + q;
+    const int kx = kwav(pos, N), k2 = kx * kx + ky * ky + kz * kz;
+    float2 a[4], b[4];
+    const float2 uz = x[idx + 2 * MM], th = x[idx + 3 * MM];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      if (A0) a[f] = u0[idx + f * MM];
+      if (B0) b[f] = bsrc[idx + f * MM];
+    }
+    float2 E[2], H[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      if (MODE != NS_RHS && MODE != NS_RK4_4) E[t] = __ldg(&upd.tab[t * upd.tab_len + k2]);
+      if (MODE >= NS_RK4_1 && MODE != NS_RK4_4) H[t] = __ldg(&upd.tab[(2 + t) * upd.tab_len + k2]);
+    }
+    const float2 dv = park[C::slot(m) * C::THREADS];
+    float2 px = cscale(park[(C::SLOTS + C::slot(m)) * C::THREADS], scale);
+    float2 py = cscale(park[(2 * C::SLOTS + C::slot(m)) * C::THREADS], scale);
+    float2 pz = cadd(cscale(V[m], scale), th);  // n + theta z, then the projection
+    float2 nv[4];
+    if (k2 == 0) {
+      nv[0] = nv[1] = nv[2] = nv[3] = make_float2(0.f, 0.f);
+    } else {
+      const float fkx = (float)kx, inv = 1.f / (float)k2;
+      const float2 kn = make_float2((fkx * px.x + fky * py.x + fkz * pz.x) * inv,
+                                    (fkx * px.y + fky * py.y + fkz * pz.y) * inv);
+      nv[0] = csub(px, cscale(kn, fkx));
+      nv[1] = csub(py, cscale(kn, fky));
+      nv[2] = csub(pz, cscale(kn, fkz));
+      nv[3] = make_float2(dv.y + uz.x, -dv.x + uz.y);  // -i k . F(u theta) + u_z
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      rbc_entry_store<MODE>(idx + f * MM, nv[f], a[f], b[f], E[f == 3 ? 1 : 0], H[f == 3 ? 1 : 0], dt, acc, out);
+  }
+}
+
+// ------------------------------------------------------------ launchers ----
+template <int N>
+static cudaError_t rbc_invx_n(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
+  using I = NICfg<N>;
+  static PerDevice once;
+  const cudaError_t e = once.run([](int) {
+    return cudaFuncSetAttribute(k_ns_invx<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I::SMEM);
+  });
+  if (e != cudaSuccess) return e;
+  constexpr int KD = (N - 1) / 3, KT = (KD + I::T) / I::T;
+  LaunchScope ls(p, KK_X_INV, st);
+  k_ns_invx<N, true><<<(2 * KD + 1) * KT, I::THREADS, I::SMEM, st>>>(x, w, KT, twiddles(p, 1 << Log2<N>::value),
+                                                                  p->d_tw3);
+  return cudaGetLastError();
+}
+
+template <int N, int SIGN>
+static cudaError_t rbc_y_ns(fftk_plan p, float2* w, cudaStream_t st) {
+  using X = NXCfg<N>;
+  static PerDevice once;
+  const cudaError_t e = once.run([](int) {
+    return cudaFuncSetAttribute(k_ns_ypass<N, SIGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::SMEM);
+  });
+  if (e != cudaSuccess) return e;
+  constexpr int KD = (N - 1) / 3, KT = (KD + X::T) / X::T;
+  LaunchScope ls(p, SIGN > 0 ? KK_Y_INV : KK_Y_FWD, st);
+  k_ns_ypass<N, SIGN><<<(SIGN > 0 ? 7 : 6) * N * KT, X::THREADS, X::SMEM, st>>>(
+      w, w, KT, twiddles(p, 1 << Log2<N>::value), p->d_tw3);
+  return cudaGetLastError();
+}
+template <int N>
+static cudaError_t rbc_y_n(fftk_plan p, float2* w, int sign, cudaStream_t st) {
+  return sign > 0 ? rbc_y_ns<N, 1>(p, w, st) : rbc_y_ns<N, -1>(p, w, st);
+}
+
+template <int N>
+static cudaError_t rbc_z_n(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st) {
+  using C = RZCfg<N>;
+  static PerDevice once;
+  const cudaError_t e = once.run([](int) {
+    return cudaFuncSetAttribute(k_rbc_z<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+  });
+  if (e != cudaSuccess) return e;
+  const long long lines = (long long)N * N;
+  LaunchScope ls(p, KK_RBC_Z, st);
+  k_rbc_z<N><<<(unsigned)((lines + C::LPC - 1) / C::LPC), C::THREADS, C::SMEM, st>>>(
+      w, sl, twiddles(p, 1 << Log2<N>::value), p->d_tw3, p->d_err);
+  return cudaGetLastError();
+}
+
+template <int N, int MODE>
+static cudaError_t rbc_fwdx_nm(fftk_plan p, const RBCStage& s, cudaStream_t st) {
+  using U = RUCfg<N>;
+  static PerDevice once;
+  const cudaError_t e = once.run([](int) {
+    return cudaFuncSetAttribute(k_rbc_fwdx<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)U::SMEM);
+  });
+  if (e != cudaSuccess) return e;
+  constexpr int KD = (N - 1) / 3, KT = (KD + U::T) / U::T;
+  LaunchScope ls(p, KK_RBC_UPDATE, st);
+  k_rbc_fwdx<N, MODE><<<(2 * KD + 1) * KT, U::THREADS, U::SMEM, st>>>(s.w, s.x, s.u0, s.s1, s.acc, s.out, KT, s.upd,
+                                                                   s.scale, twiddles(p, 1 << Log2<N>::value),
+                                                                   p->d_tw3);
+  return cudaGetLastError();
+}
+template <int N>
+static cudaError_t rbc_fwdx_n(fftk_plan p, const RBCStage& s, cudaStream_t st) {
+  switch (s.mode) {
+#define MODE(m) \
+  case m:       \
+    return rbc_fwdx_nm<N, m>(p, s, st);
+    MODE(NS_RHS) MODE(NS_STAGE1) MODE(NS_STAGE2) MODE(NS_RK4_1) MODE(NS_RK4_2) MODE(NS_RK4_3) MODE(NS_RK4_4)
+#undef MODE
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace fftk

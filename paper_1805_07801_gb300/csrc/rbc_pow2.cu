@@ -1,0 +1,54 @@
+// The fused convection passes (rbc_passes.cuh) for powers of two.
+#include "rbc_passes.cuh"
+
+namespace fftk {
+
+cudaError_t rbc_invx(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
+  switch (p->nx) {
+#define CASE(n) \
+  case n:       \
+    return rbc_invx_n<n>(p, x, w, st);
+    CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
+#undef CASE
+    default:
+      return rbc_invx3(p, x, w, st);
+  }
+}
+
+cudaError_t rbc_y(fftk_plan p, float2* w, int sign, cudaStream_t st) {
+  switch (p->nx) {
+#define CASE(n) \
+  case n:       \
+    return rbc_y_n<n>(p, w, sign, st);
+    CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
+#undef CASE
+    default:
+      return rbc_y3(p, w, sign, st);
+  }
+}
+
+cudaError_t rbc_z(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st) {
+  switch (p->nx) {
+#define CASE(n) \
+  case n:       \
+    return rbc_z_n<n>(p, w, sl, st);
+    CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
+#undef CASE
+    default:
+      return rbc_z3(p, w, sl, st);
+  }
+}
+
+cudaError_t rbc_fwdx(fftk_plan p, const RBCStage& s, cudaStream_t st) {
+  switch (p->nx) {
+#define CASE(n) \
+  case n:       \
+    return rbc_fwdx_n<n>(p, s, st);
+    CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
+#undef CASE
+    default:
+      return rbc_fwdx3(p, s, st);
+  }
+}
+
+}  // namespace fftk
