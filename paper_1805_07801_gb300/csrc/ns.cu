@@ -300,7 +300,6 @@ void ns_free(fftk_plan p) {
   cudaFree(s->part);
   cudaFree(s->dout);
   if (s->hout) cudaFreeHost(s->hout);
-  cudaFree(s->r6);
   cudaFree(s->r3);
   cudaFree(s->acc);
   rbc_free(s->rbc);

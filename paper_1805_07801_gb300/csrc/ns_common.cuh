@@ -70,8 +70,7 @@ struct NSWork {
   double* dout = nullptr;  // diag result (device)
   double* hout = nullptr;  // diag result (pinned host)
   fftk_sgs_work* sgs = nullptr;  // learned-closure scratch
-  float* r6 = nullptr;     // 6 real fields (shell-to-shell transfer)
-  float* r3 = nullptr;     // 3 real fields (shell-to-shell transfer: the advection term)
+  float* r3 = nullptr;     // 3 real fields (shell-to-shell transfer: u)
   float2* acc = nullptr;   // 3 fields (RK4 accumulator)
   RBCWork* rbc = nullptr;  // Rayleigh-Benard scratch (allocated on first use)
   double* sout = nullptr;  // per-giver shell sums of the shell-to-shell transfer
@@ -97,7 +96,9 @@ void rbc_free(RBCWork* r);
 // diagnostics (ns_diag.cu)
 int diag_blocks(int width);
 cudaError_t diag_attr();
-cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double nu, cudaStream_t st, int nf = 3);
+// (into dout, by default the workspace's)
+cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double nu, cudaStream_t st, int nf = 3,
+                        double* dout = nullptr);
 
 inline bool misaligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) != 0; }
 

@@ -227,7 +227,8 @@ cudaError_t diag_attr() {
   });
 }
 
-cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double nu, cudaStream_t st, int nf) {
+cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double nu, cudaStream_t st, int nf,
+                        double* dout) {
   NSWork* s = p->ns;
   const int width = 2 + s->kmax + 1;
   {
@@ -236,44 +237,10 @@ cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double n
   }
   {
     LaunchScope ls(p, KK_NS_REDUCE, st);
-    k_diag_final<<<(width + 127) / 128, 128, 0, st>>>(s->part, width, diag_blocks(width), s->dout);
+    k_diag_final<<<(width + 127) / 128, 128, 0, st>>>(s->part, width, diag_blocks(width),
+                                                       dout ? dout : s->dout);
   }
   return cudaGetLastError();
-}
-
-// ------------------------------------------- shell-to-shell transfer ----
-// The giver shell's gradient for one component i: w3[j] = i k_j u_i on the
-// kept modes with kmin <= nint|k| < kmax_excl, 0 elsewhere.
-__global__ void k_shell_grad(const float2* __restrict__ u, float2* __restrict__ w3, NSGeom g, int comp, int kmin,
-                             int kmax_excl) {
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < g.M;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(idx % g.h1);
-    const long long ab = idx / g.h1;
-    const int b = (int)(ab % g.n), a = (int)(ab / g.n);
-    float2 gx = make_float2(0.f, 0.f), gy = gx, gz = gx;
-    if (kept_xy(a, g.n, g.kd) && kept_xy(b, g.n, g.kd) && c < g.kc) {
-      const long long kx = kwav(a, g.n), ky = kwav(b, g.n);
-      const long long K = shell_index(kx * kx + ky * ky + (long long)c * c);
-      if (K >= kmin && K < kmax_excl) {
-        const float2 v = u[idx + comp * g.M];
-        gx = mul_i(v, (float)kx);
-        gy = mul_i(v, (float)ky);
-        gz = mul_i(v, (float)c);
-      }
-    }
-    w3[idx] = gx;
-    w3[idx + g.M] = gy;
-    w3[idx + 2 * g.M] = gz;
-  }
-}
-
-// p = u_j G_j (real space): one component of (u . grad) u_giver
-__global__ void k_shell_advect(const float* __restrict__ ur, const float* __restrict__ gr, float* __restrict__ p,
-                               long long R) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < R;
-       i += (long long)gridDim.x * blockDim.x)
-    p[i] = ur[i] * gr[i] + ur[R + i] * gr[R + i] + ur[2 * R + i] * gr[2 * R + i];
 }
 
 }  // namespace fftk
@@ -327,93 +294,6 @@ extern "C" fftk_status tarang_transfer(fftk_plan p, const void* uhat, const tara
     out_host[1 + nb + K] = pi;
   }
   return std::isfinite(out_host[0]) ? FFTK_OK : FFTK_ERR_NONFINITE;
-}
-
-extern "C" fftk_status tarang_shell_transfer(fftk_plan p, const void* uhat, int nshells, const int* bounds,
-                                             double* out_host, void* cuda_stream) {
-  if (!p || !uhat || !bounds || !out_host || misaligned16(uhat)) return FFTK_ERR_INVALID_ARG;
-  if (p->nx != p->ny || p->nx != p->nz || p->nx < 8 || p->nx > 1024 || !is_pow2(p->nx)) return FFTK_ERR_UNSUPPORTED_SIZE;
-  const int kmax = ns_kmax(p->nx);
-  if (nshells < 1 || nshells > kmax + 1 || bounds[0] < 0 || bounds[nshells] > kmax + 1)
-    return FFTK_ERR_INVALID_ARG;
-  for (int i = 0; i < nshells; ++i)
-    if (bounds[i + 1] <= bounds[i]) return FFTK_ERR_INVALID_ARG;
-  fftk_status st0 = ns_ensure(p);
-  if (st0 != FFTK_OK) return st0;
-  cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  NSWork* s = p->ns;
-  const NSGeom g = s->g;
-  const long long R = (long long)g.n * g.n * g.n;
-  const int nb = s->kmax + 1, width = 2 + nb;
-  cudaError_t e = cudaSuccess;
-  if (!s->r6) e = cudaMalloc(&s->r6, sizeof(float) * 6 * (size_t)R);
-  if (e == cudaSuccess && !s->r3) e = cudaMalloc(&s->r3, sizeof(float) * 3 * (size_t)R);
-  if (e == cudaSuccess && s->sout_rows < nshells) {
-    cudaFree(s->sout);
-    s->sout = nullptr;
-    s->sout_rows = 0;
-    e = cudaMalloc(&s->sout, sizeof(double) * (size_t)nshells * width);
-    if (e == cudaSuccess) s->sout_rows = nshells;
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return e == cudaErrorMemoryAllocation ? FFTK_ERR_OOM : FFTK_ERR_CUDA;
-  }
-  const float2* u = static_cast<const float2*>(uhat);
-  float* ur = s->r6;                 // u in real space
-  float* gr = s->r6 + 3 * R;         // one row of the giver's gradient in real space
-  float2* gh = s->w;                 // the same row on the spectrum
-  float2* ph = s->w + 3 * g.M;       // (u . grad) u_giver on the spectrum
-  const unsigned grid = 152 * 8;
-  // the largest nint|k| among the kept modes: givers beyond it are empty
-  const int kd = g.kd;
-  const int kfar = (int)std::floor(std::sqrt(3.0 * kd * kd) + 0.5);
-  if (fftk_c2r(p, u, ur, 3, cuda_stream) != FFTK_OK) return FFTK_ERR_CUDA;
-  std::vector<char> live(nshells, 0);
-  for (int gi = 0; gi < nshells && e == cudaSuccess; ++gi) {
-    if (bounds[gi] > kfar) continue;
-    live[gi] = 1;
-    for (int i = 0; i < 3 && e == cudaSuccess; ++i) {
-      {
-        LaunchScope ls(p, KK_AUX, st);
-        k_shell_grad<<<grid, 256, 0, st>>>(u, gh, g, i, bounds[gi], bounds[gi + 1]);
-      }
-      if (fftk_c2r(p, gh, gr, 3, cuda_stream) != FFTK_OK) return FFTK_ERR_CUDA;
-      {
-        LaunchScope ls(p, KK_AUX, st);
-        k_shell_advect<<<grid, 256, 0, st>>>(ur, gr, s->r3 + i * R, R);
-      }
-      e = cudaGetLastError();
-    }
-    if (e != cudaSuccess) break;
-    if (fftk_r2c(p, s->r3, ph, 3, cuda_stream) != FFTK_OK) return FFTK_ERR_CUDA;
-    {
-      LaunchScope ls(p, KK_NS_REDUCE, st);
-      k_diag<<<diag_blocks(width), DIAG_WARPS * 32, s->diag_smem, st>>>(u, ph, g, 0.0, s->kmax, s->part, 3);
-    }
-    {
-      LaunchScope ls(p, KK_NS_REDUCE, st);
-      k_diag_final<<<(width + 127) / 128, 128, 0, st>>>(s->part, width, diag_blocks(width),
-                                                         s->sout + (size_t)gi * width);
-    }
-    e = cudaGetLastError();
-  }
-  std::vector<double> h((size_t)nshells * width, 0.0);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(h.data(), s->sout, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return from_cuda(e);
-  // T[r][g] = -sum over the receiver's integer shells of w Re(conj(u) . (u . grad) u_g)
-  bool finite = true;
-  for (int r = 0; r < nshells; ++r)
-    for (int gi = 0; gi < nshells; ++gi) {
-      double t = 0.0;
-      if (live[gi])
-        for (int K = bounds[r]; K < bounds[r + 1]; ++K) t -= h[(size_t)gi * width + 2 + K];
-      out_host[(size_t)r * nshells + gi] = t;
-      finite = finite && std::isfinite(t);
-    }
-  return finite ? FFTK_OK : FFTK_ERR_NONFINITE;
 }
 
 // ------------------------------------------- diagnostics without allocation --
