@@ -310,6 +310,20 @@ void ns_free(fftk_plan p) {
 }
 
 
+// The right-hand side of a checked state into the kept modes of `out`.
+cudaError_t fftk::ns_rhs_kept(fftk_plan p, const float2* u, float2* out, const tarang_params* prm, cudaStream_t st) {
+  const NSGeom g = p->ns->g;
+  NSUpdate upd{p->ns->etab, p->ns->etab_len, nullptr, p->ns->ef, prm->force_eps, prm->force_k2min,
+               prm->force_k2max, 0.f,
+               (float)(1.0 / ((double)g.n * g.n * g.n))};
+  cudaError_t e = cudaSuccess;
+  if (prm->force_eps > 0.0) e = forced_energy(p, u, prm, st);
+  const float2* extra = nullptr;
+  if (e == cudaSuccess && prm->sgs_model) e = sgs_term(p, &p->ns->sgs, u, prm->sgs_model, st, &extra);
+  if (e == cudaSuccess) e = ns_rhs_dispatch(p, u, u, nullptr, out, upd, NS_RHS, extra, st);
+  return e;
+}
+
 extern "C" fftk_status tarang_ns_rhs(fftk_plan p, const void* uhat, void* nhat,
                                      const tarang_params* prm, void* cuda_stream) {
   fftk_status s = ns_check(p, prm, false);
@@ -319,17 +333,9 @@ extern "C" fftk_status tarang_ns_rhs(fftk_plan p, const void* uhat, void* nhat,
   s = ns_ensure(p);
   if (s != FFTK_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const NSGeom g = p->ns->g;
-  const float2* u = static_cast<const float2*>(uhat);
-  float2* out = static_cast<float2*>(nhat);
-  cudaError_t e = cudaMemsetAsync(out, 0, sizeof(float2) * 3 * (size_t)g.M, st);
-  NSUpdate upd{p->ns->etab, p->ns->etab_len, nullptr, p->ns->ef, prm->force_eps, prm->force_k2min,
-               prm->force_k2max, 0.f,
-               (float)(1.0 / ((double)g.n * g.n * g.n))};
-  if (e == cudaSuccess && prm->force_eps > 0.0) e = forced_energy(p, u, prm, st);
-  const float2* extra = nullptr;
-  if (e == cudaSuccess && prm->sgs_model) e = sgs_term(p, &p->ns->sgs, u, prm->sgs_model, st, &extra);
-  if (e == cudaSuccess) e = ns_rhs_dispatch(p, u, u, nullptr, out, upd, NS_RHS, extra, st);
+  cudaError_t e = cudaMemsetAsync(nhat, 0, sizeof(float2) * 3 * (size_t)p->ns->g.M, st);
+  if (e == cudaSuccess)
+    e = ns_rhs_kept(p, static_cast<const float2*>(uhat), static_cast<float2*>(nhat), prm, st);
   return from_cuda(e);
 }
 

@@ -91,6 +91,8 @@ NSGeom make_geom(int n);
 fftk_status ns_ensure(fftk_plan p);
 cudaError_t ns_second_workspace(fftk_plan p);  // w2, on first use
 fftk_status ns_check(fftk_plan p, const tarang_params* prm, bool need_dt);
+// the right-hand side into the kept modes of `out` (the others are not written)
+cudaError_t ns_rhs_kept(fftk_plan p, const float2* u, float2* out, const tarang_params* prm, cudaStream_t st);
 void rbc_free(RBCWork* r);
 
 // diagnostics (ns_diag.cu)

@@ -107,33 +107,48 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
   const long long items = (long long)g.nk * g.nk * nchunk;
   const bool dissip = !nh;
   double accD = 0.0;
-  for (long long it = (long long)blockIdx.x * DIAG_WARPS + warp; it < items;
-       it += (long long)gridDim.x * DIAG_WARPS) {
+  // the next item's loads are in flight while this one is reduced
+  auto fetch = [&](long long it, float (&a)[6], float (&b)[6], int& kz, long long& k2) {
     const long long line = it / nchunk;
     const int chunk = (int)(it - line * nchunk);
     const int ax = dense_to_a((int)(line / g.nk), g.n, g.kd);
     const int ay = dense_to_a((int)(line % g.nk), g.n, g.kd);
-    const int kz = chunk * 32 + lane;
-    const bool valid = kz < g.kc;
-    float a[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, b[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int shell = kmax + 1;
-    long long k2 = 0;
-    if (valid) {
-      const long long idx = ((long long)ax * g.n + ay) * g.h1 + kz;
+    kz = chunk * 32 + lane;
+    const long long kx = kwav(ax, g.n), ky = kwav(ay, g.n);
+    k2 = kx * kx + ky * ky + (long long)kz * kz;
+    const long long idx = ((long long)ax * g.n + ay) * g.h1 + kz;
 #pragma unroll
-      for (int f = 0; f < 3; ++f) {
-        if (f >= nf) break;
-        const float2 v = u[idx + f * g.M];
-        a[2 * f] = v.x;
-        a[2 * f + 1] = v.y;
-        if (nh) {
-          const float2 q = nh[idx + f * g.M];
-          b[2 * f] = q.x;
-          b[2 * f + 1] = q.y;
-        }
+    for (int f = 0; f < 3; ++f) {
+      float2 v = make_float2(0.f, 0.f), q = v;
+      if (f < nf && kz < g.kc) {
+        v = u[idx + f * g.M];
+        if (nh) q = nh[idx + f * g.M];
       }
-      const long long kx = kwav(ax, g.n), ky = kwav(ay, g.n);
-      k2 = kx * kx + ky * ky + (long long)kz * kz;
+      a[2 * f] = v.x;
+      a[2 * f + 1] = v.y;
+      b[2 * f] = q.x;
+      b[2 * f + 1] = q.y;
+    }
+  };
+  const long long stride = (long long)gridDim.x * DIAG_WARPS;
+  long long it = (long long)blockIdx.x * DIAG_WARPS + warp;
+  float an[6], bn[6];
+  int kzn = 0;
+  long long k2n = 0;
+  if (it < items) fetch(it, an, bn, kzn, k2n);
+  for (; it < items; it += stride) {
+    float a[6], b[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      a[i] = an[i];
+      b[i] = bn[i];
+    }
+    const int kz = kzn;
+    const long long k2 = k2n;
+    if (it + stride < items) fetch(it + stride, an, bn, kzn, k2n);
+    const bool valid = kz < g.kc;
+    int shell = kmax + 1;
+    if (valid) {
       const long long K = shell_index(k2);
       shell = K <= kmax ? (int)K : kmax + 1;
     }
@@ -208,13 +223,30 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
   }
 }
 
-__global__ void k_diag_final(const double* __restrict__ part, int width, int nblocks, double* out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= width) return;
+// Sums of the block partials in a fixed order: 32 slots per block, sixteen
+// threads each for every sixteenth partial, their sums in order.  (One thread
+// per slot, adding up to 1216 partials one after the other, took 60 us.)
+constexpr int kFinCols = 32, kFinRows = 16;
+__global__ void __launch_bounds__(kFinCols* kFinRows)
+    k_diag_final(const double* __restrict__ part, int width, int nblocks, double* out) {
+  __shared__ double sum[kFinRows][kFinCols + 1];
+  const int col = threadIdx.x % kFinCols, row = threadIdx.x / kFinCols;
+  const int s = blockIdx.x * kFinCols + col;
   double t = 0.0;
-  for (int b = 0; b < nblocks; ++b) t += part[(long long)b * width + s];
-  out[s] = t;
+  if (s < width) {
+#pragma unroll 8
+    for (int b = row; b < nblocks; b += kFinRows) t += part[(long long)b * width + s];
+  }
+  sum[row][col] = t;
+  __syncthreads();
+  if (row == 0 && s < width) {
+    double tot = 0.0;
+#pragma unroll
+    for (int r = 0; r < kFinRows; ++r) tot += sum[r][col];
+    out[s] = tot;
+  }
 }
+static int diag_final_blocks(int width) { return (width + kFinCols - 1) / kFinCols; }
 
 // The dynamic shared-memory limit is an attribute of the kernel (per device),
 // not of a plan: it is raised once per device to what the largest grid needs,
@@ -237,7 +269,7 @@ cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double n
   }
   {
     LaunchScope ls(p, KK_NS_REDUCE, st);
-    k_diag_final<<<(width + 127) / 128, 128, 0, st>>>(s->part, width, diag_blocks(width),
+    k_diag_final<<<diag_final_blocks(width), kFinCols * kFinRows, 0, st>>>(s->part, width, diag_blocks(width),
                                                        dout ? dout : s->dout);
   }
   return cudaGetLastError();
@@ -278,10 +310,10 @@ extern "C" fftk_status tarang_transfer(fftk_plan p, const void* uhat, const tara
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   NSWork* w = p->ns;
   const int nb = w->kmax + 1, width = 2 + nb;
-  // the right-hand side goes to the stage buffer, free between steps
-  s = tarang_ns_rhs(p, uhat, w->u1, prm ? prm : &none, cuda_stream);
-  if (s != FFTK_OK) return s;
-  cudaError_t e = diag_launch(p, static_cast<const float2*>(uhat), w->u1, 0.0, st);
+  // the right-hand side goes to the stage buffer, free between steps; the
+  // reduction reads its kept modes only
+  cudaError_t e = ns_rhs_kept(p, static_cast<const float2*>(uhat), w->u1, prm ? prm : &none, st);
+  if (e == cudaSuccess) e = diag_launch(p, static_cast<const float2*>(uhat), w->u1, 0.0, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(w->hout, w->dout, sizeof(double) * width, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -361,6 +393,6 @@ extern "C" fftk_status tarang_diag_noalloc(int n, const void* uhat, double nu, d
   const int smem = (int)(sizeof(double) * DIAG_WARPS * (kmax + 1));
   k_diag<<<diag_blocks(width), DIAG_WARPS * 32, smem, st>>>(static_cast<const float2*>(uhat), nullptr, g, nu, kmax,
                                                    scratch, 3);
-  k_diag_final<<<(width + 127) / 128, 128, 0, st>>>(scratch, width, diag_blocks(width), diag_dev);
+  k_diag_final<<<diag_final_blocks(width), kFinCols * kFinRows, 0, st>>>(scratch, width, diag_blocks(width), diag_dev);
   return from_cuda(cudaGetLastError());
 }

@@ -344,9 +344,8 @@ extern "C" fftk_status tarang_rbc_transfer(fftk_plan p, const void* state, doubl
   const NSGeom g = w->g;
   const float2* x = static_cast<const float2*>(state);
   float2* nh = r->acc;  // free between steps
-  cudaError_t e = cudaMemsetAsync(nh, 0, sizeof(float2) * 4 * (size_t)g.M, st);
   const RBCUpdate upd{r->tab, r->tab_len, 0.f};
-  if (e == cudaSuccess) e = rbc_stage(p, x, x, nh, upd, NS_RHS, TARANG_RBC_FFF, st);
+  cudaError_t e = rbc_stage(p, x, x, nh, upd, NS_RHS, TARANG_RBC_FFF, st);
   const int nb = w->kmax + 1, width = 2 + nb;
   // three reductions: u . N_u (3 components), u_z theta, theta N_theta
   const float2* ua[3] = {x, x + 2 * g.M, x + 3 * g.M};
