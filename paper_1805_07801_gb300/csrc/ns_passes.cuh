@@ -216,18 +216,21 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
 // fewer values (8 at 128 and 256, 4 below), which fills the chip (per RK2 step,
 // 16 values -> these: 32^3 82 -> 53 us, 64^3 101 -> 62 us, 128^3 180 -> 139 us,
 // 256^3 929 -> 843 us).
-// 3 * 2^m lines: 12 values (radices 4, 4, 4, 6 at n = 768), 32 threads a line.
+// 3 * 2^m lines: 12 values per thread, at n = 768 24 (radices 8, 8, 6 instead of
+// 4, 4, 4, 6) with one staging buffer, so that two CTAs fit: 5.95 -> 4.85 ms
+// per launch (at 384 and 192 with 24: 3.06 against 3.03 ms, 514 against 479 us
+// per step).
 // Measured and dropped: three CTAs per SM with one staging buffer (168
 // registers, 1.120 against 1.126 ms), CTAs of 64 or 32 threads with five or
 // ten per SM (spills; 1.20 ms), the velocity parked in TMEM (slower).
-template <int N>
+template <int N, int MIN24 = 768>  // MIN24: 3 * 2^m lines from here on hold 24 values per thread
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-    static constexpr int G = N % 3 == 0 ? (H >= 48 ? 12 : 6) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
+    static constexpr int G = N % 3 == 0 ? (N >= MIN24 ? 24 : (H >= 48 ? 12 : 6)) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
-  static constexpr int NBUF = 2;                  // staging buffers per line
+  static constexpr int NBUF = G == 24 ? 1 : 2;    // staging buffers per line
   static constexpr int THREADS = LPC * S;
   static constexpr bool WARP = S <= 32;
   static constexpr int KC = (N - 1) / 3 + 1;      // kept k_z count (2/3 rule)
@@ -235,7 +238,7 @@ struct NZCfg {
   static constexpr size_t FIELDS = sizeof(float2) * (size_t)LPC * (HB + 3 * H);  // exchange + 3 parked fields
   static constexpr size_t STAGE = sizeof(float2) * (size_t)LPC * NBUF * KCP;  // staging buffers
   static constexpr size_t SMEM = FIELDS + STAGE + sizeof(uint64_t) * NBUF * LPC;  // + one mbarrier per buffer
-  static constexpr int MINB = G == 16 ? 2 : (G == 12 || N == 256 ? 3 : 4);  // CTAs per SM the registers must allow
+  static constexpr int MINB = G == 16 || G == 24 ? 2 : (G == 12 || N == 256 ? 3 : 4);  // CTAs per SM the registers must allow
 };
 
 // 3. per (x, y) line: the six c2r transforms, the product n = u x omega and

@@ -94,7 +94,7 @@ cudaError_t rbc_fwdx3(fftk_plan p, const RBCStage& s, cudaStream_t st);
 // thread and plain loads, 1679 us so; 256^3: 265 and 225 us.
 template <int N>
 struct RZCfg {
-  using Z = NZCfg<N>;
+  using Z = NZCfg<N, 4096>;  // (with 24 values only one CTA of four parked fields would fit)
   static constexpr int H = Z::H, HB = Z::HB, G = Z::G, S = Z::S, LPC = Z::LPC, NBUF = Z::NBUF, THREADS = Z::THREADS;
   static constexpr bool WARP = Z::WARP;
   static constexpr int KC = Z::KC, KCP = Z::KCP;
