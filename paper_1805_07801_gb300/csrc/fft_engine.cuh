@@ -313,14 +313,40 @@ __device__ __forceinline__ int swz_line(int pos) {
   return (pos & ~15) | ((pos ^ h) & 15);
 }
 
-// Exchange buffer for one contiguous line; WARP_SYNC when a line's threads
-// live in one warp.
-template <bool WARP_SYNC>
+// The same with the map {7, 10, 12, 8, ...}, which also keeps the radix-4
+// exchanges (4 or 12 values per thread) free of conflicts, at a few more
+// integer operations.
+__device__ __forceinline__ int swz_line4(int pos) {
+  const int b = pos >> 4;
+  const int lo = b & 15;
+  const int h = lo ^ ((lo & 1) * 6) ^ ((lo & 2) << 2) ^ ((lo & 4) << 1) ^ (b >> 4) ^ (b >> 8);
+  return (pos & ~15) | ((pos ^ h) & 15);
+}
+
+// Lines of S < 16 threads share a half warp: line li of a CTA permutes its
+// slots by one more XOR, so that the lines' equal positions lie in different
+// banks.  (Simulated over all exchanges, packed lines of 48 values on 4
+// threads: 4.0 -> 1.25 times the least number of wavefronts; 96 on 8: 2.4 ->
+// 1.15; 192 on 16 through swz_line4: 1.67 -> 1.17.)
+template <int S>
+__device__ __forceinline__ int line_xor(int li) {
+  if constexpr (S == 8) return (li & 1) * 9;
+  if constexpr (S == 4) return ((li & 1) * 5) ^ ((li & 2) * 5);
+  if constexpr (S == 2) return (li & 7) * 2;
+  return 0;
+}
+
+// Exchange buffer for one contiguous line of S threads with G values each;
+// WARP_SYNC when a line's threads live in one warp.
+template <bool WARP_SYNC, int S = 32, int G = 16>
 struct LineX {
   static constexpr bool kStageTables = true;  // a warp spans 32 consecutive butterflies
+  static constexpr bool kMap4 = G != 16 && (S < 16 || G % 8 != 0);
   float2* s;
-  __device__ __forceinline__ void st(int pos, float2 v) const { s[swz_line(pos)] = v; }
-  __device__ __forceinline__ float2 ld(int pos) const { return s[swz_line(pos)]; }
+  int x = 0;  // line_xor
+  __device__ __forceinline__ int at(int pos) const { return (kMap4 ? swz_line4(pos) : swz_line(pos)) ^ x; }
+  __device__ __forceinline__ void st(int pos, float2 v) const { s[at(pos)] = v; }
+  __device__ __forceinline__ float2 ld(int pos) const { return s[at(pos)]; }
   __device__ __forceinline__ void sync() const {
     if constexpr (WARP_SYNC)
       __syncwarp();
@@ -454,9 +480,9 @@ __host__ __device__ constexpr int elems_per_thread(int L) {
   if (L % 3 == 0) return L >= 96 ? 24 : (L >= 12 ? 12 : L);
   return L < 16 ? L : 16;
 }
-// slots of the exchange buffer of one contiguous line of H values (swz_line
-// permutes within blocks of 16)
-__host__ __device__ constexpr int line_slots(int H) { return H % 3 == 0 ? (H + 15) / 16 * 16 : H; }
+// slots of the exchange buffer of one contiguous line of H values (the
+// permutations stay within blocks of 16)
+__host__ __device__ constexpr int line_slots(int H) { return (H + 15) / 16 * 16; }
 
 }  // inline namespace
 }  // namespace fftk

@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   const int li = threadIdx.x / S, j = threadIdx.x % S;
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < nlines;
-  const LineX<C::WARP> xc{sm + li * C::HB};
+  const LineX<C::WARP, S, G> xc{sm + li * C::HB, line_xor<S>(li)};
   float2 v[G];
   const float2* src = reinterpret_cast<const float2*>(in + line * N);
 #pragma unroll
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   const int li = threadIdx.x / S, j = threadIdx.x % S;
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < nlines;
-  const LineX<C::WARP> xc{sm + li * C::HB};
+  const LineX<C::WARP, S, G> xc{sm + li * C::HB, line_xor<S>(li)};
   const float2* src = in + line * (H + 1);
   // X[0..H-1] of the line pass through the exchange buffer once, so the
   // mirror X[H - k] is read from there instead of a second global load

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
   const int li = threadIdx.x / S, j = threadIdx.x % S;
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < (long long)N * N;
-  const LineX<C::WARP> xc{smz + li * C::HB};
+  const LineX<C::WARP, S, G> xc{smz + li * C::HB, line_xor<S>(li)};
   float2* park = smz + C::LPC * C::HB + li * 3 * H + j;  // [3][G][S] per line, this thread's column
   constexpr int NB = C::NBUF;
   float2* stage = smz + C::FIELDS / sizeof(float2) + li * NB * C::KCP;  // this line's buffers

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
   const int li = threadIdx.x / S, j = threadIdx.x % S;
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < (long long)N * N;
-  const LineX<C::WARP> xc{smz + li * C::HB};
+  const LineX<C::WARP, S, G> xc{smz + li * C::HB, line_xor<S>(li)};
   float2* park = smz + C::LPC * C::HB + li * 4 * H + j;  // [4][G][S]: u_x, u_y, u_z, theta
   float2* stage = smz + C::FIELDS / sizeof(float2) + li * NB * C::KCP;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smz + (C::FIELDS + C::STAGE) / sizeof(float2)) + NB * li;
