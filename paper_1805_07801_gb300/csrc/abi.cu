@@ -210,8 +210,8 @@ extern "C" fftk_status fftk_plan_create(int nx, int ny, int nz, fftk_dtype dtype
       e = cudaMemcpy(p->d_tw3_alloc, h3.data(), sizeof(float2) * h3.size(), cudaMemcpyHostToDevice);
     }
   }
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_err, 3 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, 3 * sizeof(int));
   if (e == cudaSuccess && dtype == FFTK_R32_SPLIT16) e = upload_dft16_operands(p);
   if (e != cudaSuccess) {
     fftk_status s = from_cuda(e);

@@ -226,6 +226,31 @@ __device__ __forceinline__ void dft16(float2 (&x)[16]) {
     for (int k2 = 0; k2 < 4; ++k2) x[k1 + 4 * k2] = t[4 * k1 + k2];
 }
 
+// a * exp(SIGN 2 pi i q / 32), q known at compile time after unrolling
+template <int SIGN>
+__device__ __forceinline__ float2 rot32(float2 a, int q) {
+  return mul_root32(a, SIGN < 0 ? q : (32 - q) & 31);
+}
+
+// 32 = 4 x 8: X[k1 + 4 k2] = sum_{n2} W32^{n2 k1} W8^{n2 k2} sum_{n1} x[8 n1 + n2] W4^{n1 k1}
+template <int SIGN>
+__device__ __forceinline__ void dft32(float2 (&x)[32]) {
+#pragma unroll
+  for (int n2 = 0; n2 < 8; ++n2) dft4<SIGN>(x[n2], x[8 + n2], x[16 + n2], x[24 + n2]);
+  float2 o[32];
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) {
+    float2 t[8];
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) t[n2] = rot32<SIGN>(x[8 * k1 + n2], n2 * k1);
+    dft8<SIGN>(t);
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) o[k1 + 4 * k2] = t[k2];
+  }
+#pragma unroll
+  for (int k = 0; k < 32; ++k) x[k] = o[k];
+}
+
 // X1,2 = a - (b + c)/2 +- SIGN i sin(pi/3) (b - c)
 template <int SIGN>
 __device__ __forceinline__ void dft3(float2& a, float2& b, float2& c) {

@@ -154,9 +154,9 @@ struct CCfg {
 
 // AHEAD > 0: while it transforms, the CTA asks for the rows of the tile AHEAD
 // places on (the one that comes next on some SM) in L2.  For lines that leave
-// room for one CTA per SM, whose loads nothing else covers.  y passes: 1024^3
-// 2.07 -> 1.95 ms each, 768^3 pair 4.87 -> 4.60 ms; x passes, whose rows lie
-// megabytes apart: 768^3 pair 4.60 -> 4.41 ms, but 1024^3 2.01 against 2.12 ms.
+// room for one CTA per SM, whose loads nothing else covers: 768^3 pair 4.87 ->
+// 4.41 ms.  (1024^3, where fft_stream.cu has a pipelined pass: y 2.07 -> 1.95
+// ms, but x, with 32 warps on the SM, 2.01 against 2.12 ms.)
 template <int L, int SIGN, int AHEAD>
 __global__ void __launch_bounds__(CCfg<L>::THREADS, CCfg<L>::MINB)
     k_cpass(const float2* in, float2* out, long long Q, long long qtiles,

@@ -7,9 +7,8 @@
 // 256 rows) instead of 16 global loads per thread, and starts the next tile's
 // copy as soon as the line engine has released the tile buffer, so the copy
 // overlaps the last radix stage and the stores of the current tile.  Two
-// such CTAs (512 threads, 64 KB each) share an SM.  For 1024-point lines the
-// tile fills 128 KB and one CTA of 1024 threads holds the SM; there the copy
-// has nothing to overlap and the pass with plain loads is the faster one.
+// such CTAs (512 threads, 64 KB each) share an SM.  Lines of 1024 points, whose
+// tile fills 128 KB, take k_cpass_pipe below.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -103,6 +102,137 @@ __global__ void __launch_bounds__(PFCfg<L>::THREADS, PFCfg<L>::MINB)
 #pragma unroll
       for (int m = 0; m < G; ++m) dst[(long long)(j + m * S) * Q] = cscale(v[m], scale);
     }
+  }
+}
+
+// Strided pass for lines of 1024 points.  A tile of 16 columns fills 128 KB,
+// so two tiles of the exchange-in-place kind do not fit beside each other and
+// the phases of one CTA (load, transform, store) run in turn (k_cpass: 1.95 to
+// 2.01 ms per 1024^3 pass, 0.63 of the copy rate).  Here the next tile streams
+// into a staging buffer while this one, held in registers (32 values on each
+// of 512 threads, two radix-32 stages), exchanges once through 64 KB: real
+// parts first, then imaginary parts.  The twiddles lie in shared memory (from
+// global memory their 31 gathers per tile cost 50 us per pass).  Bound by HBM:
+// 1024^3, per pass, x 1.35 ms and y 1.37 ms (0.93 of the copy rate).
+//
+// Q even: rows start on 16-byte boundaries and the tile arrives as four boxes
+// of 16 columns x 256 rows.  Q odd (PAIR; the y pass, whose rows of n/2 + 1
+// values start on and 8 bytes past such boundaries in turn): even and odd rows
+// are two tensors whose row stride, 16 Q bytes, is a multiple of 16, the second
+// one starting 8 bytes early, in boxes of 18 columns.  (One bulk copy of 144
+// bytes per row instead: 2.43 ms.)
+constexpr int kPL = 1024, kPG = 32, kPS = 32, kPT = 16, kPThreads = kPS * kPT;
+template <bool PAIR>
+struct PipeCfg {
+  static constexpr int ODD = PAIR ? kPT + 2 : kPT;  // float2 per staged odd row
+  static constexpr size_t STAGE = sizeof(float2) * (kPL / 2) * (kPT + ODD);
+  static constexpr size_t EX = sizeof(float) * kPL * kPT;
+  static constexpr size_t SMEM = STAGE + EX + sizeof(float2) * kPL + 16;
+};
+
+template <int SIGN, bool PAIR>
+__global__ void __launch_bounds__(kPThreads, 1)
+    k_cpass_pipe(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_odd, float2* out,
+                 long long Q, int qtiles, int ntiles, const float2* __restrict__ tw, float scale, int* err) {
+  using C = PipeCfg<PAIR>;
+  extern __shared__ __align__(128) unsigned char smp[];
+  __shared__ int ok_flag, next_tile;
+  float2* stage = reinterpret_cast<float2*>(smp);
+  float2* odd = stage + (size_t)(kPL / 2) * kPT;  // PAIR: the odd rows
+  float* ex = reinterpret_cast<float*>(smp + C::STAGE);
+  float2* stw = reinterpret_cast<float2*>(smp + C::STAGE + C::EX);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smp + C::SMEM - 16);
+  const int tid = threadIdx.x, c = tid % kPT, j = tid / kPT;
+  for (int i = tid; i < kPL; i += kPThreads) stw[i] = tw[i];
+
+  auto fetch = [&](int t) {  // thread 0
+    const int p = t / qtiles, q0 = (t - p * qtiles) * kPT;
+    mbar_expect(bar, (uint32_t)C::STAGE);
+    if constexpr (PAIR) {
+#pragma unroll 1
+      for (int b = 0; b < 2; ++b) {
+        tma_load3(stage + (size_t)b * 256 * kPT, &map, 2 * q0, b * 256, p, bar);
+        tma_load3(odd + (size_t)b * 256 * C::ODD, &map_odd, 2 * q0, b * 256, p, bar);
+      }
+    } else {
+#pragma unroll 1
+      for (int b = 0; b < 4; ++b) tma_load3(stage + (size_t)b * 256 * kPT, &map, 2 * q0, b * 256, p, bar);
+    }
+  };
+  // a warp holds two rows: rows 32 apart (the stores of the first stage) and
+  // neighbouring rows (the loads) each fall into different halves of the banks
+  auto slot = [&](int pos) { return ((pos ^ ((pos >> 5) & 1)) * kPT) + c; };
+  if (tid == 0) tcg::mbar_init(bar);
+  __syncthreads();
+  // Tiles are handed out in order (a counter; each CTA draws one ahead): were
+  // each CTA to take every gridDim-th tile, the CTAs would drift apart over a
+  // long pass, and neighbouring tiles, which share the lines of misaligned
+  // rows, would meet in L2 no longer (1024^3 with every gridDim-th tile: x
+  // 1.60 ms, y 2.14 ms).
+  int* queue = err + 1;  // next tile, CTAs that are done
+  uint32_t phase = 0;
+  int t = blockIdx.x, drawn = 0;
+  if (tid == 0) {
+    fetch(t);
+    drawn = (int)gridDim.x + atomicAdd(queue, 1);
+  }
+  while (t < ntiles) {
+    if (tid == 0) {
+      ok_flag = tcg::mbar_wait(bar, phase) ? 1 : 0;
+      next_tile = drawn;
+    }
+    __syncthreads();
+    if (!ok_flag) {  // see k_cpass_tma
+      if (tid == 0) {
+        atomicOr(err, 1);
+        tcg::mbar_wait(bar, phase);
+      }
+      break;
+    }
+    const int tn = next_tile;
+    phase ^= 1;
+    float2 v[kPG];
+    const float2* src = !PAIR ? stage + j * kPT + c
+                              : (j & 1 ? odd + (j >> 1) * C::ODD + 1 + c : stage + (j >> 1) * kPT + c);
+    const int step = !PAIR ? kPS * kPT : (kPS / 2) * (j & 1 ? C::ODD : kPT);
+#pragma unroll
+    for (int m = 0; m < kPG; ++m) v[m] = src[m * step];
+    __syncthreads();  // the staging buffer is free, and so is the exchange buffer
+    if (tid == 0 && tn < ntiles) {
+      tcg::fence_smem_async();
+      fetch(tn);
+      drawn = (int)gridDim.x + atomicAdd(queue, 1);
+    }
+    dft32<SIGN>(v);
+#pragma unroll
+    for (int r = 0; r < kPG; ++r) ex[slot(j * kPG + r)] = v[r].x;
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < kPG; ++m) v[m].x = ex[slot(j + m * kPS)];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kPG; ++r) ex[slot(j * kPG + r)] = v[r].y;
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < kPG; ++m) v[m].y = ex[slot(j + m * kPS)];
+#pragma unroll
+    for (int r = 1; r < kPG; ++r) {
+      const float2 w = stw[r * j];
+      v[r] = SIGN < 0 ? cmul(v[r], w) : cmulc(v[r], w);
+    }
+    dft32<SIGN>(v);
+    const int p = t / qtiles;
+    const long long q = (long long)(t - p * qtiles) * kPT + c;
+    if (q < Q) {
+      float2* dst = out + (long long)p * kPL * Q + q;
+#pragma unroll
+      for (int m = 0; m < kPG; ++m) dst[(long long)(j + m * kPS) * Q] = cscale(v[m], scale);
+    }
+    t = tn;
+  }
+  if (tid == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {  // the last CTA leaves the counters at zero
+    queue[0] = 0;
+    queue[1] = 0;
   }
 }
 
@@ -202,10 +332,60 @@ static bool tma_map_l(CUtensorMap* m, const float2* in, long long P, long long Q
   return make_map<L>(m, in, P, Q);
 }
 
+template <int SIGN, bool PAIR>
+static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorMap& mo, float2* out, long long P,
+                              long long Q, float scale, int kind, cudaStream_t st) {
+  using C = PipeCfg<PAIR>;
+  static PerDevice once;
+  static int nsm[kMaxDevices];
+  int dev = 0;
+  const cudaError_t e = once.run(
+      [](int d) {
+        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<SIGN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)C::SMEM);
+        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d);
+        return err;
+      },
+      &dev);
+  if (e != cudaSuccess) return e;
+  const long long qtiles = (Q + kPT - 1) / kPT, ntiles = P * qtiles;
+  const unsigned grid = (unsigned)(ntiles < nsm[dev] ? ntiles : nsm[dev]);
+  LaunchScope ls(p, kind, st);
+  k_cpass_pipe<SIGN, PAIR><<<grid, kPThreads, C::SMEM, st>>>(m, mo, out, Q, (int)qtiles, (int)ntiles,
+                                                            twiddles(p, kPL), scale, p->d_err);
+  return cudaGetLastError();
+}
+
+// The maps of even and odd rows for odd Q: [P][kPL / 2][2 Q] and, 8 bytes
+// before row 1, [P][kPL / 2][2 (Q + 1)] floats, row stride 16 Q bytes.  The
+// last element of the second is the last of the array.
+static bool pair_maps(CUtensorMap* even, CUtensorMap* odd, const float2* in, long long P, long long Q) {
+  if (8LL * Q * kPL >= (1LL << 40) || 2 * (Q + 1) >= (1LL << 31) || P >= (1LL << 31)) return false;
+  const uint64_t strides[2] = {(uint64_t)(16 * Q), (uint64_t)(8 * Q * kPL)};
+  const uint64_t de[3] = {(uint64_t)(2 * Q), kPL / 2, (uint64_t)P}, dd[3] = {(uint64_t)(2 * (Q + 1)), kPL / 2, (uint64_t)P};
+  const uint32_t be[3] = {2 * kPT, 256, 1}, bo[3] = {2 * PipeCfg<true>::ODD, 256, 1};
+  return encode_f32_map(even, in, 3, de, strides, be) && encode_f32_map(odd, in + Q - 1, 3, dd, strides, bo);
+}
+
 bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
                       float scale, int kind, cudaStream_t st, cudaError_t* e) {
   if (P <= 0 || Q <= 0) return false;
-  CUtensorMap m;
+  CUtensorMap m{};
+  if (L == kPL) {
+    // narrow arrays and bases off 16 bytes keep the general pass
+    if (Q < kPT || reinterpret_cast<uintptr_t>(in) % 16 != 0 || P * ((Q + kPT - 1) / kPT) >= (1LL << 31)) return false;
+    if (Q % 2 == 0) {
+      if (!tma_map_l<kPL>(&m, in, P, Q)) return false;
+      *e = sign < 0 ? cpass_pipe<-1, false>(p, m, m, out, P, Q, scale, kind, st)
+                    : cpass_pipe<+1, false>(p, m, m, out, P, Q, scale, kind, st);
+    } else {
+      CUtensorMap mo{};
+      if (!pair_maps(&m, &mo, in, P, Q)) return false;
+      *e = sign < 0 ? cpass_pipe<-1, true>(p, m, mo, out, P, Q, scale, kind, st)
+                    : cpass_pipe<+1, true>(p, m, mo, out, P, Q, scale, kind, st);
+    }
+    return true;
+  }
 #define CASE(n)                                                                                  \
   case n:                                                                                        \
     if (!tma_map_l<n>(&m, in, P, Q)) return false;                                               \

@@ -67,7 +67,7 @@ struct fftk_plan_s {
   float2* d_tw3_alloc = nullptr;  // per-stage tables of the 3 * 2^m lines (kStage3Twiddles entries), then d_tw3
   float2* d_tw3 = nullptr;   // the same as d_tw for L = 3, 6, 12, ... up to the largest 3 * 2^m dimension
   __half* d_dft16 = nullptr; // split-FP16 DFT-16 operands (FFTK_R32_SPLIT16): forward, inverse
-  int* d_err = nullptr;      // device error word (bounded waits that expired)
+  int* d_err = nullptr;      // device error word (bounded waits that expired), then two tile counters (fft_stream.cu)
   // c2r workspace (one complex field per batch element)
   void* ws = nullptr;
   size_t ws_bytes = 0;

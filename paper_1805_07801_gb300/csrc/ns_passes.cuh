@@ -227,7 +227,7 @@ template <int N, int MIN24 = 768>  // MIN24: 3 * 2^m lines from here on hold 24 
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-    static constexpr int G = N % 3 == 0 ? (N >= MIN24 ? 24 : (H >= 48 ? 12 : 6)) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
+  static constexpr int G = N % 3 == 0 ? (N >= MIN24 ? 24 : (H >= 48 ? 12 : 6)) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
   static constexpr int NBUF = G == 24 ? 1 : 2;    // staging buffers per line
