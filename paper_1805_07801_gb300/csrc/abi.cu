@@ -293,11 +293,11 @@ extern "C" fftk_status fftk_set_workspace(fftk_plan p, void* dev_ptr, size_t byt
 // and the line length has two radix-16 stages, the FP32 kernel otherwise.
 static cudaError_t strided_pass(fftk_plan p, int L, int sign, const float2* in, float2* out,
                                 long long P, long long Q, float scale, int kind, cudaStream_t st) {
-  if (!is_pow2(L)) return launch_cpass3(p, L, sign, in, out, P, Q, scale, kind, st);
   if (p->dtype == FFTK_R32_SPLIT16 && cpass_tc_supported(L))
     return launch_cpass_tc(p, L, sign, in, out, P, Q, scale, kind, st);
   cudaError_t e = cudaSuccess;
   if (launch_cpass_tma(p, L, sign, in, out, P, Q, scale, kind, st, &e)) return e;
+  if (!is_pow2(L)) return launch_cpass3(p, L, sign, in, out, P, Q, scale, kind, st);
   return launch_cpass(p, L, sign, in, out, P, Q, scale, kind, st);
 }
 

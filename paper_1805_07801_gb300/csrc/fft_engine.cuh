@@ -291,6 +291,8 @@ __device__ __forceinline__ void dftR(float2 (&a)[R]) {
     dft8<SIGN>(a);
   } else if constexpr (R == 16) {
     dft16<SIGN>(a);
+  } else if constexpr (R == 32) {
+    dft32<SIGN>(a);
   }
 }
 

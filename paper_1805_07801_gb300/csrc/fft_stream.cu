@@ -1,14 +1,22 @@
-// Strided pass for lines of 512 points with TMA tile loads.
+// Pipelined strided pass for lines of 256 to 1024 points and of 3 * 2^m from
+// 384 to 1536.
 //
 // The strided pass of the 3D transform (the y and x line transforms of
-// Sec. 3) works on tiles of T = 16 adjacent columns x L rows.  Where the row
-// stride Q is a multiple of 16 bytes (the x pass, Q = ny (nz/2+1)), a
-// persistent CTA loads its tiles with TMA tiled copies (boxes of 16 columns x
-// 256 rows) instead of 16 global loads per thread, and starts the next tile's
-// copy as soon as the line engine has released the tile buffer, so the copy
-// overlaps the last radix stage and the stores of the current tile.  Two
-// such CTAs (512 threads, 64 KB each) share an SM.  Lines of 1024 points, whose
-// tile fills 128 KB, take k_cpass_pipe below.
+// Sec. 3) works on tiles of 16 adjacent columns x L rows.  Persistent CTAs
+// stream their next tile into a staging buffer (TMA) while this one, held in
+// registers, takes two long-radix stages (32 x 32, 32 x 16, 16 x 16) with one
+// exchange through a buffer of half the tile's size: real parts first, then
+// imaginary parts.  So the copies overlap the transforms and the stores, and
+// the pass is bound by HBM (k_cpass, which loads, transforms and stores in
+// turn with one to four CTAs per SM, by its latencies).  Per pass, x / y, with
+// k_cpass (512^3 x: with a tile streamed into the exchange buffer) and so:
+//   1024^3      2.01 / 2.07 -> 1.35 / 1.37 ms   (0.94 of the copy rate)
+//   512^3       187 / 225 -> 168 / 206 us       (0.95 / 0.77)
+//   16 x 256^3  423 / 439 -> 322 / 418 us       (0.99 / 0.76)
+//   768^3       797 / 858 -> 622 / 698 us       (0.86 / 0.77)
+//   2 x 1536 x 1536 x 96   1180 / 1357 -> 823 / 1011 us
+// The y passes' rows of n/2 + 1 values leave one column for a last tile and
+// store across line boundaries, which the shorter lines' transforms feel.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -22,153 +30,77 @@
 
 namespace fftk {
 
-template <int L>
-struct PFCfg {
-  static constexpr int G = 16;                                // values per thread
-  static constexpr int S = L / G;                             // threads per line
-  static constexpr int T = 16;                                // columns per tile (128-byte rows)
-  static constexpr int THREADS = S * T;
-  static constexpr int MINB = THREADS <= 512 ? 2 : 1;
-  static constexpr int BOXR = 256;                            // rows per TMA box
-  static constexpr int NBOX = L / BOXR;
-  static constexpr size_t PBYTES = sizeof(float2) * (size_t)L * T;
-  static constexpr size_t SMEM = PBYTES + 16;                 // + the tile mbarrier
-};
-
 using tcg::mbar_expect;
 using tcg::tma_load3;
 
-// Array [P][L][Q] of complex values, transform along L (element stride Q);
-// tile t = (p, q-tile); in may equal out (tiles are disjoint column sets).
-// The tile buffer doubles as the exchange buffer of the line engine; once the
-// last exchange has been read, thread 0 starts the next tile's loads, which
-// then overlap the last stage and the stores of this tile.
-template <int L, int SIGN>
-__global__ void __launch_bounds__(PFCfg<L>::THREADS, PFCfg<L>::MINB)
-    k_cpass_tma(const __grid_constant__ CUtensorMap tmap, float2* out, int Q, int qtiles, int ntiles,
-                const float2* __restrict__ tw, float scale, int* err) {
-  using C = PFCfg<L>;
-  constexpr int G = C::G, S = C::S, T = C::T;
-  extern __shared__ __align__(128) float2 smf[];
-  __shared__ int ok_flag;
-  float2* P = smf;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smf + (size_t)L * T);
-  const int tid = threadIdx.x;
-  const int c = tid % T, j = tid / T;
-
-  auto fetch = [&](int t) {  // thread 0: the NBOX boxes of tile t into P
-    const int p = t / qtiles;
-    const int q0 = (t - p * qtiles) * T;
-    mbar_expect(bar, (uint32_t)C::PBYTES);
-#pragma unroll 1
-    for (int b = 0; b < C::NBOX; ++b) tma_load3(P + (size_t)b * C::BOXR * T, &tmap, 2 * q0, b * C::BOXR, p, bar);
-  };
-
-  if (tid == 0) tcg::mbar_init(bar);
-  __syncthreads();
-  uint32_t phase = 0;
-  int t = blockIdx.x;
-  if (tid == 0 && t < ntiles) fetch(t);
-  for (; t < ntiles; t += gridDim.x) {
-    if (tid == 0) ok_flag = tcg::mbar_wait(bar, phase) ? 1 : 0;
-    __syncthreads();
-    if (!ok_flag) {
-      // The tile never arrived: its copy may still be pending, writing into
-      // this CTA's shared memory and completing on the mbarrier there.  Thread
-      // 0 reports, then waits once more (bounded) for that copy before the
-      // CTA's shared memory is released; the other threads may leave.  The
-      // error word is the only signal: the host treats it as fatal for the plan.
-      if (tid == 0) {
-        atomicOr(err, 1);
-        tcg::mbar_wait(bar, phase);
-      }
-      return;
-    }
-    phase ^= 1;
-    float2 v[G];
-#pragma unroll
-    for (int m = 0; m < G; ++m) v[m] = P[(j + m * S) * T + c];
-    __syncthreads();  // the exchanges below overwrite P
-    fft_line<L, G, SIGN>(v, j, ColX<T>{P, c}, tw);
-    const int tn = t + (int)gridDim.x;
-    if (tid == 0 && tn < ntiles) {  // every thread has read the last exchange: P is free
-      tcg::fence_smem_async();
-      fetch(tn);
-    }
-    const int p = t / qtiles;
-    const int q = (t - p * qtiles) * T + c;
-    if (q < Q) {
-      float2* dst = out + (long long)p * L * Q + q;
-#pragma unroll
-      for (int m = 0; m < G; ++m) dst[(long long)(j + m * S) * Q] = cscale(v[m], scale);
-    }
-  }
-}
-
-// Strided pass for lines of 1024 points.  A tile of 16 columns fills 128 KB,
-// so two tiles of the exchange-in-place kind do not fit beside each other and
-// the phases of one CTA (load, transform, store) run in turn (k_cpass: 1.95 to
-// 2.01 ms per 1024^3 pass, 0.63 of the copy rate).  Here the next tile streams
-// into a staging buffer while this one, held in registers (32 values on each
-// of 512 threads, two radix-32 stages), exchanges once through 64 KB: real
-// parts first, then imaginary parts.  The twiddles lie in shared memory (from
-// global memory their 31 gathers per tile cost 50 us per pass).  Bound by HBM:
-// 1024^3, per pass, x 1.35 ms and y 1.37 ms (0.93 of the copy rate).
-//
-// Q even: rows start on 16-byte boundaries and the tile arrives as four boxes
-// of 16 columns x 256 rows.  Q odd (PAIR; the y pass, whose rows of n/2 + 1
-// values start on and 8 bytes past such boundaries in turn): even and odd rows
-// are two tensors whose row stride, 16 Q bytes, is a multiple of 16, the second
+// Q even: rows start on 16-byte boundaries and a tile arrives as boxes of 16
+// columns x 256 rows.  Q odd (PAIR; the y pass, whose rows of n/2 + 1 values
+// start on and 8 bytes past such boundaries in turn): even and odd rows are
+// two tensors whose row stride, 16 Q bytes, is a multiple of 16, the second
 // one starting 8 bytes early, in boxes of 18 columns.  (One bulk copy of 144
-// bytes per row instead: 2.43 ms.)
-constexpr int kPL = 1024, kPG = 32, kPS = 32, kPT = 16, kPThreads = kPS * kPT;
-template <bool PAIR>
+// bytes per row instead: 2.43 against 2.14 ms at 1024^3.)
+template <int L_, bool PAIR_>
 struct PipeCfg {
-  static constexpr int ODD = PAIR ? kPT + 2 : kPT;  // float2 per staged odd row
-  static constexpr size_t STAGE = sizeof(float2) * (kPL / 2) * (kPT + ODD);
-  static constexpr size_t EX = sizeof(float) * kPL * kPT;
-  static constexpr size_t SMEM = STAGE + EX + sizeof(float2) * kPL + 16;
+  static constexpr int L = L_;
+  static constexpr bool PAIR = PAIR_;
+  // powers of two: two stages (radix G, then R2) with the half-size exchange;
+  // 3 * 2^m: the line engine (24 values, radices 8, 8, 12 at 768) with an
+  // exchange buffer of the tile's size
+  static constexpr bool ENGINE = L % 3 == 0;
+  static constexpr int G = ENGINE ? elems_per_thread(L) : (L >= 512 ? 32 : 16);  // values per thread
+  static constexpr int R2 = L / G;                  // radix of the second stage
+  static constexpr int S = L / G;                   // threads per line
+  static constexpr int T = L > 1024 ? 8 : 16;       // columns per tile (128-byte rows)
+  static constexpr int THREADS = S * T;
+  static constexpr int MINB = L >= 768 ? 1 : (L >= 384 ? 2 : 4);
+  static constexpr int ODD = PAIR ? T + 2 : T;      // float2 per staged odd row
+  static constexpr int ROWS = PAIR ? L / 2 : L;     // rows of a tensor
+  static constexpr int NBOX = (ROWS + 255) / 256;
+  static constexpr int BOXR = ROWS / NBOX;          // rows per box
+  static constexpr size_t STAGE = sizeof(float2) * (L / 2) * (T + ODD);
+  static constexpr size_t EX = (ENGINE ? sizeof(float2) : sizeof(float)) * L * T;
+  static constexpr size_t SMEM = STAGE + EX + (ENGINE ? 0 : sizeof(float2) * L) + 16;  // + the twiddles, the mbarrier
 };
 
-template <int SIGN, bool PAIR>
-__global__ void __launch_bounds__(kPThreads, 1)
+// Array [P][L][Q] of complex values, transform along L (element stride Q);
+// tile t = (p, q-tile).
+template <int L, int SIGN, bool PAIR>
+__global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::MINB)
     k_cpass_pipe(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_odd, float2* out,
-                 long long Q, int qtiles, int ntiles, const float2* __restrict__ tw, float scale, int* err) {
-  using C = PipeCfg<PAIR>;
+                 long long Q, int qtiles, int ntiles, const float2* __restrict__ tw, const float2* __restrict__ t3,
+                 float scale, int* err) {
+  using C = PipeCfg<L, PAIR>;
+  constexpr int G = C::G, S = C::S, T = C::T;
   extern __shared__ __align__(128) unsigned char smp[];
   __shared__ int ok_flag, next_tile;
   float2* stage = reinterpret_cast<float2*>(smp);
-  float2* odd = stage + (size_t)(kPL / 2) * kPT;  // PAIR: the odd rows
+  float2* odd = stage + (size_t)(L / 2) * T;  // PAIR: the odd rows
   float* ex = reinterpret_cast<float*>(smp + C::STAGE);
-  float2* stw = reinterpret_cast<float2*>(smp + C::STAGE + C::EX);
+  float2* stw = reinterpret_cast<float2*>(smp + C::STAGE + C::EX);  // (from global memory the gathers cost 3 %)
   uint64_t* bar = reinterpret_cast<uint64_t*>(smp + C::SMEM - 16);
-  const int tid = threadIdx.x, c = tid % kPT, j = tid / kPT;
-  for (int i = tid; i < kPL; i += kPThreads) stw[i] = tw[i];
+  const int tid = threadIdx.x, c = tid % T, j = tid / T;
+  if constexpr (!C::ENGINE)
+    for (int i = tid; i < L; i += C::THREADS) stw[i] = tw[i];
 
   auto fetch = [&](int t) {  // thread 0
-    const int p = t / qtiles, q0 = (t - p * qtiles) * kPT;
+    const int p = t / qtiles, q0 = (t - p * qtiles) * T;
     mbar_expect(bar, (uint32_t)C::STAGE);
-    if constexpr (PAIR) {
 #pragma unroll 1
-      for (int b = 0; b < 2; ++b) {
-        tma_load3(stage + (size_t)b * 256 * kPT, &map, 2 * q0, b * 256, p, bar);
-        tma_load3(odd + (size_t)b * 256 * C::ODD, &map_odd, 2 * q0, b * 256, p, bar);
-      }
-    } else {
-#pragma unroll 1
-      for (int b = 0; b < 4; ++b) tma_load3(stage + (size_t)b * 256 * kPT, &map, 2 * q0, b * 256, p, bar);
+    for (int b = 0; b < C::NBOX; ++b) {
+      tma_load3(stage + (size_t)b * C::BOXR * T, &map, 2 * q0, b * C::BOXR, p, bar);
+      if constexpr (PAIR) tma_load3(odd + (size_t)b * C::BOXR * C::ODD, &map_odd, 2 * q0, b * C::BOXR, p, bar);
     }
   };
-  // a warp holds two rows: rows 32 apart (the stores of the first stage) and
+  // a warp holds two rows: rows G apart (the stores of the first stage) and
   // neighbouring rows (the loads) each fall into different halves of the banks
-  auto slot = [&](int pos) { return ((pos ^ ((pos >> 5) & 1)) * kPT) + c; };
+  auto slot = [&](int pos) { return ((pos ^ ((pos / G) & 1)) * T) + c; };
   if (tid == 0) tcg::mbar_init(bar);
   __syncthreads();
   // Tiles are handed out in order (a counter; each CTA draws one ahead): were
   // each CTA to take every gridDim-th tile, the CTAs would drift apart over a
   // long pass, and neighbouring tiles, which share the lines of misaligned
   // rows, would meet in L2 no longer (1024^3 with every gridDim-th tile: x
-  // 1.60 ms, y 2.14 ms).
+  // 1.60 against 1.35 ms, y 2.14 against 1.37 ms).
   int* queue = err + 1;  // next tile, CTAs that are done
   uint32_t phase = 0;
   int t = blockIdx.x, drawn = 0;
@@ -182,7 +114,12 @@ __global__ void __launch_bounds__(kPThreads, 1)
       next_tile = drawn;
     }
     __syncthreads();
-    if (!ok_flag) {  // see k_cpass_tma
+    if (!ok_flag) {
+      // The tile never arrived: its copy may still be pending, writing into
+      // this CTA's shared memory and completing on the mbarrier there.  Thread
+      // 0 reports, then waits once more (bounded) for that copy before the
+      // CTA's shared memory is released; the other threads may leave.  The
+      // error word is the only signal: the host treats it as fatal for the plan.
       if (tid == 0) {
         atomicOr(err, 1);
         tcg::mbar_wait(bar, phase);
@@ -191,42 +128,55 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
     const int tn = next_tile;
     phase ^= 1;
-    float2 v[kPG];
-    const float2* src = !PAIR ? stage + j * kPT + c
-                              : (j & 1 ? odd + (j >> 1) * C::ODD + 1 + c : stage + (j >> 1) * kPT + c);
-    const int step = !PAIR ? kPS * kPT : (kPS / 2) * (j & 1 ? C::ODD : kPT);
+    float2 v[G];
+    const float2* src = !PAIR ? stage + j * T + c : (j & 1 ? odd + (j >> 1) * C::ODD + 1 + c : stage + (j >> 1) * T + c);
+    const int step = !PAIR ? S * T : (S / 2) * (j & 1 ? C::ODD : T);
 #pragma unroll
-    for (int m = 0; m < kPG; ++m) v[m] = src[m * step];
+    for (int m = 0; m < G; ++m) v[m] = src[m * step];
     __syncthreads();  // the staging buffer is free, and so is the exchange buffer
     if (tid == 0 && tn < ntiles) {
       tcg::fence_smem_async();
       fetch(tn);
       drawn = (int)gridDim.x + atomicAdd(queue, 1);
     }
-    dft32<SIGN>(v);
+    if constexpr (C::ENGINE) {
+      fft_line<L, G, SIGN>(v, j, ColX<T>{reinterpret_cast<float2*>(ex), c}, tw, t3);
+    } else {
+      constexpr int R2 = C::R2, B = G / R2;
+      dftR<G, SIGN>(v);
 #pragma unroll
-    for (int r = 0; r < kPG; ++r) ex[slot(j * kPG + r)] = v[r].x;
-    __syncthreads();
+      for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].x;
+      __syncthreads();
 #pragma unroll
-    for (int m = 0; m < kPG; ++m) v[m].x = ex[slot(j + m * kPS)];
-    __syncthreads();
+      for (int m = 0; m < G; ++m) v[m].x = ex[slot(j + m * S)];
+      __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kPG; ++r) ex[slot(j * kPG + r)] = v[r].y;
-    __syncthreads();
+      for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].y;
+      __syncthreads();
 #pragma unroll
-    for (int m = 0; m < kPG; ++m) v[m].y = ex[slot(j + m * kPS)];
+      for (int m = 0; m < G; ++m) v[m].y = ex[slot(j + m * S)];
+      // second stage: butterfly b = j + i S takes the values i + r B
 #pragma unroll
-    for (int r = 1; r < kPG; ++r) {
-      const float2 w = stw[r * j];
-      v[r] = SIGN < 0 ? cmul(v[r], w) : cmulc(v[r], w);
+      for (int i = 0; i < B; ++i) {
+        float2 a[R2];
+#pragma unroll
+        for (int r = 0; r < R2; ++r) a[r] = v[i + r * B];
+#pragma unroll
+        for (int r = 1; r < R2; ++r) {
+          const float2 w = stw[r * (j + i * S)];
+          a[r] = SIGN < 0 ? cmul(a[r], w) : cmulc(a[r], w);
+        }
+        dftR<R2, SIGN>(a);
+#pragma unroll
+        for (int r = 0; r < R2; ++r) v[i + r * B] = a[r];
+      }
     }
-    dft32<SIGN>(v);
     const int p = t / qtiles;
-    const long long q = (long long)(t - p * qtiles) * kPT + c;
+    const long long q = (long long)(t - p * qtiles) * T + c;
     if (q < Q) {
-      float2* dst = out + (long long)p * kPL * Q + q;
+      float2* dst = out + (long long)p * L * Q + q;
 #pragma unroll
-      for (int m = 0; m < kPG; ++m) dst[(long long)(j + m * kPS) * Q] = cscale(v[m], scale);
+      for (int m = 0; m < G; ++m) dst[(long long)(j + m * S) * Q] = cscale(v[m], scale);
     }
     t = tn;
   }
@@ -275,125 +225,80 @@ bool encode_f32_map(CUtensorMap* m, const void* base, int rank, const uint64_t* 
   return r == CUDA_SUCCESS;
 }
 
-// The 3D map [P][L][2Q] floats with boxes of 2T floats x 256 rows x 1; false
-// where the layout breaks a TMA rule (row stride not a multiple of 16 bytes,
-// base not 16-byte aligned, extents out of range) or no encoder exists.
-template <int L>
-static bool make_map(CUtensorMap* m, const float2* in, long long P, long long Q) {
-  using C = PFCfg<L>;
-  if (Q % 2 != 0 || reinterpret_cast<uintptr_t>(in) % 16 != 0) return false;
-  if (2 * Q >= (1LL << 31) || P >= (1LL << 31) || (long long)L * Q * 8 >= (1LL << 40)) return false;
-  auto enc = tensor_map_encoder();
-  if (!enc) return false;
-  std::memset(m, 0, sizeof(*m));
-  const cuuint64_t dims[3] = {(cuuint64_t)(2 * Q), (cuuint64_t)L, (cuuint64_t)P};
-  const cuuint64_t strides[2] = {(cuuint64_t)(8 * Q), (cuuint64_t)(8 * Q * L)};
-  const cuuint32_t box[3] = {(cuuint32_t)(2 * C::T), (cuuint32_t)C::BOXR, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float2*>(in), dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS;
-}
-
-template <int L, int SIGN>
-static cudaError_t cpass_tma_l(fftk_plan p, const CUtensorMap& m, float2* out, long long P, long long Q, float scale,
-                               int kind, cudaStream_t st) {
-  using C = PFCfg<L>;
-  static PerDevice once;
-  static int per_sm[kMaxDevices], nsm[kMaxDevices];
-  int dev = 0;
-  const cudaError_t attr_err = once.run(
-      [](int d) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_cpass_tma<L, SIGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-        if (e == cudaSuccess)
-          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[d], k_cpass_tma<L, SIGN>, C::THREADS, C::SMEM);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d);
-        if (e == cudaSuccess && per_sm[d] < 1) e = cudaErrorInvalidConfiguration;
-        return e;
-      },
-      &dev);
-  if (attr_err != cudaSuccess) return attr_err;
-  const long long qtiles = (Q + C::T - 1) / C::T;
-  const long long ntiles = P * qtiles;
-  const long long cap = (long long)nsm[dev] * per_sm[dev];
-  const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
-  LaunchScope ls(p, kind, st);
-  k_cpass_tma<L, SIGN><<<grid, C::THREADS, C::SMEM, st>>>(m, out, (int)Q, (int)qtiles, (int)ntiles, twiddles(p, L),
-                                                         scale, p->d_err);
-  return cudaGetLastError();
-}
-
-template <int L>
-static bool tma_map_l(CUtensorMap* m, const float2* in, long long P, long long Q) {
-  using C = PFCfg<L>;
-  if ((Q + C::T - 1) / C::T * P >= (1LL << 31)) return false;  // 32-bit tile indices
-  return make_map<L>(m, in, P, Q);
-}
-
-template <int SIGN, bool PAIR>
+template <int L, int SIGN, bool PAIR>
 static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorMap& mo, float2* out, long long P,
                               long long Q, float scale, int kind, cudaStream_t st) {
-  using C = PipeCfg<PAIR>;
+  using C = PipeCfg<L, PAIR>;
   static PerDevice once;
   static int nsm[kMaxDevices];
   int dev = 0;
   const cudaError_t e = once.run(
       [](int d) {
-        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<SIGN, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)C::SMEM);
+        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<L, SIGN, PAIR>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d);
         return err;
       },
       &dev);
   if (e != cudaSuccess) return e;
-  const long long qtiles = (Q + kPT - 1) / kPT, ntiles = P * qtiles;
-  const unsigned grid = (unsigned)(ntiles < nsm[dev] ? ntiles : nsm[dev]);
+  const long long qtiles = (Q + C::T - 1) / C::T, ntiles = P * qtiles, cap = (long long)nsm[dev] * C::MINB;
+  const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   LaunchScope ls(p, kind, st);
-  k_cpass_pipe<SIGN, PAIR><<<grid, kPThreads, C::SMEM, st>>>(m, mo, out, Q, (int)qtiles, (int)ntiles,
-                                                            twiddles(p, kPL), scale, p->d_err);
+  k_cpass_pipe<L, SIGN, PAIR><<<grid, C::THREADS, C::SMEM, st>>>(
+      m, mo, out, Q, (int)qtiles, (int)ntiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3, scale, p->d_err);
   return cudaGetLastError();
 }
 
-// The maps of even and odd rows for odd Q: [P][kPL / 2][2 Q] and, 8 bytes
-// before row 1, [P][kPL / 2][2 (Q + 1)] floats, row stride 16 Q bytes.  The
-// last element of the second is the last of the array.
-static bool pair_maps(CUtensorMap* even, CUtensorMap* odd, const float2* in, long long P, long long Q) {
-  if (8LL * Q * kPL >= (1LL << 40) || 2 * (Q + 1) >= (1LL << 31) || P >= (1LL << 31)) return false;
-  const uint64_t strides[2] = {(uint64_t)(16 * Q), (uint64_t)(8 * Q * kPL)};
-  const uint64_t de[3] = {(uint64_t)(2 * Q), kPL / 2, (uint64_t)P}, dd[3] = {(uint64_t)(2 * (Q + 1)), kPL / 2, (uint64_t)P};
-  const uint32_t be[3] = {2 * kPT, 256, 1}, bo[3] = {2 * PipeCfg<true>::ODD, 256, 1};
-  return encode_f32_map(even, in, 3, de, strides, be) && encode_f32_map(odd, in + Q - 1, 3, dd, strides, bo);
+// The maps of a pass: [P][L][2 Q] floats for even Q; for odd Q those of the
+// even rows, [P][L / 2][2 Q], and, from 8 bytes before row 1, of the odd rows,
+// [P][L / 2][2 (Q + 1)], with a row stride of 16 Q bytes (the last element of
+// the second is the last of the array).
+template <int L>
+static bool pipe_maps(CUtensorMap* m, CUtensorMap* mo, const float2* in, long long P, long long Q) {
+  using E = PipeCfg<L, false>;
+  using O = PipeCfg<L, true>;
+  if (8LL * Q * L >= (1LL << 40) || 2 * (Q + 1) >= (1LL << 31) || P >= (1LL << 31)) return false;
+  const uint64_t rows = Q % 2 == 0 ? L : L / 2;
+  const uint64_t strides[2] = {(uint64_t)(8 * Q * (L / (long long)rows)), (uint64_t)(8 * Q * L)};
+  const uint64_t dims[3] = {(uint64_t)(2 * Q), rows, (uint64_t)P};
+  const uint32_t box[3] = {2 * E::T, (uint32_t)(Q % 2 == 0 ? E::BOXR : O::BOXR), 1};
+  if (!encode_f32_map(m, in, 3, dims, strides, box)) return false;
+  if (Q % 2 == 0) return true;
+  const uint64_t dims_odd[3] = {(uint64_t)(2 * (Q + 1)), rows, (uint64_t)P};
+  const uint32_t box_odd[3] = {2 * O::ODD, O::BOXR, 1};
+  return encode_f32_map(mo, in + Q - 1, 3, dims_odd, strides, box_odd);
 }
 
+template <int L>
+static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long long P, long long Q, float scale, int kind,
+                   cudaStream_t st, cudaError_t* e) {
+  CUtensorMap m{}, mo{};
+  if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
+  if (Q % 2 == 0)
+    *e = sign < 0 ? cpass_pipe<L, -1, false>(p, m, m, out, P, Q, scale, kind, st)
+                  : cpass_pipe<L, +1, false>(p, m, m, out, P, Q, scale, kind, st);
+  else
+    *e = sign < 0 ? cpass_pipe<L, -1, true>(p, m, mo, out, P, Q, scale, kind, st)
+                  : cpass_pipe<L, +1, true>(p, m, mo, out, P, Q, scale, kind, st);
+  return true;
+}
+
+// Arrays narrower than a tile, bases off 16 bytes and (below 768 points, where
+// the general pass has several CTAs per SM) passes of less than two tiles per
+// SM keep the general pass: false, nothing launched.  (64 fields of 512 x 32:
+// 37 us a pair through k_cpass, 42 us here; 450 tiles of 256 x 16: the same.)
 bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
                       float scale, int kind, cudaStream_t st, cudaError_t* e) {
-  if (P <= 0 || Q <= 0) return false;
-  CUtensorMap m{};
-  if (L == kPL) {
-    // narrow arrays and bases off 16 bytes keep the general pass
-    if (Q < kPT || reinterpret_cast<uintptr_t>(in) % 16 != 0 || P * ((Q + kPT - 1) / kPT) >= (1LL << 31)) return false;
-    if (Q % 2 == 0) {
-      if (!tma_map_l<kPL>(&m, in, P, Q)) return false;
-      *e = sign < 0 ? cpass_pipe<-1, false>(p, m, m, out, P, Q, scale, kind, st)
-                    : cpass_pipe<+1, false>(p, m, m, out, P, Q, scale, kind, st);
-    } else {
-      CUtensorMap mo{};
-      if (!pair_maps(&m, &mo, in, P, Q)) return false;
-      *e = sign < 0 ? cpass_pipe<-1, true>(p, m, mo, out, P, Q, scale, kind, st)
-                    : cpass_pipe<+1, true>(p, m, mo, out, P, Q, scale, kind, st);
-    }
-    return true;
-  }
-#define CASE(n)                                                                                  \
-  case n:                                                                                        \
-    if (!tma_map_l<n>(&m, in, P, Q)) return false;                                               \
-    *e = sign < 0 ? cpass_tma_l<n, -1>(p, m, out, P, Q, scale, kind, st)                         \
-                  : cpass_tma_l<n, +1>(p, m, out, P, Q, scale, kind, st);                        \
-    return true;
-  switch (L) { CASE(512) }
+  if (P <= 0 || Q < 16 || reinterpret_cast<uintptr_t>(in) % 16 != 0) return false;
+  const long long tiles = P * ((Q + 7) / 8);  // of eight columns
+  if (tiles >= (1LL << 31) || (L < 768 && tiles < 4 * 152)) return false;
+  switch (L) {
+#define CASE(n) \
+  case n:       \
+    return pipe_l<n>(p, sign, in, out, P, Q, scale, kind, st, e);
+    CASE(256) CASE(384) CASE(512) CASE(768) CASE(1024) CASE(1536)
 #undef CASE
+  }
   return false;
 }
 
