@@ -23,24 +23,9 @@
 #include "fft_engine.cuh"
 #include "internal.h"
 #include "ns_common.cuh"
+#include "sc_algebra.cuh"
 
 namespace fftk {
-
-__device__ __forceinline__ int mk_perm(int r, int L) { return r < L / 2 ? 2 * r : 2 * (L - 1 - r) + 1; }
-// position r of element i in the permuted line
-__device__ __forceinline__ int mk_unperm(int i, int L) { return (i & 1) ? L - 1 - (i >> 1) : (i >> 1); }
-
-// C_k from V_k, V_{L-k} and W_k
-__device__ __forceinline__ float2 mk_post(float2 vk, float2 vn, float2 w) {
-  const float2 a = cmul(w, vk), b = cmulc(vn, w);  // W V_k, conj(W) V_{L-k}
-  return make_float2(0.5f * (a.x + b.x), 0.5f * (a.y + b.y));
-}
-
-// V_k = conj(W_k) (C_k - i C_{L-k})
-__device__ __forceinline__ float2 mk_pre(float2 ck, float2 cn, float2 w) {
-  const float2 d = make_float2(ck.x + cn.y, ck.y - cn.x);  // C_k - i C_{L-k}
-  return cmulc(d, w);
-}
 
 // --------------------------------------------------------- strided pass --
 template <int L>
@@ -75,7 +60,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int r = j + m * S;
-      float2 x = valid ? in[base + (long long)mk_perm(r, L) * Q] : make_float2(0.f, 0.f);
+      float2 x = valid ? in[base + (long long)sc_perm(r, L) * Q] : make_float2(0.f, 0.f);
       if (SINE && r >= L / 2) x = make_float2(-x.x, -x.y);  // (-1)^j at odd j
       v[m] = x;
     }
@@ -87,7 +72,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
 #pragma unroll
       for (int m = 0; m < G; ++m) {
         const int k = j + m * S;
-        const float2 ck = mk_post(v[m], xc.ld((L - k) & (L - 1)), __ldg(&tq[k]));
+        const float2 ck = sc_post(v[m], xc.ld((L - k) & (L - 1)), __ldg(&tq[k]));
         const float f = (k == 0 ? 0.5f : 1.f) * scale;
         const int row = SINE ? L - 1 - k : k;
         out[base + (long long)row * Q] = cscale(ck, f);
@@ -110,7 +95,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
       const float2 cn = k == 0 ? make_float2(0.f, 0.f) : xc.ld(L - k);
-      w[m] = mk_pre(v[m], cn, __ldg(&tq[k]));
+      w[m] = sc_pre(v[m], cn, __ldg(&tq[k]));
     }
     xc.sync();
     fft_line<L, G, +1>(w, j, xc, tw);
@@ -120,7 +105,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
         const int r = j + m * S;
         float2 x = w[m];
         if (SINE && r >= L / 2) x = make_float2(-x.x, -x.y);
-        out[base + (long long)mk_perm(r, L) * Q] = cscale(x, scale);
+        out[base + (long long)sc_perm(r, L) * Q] = cscale(x, scale);
       }
     }
   }
@@ -157,7 +142,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int r = j + m * S;
-      float2 x = valid ? in[base + (long long)mk_perm(r, L) * Q] : make_float2(0.f, 0.f);
+      float2 x = valid ? in[base + (long long)sc_perm(r, L) * Q] : make_float2(0.f, 0.f);
       if (SINE && r >= L / 2) x = make_float2(-x.x, -x.y);
       v[m] = x;
     }
@@ -171,7 +156,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
         const int k = j + m * S;
         const int row = SINE ? L - 1 - k : k;
         if (!kept_row(row)) continue;
-        const float2 ck = mk_post(v[m], xc.ld((L - k) & (L - 1)), __ldg(&tq[k]));
+        const float2 ck = sc_post(v[m], xc.ld((L - k) & (L - 1)), __ldg(&tq[k]));
         out[base + (long long)row * Q] = cscale(ck, (k == 0 ? 0.5f : 1.f) * scale);
       }
     }
@@ -191,7 +176,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
       const float2 cn = k == 0 ? make_float2(0.f, 0.f) : xc.ld(L - k);
-      w[m] = mk_pre(v[m], cn, __ldg(&tq[k]));
+      w[m] = sc_pre(v[m], cn, __ldg(&tq[k]));
     }
     xc.sync();
     fft_line<L, G, +1>(w, j, xc, tw);
@@ -201,7 +186,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
         const int r = j + m * S;
         float2 x = w[m];
         if (SINE && r >= L / 2) x = make_float2(-x.x, -x.y);
-        out[base + (long long)mk_perm(r, L) * Q] = cscale(x, scale);
+        out[base + (long long)sc_perm(r, L) * Q] = cscale(x, scale);
       }
     }
   }
@@ -242,7 +227,7 @@ __global__ void __launch_bounds__(SZCfg<N>::THREADS)
       const int i = j + m * S;
       float2 x = make_float2(va ? ia[i] : 0.f, vb ? ib[i] : 0.f);
       if (SINE && (i & 1)) x = make_float2(-x.x, -x.y);
-      xc.st(mk_unperm(i, N), x);
+      xc.st(sc_unperm(i, N), x);
     }
     xc.sync();
 #pragma unroll
@@ -255,7 +240,7 @@ __global__ void __launch_bounds__(SZCfg<N>::THREADS)
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
-      const float2 ck = mk_post(v[m], xc.ld((N - k) & (N - 1)), __ldg(&tq[k]));
+      const float2 ck = sc_post(v[m], xc.ld((N - k) & (N - 1)), __ldg(&tq[k]));
       const float f = (k == 0 ? 0.5f : 1.f) * scale;
       const int row = SINE ? N - 1 - k : k;
       if (va) oa[row] = ck.x * f;
@@ -277,7 +262,7 @@ __global__ void __launch_bounds__(SZCfg<N>::THREADS)
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
       const float2 cn = k == 0 ? make_float2(0.f, 0.f) : xc.ld(N - k);
-      w[m] = mk_pre(v[m], cn, __ldg(&tq[k]));
+      w[m] = sc_pre(v[m], cn, __ldg(&tq[k]));
     }
     xc.sync();
     fft_line<N, G, +1, LOGN>(w, j, xc, tw);
@@ -287,7 +272,7 @@ __global__ void __launch_bounds__(SZCfg<N>::THREADS)
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int i = j + m * S;
-      float2 x = xc.ld(mk_unperm(i, N));
+      float2 x = xc.ld(sc_unperm(i, N));
       if (SINE && (i & 1)) x = make_float2(-x.x, -x.y);
       if (va) oa[i] = x.x * scale;
       if (vb) ob[i] = x.y * scale;
@@ -346,6 +331,8 @@ static cudaError_t scpass_pr_l(fftk_plan p, const float2* in, float2* out, long 
 cudaError_t launch_scpass(fftk_plan p, int L, bool sine, int dir, const float2* in, float2* out, long long P,
                           long long Q, float scale, int kind, cudaStream_t st) {
   if (P <= 0 || Q <= 0) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  if (launch_scpass_tma(p, L, sine, dir, in, out, P, Q, scale, kind, st, &e)) return e;
 #define CASE(n)                                                                                   \
   case n:                                                                                         \
     if (sine)                                                                                     \

@@ -26,6 +26,7 @@
 
 #include "fft_engine.cuh"
 #include "internal.h"
+#include "sc_algebra.cuh"
 #include "tcgen05.cuh"
 
 namespace fftk {
@@ -49,6 +50,7 @@ struct PipeCfg {
   static constexpr bool ENGINE = L % 3 == 0;
   static constexpr int G = ENGINE ? elems_per_thread(L) : (L >= 512 ? 32 : 16);  // values per thread
   static constexpr int R2 = L / G;                  // radix of the second stage
+  static constexpr bool PAIRED = L == 512;          // two butterflies per thread in the second stage
   static constexpr int S = L / G;                   // threads per line
   static constexpr int T = L > 1024 ? 8 : 16;       // columns per tile (128-byte rows)
   static constexpr int THREADS = S * T;
@@ -64,11 +66,16 @@ struct PipeCfg {
 
 // Array [P][L][Q] of complex values, transform along L (element stride Q);
 // tile t = (p, q-tile).
-template <int L, int SIGN, bool PAIR>
+// BASIS: 0 Fourier, 1 cosine, 2 sine (fft_sc.cu states the reduction to one
+// complex transform): forward (SIGN -1), the samples are read from the staged
+// tile in permuted order and the result is combined with its mirror through
+// the exchange buffer; inverse, the mirror coefficient comes from the staged
+// tile and the rows are stored in permuted order.
+template <int L, int SIGN, bool PAIR, int BASIS>
 __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::MINB)
     k_cpass_pipe(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_odd, float2* out,
                  long long Q, int qtiles, int ntiles, const float2* __restrict__ tw, const float2* __restrict__ t3,
-                 float scale, int* err) {
+                 const float2* __restrict__ tq, float scale, int* err) {
   using C = PipeCfg<L, PAIR>;
   constexpr int G = C::G, S = C::S, T = C::T;
   extern __shared__ __align__(128) unsigned char smp[];
@@ -129,10 +136,34 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
     const int tn = next_tile;
     phase ^= 1;
     float2 v[G];
-    const float2* src = !PAIR ? stage + j * T + c : (j & 1 ? odd + (j >> 1) * C::ODD + 1 + c : stage + (j >> 1) * T + c);
-    const int step = !PAIR ? S * T : (S / 2) * (j & 1 ? C::ODD : T);
+    auto staged = [&](int row) -> float2 {
+      return !PAIR ? stage[row * T + c] : (row & 1 ? odd[(row >> 1) * C::ODD + 1 + c] : stage[(row >> 1) * T + c]);
+    };
+    if constexpr (BASIS == 0) {
+      const float2* src =
+          !PAIR ? stage + j * T + c : (j & 1 ? odd + (j >> 1) * C::ODD + 1 + c : stage + (j >> 1) * T + c);
+      const int step = !PAIR ? S * T : (S / 2) * (j & 1 ? C::ODD : T);
 #pragma unroll
-    for (int m = 0; m < G; ++m) v[m] = src[m * step];
+      for (int m = 0; m < G; ++m) v[m] = src[m * step];
+    } else if constexpr (SIGN < 0) {
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        const int r = j + m * S;
+        const float2 x = staged(sc_perm(r, L));
+        v[m] = BASIS == 2 && r >= L / 2 ? make_float2(-x.x, -x.y) : x;  // (-1)^j at odd j
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        const int k = j + m * S;
+        float2 x = staged(BASIS == 2 ? L - 1 - k : k), n = make_float2(0.f, 0.f);
+        if (k == 0)
+          x = cscale(x, 2.f);
+        else
+          n = staged(BASIS == 2 ? k - 1 : L - k);
+        v[m] = sc_pre(x, n, __ldg(&tq[k]));
+      }
+    }
     __syncthreads();  // the staging buffer is free, and so is the exchange buffer
     if (tid == 0 && tn < ntiles) {
       tcg::fence_smem_async();
@@ -143,19 +174,23 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
       fft_line<L, G, SIGN>(v, j, ColX<T>{reinterpret_cast<float2*>(ex), c}, tw, t3);
     } else {
       constexpr int R2 = C::R2, B = G / R2;
+      // butterfly i of this thread's second stage; with two of them a thread
+      // of a forward sine/cosine line takes b and G - b, whose outputs are
+      // each other's mirrors (of j = 0: 0 and G / 2, their own)
+      auto bf = [&](int i) { return C::PAIRED && BASIS && SIGN < 0 && i == 1 ? (j == 0 ? G / 2 : G - j) : j + i * S; };
       dftR<G, SIGN>(v);
 #pragma unroll
       for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].x;
       __syncthreads();
 #pragma unroll
-      for (int m = 0; m < G; ++m) v[m].x = ex[slot(j + m * S)];
+      for (int m = 0; m < G; ++m) v[m].x = ex[slot(bf(m % B) + m / B * G)];
       __syncthreads();
 #pragma unroll
       for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].y;
       __syncthreads();
 #pragma unroll
-      for (int m = 0; m < G; ++m) v[m].y = ex[slot(j + m * S)];
-      // second stage: butterfly b = j + i S takes the values i + r B
+      for (int m = 0; m < G; ++m) v[m].y = ex[slot(bf(m % B) + m / B * G)];
+      // second stage: butterfly i takes the values i + r B
 #pragma unroll
       for (int i = 0; i < B; ++i) {
         float2 a[R2];
@@ -163,7 +198,7 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
         for (int r = 0; r < R2; ++r) a[r] = v[i + r * B];
 #pragma unroll
         for (int r = 1; r < R2; ++r) {
-          const float2 w = stw[r * (j + i * S)];
+          const float2 w = stw[r * bf(i)];
           a[r] = SIGN < 0 ? cmul(a[r], w) : cmulc(a[r], w);
         }
         dftR<R2, SIGN>(a);
@@ -173,10 +208,58 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
     }
     const int p = t / qtiles;
     const long long q = (long long)(t - p * qtiles) * T + c;
-    if (q < Q) {
-      float2* dst = out + (long long)p * L * Q + q;
+    float2* dst = out + (long long)p * L * Q + q;
+    if constexpr (BASIS == 0) {
+      if (q < Q) {
 #pragma unroll
-      for (int m = 0; m < G; ++m) dst[(long long)(j + m * S) * Q] = cscale(v[m], scale);
+        for (int m = 0; m < G; ++m) dst[(long long)(j + m * S) * Q] = cscale(v[m], scale);
+      }
+    } else if constexpr (SIGN > 0) {
+      if (q < Q) {
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+          const int r = j + m * S;
+          const float2 x = BASIS == 2 && r >= L / 2 ? make_float2(-v[m].x, -v[m].y) : v[m];
+          dst[(long long)sc_perm(r, L) * Q] = cscale(x, scale);
+        }
+      }
+    } else if constexpr (C::PAIRED) {
+      constexpr int R2 = C::R2;
+      if (q < Q) {
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+          const int i = m & 1, r = m >> 1;
+          const int k = (i == 0 ? j : (j == 0 ? G / 2 : G - j)) + r * G;
+          const float2 own = v[i == 0 ? 2 * ((R2 - r) % R2) : 1 + 2 * (R2 - 1 - r)];  // j = 0
+          const float2 other = v[(1 - i) + 2 * (R2 - 1 - r)];
+          const float2 n = j == 0 ? own : other;
+          const float2 ck = sc_post(v[m], n, __ldg(&tq[k]));
+          dst[(long long)(BASIS == 2 ? L - 1 - k : k) * Q] = cscale(ck, (k == 0 ? 0.5f : 1.f) * scale);
+        }
+      }
+    } else {
+      // the mirrors V[L - k], real parts and then imaginary ones
+      float2 n[G];
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < G; ++m) ex[slot(j + m * S)] = v[m].x;
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < G; ++m) n[m].x = ex[slot((L - (j + m * S)) & (L - 1))];
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < G; ++m) ex[slot(j + m * S)] = v[m].y;
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < G; ++m) n[m].y = ex[slot((L - (j + m * S)) & (L - 1))];
+      if (q < Q) {
+#pragma unroll
+        for (int m = 0; m < G; ++m) {
+          const int k = j + m * S;
+          const float2 ck = sc_post(v[m], n[m], __ldg(&tq[k]));
+          dst[(long long)(BASIS == 2 ? L - 1 - k : k) * Q] = cscale(ck, (k == 0 ? 0.5f : 1.f) * scale);
+        }
+      }
     }
     t = tn;
   }
@@ -225,7 +308,7 @@ bool encode_f32_map(CUtensorMap* m, const void* base, int rank, const uint64_t* 
   return r == CUDA_SUCCESS;
 }
 
-template <int L, int SIGN, bool PAIR>
+template <int L, int SIGN, bool PAIR, int BASIS>
 static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorMap& mo, float2* out, long long P,
                               long long Q, float scale, int kind, cudaStream_t st) {
   using C = PipeCfg<L, PAIR>;
@@ -234,7 +317,7 @@ static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorM
   int dev = 0;
   const cudaError_t e = once.run(
       [](int d) {
-        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<L, SIGN, PAIR>,
+        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<L, SIGN, PAIR, BASIS>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d);
         return err;
@@ -244,8 +327,9 @@ static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorM
   const long long qtiles = (Q + C::T - 1) / C::T, ntiles = P * qtiles, cap = (long long)nsm[dev] * C::MINB;
   const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   LaunchScope ls(p, kind, st);
-  k_cpass_pipe<L, SIGN, PAIR><<<grid, C::THREADS, C::SMEM, st>>>(
-      m, mo, out, Q, (int)qtiles, (int)ntiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3, scale, p->d_err);
+  k_cpass_pipe<L, SIGN, PAIR, BASIS><<<grid, C::THREADS, C::SMEM, st>>>(
+      m, mo, out, Q, (int)qtiles, (int)ntiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3,
+      BASIS ? twiddles(p, 4 * L) : nullptr, scale, p->d_err);
   return cudaGetLastError();
 }
 
@@ -269,17 +353,17 @@ static bool pipe_maps(CUtensorMap* m, CUtensorMap* mo, const float2* in, long lo
   return encode_f32_map(mo, in + Q - 1, 3, dims_odd, strides, box_odd);
 }
 
-template <int L>
+template <int L, int BASIS>
 static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long long P, long long Q, float scale, int kind,
                    cudaStream_t st, cudaError_t* e) {
   CUtensorMap m{}, mo{};
   if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
   if (Q % 2 == 0)
-    *e = sign < 0 ? cpass_pipe<L, -1, false>(p, m, m, out, P, Q, scale, kind, st)
-                  : cpass_pipe<L, +1, false>(p, m, m, out, P, Q, scale, kind, st);
+    *e = sign < 0 ? cpass_pipe<L, -1, false, BASIS>(p, m, m, out, P, Q, scale, kind, st)
+                  : cpass_pipe<L, +1, false, BASIS>(p, m, m, out, P, Q, scale, kind, st);
   else
-    *e = sign < 0 ? cpass_pipe<L, -1, true>(p, m, mo, out, P, Q, scale, kind, st)
-                  : cpass_pipe<L, +1, true>(p, m, mo, out, P, Q, scale, kind, st);
+    *e = sign < 0 ? cpass_pipe<L, -1, true, BASIS>(p, m, mo, out, P, Q, scale, kind, st)
+                  : cpass_pipe<L, +1, true, BASIS>(p, m, mo, out, P, Q, scale, kind, st);
   return true;
 }
 
@@ -287,16 +371,34 @@ static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long lo
 // the general pass has several CTAs per SM) passes of less than two tiles per
 // SM keep the general pass: false, nothing launched.  (64 fields of 512 x 32:
 // 37 us a pair through k_cpass, 42 us here; 450 tiles of 256 x 16: the same.)
-bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
-                      float scale, int kind, cudaStream_t st, cudaError_t* e) {
+static bool pipe_applies(int L, const float2* in, long long P, long long Q) {
   if (P <= 0 || Q < 16 || reinterpret_cast<uintptr_t>(in) % 16 != 0) return false;
   const long long tiles = P * ((Q + 7) / 8);  // of eight columns
-  if (tiles >= (1LL << 31) || (L < 768 && tiles < 4 * 152)) return false;
+  return tiles < (1LL << 31) && (L >= 768 || tiles >= 4 * 152);
+}
+
+bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
+                      float scale, int kind, cudaStream_t st, cudaError_t* e) {
+  if (!pipe_applies(L, in, P, Q)) return false;
   switch (L) {
 #define CASE(n) \
   case n:       \
-    return pipe_l<n>(p, sign, in, out, P, Q, scale, kind, st, e);
+    return pipe_l<n, 0>(p, sign, in, out, P, Q, scale, kind, st, e);
     CASE(256) CASE(384) CASE(512) CASE(768) CASE(1024) CASE(1536)
+#undef CASE
+  }
+  return false;
+}
+
+bool launch_scpass_tma(fftk_plan p, int L, bool sine, int dir, const float2* in, float2* out, long long P, long long Q,
+                       float scale, int kind, cudaStream_t st, cudaError_t* e) {
+  if (!pipe_applies(L, in, P, Q)) return false;
+  switch (L) {
+#define CASE(n) \
+  case n:       \
+    return sine ? pipe_l<n, 2>(p, dir, in, out, P, Q, scale, kind, st, e) \
+                : pipe_l<n, 1>(p, dir, in, out, P, Q, scale, kind, st, e);
+    CASE(256) CASE(512) CASE(1024)
 #undef CASE
   }
   return false;

@@ -164,6 +164,9 @@ bool cpass_tc_supported(int L);
 // a tile, base not 16-byte aligned), else true with the launch status in *e
 bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
                       float scale, int kind, cudaStream_t st, cudaError_t* e);
+// the same for sine/cosine lines of 256, 512 and 1024 points
+bool launch_scpass_tma(fftk_plan p, int L, bool sine, int dir, const float2* in, float2* out, long long P, long long Q,
+                       float scale, int kind, cudaStream_t st, cudaError_t* e);
 // the split-FP16 pass restricted to the 2/3-rule set of an n^3 spectrum
 // (axis 0: x lines, 1: y lines; n of 256, 512 or 1024), as launch_pruned_x/y
 cudaError_t launch_cpass_tc_pruned(fftk_plan p, int axis, int sign, const float2* in, float2* out, long long B,

@@ -54,3 +54,32 @@ def test_pipelined_passes_match_oracle(fk, oracle_mod, shape):
     assert rel_l2(Fg, want) < 2e-6
     assert np.max(np.abs(Fg - want)) < 1e-5 * np.max(np.abs(want))
     assert rel_l2(yg, f) < 2e-6
+
+
+@pytest.mark.parametrize("basis", ["SCF", "CSF", "SCC", "SFF"])
+@pytest.mark.parametrize("shape", [(128, 256, 64), (256, 128, 64), (128, 512, 64), (512, 64, 128), (8, 1024, 64),
+                                   (1024, 16, 32)])
+def test_pipelined_sine_cosine_passes_match_oracle(fk, oracle_mod, shape, basis):
+    import torch
+
+    f = synth.uniform_pm1(62, 0, shape)
+    nx, ny, nz = shape
+    plan = fk.fftk_plan_create(nx, ny, nz)
+    try:
+        x = torch.from_numpy(np.ascontiguousarray(f, dtype=np.float32)).to("cuda:0")
+        half = basis[2] == "F"
+        F = torch.empty((nx, ny, nz // 2 + 1, 2) if half else (nx, ny, nz), dtype=torch.float32, device="cuda:0")
+        y = torch.empty_like(x)
+        for _ in range(2):
+            fk.fftk_forward(plan, basis, x.data_ptr(), F.data_ptr(), 1, stream())
+            fk.fftk_inverse(plan, basis, F.data_ptr(), y.data_ptr(), 1, stream())
+        fk.fftk_sync(plan, stream())
+        sync()
+        Fg = from_dev_c64(F) if half else F.cpu().numpy().astype(np.float64)
+        yg = y.cpu().numpy()
+    finally:
+        fk.fftk_plan_destroy(plan)
+    want = oracle_mod.transform3(f.astype(np.float64), basis)
+    assert rel_l2(Fg, want) < 2e-6
+    assert np.max(np.abs(Fg - want)) < 1e-5 * np.max(np.abs(want))
+    assert rel_l2(yg, f) < 2e-6
