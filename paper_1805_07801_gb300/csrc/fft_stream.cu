@@ -24,7 +24,7 @@
 #include <cstring>
 #include <mutex>
 
-#include "fft_engine.cuh"
+#include "fft_pipe.cuh"
 #include "internal.h"
 #include "sc_algebra.cuh"
 #include "tcgen05.cuh"
@@ -98,17 +98,10 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
       if constexpr (PAIR) tma_load3(odd + (size_t)b * C::BOXR * C::ODD, &map_odd, 2 * q0, b * C::BOXR, p, bar);
     }
   };
-  // a warp holds two rows: rows G apart (the stores of the first stage) and
-  // neighbouring rows (the loads) each fall into different halves of the banks
-  auto slot = [&](int pos) { return ((pos ^ ((pos / G) & 1)) * T) + c; };
+  auto slot = [&](int pos) { return pipe_slot<G, T>(pos, c); };
   if (tid == 0) tcg::mbar_init(bar);
   __syncthreads();
-  // Tiles are handed out in order (a counter; each CTA draws one ahead): were
-  // each CTA to take every gridDim-th tile, the CTAs would drift apart over a
-  // long pass, and neighbouring tiles, which share the lines of misaligned
-  // rows, would meet in L2 no longer (1024^3 with every gridDim-th tile: x
-  // 1.60 against 1.35 ms, y 2.14 against 1.37 ms).
-  int* queue = err + 1;  // next tile, CTAs that are done
+  int* queue = err + 1;  // next tile, CTAs that are done (fft_pipe.cuh)
   uint32_t phase = 0;
   int t = blockIdx.x, drawn = 0;
   if (tid == 0) {
@@ -170,42 +163,10 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
       fetch(tn);
       drawn = (int)gridDim.x + atomicAdd(queue, 1);
     }
-    if constexpr (C::ENGINE) {
+    if constexpr (C::ENGINE)
       fft_line<L, G, SIGN>(v, j, ColX<T>{reinterpret_cast<float2*>(ex), c}, tw, t3);
-    } else {
-      constexpr int R2 = C::R2, B = G / R2;
-      // butterfly i of this thread's second stage; with two of them a thread
-      // of a forward sine/cosine line takes b and G - b, whose outputs are
-      // each other's mirrors (of j = 0: 0 and G / 2, their own)
-      auto bf = [&](int i) { return C::PAIRED && BASIS && SIGN < 0 && i == 1 ? (j == 0 ? G / 2 : G - j) : j + i * S; };
-      dftR<G, SIGN>(v);
-#pragma unroll
-      for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].x;
-      __syncthreads();
-#pragma unroll
-      for (int m = 0; m < G; ++m) v[m].x = ex[slot(bf(m % B) + m / B * G)];
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < G; ++r) ex[slot(j * G + r)] = v[r].y;
-      __syncthreads();
-#pragma unroll
-      for (int m = 0; m < G; ++m) v[m].y = ex[slot(bf(m % B) + m / B * G)];
-      // second stage: butterfly i takes the values i + r B
-#pragma unroll
-      for (int i = 0; i < B; ++i) {
-        float2 a[R2];
-#pragma unroll
-        for (int r = 0; r < R2; ++r) a[r] = v[i + r * B];
-#pragma unroll
-        for (int r = 1; r < R2; ++r) {
-          const float2 w = stw[r * bf(i)];
-          a[r] = SIGN < 0 ? cmul(a[r], w) : cmulc(a[r], w);
-        }
-        dftR<R2, SIGN>(a);
-#pragma unroll
-        for (int r = 0; r < R2; ++r) v[i + r * B] = a[r];
-      }
-    }
+    else
+      pipe_transform<L, G, SIGN, T, (C::PAIRED && BASIS != 0 && SIGN < 0)>(v, j, c, ex, stw);
     const int p = t / qtiles;
     const long long q = (long long)(t - p * qtiles) * T + c;
     float2* dst = out + (long long)p * L * Q + q;
@@ -263,10 +224,7 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
     }
     t = tn;
   }
-  if (tid == 0 && atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {  // the last CTA leaves the counters at zero
-    queue[0] = 0;
-    queue[1] = 0;
-  }
+  if (tid == 0) pipe_leave(queue);
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {

@@ -51,23 +51,7 @@ __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
   for (int m = 0; m < G; ++m) {
     const int pos = j + m * S;
     const bool rd = valid && (SIGN < 0 || kept_xy(pos, N, KD));
-    v[m] = rd ? (SIGN < 0 ? wo[off + (long long)pos * H1] : __ldg(&w[off + (long long)pos * H1]))
-              : make_float2(0.f, 0.f);
-  }
-  constexpr int AHEAD = N >= 768 ? 152 : (N == 512 && SIGN > 0 ? 304 : 0);  // tiles
-  if constexpr (AHEAD > 0) {
-    // One CTA holds the SM: while it transforms, the rows of the tile that
-    // comes next on some SM (CTAs start in order) go to L2.  768^3, per launch:
-    // inverse 3.06 -> 2.43 ms, forward 1.52 -> 1.16 ms.  512^3 (two CTAs per
-    // SM): inverse in place (convection) 795 -> 747 us, out of place 646 -> 641;
-    // the forward pass, 310 against 315 us, does without.
-    const long long nb = (long long)blockIdx.x + AHEAD;
-    if (nb < gridDim.x) {
-      const long long nr = nb / ktiles;  // f N + x of that tile
-      const float2* src = (SIGN < 0 ? wo : w) + (nr / N) * MM + (nr % N) * N * H1 + (nb - nr * ktiles) * T;
-      for (int r = threadIdx.x; r < (SIGN < 0 ? N : 2 * KD + 1); r += C::THREADS)
-        prefetch_l2(src + (long long)(SIGN < 0 ? r : dense_to_a(r, N, KD)) * H1);
-    }
+    v[m] = rd ? w[off + (long long)pos * H1] : make_float2(0.f, 0.f);
   }
   fft_line<N, G, SIGN>(v, j, ColX<T>{smn, c}, tw, t3);
   if (valid) {
@@ -401,6 +385,11 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
   r2c(1, Ny);
 }
 
+// y pass of `fields` fields on padded rows (ns_ypass.cu): sign +1 reads the kept
+// rows and writes every row, -1 reads every row and writes the kept ones; out
+// may be in.
+cudaError_t ns_ypass(fftk_plan p, const float2* in, float2* out, int fields, int sign, int kind, cudaStream_t st);
+
 // One right-hand side and update on a cube of 3 * 2^m points (ns_radix3.cu).
 cudaError_t ns_rhs_radix3(fftk_plan p, const float2* u, const float2* u0, const float2* u1, float2* out,
                           const NSUpdate& upd, int mode, const float2* extra, cudaStream_t st);
@@ -411,13 +400,8 @@ struct NSLaunch {
   static cudaError_t attrs() {
     static PerDevice once;
     return once.run([](int) {
-      const int sx = (int)NXCfg<N>::SMEM;
       cudaError_t err = cudaFuncSetAttribute(k_ns_invx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)NICfg<N>::SMEM);
-      if (err == cudaSuccess)
-        err = cudaFuncSetAttribute(k_ns_ypass<N, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
-      if (err == cudaSuccess)
-        err = cudaFuncSetAttribute(k_ns_ypass<N, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
       if (err == cudaSuccess)
         err = cudaFuncSetAttribute(k_ns_z<N, (int)ns_row(N)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)NZCfg<N>::SMEM);
@@ -447,13 +431,11 @@ struct NSLaunch {
   static cudaError_t rhs(fftk_plan p, const float2* u, const float2* u0, const float2* u1,
                          float2* out, const NSUpdate& upd, int mode, const float2* extra,
                          cudaStream_t st) {
-    using X = NXCfg<N>;
     using Z = NZCfg<N>;
     cudaError_t e = attrs();
     if (e != cudaSuccess) return e;
     NSWork* s = p->ns;
     const NSGeom g = s->g;
-    const int kx = (g.kc + X::T - 1) / X::T;
     using I = NICfg<N>;
     const int ki = (g.kc + I::T - 1) / I::T;
     // invx u -> A, inverse y A -> B, z B -> A (fields 0..2), forward y A -> A,
@@ -470,21 +452,16 @@ struct NSLaunch {
       LaunchScope ls(p, KK_NS_INVX, st);
       k_ns_invx<N><<<g.nk * ki, I::THREADS, I::SMEM, st>>>(u, A, ki, tw, t3);
     }
-    {
-      LaunchScope ls(p, KK_NS_INVY, st);
-      k_ns_ypass<N, 1><<<6 * N * kx, X::THREADS, X::SMEM, st>>>(A, Bw, kx, tw, t3);
-    }
+    e = ns_ypass(p, A, Bw, 6, +1, KK_NS_INVY, st);
+    if (e != cudaSuccess) return e;
     {
       LaunchScope ls(p, KK_NS_Z, st);
       const long long lines = (long long)N * N;
       k_ns_z<N, (int)ns_row(N)><<<(unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st>>>(
           Bw, A, tw, t3, p->d_err);
     }
-    {
-      LaunchScope ls(p, KK_NS_FWDY, st);
-      k_ns_ypass<N, -1><<<3 * N * kx, X::THREADS, X::SMEM, st>>>(A, A, kx, tw, t3);
-    }
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = ns_ypass(p, A, A, 3, -1, KK_NS_FWDY, st);
     return e == cudaSuccess ? ns_fwdx(p, A, u0, u1, out, upd, mode, extra, st) : e;
   }
 };

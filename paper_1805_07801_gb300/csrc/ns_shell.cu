@@ -223,8 +223,6 @@ static cudaError_t shell_advect_n(fftk_plan p, const float2* u, const float* ur,
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_shell_invy<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
     if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(k_ns_ypass<N, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
-    if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_shell_fwdx<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sx);
     if (err == cudaSuccess)
       err = cudaFuncSetAttribute(k_shell_z<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SZCfg3<N>::SMEM);
@@ -249,10 +247,8 @@ static cudaError_t shell_advect_n(fftk_plan p, const float2* u, const float* ur,
     k_shell_z<N><<<(unsigned)(((long long)N * N + Z::LPC - 1) / Z::LPC), Z::THREADS, SZCfg3<N>::SMEM, st>>>(
         A, B, ur, sh.kb, tw);
   }
-  {
-    LaunchScope ls(p, KK_Y_FWD, st);
-    k_ns_ypass<N, -1><<<3 * N * KT, X::THREADS, X::SMEM, st>>>(A, A, KT, tw, nullptr);
-  }
+  const cudaError_t ey = ns_ypass(p, A, A, 3, -1, KK_Y_FWD, st);
+  if (ey != cudaSuccess) return ey;
   {
     LaunchScope ls(p, KK_X_FWD, st);
     k_shell_fwdx<N><<<3 * (2 * KD + 1) * KT, X::THREADS, X::SMEM, st>>>(

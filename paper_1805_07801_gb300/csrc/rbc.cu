@@ -239,11 +239,11 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
     }
     e = launch_scpass_pruned(p, true, +1, w, w, 4, 1.f, st);
     if (e == cudaSuccess) e = launch_scpass_pruned(p, false, +1, w + 4 * mw, w + 4 * mw, 3, 1.f, st);
-    if (e == cudaSuccess) e = rbc_y(p, w, +1, st);
+    if (e == cudaSuccess) e = ns_ypass(p, w, w, 7, +1, KK_Y_INV, st);
     // products: [(u x omega)_x, u_y theta, u_z theta | (u x omega)_y, (u x omega)_z, u_x theta]
     const RBCSlots sl{{0, 4, 5, 6, 1, 2, 3}, {0, 3, 4, 5, 1, 2}};
     if (e == cudaSuccess) e = rbc_z(p, w, sl, st);
-    if (e == cudaSuccess) e = rbc_y(p, w, -1, st);
+    if (e == cudaSuccess) e = ns_ypass(p, w, w, 6, -1, KK_Y_FWD, st);
     if (e == cudaSuccess) e = launch_scpass_pruned(p, true, -1, w, w, 3, scale, st);
     if (e == cudaSuccess) e = launch_scpass_pruned(p, false, -1, w + 3 * mw, w + 3 * mw, 3, scale, st);
     if (e != cudaSuccess) return e;
@@ -255,10 +255,10 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
   }
   // w7 = [u_x, u_y, u_z, omega_x, omega_y, omega_z, theta] -> [n_x, n_y, n_z, u_x theta, ...]
   e = rbc_invx(p, x, w, st);
-  if (e == cudaSuccess) e = rbc_y(p, w, +1, st);
+  if (e == cudaSuccess) e = ns_ypass(p, w, w, 7, +1, KK_Y_INV, st);
   const RBCSlots sl{{0, 1, 2, 3, 4, 5, 6}, {0, 1, 2, 3, 4, 5}};
   if (e == cudaSuccess) e = rbc_z(p, w, sl, st);
-  if (e == cudaSuccess) e = rbc_y(p, w, -1, st);
+  if (e == cudaSuccess) e = ns_ypass(p, w, w, 6, -1, KK_Y_FWD, st);
   if (e != cudaSuccess) return e;
   return rbc_fwdx(p, RBCStage{w, x, u0, r->s1, r->acc, out, upd, mode, scale}, st);
 }

@@ -71,9 +71,7 @@ struct RBCStage {
   float scale;        // 1 / n^3
 };
 
-// y passes (sign +1: 7 fields, -1: 6) and the fused z pass on the padded workspace
-cudaError_t rbc_y(fftk_plan p, float2* w, int sign, cudaStream_t st);
-cudaError_t rbc_y3(fftk_plan p, float2* w, int sign, cudaStream_t st);
+// the fused z pass on the padded workspace
 cudaError_t rbc_z(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
 cudaError_t rbc_z3(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
 // periodic cube: the inverse x pass with the curl (state -> 7 fields), and the
@@ -384,25 +382,6 @@ static cudaError_t rbc_invx_n(fftk_plan p, const float2* x, float2* w, cudaStrea
   k_ns_invx<N, true><<<(2 * KD + 1) * KT, I::THREADS, I::SMEM, st>>>(x, w, KT, twiddles(p, 1 << Log2<N>::value),
                                                                   p->d_tw3);
   return cudaGetLastError();
-}
-
-template <int N, int SIGN>
-static cudaError_t rbc_y_ns(fftk_plan p, float2* w, cudaStream_t st) {
-  using X = NXCfg<N>;
-  static PerDevice once;
-  const cudaError_t e = once.run([](int) {
-    return cudaFuncSetAttribute(k_ns_ypass<N, SIGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::SMEM);
-  });
-  if (e != cudaSuccess) return e;
-  constexpr int KD = (N - 1) / 3, KT = (KD + X::T) / X::T;
-  LaunchScope ls(p, SIGN > 0 ? KK_Y_INV : KK_Y_FWD, st);
-  k_ns_ypass<N, SIGN><<<(SIGN > 0 ? 7 : 6) * N * KT, X::THREADS, X::SMEM, st>>>(
-      w, w, KT, twiddles(p, 1 << Log2<N>::value), p->d_tw3);
-  return cudaGetLastError();
-}
-template <int N>
-static cudaError_t rbc_y_n(fftk_plan p, float2* w, int sign, cudaStream_t st) {
-  return sign > 0 ? rbc_y_ns<N, 1>(p, w, st) : rbc_y_ns<N, -1>(p, w, st);
 }
 
 template <int N>

@@ -15,18 +15,6 @@ cudaError_t rbc_invx(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
   }
 }
 
-cudaError_t rbc_y(fftk_plan p, float2* w, int sign, cudaStream_t st) {
-  switch (p->nx) {
-#define CASE(n) \
-  case n:       \
-    return rbc_y_n<n>(p, w, sign, st);
-    CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
-#undef CASE
-    default:
-      return rbc_y3(p, w, sign, st);
-  }
-}
-
 cudaError_t rbc_z(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st) {
   switch (p->nx) {
 #define CASE(n) \

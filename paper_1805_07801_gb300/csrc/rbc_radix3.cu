@@ -14,17 +14,6 @@ cudaError_t rbc_invx3(fftk_plan p, const float2* x, float2* w, cudaStream_t st) 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t rbc_y3(fftk_plan p, float2* w, int sign, cudaStream_t st) {
-  switch (p->nx) {
-#define CASE(n) \
-  case n:       \
-    return rbc_y_n<n>(p, w, sign, st);
-    CASE(12) CASE(24) CASE(48) CASE(96) CASE(192) CASE(384) CASE(768)
-#undef CASE
-  }
-  return cudaErrorInvalidValue;
-}
-
 cudaError_t rbc_z3(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st) {
   switch (p->nx) {
 #define CASE(n) \
