@@ -264,11 +264,11 @@ __device__ __forceinline__ void dft3(float2& a, float2& b, float2& c) {
 template <int R, int SIGN>
 __device__ __forceinline__ void dftR(float2 (&a)[R]) {
   if constexpr (R % 3 == 0) {
-    // R = 3 P, P = 1, 2, 4 or 8: 3 and P have no common factor, so the DFT is
+    // R = 3 P, P = 1, 2, 4, 8 or 16: 3 and P have no common factor, so the DFT is
     // the two-dimensional 3 x P one without twiddles (Good's mapping):
     // n = P n1 + 3 n2, k = k1 (mod 3) = k2 (mod P)
     constexpr int P = R / 3;
-    constexpr int E1 = P == 1 ? 1 : (P == 8 ? 16 : 4), E2 = P == 1 ? 0 : (P == 2 ? 3 : 9);
+    constexpr int E1 = P == 1 ? 1 : (P >= 8 ? 16 : 4), E2 = P == 1 ? 0 : (P == 2 ? 3 : (P == 16 ? 33 : 9));
 #pragma unroll
     for (int n2 = 0; n2 < P; ++n2) dft3<SIGN>(a[3 * n2], a[(P + 3 * n2) % R], a[(2 * P + 3 * n2) % R]);
     float2 o[R];

@@ -13,7 +13,7 @@
 //   1024^3      2.01 / 2.07 -> 1.35 / 1.37 ms   (0.94 of the copy rate)
 //   512^3       187 / 225 -> 168 / 206 us       (0.95 / 0.77)
 //   16 x 256^3  423 / 439 -> 322 / 418 us       (0.99 / 0.76)
-//   768^3       797 / 858 -> 622 / 698 us       (0.86 / 0.77)
+//   768^3       797 / 858 -> 587 / 626 us       (0.92 / 0.86)
 //   2 x 1536 x 1536 x 96   1180 / 1357 -> 823 / 1011 us
 // The y passes' rows of n/2 + 1 values leave one column for a last tile and
 // store across line boundaries, which the shorter lines' transforms feel.
@@ -44,11 +44,12 @@ template <int L_, bool PAIR_>
 struct PipeCfg {
   static constexpr int L = L_;
   static constexpr bool PAIR = PAIR_;
-  // powers of two: two stages (radix G, then R2) with the half-size exchange;
-  // 3 * 2^m: the line engine (24 values, radices 8, 8, 12 at 768) with an
-  // exchange buffer of the tile's size
-  static constexpr bool ENGINE = L % 3 == 0;
-  static constexpr int G = ENGINE ? elems_per_thread(L) : (L >= 512 ? 32 : 16);  // values per thread
+  // powers of two and 768: two stages (radix G, then R2) with the half-size
+  // exchange; 384 and 1536: the line engine (24 values) with an exchange buffer
+  // of the tile's size.  (768 with the engine, radices 8, 8, 12 on 512 threads:
+  // 622 / 698 us per 768^3 x / y pass against 587 / 626 us with 48 x 16 on 256.)
+  static constexpr bool ENGINE = L % 3 == 0 && L != 768;
+  static constexpr int G = ENGINE ? elems_per_thread(L) : (L == 768 ? 48 : (L >= 512 ? 32 : 16));  // values per thread
   static constexpr int R2 = L / G;                  // radix of the second stage
   static constexpr bool PAIRED = L == 512;          // two butterflies per thread in the second stage
   static constexpr int S = L / G;                   // threads per line
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
   uint64_t* bar = reinterpret_cast<uint64_t*>(smp + C::SMEM - 16);
   const int tid = threadIdx.x, c = tid % T, j = tid / T;
   if constexpr (!C::ENGINE)
-    for (int i = tid; i < L; i += C::THREADS) stw[i] = tw[i];
+    for (int i = tid; i < L; i += C::THREADS) stw[i] = L % 3 == 0 ? t3[L + i] : tw[i];
 
   auto fetch = [&](int t) {  // thread 0
     const int p = t / qtiles, q0 = (t - p * qtiles) * T;

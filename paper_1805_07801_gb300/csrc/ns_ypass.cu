@@ -1,9 +1,12 @@
 // The y passes of the solvers (padded rows, 2/3 rule; see k_ns_ypass for the
-// general kernel): from 256 points on pipelined (fft_pipe.cuh).  The inverse
+// general kernel): from 384 points on pipelined (fft_pipe.cuh).  The inverse
 // pass stages only the kept rows, the forward pass stores only those.
 // Per launch, one tile after the other with one or two CTAs per SM, and so:
-// 768^3, six fields inverse 2.43 -> II ms, three forward 1.16 -> FF ms; 512^3,
-// 641 -> ii us, 310 -> ff us.
+// 768^3, six fields inverse 2.43 -> 1.95 ms, three forward 1.16 -> 0.91 ms
+// (radix 48, then 16; 2.27 and 1.04 ms with radices 8, 8, 12); 512^3,
+// 641 -> 586 us, 310 -> 277 us (0.95 of the copy rate).  At 256 points the
+// general kernel, with more CTAs per SM, is as fast (79 / 101 against 82 / 102
+// us for six and seven fields).
 #include <mutex>
 
 #include "fft_pipe.cuh"
@@ -13,8 +16,8 @@ namespace fftk {
 
 template <int N, int SIGN>
 struct YPipeCfg {
-  static constexpr bool ENGINE = N % 3 == 0;  // else two long-radix stages
-  static constexpr int G = ENGINE ? elems_per_thread(N) : (N >= 512 ? 32 : 16);
+  static constexpr bool ENGINE = N % 3 == 0 && N != 768;  // else two long-radix stages
+  static constexpr int G = ENGINE ? elems_per_thread(N) : (N == 768 ? 48 : (N >= 512 ? 32 : 16));
   static constexpr int S = N / G, T = 16, THREADS = S * T;
   static constexpr int MINB = N >= 768 ? 1 : (N >= 384 ? 2 : 4);
   static constexpr int KD = (N - 1) / 3;
@@ -45,7 +48,7 @@ __global__ void __launch_bounds__(YPipeCfg<N, SIGN>::THREADS, YPipeCfg<N, SIGN>:
   uint64_t* bar = reinterpret_cast<uint64_t*>(smy + C::SMEM - 16);
   const int tid = threadIdx.x, c = tid % T, j = tid / T;
   if constexpr (!C::ENGINE)
-    for (int i = tid; i < N; i += C::THREADS) stw[i] = tw[i];
+    for (int i = tid; i < N; i += C::THREADS) stw[i] = N % 3 == 0 ? t3[N + i] : tw[i];
   constexpr int HIGH0 = N - C::SPLIT * C::BOXR;  // first row of the upper part (inverse)
   auto fetch = [&](int t) {  // thread 0
     const int plane = t / KT, x0 = 2 * T * (t - plane * KT);
@@ -123,7 +126,7 @@ template <int N, int SIGN>
 static cudaError_t ypass_n(fftk_plan p, const float2* in, float2* out, int fields, int kind, cudaStream_t st) {
   constexpr int KD = (N - 1) / 3;
   const float2* tw = twiddles(p, 1 << Log2<N>::value);
-  if constexpr (N >= 256) {
+  if constexpr (N >= 384) {
     using C = YPipeCfg<N, SIGN>;
     static PerDevice once;
     static int nsm[kMaxDevices];
