@@ -15,27 +15,32 @@ namespace fftk {
 // 512^3, RK2: 648 us per launch with the update's loads one mode at a time,
 // 567 us with the loads of two modes in flight (the mode a template argument,
 // so that they fit into 64 registers), 484 us with the L2 prefetches below
-// (546 us with all of them at the start); 64^3: 12.6 -> 8.3 us.
+// (546 us with all of them at the start), 468 us with two long-radix stages
+// instead of three; 64^3: 12.6 -> 8.3 us; 768^3: 2.87 -> 2.26 ms, with radix 48
+// and 16 instead of 8, 8, 12 1.76 ms.
 //
-// Forward x pass (one field in registers, two parked): 1024 threads, 8 values
-// per thread, 16 columns per tile at n = 512 and 8 at n = 1024; 3 * 2^m: 24
-// values per thread, 16 columns; there only the slots m whose rows j + m S can
-// be kept by the 2/3 rule are parked, the first LOW and those from HIGH on
-// (all slots would not fit beside the exchange buffer at n = 768).
+// One field is in registers and two are parked.  n = 512 and 768: two stages
+// with the half-size exchange (XTransform), 256 threads, 16 columns per tile;
+// other 3 * 2^m: 24 values per thread, 16 columns; other powers of two: 8
+// values per thread, 16 columns (8 at n = 1024).  At 512 and for 3 * 2^m only
+// the slots m whose rows j + m S can be kept by the 2/3 rule are parked, the
+// first LOW and those from HIGH on.
 template <int N>
 struct NUCfg {
-  static constexpr int G = N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G;
+  static constexpr bool TWO = N == 768 || N == 512;  // radix 48 or 32, then 16
+  static constexpr int G = N == 768 ? 48 : TWO ? 32 : (N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G);
   static constexpr int S = N / G;
   static constexpr int T = N % 3 == 0 || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
   static constexpr int THREADS = T * S;
   static constexpr int KD = (N - 1) / 3;
-  static constexpr int LOW = N % 3 != 0 ? G : KD / S + 1;
+  static constexpr int LOW = N % 3 != 0 && !TWO ? G : KD / S + 1;
   static constexpr int HIGH = (N - KD) / S > LOW ? (N - KD) / S : LOW;
   static constexpr int SLOTS = LOW + G - HIGH;
-  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N * T + 2 * (size_t)SLOTS * THREADS);
-  static constexpr int MINB = N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
+  using X = XTransform<N, G, -1, T, TWO>;
+  static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 2 * (size_t)SLOTS * THREADS);
+  static constexpr int MINB = TWO ? 1 : N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
                                          : (N >= 512 ? 1024 / THREADS : (512 / THREADS < 8 ? 512 / THREADS : 8));  // 64 registers, 128
-  static constexpr int GROUP = N % 3 != 0 && N >= 512 ? 2 : 4;  // modes whose loads are in flight together
+  static constexpr int GROUP = N % 3 != 0 && N >= 512 && !TWO ? 2 : 4;  // modes whose loads are in flight together
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };
@@ -64,10 +69,10 @@ __global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
   const long long q = (long long)ay * H1 + kz;
   const long long rs = (long long)N * H1;
   const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
-  const ColX<T> xc{smn, c};
   // fields 0 and 1 are parked in shared memory after their transforms (this
   // thread's slots only), so one field at a time is held in registers
-  float2* park = smn + (size_t)N * T + threadIdx.x;
+  float2* park = smn + C::X::WORDS + threadIdx.x;
+  C::X::init(smn, tw, t3);
   const float2* bsrc = MODE == NS_STAGE2 ? u1 : upd.acc;
   constexpr bool A0 = MODE != NS_RHS && MODE != NS_RK4_4, B0 = MODE == NS_STAGE2 || MODE >= NS_RK4_2;
   float2 V[G];
@@ -91,7 +96,7 @@ __global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
         }
       }
     }
-    fft_line<N, G, -1>(V, j, xc, tw, t3);
+    C::X::run(V, j, c, smn, tw, t3);
     if (f < 2) {
 #pragma unroll
       for (int m = 0; m < G; ++m)

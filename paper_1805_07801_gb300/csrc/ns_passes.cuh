@@ -75,7 +75,8 @@ struct NICfg {
   static constexpr int T = PARK || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
   static constexpr int THREADS = T * S;
   static constexpr int MINB = PARK ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1)) : (THREADS <= 256 ? 2 : 1);
-  static constexpr size_t SMEM = sizeof(float2) * (size_t)N * T * (PARK ? 2 : 1);
+  using X = XTransform<N, G, +1, T, false>;
+  static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + (PARK ? (size_t)N * T : 0));
 };
 
 // 1. inverse x pass with the curl.  Columns: kept (k_y, k_z); rows: k_x.
@@ -103,7 +104,6 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
   const long long rs = (long long)N * H1;
   const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
   const float ky = (float)kwav(ay, N), kzf = (float)kz;
-  const ColX<T> xc{smn, c};
   auto load = [&](int f, float2(&v)[G], bool ikx) {
 #pragma unroll
     for (int m = 0; m < G; ++m) {
@@ -120,30 +120,31 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     }
   };
   if constexpr (C::PARK) {
-    float2* park = smn + (size_t)N * T + threadIdx.x;  // this thread's slots
+    float2* park = smn + C::X::WORDS + threadIdx.x;  // this thread's slots
+    C::X::init(smn, tw, t3);
     float2 a[G];
     load(0, a, false);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_x
+    C::X::run(a, j, c, smn, tw, t3);  // U_x
     store(0, a);
 #pragma unroll
     for (int m = 0; m < G; ++m) park[m * C::THREADS] = a[m];
     load(1, a, true);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_y
+    C::X::run(a, j, c, smn, tw, t3);  // D_y
 #pragma unroll
     for (int m = 0; m < G; ++m) a[m] = csub(a[m], mul_i(park[m * C::THREADS], ky));  // omega_z
     store(5, a);
     load(2, a, true);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_z
+    C::X::run(a, j, c, smn, tw, t3);  // D_z
 #pragma unroll
     for (int m = 0; m < G; ++m) a[m] = csub(mul_i(park[m * C::THREADS], kzf), a[m]);  // omega_y
     store(4, a);
     load(1, a, false);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_y
+    C::X::run(a, j, c, smn, tw, t3);  // U_y
     store(1, a);
 #pragma unroll
     for (int m = 0; m < G; ++m) park[m * C::THREADS] = a[m];
     load(2, a, false);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_z
+    C::X::run(a, j, c, smn, tw, t3);  // U_z
     store(2, a);
 #pragma unroll
     for (int m = 0; m < G; ++m) {
@@ -153,29 +154,29 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     store(3, a);
     if constexpr (THETA) {
       load(3, a, false);
-      fft_line<N, G, +1>(a, j, xc, tw, t3);
+      C::X::run(a, j, c, smn, tw, t3);
       store(6, a);
     }
   } else {
     float2 a[G], b[G];
     load(1, a, true);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_y
+    C::X::run(a, j, c, smn, tw, t3);  // D_y
     load(0, b, false);
-    fft_line<N, G, +1>(b, j, xc, tw, t3);  // U_x
+    C::X::run(b, j, c, smn, tw, t3);  // U_x
     store(0, b);
   #pragma unroll
     for (int m = 0; m < G; ++m) a[m] = csub(a[m], mul_i(b[m], ky));  // omega_z
     store(5, a);
     load(2, a, true);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // D_z
+    C::X::run(a, j, c, smn, tw, t3);  // D_z
   #pragma unroll
     for (int m = 0; m < G; ++m) a[m] = csub(mul_i(b[m], kzf), a[m]);  // omega_y
     store(4, a);
     load(1, a, false);
-    fft_line<N, G, +1>(a, j, xc, tw, t3);  // U_y
+    C::X::run(a, j, c, smn, tw, t3);  // U_y
     store(1, a);
     load(2, b, false);
-    fft_line<N, G, +1>(b, j, xc, tw, t3);  // U_z
+    C::X::run(b, j, c, smn, tw, t3);  // U_z
     store(2, b);
   #pragma unroll
     for (int m = 0; m < G; ++m)
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     store(3, b);
     if constexpr (THETA) {
       load(3, a, false);
-      fft_line<N, G, +1>(a, j, xc, tw, t3);
+      C::X::run(a, j, c, smn, tw, t3);
       store(6, a);
     }
   }

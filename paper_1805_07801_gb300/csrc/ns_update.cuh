@@ -3,6 +3,7 @@
 #pragma once
 
 #include "fft_engine.cuh"
+#include "fft_pipe.cuh"
 #include "ns_common.cuh"
 
 namespace fftk {
@@ -132,6 +133,27 @@ __device__ __forceinline__ void ns_mode_update(const NSModeIn& in, float2 nx, fl
     }
   }
 }
+
+// Transform of an x pass with its tile's buffers at `sm`: the line engine with
+// an exchange buffer of the tile's size, or (TWO, 768 points) two stages of
+// radix 48 and 16 with a half-size buffer and the twiddles behind it.
+template <int N, int G, int SIGN, int T, bool TWO>
+struct XTransform {
+  static constexpr size_t WORDS = TWO ? (size_t)N * T / 2 + N : (size_t)N * T;  // float2 at sm
+  __device__ __forceinline__ static void init(float2* sm, const float2* tw, const float2* t3) {
+    if constexpr (TWO)
+      for (int i = threadIdx.x; i < N; i += N / G * T) sm[(size_t)N * T / 2 + i] = N % 3 == 0 ? t3[N + i] : tw[i];
+  }
+  __device__ __forceinline__ static void run(float2 (&v)[G], int j, int c, float2* sm, const float2* tw,
+                                             const float2* t3) {
+    if constexpr (TWO) {
+      __syncthreads();  // the buffer may still be read
+      pipe_transform<N, G, SIGN, T>(v, j, c, reinterpret_cast<float*>(sm), sm + (size_t)N * T / 2);
+    } else {
+      fft_line<N, G, SIGN>(v, j, ColX<T>{sm, c}, tw, t3);
+    }
+  }
+};
 
 // The forward x pass with the update of `mode` (ns_fwdx.cu, ns_fwdx3.cu).
 cudaError_t ns_fwdx(fftk_plan p, const float2* nh, const float2* u0, const float2* u1, float2* out,

@@ -241,11 +241,13 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
 // As the Navier-Stokes forward x pass (ns_fwdx.cuh), with six fields and three
 // parked arrays: the divergence k . F(u theta), summed as its three fields are
 // transformed, then n_x and n_y.  512^3, per launch: forward x pass 528 us and
-// update 922 us as kernels of their own, 1355 us fused (1607 us with all its L2
-// prefetches at the start instead of one field ahead).
+// update 922 us as kernels of their own, 1135 us fused (1607 us with all its L2
+// prefetches at the start instead of one field ahead, 1351 us with radices 8, 8,
+// 8 on 1024 threads instead of 32, 16 on 256).
 template <int N>
 struct RUCfg {
-  static constexpr int G = N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G;
+  static constexpr bool TWO = N == 512;  // radix 32, then 16
+  static constexpr int G = TWO ? 32 : (N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G);
   static constexpr int S = N / G;
   static constexpr int T = N == 512 ? 16 : (N >= 768 ? 8 : (N % 3 == 0 ? 16 : NFCfg<N>::T));
   static constexpr int THREADS = T * S;
@@ -253,8 +255,9 @@ struct RUCfg {
   static constexpr int LOW = KD / S + 1;
   static constexpr int HIGH = (N - KD) / S > LOW ? (N - KD) / S : LOW;
   static constexpr int SLOTS = LOW + G - HIGH;
-  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N * T + 3 * (size_t)SLOTS * THREADS);
-  static constexpr int MINB = THREADS >= 512 ? 1 : (THREADS == 256 ? (N == 768 ? 1 : 2) : 4);
+  using X = XTransform<N, G, -1, T, TWO>;
+  static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 3 * (size_t)SLOTS * THREADS);
+  static constexpr int MINB = THREADS >= 512 ? 1 : (THREADS == 256 ? (N == 768 || TWO ? 1 : 2) : 4);
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };
@@ -279,8 +282,8 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
   const bool valid = kz < (KD + 1);
   const long long q = (long long)ay * H1 + kz, rs = (long long)N * H1;
   const long long qw = (long long)ay * HW + kz, rw = (long long)N * HW;
-  const ColX<T> xc{smn, c};
-  float2* park = smn + (size_t)N * T + threadIdx.x;
+  float2* park = smn + C::X::WORDS + threadIdx.x;
+  C::X::init(smn, tw, t3);
   const int ky = kwav(ay, N);
   const float2* bsrc = MODE == NS_STAGE2 ? s1 : acc;
   float2 V[G];
@@ -309,7 +312,7 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
           }
         }
     }
-    fft_line<N, G, -1>(V, j, xc, tw, t3);
+    C::X::run(V, j, c, smn, tw, t3);
     if (i < 3) {
 #pragma unroll
       for (int m = 0; m < G; ++m)
