@@ -128,6 +128,7 @@ __global__ void k_les_products(const float* __restrict__ ubar, const float* __re
 }
 
 __global__ void k_grad_spectra(const float2* __restrict__ uh, float2* __restrict__ gh, int n) {
+  pdl_wait();
   const int h1 = n / 2 + 1;
   const long long M = (long long)n * n * h1;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < M;
@@ -292,7 +293,9 @@ struct SGSConst {
 namespace mlptc {
 constexpr int kThreads = 256;
 constexpr int kBlocks = 2;
-constexpr int kPerSm = 3;  // CTAs per SM (shared memory, 80 registers); 128^3 step with the model: 1445 us with 2, 1371 with 3
+// CTAs per SM (shared memory, 80 registers); 128^3 step with the model: 1445 us
+// with 2, 1371 us with 3
+constexpr int kPerSm = 3;
 constexpr int kW1 = 64 * 16 * 2;  // bytes of one BF16 part of W1 as B [64 x 16]
 constexpr int kW2 = 64 * 64 * 2;  // W2, W3 as B [64 x 64]
 constexpr int kW4 = 16 * 64 * 2;  // W4 as B [16 x 64]
@@ -503,6 +506,7 @@ __device__ __forceinline__ void finish(unsigned char* base, uint32_t tmem, uint3
 __global__ void __launch_bounds__(mlptc::kThreads, mlptc::kPerSm)
     k_sgs_pointwise_tc(const float* __restrict__ A9, long long R, const float* __restrict__ params, SGSConst cst,
                        float* __restrict__ tau6, int* err) {
+  pdl_wait();
   extern __shared__ __align__(1024) unsigned char smraw_tc[];
   unsigned char* base = mlptc::aligned_base(smraw_tc);
   uint64_t* bar = reinterpret_cast<uint64_t*>(base + mlptc::oBar);
@@ -578,6 +582,7 @@ __global__ void __launch_bounds__(mlptc::kThreads, mlptc::kPerSm)
 
 // SGS force s_i = -i k_j tau_hat_ij on the 2/3 set, projected; written to s (3 fields)
 __global__ void k_sgs_divergence(const float2* __restrict__ th, float2* __restrict__ s, int n) {
+  pdl_wait();
   const int h1 = n / 2 + 1;
   const long long M = (long long)n * n * h1;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < M;
@@ -720,7 +725,7 @@ extern "C" fftk_status tarang_closure_features(fftk_plan p, const float* ubar, c
   if (s == FFTK_OK) s = fftk_r2c(p, ubar, uh, 3, cuda_stream);
   if (s == FFTK_OK) {
     LaunchScope ls(p, KK_AUX, st);
-    k_grad_spectra<<<grid_for(M, 256), 256, 0, st>>>(uh, gh, n);
+    launch_pdl(k_grad_spectra, grid_for(M, 256), 256, 0, st, uh, gh, n);
   }
   if (s == FFTK_OK) s = fftk_c2r(p, gh, A, 9, cuda_stream);
   if (s == FFTK_OK) {
@@ -965,7 +970,7 @@ cudaError_t sgs_term(fftk_plan p, fftk_sgs_work** wp, const float2* u, const tar
   fftk_sgs_work* w = *wp;
   {
     LaunchScope ls(p, KK_AUX, st);
-    k_grad_spectra<<<grid_for(M, 256), 256, 0, st>>>(u, w->gh, n);
+    launch_pdl(k_grad_spectra, grid_for(M, 256), 256, 0, st, u, w->gh, n);
   }
   if (fftk_c2r(p, w->gh, w->A, 9, st) != FFTK_OK) return cudaErrorLaunchFailure;
   SGSConst c;
@@ -974,13 +979,13 @@ cudaError_t sgs_term(fftk_plan p, fftk_sgs_work** wp, const float2* u, const tar
   std::memcpy(c.out_scale, model->out_scale, sizeof(c.out_scale));
   {
     LaunchScope ls(p, KK_AUX, st);
-    k_sgs_pointwise_tc<<<mlptc_grid(R), mlptc::kThreads, mlptc::kSmem, st>>>(w->A, R, model->params, c, w->tau,
+    launch_pdl(k_sgs_pointwise_tc, mlptc_grid(R), mlptc::kThreads, mlptc::kSmem, st, w->A, R, model->params, c, w->tau,
                                                                             p->d_err);
   }
   if (fftk_r2c(p, w->tau, w->th, 6, st) != FFTK_OK) return cudaErrorLaunchFailure;
   {
     LaunchScope ls(p, KK_AUX, st);
-    k_sgs_divergence<<<grid_for(M, 256), 256, 0, st>>>(w->th, w->s, n);
+    launch_pdl(k_sgs_divergence, grid_for(M, 256), 256, 0, st, w->th, w->s, n);
   }
   *out = w->s;
   return cudaGetLastError();

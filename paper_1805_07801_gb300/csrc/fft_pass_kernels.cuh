@@ -48,6 +48,7 @@ template <int N>
 __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     k_z_r2c(const float* __restrict__ in, float2* __restrict__ out, long long nlines,
             const float2* __restrict__ tw, const float2* __restrict__ t3, float scale) {  // tw: size-2^LOGN table
+  pdl_wait();
   using C = ZCfg<N>;
   constexpr int H = C::H, G = C::G, S = C::S;
   constexpr int LOGN = Log2<N>::value;
@@ -66,7 +67,8 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   xc.sync();
   if (valid) {
     float2* dst = out + line * (H + 1);
-    const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);  // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
+    // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
+    const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
@@ -89,6 +91,7 @@ template <int N>
 __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     k_z_c2r(const float2* __restrict__ in, float* __restrict__ out, long long nlines,
             const float2* __restrict__ tw, const float2* __restrict__ t3) {  // tw: size-2^LOGN table
+  pdl_wait();
   using C = ZCfg<N>;
   constexpr int H = C::H, G = C::G, S = C::S;
   constexpr int LOGN = Log2<N>::value;
@@ -108,7 +111,8 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     xc.st(j + m * S, v[m]);
   }
   const float2 XH = valid ? src[H] : make_float2(0.f, 0.f);
-  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);  // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
+  // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
+  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
   xc.sync();
 #pragma unroll
   for (int m = 0; m < G; ++m) {
@@ -161,6 +165,7 @@ template <int L, int SIGN, int AHEAD>
 __global__ void __launch_bounds__(CCfg<L>::THREADS, CCfg<L>::MINB)
     k_cpass(const float2* in, float2* out, long long Q, long long qtiles,
             const float2* __restrict__ tw, const float2* __restrict__ t3, float scale) {
+  pdl_wait();
   using C = CCfg<L>;
   constexpr int G = C::G, S = C::S, T = C::T;
   extern __shared__ float2 smc[];
@@ -196,7 +201,8 @@ static cudaError_t z_r2c_n(fftk_plan p, const float* in, float2* out, long long 
   using C = ZCfg<N>;
   const long long blocks = (nl + C::LPC - 1) / C::LPC;
   LaunchScope ls(p, KK_Z_R2C, st);
-  k_z_r2c<N><<<(unsigned)blocks, C::THREADS, 0, st>>>(in, out, nl, twiddles(p, 1 << Log2<N>::value), p->d_tw3, scale);
+  launch_pdl(k_z_r2c<N>, (unsigned)blocks, C::THREADS, 0, st, in, out, nl, twiddles(p, 1 << Log2<N>::value), p->d_tw3,
+             scale);
   return cudaGetLastError();
 }
 
@@ -206,7 +212,7 @@ static cudaError_t z_c2r_n(fftk_plan p, const float2* in, float* out, long long 
   using C = ZCfg<N>;
   const long long blocks = (nl + C::LPC - 1) / C::LPC;
   LaunchScope ls(p, KK_Z_C2R, st);
-  k_z_c2r<N><<<(unsigned)blocks, C::THREADS, 0, st>>>(in, out, nl, twiddles(p, 1 << Log2<N>::value), p->d_tw3);
+  launch_pdl(k_z_c2r<N>, (unsigned)blocks, C::THREADS, 0, st, in, out, nl, twiddles(p, 1 << Log2<N>::value), p->d_tw3);
   return cudaGetLastError();
 }
 
@@ -222,8 +228,8 @@ static cudaError_t cpass_la(fftk_plan p, const float2* in, float2* out, long lon
   const long long qtiles = (Q + C::T - 1) / C::T;
   const long long blocks = P * qtiles;
   LaunchScope ls(p, kind, st);
-  k_cpass<L, SIGN, AHEAD><<<(unsigned)blocks, C::THREADS, C::SMEM, st>>>(
-      in, out, Q, qtiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3, scale);
+  launch_pdl(k_cpass<L, SIGN, AHEAD>, (unsigned)blocks, C::THREADS, C::SMEM, st, in, out, Q, qtiles,
+             twiddles(p, 1 << Log2<L>::value), p->d_tw3, scale);
   return cudaGetLastError();
 }
 

@@ -45,6 +45,7 @@ template <int L, bool SINE, int DIR>
 __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
     k_scpass(const float2* in, float2* out, long long Q, long long qtiles, const float2* __restrict__ tw,
              const float2* __restrict__ tq, float scale) {
+  pdl_wait();
   using C = SCfg<L>;
   constexpr int G = C::G, S = C::S, T = C::T;
   extern __shared__ float2 smc[];
@@ -120,6 +121,7 @@ template <int L, bool SINE, int DIR>
 __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
     k_scpass_pr(const float2* in, float2* out, int ktiles, const float2* __restrict__ tw,
                 const float2* __restrict__ tq, float scale) {
+  pdl_wait();
   using C = SCfg<L>;
   constexpr int G = C::G, S = C::S, T = C::T;
   constexpr long long H1 = ns_row(L), M = (long long)L * L * H1, Q = (long long)L * H1;
@@ -208,6 +210,7 @@ template <int N, bool SINE, int DIR>
 __global__ void __launch_bounds__(SZCfg<N>::THREADS)
     k_scz(const float* in, float* out, long long nlines, const float2* __restrict__ tw,
           const float2* __restrict__ tq, float scale) {
+  pdl_wait();
   using C = SZCfg<N>;
   constexpr int G = C::G, S = C::S;
   constexpr int LOGN = Log2<N>::value;
@@ -292,8 +295,8 @@ static cudaError_t scpass_l(fftk_plan p, const float2* in, float2* out, long lon
   if (attr_err != cudaSuccess) return attr_err;
   const long long qtiles = (Q + C::T - 1) / C::T;
   LaunchScope ls(p, kind, st);
-  k_scpass<L, SINE, DIR><<<(unsigned)(P * qtiles), C::THREADS, C::SMEM, st>>>(in, out, Q, qtiles, twiddles(p, L),
-                                                                              twiddles(p, 4 * L), scale);
+  launch_pdl(k_scpass<L, SINE, DIR>, (unsigned)(P * qtiles), C::THREADS, C::SMEM, st, in, out, Q, qtiles,
+             twiddles(p, L), twiddles(p, 4 * L), scale);
   return cudaGetLastError();
 }
 
@@ -303,8 +306,8 @@ static cudaError_t scz_n(fftk_plan p, const float* in, float* out, long long nli
   using C = SZCfg<N>;
   const long long pairs = (nlines + 1) / 2;
   LaunchScope ls(p, kind, st);
-  k_scz<N, SINE, DIR><<<(unsigned)((pairs + C::LPC - 1) / C::LPC), C::THREADS, 0, st>>>(
-      in, out, nlines, twiddles(p, N), twiddles(p, 4 * N), scale);
+  launch_pdl(k_scz<N, SINE, DIR>, (unsigned)((pairs + C::LPC - 1) / C::LPC), C::THREADS, 0, st, in, out, nlines,
+             twiddles(p, N), twiddles(p, 4 * N), scale);
   return cudaGetLastError();
 }
 
@@ -321,8 +324,8 @@ static cudaError_t scpass_pr_l(fftk_plan p, const float2* in, float2* out, long 
   constexpr int KD = (L - 1) / 3, KC = KD + 1;
   const int ktiles = (KC + C::T - 1) / C::T;
   LaunchScope ls(p, DIR < 0 ? KK_SC_FWD : KK_SC_INV, st);
-  k_scpass_pr<L, SINE, DIR><<<(unsigned)(B * (2 * KD + 1) * ktiles), C::THREADS, C::SMEM, st>>>(
-      in, out, ktiles, twiddles(p, L), twiddles(p, 4 * L), scale);
+  launch_pdl(k_scpass_pr<L, SINE, DIR>, (unsigned)(B * (2 * KD + 1) * ktiles), C::THREADS, C::SMEM, st, in, out,
+             ktiles, twiddles(p, L), twiddles(p, 4 * L), scale);
   return cudaGetLastError();
 }
 

@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(PipeCfg<L, PAIR>::THREADS, PipeCfg<L, PAIR>::M
     k_cpass_pipe(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_odd, float2* out,
                  long long Q, int qtiles, int ntiles, const float2* __restrict__ tw, const float2* __restrict__ t3,
                  const float2* __restrict__ tq, float scale, int* err) {
+  pdl_wait();
   using C = PipeCfg<L, PAIR>;
   constexpr int G = C::G, S = C::S, T = C::T;
   extern __shared__ __align__(128) unsigned char smp[];
@@ -286,9 +287,9 @@ static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorM
   const long long qtiles = (Q + C::T - 1) / C::T, ntiles = P * qtiles, cap = (long long)nsm[dev] * C::MINB;
   const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   LaunchScope ls(p, kind, st);
-  k_cpass_pipe<L, SIGN, PAIR, BASIS><<<grid, C::THREADS, C::SMEM, st>>>(
-      m, mo, out, Q, (int)qtiles, (int)ntiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3,
-      BASIS ? twiddles(p, 4 * L) : nullptr, scale, p->d_err);
+  launch_pdl(k_cpass_pipe<L, SIGN, PAIR, BASIS>, grid, C::THREADS, C::SMEM, st, m, mo, out, Q, (int)qtiles,
+             (int)ntiles, twiddles(p, 1 << Log2<L>::value), p->d_tw3, BASIS ? twiddles(p, 4 * L) : nullptr, scale,
+             p->d_err);
   return cudaGetLastError();
 }
 
@@ -313,8 +314,8 @@ static bool pipe_maps(CUtensorMap* m, CUtensorMap* mo, const float2* in, long lo
 }
 
 template <int L, int BASIS>
-static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long long P, long long Q, float scale, int kind,
-                   cudaStream_t st, cudaError_t* e) {
+static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long long P, long long Q, float scale,
+                   int kind, cudaStream_t st, cudaError_t* e) {
   CUtensorMap m{}, mo{};
   if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
   if (Q % 2 == 0)

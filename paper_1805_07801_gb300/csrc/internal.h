@@ -9,6 +9,7 @@
 
 #include <atomic>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 #include "../../include/fftk.h"
@@ -111,6 +112,30 @@ struct PerDevice {
     return err[dev];
   }
 };
+
+// Programmatic dependent launch: a kernel launched by launch_pdl comes up as
+// soon as the last CTA of the kernel before it in the stream has ended, without
+// waiting for that one's memory to be flushed and its end to be signalled;
+// pdl_wait, the first statement of such a kernel, then waits until every
+// kernel before it has ended and its memory is visible.  Nothing that another
+// kernel writes or reads is touched before it.  (Launched in the plain way it
+// does nothing.)
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // Launch bracketing: counts the launch and records profiling events.
 struct LaunchScope {

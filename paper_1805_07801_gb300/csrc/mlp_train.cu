@@ -244,6 +244,7 @@ template <bool BF16>
 __global__ void __launch_bounds__(mlpcc::kThreads, mlpcc::kPerSm)
     k_mlp_grad(const float* __restrict__ params, const float* __restrict__ x, const float* __restrict__ t, int B,
                int chunks, float* __restrict__ part, double* __restrict__ loss_part) {
+  pdl_wait();
   using namespace mlpcc;
   extern __shared__ __align__(16) unsigned char smem_mlp[];
   Smem& s = *reinterpret_cast<Smem*>(smem_mlp);
@@ -372,6 +373,7 @@ template <bool ADAM>
 __global__ void __launch_bounds__(kRedCols* kRedRows)
     k_mlp_reduce(const float* __restrict__ part, int nblk, float* __restrict__ grad,
                  const double* __restrict__ loss_part, double* __restrict__ loss, double inv_count, AdamStep adam) {
+  pdl_wait();
   __shared__ double sum[kRedRows][kRedCols + 1];
   const int col = threadIdx.x % kRedCols, row = threadIdx.x / kRedCols;
   const int i = blockIdx.x * kRedCols + col;
@@ -400,6 +402,7 @@ __global__ void __launch_bounds__(kRedCols* kRedRows)
 }
 
 __global__ void k_adam(AdamStep a, const float* __restrict__ g, int n) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) adam_update(a, i, g[i]);
 }
@@ -433,9 +436,11 @@ cudaError_t launch_mlp_grad(bool bf16, const float* params, const float* x, cons
   if (e != cudaSuccess) return e;
   const int blocks = mlp_grad_blocks(B), chunks = mlp_chunks(B);
   if (bf16)
-    k_mlp_grad<true><<<blocks, mlpcc::kThreads, sizeof(mlpcc::Smem), st>>>(params, x, t, B, chunks, part, loss_part);
+    launch_pdl(k_mlp_grad<true>, blocks, mlpcc::kThreads, sizeof(mlpcc::Smem), st, params, x, t, B, chunks, part,
+               loss_part);
   else
-    k_mlp_grad<false><<<blocks, mlpcc::kThreads, sizeof(mlpcc::Smem), st>>>(params, x, t, B, chunks, part, loss_part);
+    launch_pdl(k_mlp_grad<false>, blocks, mlpcc::kThreads, sizeof(mlpcc::Smem), st, params, x, t, B, chunks, part,
+               loss_part);
   return cudaGetLastError();
 }
 
@@ -444,9 +449,10 @@ cudaError_t launch_mlp_reduce(int B, const float* part, const double* loss_part,
   const int blocks = (kNP + kRedCols - 1) / kRedCols, nblk = mlp_grad_blocks(B);
   const double inv = 1.0 / (6.0 * (double)B);
   if (adam)
-    k_mlp_reduce<true><<<blocks, kRedCols * kRedRows, 0, st>>>(part, nblk, grad, loss_part, loss, inv, *adam);
+    launch_pdl(k_mlp_reduce<true>, blocks, kRedCols * kRedRows, 0, st, part, nblk, grad, loss_part, loss, inv, *adam);
   else
-    k_mlp_reduce<false><<<blocks, kRedCols * kRedRows, 0, st>>>(part, nblk, grad, loss_part, loss, inv, AdamStep{});
+    launch_pdl(k_mlp_reduce<false>, blocks, kRedCols * kRedRows, 0, st, part, nblk, grad, loss_part, loss, inv,
+               AdamStep{});
   return cudaGetLastError();
 }
 
@@ -462,7 +468,7 @@ cudaError_t launch_mlp_forward_cc(bool bf16, const float* params, const float* x
 }
 
 cudaError_t launch_adam(const AdamStep& a, const float* grad, cudaStream_t st) {
-  k_adam<<<(kNP + 255) / 256, 256, 0, st>>>(a, grad, kNP);
+  launch_pdl(k_adam, (kNP + 255) / 256, 256, 0, st, a, grad, kNP);
   return cudaGetLastError();
 }
 

@@ -30,6 +30,7 @@ namespace fftk {
 // in FP64; one block, fixed order.
 __global__ void k_forced_energy(const float2* __restrict__ u, NSGeom g, int kr, int k2min,
                                 int k2max, double* ef) {
+  pdl_wait();
   __shared__ double red[256];
   const int side = 2 * kr + 1;
   const int count = side * side * (kr + 1);
@@ -262,7 +263,7 @@ static cudaError_t forced_energy(fftk_plan p, const float2* u, const tarang_para
   int kr = 0;
   while ((kr + 1) * (kr + 1) <= prm->force_k2max) ++kr;
   LaunchScope ls(p, KK_NS_REDUCE, st);
-  k_forced_energy<<<1, 256, 0, st>>>(u, p->ns->g, kr, prm->force_k2min, prm->force_k2max,
+  launch_pdl(k_forced_energy, 1, 256, 0, st, u, p->ns->g, kr, prm->force_k2min, prm->force_k2max,
                                      p->ns->ef);
   return cudaGetLastError();
 }

@@ -96,6 +96,7 @@ __device__ __forceinline__ float scale2(float v, int k) {
 __global__ void __launch_bounds__(DIAG_WARPS * 32)
     k_diag(const float2* __restrict__ u, const float2* __restrict__ nh, NSGeom g, double nu, int kmax,
            double* part, int nf) {
+  pdl_wait();
   extern __shared__ double hist[];  // [DIAG_WARPS][kmax+1]
   __shared__ double wd[DIAG_WARPS];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
 constexpr int kFinCols = 32, kFinRows = 16;
 __global__ void __launch_bounds__(kFinCols* kFinRows)
     k_diag_final(const double* __restrict__ part, int width, int nblocks, double* out) {
+  pdl_wait();
   __shared__ double sum[kFinRows][kFinCols + 1];
   const int col = threadIdx.x % kFinCols, row = threadIdx.x / kFinCols;
   const int s = blockIdx.x * kFinCols + col;
@@ -265,11 +267,11 @@ cudaError_t diag_launch(fftk_plan p, const float2* u, const float2* nh, double n
   const int width = 2 + s->kmax + 1;
   {
     LaunchScope ls(p, KK_NS_REDUCE, st);
-    k_diag<<<diag_blocks(width), DIAG_WARPS * 32, s->diag_smem, st>>>(u, nh, s->g, nu, s->kmax, s->part, nf);
+    launch_pdl(k_diag, diag_blocks(width), DIAG_WARPS * 32, s->diag_smem, st, u, nh, s->g, nu, s->kmax, s->part, nf);
   }
   {
     LaunchScope ls(p, KK_NS_REDUCE, st);
-    k_diag_final<<<diag_final_blocks(width), kFinCols * kFinRows, 0, st>>>(s->part, width, diag_blocks(width),
+    launch_pdl(k_diag_final, diag_final_blocks(width), kFinCols * kFinRows, 0, st, s->part, width, diag_blocks(width),
                                                        dout ? dout : s->dout);
   }
   return cudaGetLastError();
@@ -391,8 +393,9 @@ extern "C" fftk_status tarang_diag_noalloc(int n, const void* uhat, double nu, d
   // Every entry of the partials that k_diag_final reads is written by k_diag
   // in the same call, so nothing in the shared scratch needs clearing.
   const int smem = (int)(sizeof(double) * DIAG_WARPS * (kmax + 1));
-  k_diag<<<diag_blocks(width), DIAG_WARPS * 32, smem, st>>>(static_cast<const float2*>(uhat), nullptr, g, nu, kmax,
-                                                   scratch, 3);
-  k_diag_final<<<diag_final_blocks(width), kFinCols * kFinRows, 0, st>>>(scratch, width, diag_blocks(width), diag_dev);
+  launch_pdl(k_diag, diag_blocks(width), DIAG_WARPS * 32, smem, st, static_cast<const float2*>(uhat), nullptr, g, nu,
+             kmax, scratch, 3);
+  launch_pdl(k_diag_final, diag_final_blocks(width), kFinCols * kFinRows, 0, st, scratch, width, diag_blocks(width),
+             diag_dev);
   return from_cuda(cudaGetLastError());
 }

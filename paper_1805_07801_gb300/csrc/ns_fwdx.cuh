@@ -38,8 +38,10 @@ struct NUCfg {
   static constexpr int SLOTS = LOW + G - HIGH;
   using X = XTransform<N, G, -1, T, TWO>;
   static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 2 * (size_t)SLOTS * THREADS);
-  static constexpr int MINB = TWO ? 1 : N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
-                                         : (N >= 512 ? 1024 / THREADS : (512 / THREADS < 8 ? 512 / THREADS : 8));  // 64 registers, 128
+  static constexpr int MINB = TWO ? 1
+                                  : N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
+                                  : N >= 512   ? 1024 / THREADS  // 64 registers; below 512 points 128
+                                               : (512 / THREADS < 8 ? 512 / THREADS : 8);
   static constexpr int GROUP = N % 3 != 0 && N >= 512 && !TWO ? 2 : 4;  // modes whose loads are in flight together
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
@@ -55,6 +57,7 @@ __global__ void __launch_bounds__(NUCfg<N>::THREADS, NUCfg<N>::MINB)
     k_ns_fwdx(const float2* __restrict__ nh, const float2* u0, const float2* u1, float2* out,
               int ktiles, NSUpdate upd, const float2* __restrict__ extra, const float2* __restrict__ tw,
               const float2* __restrict__ t3) {
+  pdl_wait();
   constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace (nh)
   constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
@@ -142,7 +145,7 @@ static cudaError_t fwdx_nm(fftk_plan p, const float2* nh, const float2* u0, cons
   if (e != cudaSuccess) return e;
   constexpr int KD = (N - 1) / 3, KT = (KD + U::T) / U::T;  // k_z tiles of KD + 1 columns
   LaunchScope ls(p, KK_NS_FWDX, st);
-  k_ns_fwdx<N, MODE><<<(2 * KD + 1) * KT, U::THREADS, U::SMEM, st>>>(nh, u0, u1, out, KT, upd, extra,
+  launch_pdl(k_ns_fwdx<N, MODE>, (2 * KD + 1) * KT, U::THREADS, U::SMEM, st, nh, u0, u1, out, KT, upd, extra,
                                                                   twiddles(p, 1 << Log2<N>::value), p->d_tw3);
   return cudaGetLastError();
 }

@@ -33,6 +33,7 @@ template <int N, int SIGN>
 __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
     k_ns_ypass(const float2* w, float2* wo, int ktiles, const float2* __restrict__ tw,
                const float2* __restrict__ t3) {  // wo may be w
+  pdl_wait();
   constexpr long long H1 = ns_row(N), MM = (long long)N * N * H1;  // the padded workspace
   constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
   using C = NXCfg<N>;
@@ -89,6 +90,7 @@ template <int N, bool THETA = false>
 __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     k_ns_invx(const float2* __restrict__ u, float2* __restrict__ w, int ktiles, const float2* __restrict__ tw,
               const float2* __restrict__ t3) {
+  pdl_wait();
   constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace
   constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
@@ -212,7 +214,8 @@ template <int N, int MIN24 = 768>  // MIN24: 3 * 2^m lines from here on hold 24 
 struct NZCfg {
   static constexpr int H = N / 2;
   static constexpr int HB = line_slots(H);        // exchange slots per line
-  static constexpr int G = N % 3 == 0 ? (N >= MIN24 ? 24 : (H >= 48 ? 12 : 6)) : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
+  static constexpr int G = N % 3 == 0 ? (N >= MIN24 ? 24 : (H >= 48 ? 12 : 6))
+                                      : (N >= 512 ? 16 : (N >= 128 ? 8 : (H < 4 ? H : 4)));
   static constexpr int S = H / G;
   static constexpr int LPC = S >= 128 ? 1 : 128 / S;
   static constexpr int NBUF = G == 24 ? 1 : 2;    // staging buffers per line
@@ -223,7 +226,7 @@ struct NZCfg {
   static constexpr size_t FIELDS = sizeof(float2) * (size_t)LPC * (HB + 3 * H);  // exchange + 3 parked fields
   static constexpr size_t STAGE = sizeof(float2) * (size_t)LPC * NBUF * KCP;  // staging buffers
   static constexpr size_t SMEM = FIELDS + STAGE + sizeof(uint64_t) * NBUF * LPC;  // + one mbarrier per buffer
-  static constexpr int MINB = G == 16 || G == 24 ? 2 : (G == 12 || N == 256 ? 3 : 4);  // CTAs per SM the registers must allow
+  static constexpr int MINB = G == 16 || G == 24 ? 2 : (G == 12 || N == 256 ? 3 : 4);  // CTAs per SM
 };
 
 // 3. per (x, y) line: the six c2r transforms, the product n = u x omega and
@@ -240,6 +243,7 @@ struct NZCfg {
 template <int N, int HW>  // HW: row length of the workspace (n/2 + 1, or the fused path's padded rows)
 __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
     k_ns_z(const float2* w, float2* wo, const float2* __restrict__ tw, const float2* __restrict__ t3, int* err) {
+  pdl_wait();
   constexpr long long H1 = HW, MM = (long long)N * N * H1;  // geometry of the workspace
   using C = NZCfg<N>;
   constexpr int H = C::H, G = C::G, S = C::S;
@@ -423,8 +427,8 @@ struct NSLaunch {
     NSWork* s = p->ns;
     LaunchScope ls(p, KK_NS_Z, st);
     const long long lines = (long long)N * N;
-    k_ns_z<N, N / 2 + 1><<<(unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st>>>(
-        s->w, s->w, twiddles(p, N), nullptr, p->d_err);
+    launch_pdl(k_ns_z<N, N / 2 + 1>, (unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st, s->w, s->w,
+               twiddles(p, N), nullptr, p->d_err);
     return cudaGetLastError();
   }
 
@@ -451,15 +455,15 @@ struct NSLaunch {
     const float2* t3 = p->d_tw3;
     {
       LaunchScope ls(p, KK_NS_INVX, st);
-      k_ns_invx<N><<<g.nk * ki, I::THREADS, I::SMEM, st>>>(u, A, ki, tw, t3);
+      launch_pdl(k_ns_invx<N>, g.nk * ki, I::THREADS, I::SMEM, st, u, A, ki, tw, t3);
     }
     e = ns_ypass(p, A, Bw, 6, +1, KK_NS_INVY, st);
     if (e != cudaSuccess) return e;
     {
       LaunchScope ls(p, KK_NS_Z, st);
       const long long lines = (long long)N * N;
-      k_ns_z<N, (int)ns_row(N)><<<(unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st>>>(
-          Bw, A, tw, t3, p->d_err);
+      launch_pdl(k_ns_z<N, (int)ns_row(N)>, (unsigned)((lines + Z::LPC - 1) / Z::LPC), Z::THREADS, Z::SMEM, st, Bw, A,
+                 tw, t3, p->d_err);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = ns_ypass(p, A, A, 3, -1, KK_NS_FWDY, st);

@@ -31,6 +31,7 @@ template <int N>
 __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
     k_shell_invx(const float2* __restrict__ u, float2* __restrict__ w, ShellRange sh, int ktiles,
                  const float2* __restrict__ tw) {
+  pdl_wait();
   constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;
   using C = NXCfg<N>;
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
 template <int N>
 __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
     k_shell_invy(float2* a, float2* __restrict__ b, int kb, int ktiles, const float2* __restrict__ tw) {
+  pdl_wait();
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;
   using C = NXCfg<N>;
   constexpr int G = C::G, S = C::S, T = C::T;
@@ -110,6 +112,7 @@ template <int N>
 __global__ void __launch_bounds__(NZCfg<N>::THREADS, SZCfg3<N>::MINB)
     k_shell_z(float2* a, const float2* __restrict__ b, const float* __restrict__ ur, int kb,
               const float2* __restrict__ tw) {
+  pdl_wait();
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW, R = (long long)N * N * N;
   using C = NZCfg<N>;
   constexpr int H = C::H, G = C::G, S = C::S, KC = C::KC;
@@ -184,6 +187,7 @@ template <int N>
 __global__ void __launch_bounds__(NXCfg<N>::THREADS, NXCfg<N>::MINB)
     k_shell_fwdx(const float2* __restrict__ a, float2* __restrict__ out, int ktiles, float scale,
                  const float2* __restrict__ tw) {
+  pdl_wait();
   constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;
   constexpr int KD = (N - 1) / 3, NK = 2 * KD + 1;
@@ -236,23 +240,23 @@ static cudaError_t shell_advect_n(fftk_plan p, const float2* u, const float* ur,
   float2* B = p->ns->w2;
   {
     LaunchScope ls(p, KK_X_INV, st);
-    k_shell_invx<N><<<3 * (2 * sh.kb + 1) * kt, X::THREADS, X::SMEM, st>>>(u, A, sh, kt, tw);
+    launch_pdl(k_shell_invx<N>, 3 * (2 * sh.kb + 1) * kt, X::THREADS, X::SMEM, st, u, A, sh, kt, tw);
   }
   {
     LaunchScope ls(p, KK_Y_INV, st);
-    k_shell_invy<N><<<6 * N * kt, X::THREADS, X::SMEM, st>>>(A, B, sh.kb, kt, tw);
+    launch_pdl(k_shell_invy<N>, 6 * N * kt, X::THREADS, X::SMEM, st, A, B, sh.kb, kt, tw);
   }
   {
     LaunchScope ls(p, KK_AUX, st);
-    k_shell_z<N><<<(unsigned)(((long long)N * N + Z::LPC - 1) / Z::LPC), Z::THREADS, SZCfg3<N>::SMEM, st>>>(
-        A, B, ur, sh.kb, tw);
+    launch_pdl(k_shell_z<N>, (unsigned)(((long long)N * N + Z::LPC - 1) / Z::LPC), Z::THREADS, SZCfg3<N>::SMEM, st, A,
+               B, ur, sh.kb, tw);
   }
   const cudaError_t ey = ns_ypass(p, A, A, 3, -1, KK_Y_FWD, st);
   if (ey != cudaSuccess) return ey;
   {
     LaunchScope ls(p, KK_X_FWD, st);
-    k_shell_fwdx<N><<<3 * (2 * KD + 1) * KT, X::THREADS, X::SMEM, st>>>(
-        A, out, KT, (float)(1.0 / ((double)N * N * N)), tw);
+    launch_pdl(k_shell_fwdx<N>, 3 * (2 * KD + 1) * KT, X::THREADS, X::SMEM, st, A, out, KT,
+               (float)(1.0 / ((double)N * N * N)), tw);
   }
   return cudaGetLastError();
 }

@@ -37,6 +37,7 @@ template <int N, int SIGN>
 __global__ void __launch_bounds__(YPipeCfg<N, SIGN>::THREADS, YPipeCfg<N, SIGN>::MINB)
     k_ns_ypipe(const __grid_constant__ CUtensorMap map, float2* out, int ntiles, const float2* __restrict__ tw,
                const float2* __restrict__ t3, int* err) {
+  pdl_wait();
   using C = YPipeCfg<N, SIGN>;
   constexpr long long HW = ns_row(N);
   constexpr int G = C::G, S = C::S, T = C::T, KD = C::KD, KT = (KD + T) / T;
@@ -148,7 +149,8 @@ static cudaError_t ypass_n(fftk_plan p, const float2* in, float2* out, int field
     if (encode_f32_map(&m, in, 3, dims, strides, box)) {
       const int ntiles = fields * N * ((KD + C::T) / C::T), cap = nsm[dev] * C::MINB;
       LaunchScope ls(p, kind, st);
-      k_ns_ypipe<N, SIGN><<<ntiles < cap ? ntiles : cap, C::THREADS, C::SMEM, st>>>(m, out, ntiles, tw, p->d_tw3,
+      launch_pdl(k_ns_ypipe<N, SIGN>, ntiles < cap ? ntiles : cap, C::THREADS, C::SMEM, st, m, out, ntiles, tw,
+                 p->d_tw3,
                                                                                   p->d_err);
       return cudaGetLastError();
     }
@@ -161,7 +163,7 @@ static cudaError_t ypass_n(fftk_plan p, const float2* in, float2* out, int field
   if (e != cudaSuccess) return e;
   constexpr int KT = (KD + X::T) / X::T;
   LaunchScope ls(p, kind, st);
-  k_ns_ypass<N, SIGN><<<fields * N * KT, X::THREADS, X::SMEM, st>>>(in, out, KT, tw, p->d_tw3);
+  launch_pdl(k_ns_ypass<N, SIGN>, fields * N * KT, X::THREADS, X::SMEM, st, in, out, KT, tw, p->d_tw3);
   return cudaGetLastError();
 }
 

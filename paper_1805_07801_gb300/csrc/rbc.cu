@@ -96,6 +96,7 @@ static fftk_status rbc_tables(fftk_plan p, double Ra, double Pr, double dt) {
 // w7 = [u_x, omega_y, omega_z, theta | u_y, u_z, omega_x]: sine group, then
 // cosine group (each contiguous, for one batched transform per group)
 __global__ void k_rbc_sff_prep(const float2* __restrict__ x, float2* __restrict__ w7, NSGeom g) {
+  pdl_wait();
   const long long M = g.M, rowa = (long long)g.n * g.h1;  // one step of the x index
   const long long HW = ns_row(g.n), MW = (long long)g.n * g.n * HW, roww = (long long)g.n * HW;  // of w7
   // the kept modes only (the pruned inverse passes read nothing else; the
@@ -164,6 +165,7 @@ __device__ __forceinline__ void rbc_entry_update(long long i, float2 n, float2 E
 // gradient of the cosine pressure p = -div v / k^2; N_theta = -div(u theta) + u_x.
 __global__ void k_rbc_sff_update(const float2* __restrict__ w7, const float2* x, const float2* u0, float2* s1,
                                  float2* acc, float2* out, NSGeom g, RBCUpdate upd, int mode) {
+  pdl_wait();
   const long long M = g.M, rowa = (long long)g.n * g.h1;
   const long long HW = ns_row(g.n), MW = (long long)g.n * g.n * HW, roww = (long long)g.n * HW;  // of w7
   const int nx = (2 * g.n - 1) / 3 + 1;  // the kept modes, k_z fastest
@@ -235,7 +237,7 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
     // w7 = [u_x, omega_y, omega_z, theta | u_y, u_z, omega_x]: sine group, cosine group
     {
       LaunchScope ls(p, KK_RBC_PREP, st);
-      k_rbc_sff_prep<<<grid, 256, 0, st>>>(x, w, g);
+      launch_pdl(k_rbc_sff_prep, grid, 256, 0, st, x, w, g);
     }
     e = launch_scpass_pruned(p, true, +1, w, w, 4, 1.f, st);
     if (e == cudaSuccess) e = launch_scpass_pruned(p, false, +1, w + 4 * mw, w + 4 * mw, 3, 1.f, st);
@@ -249,7 +251,7 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
     if (e != cudaSuccess) return e;
     {
       LaunchScope ls(p, KK_RBC_UPDATE, st);
-      k_rbc_sff_update<<<grid, 256, 0, st>>>(w, x, u0, r->s1, r->acc, out, g, upd, mode);
+      launch_pdl(k_rbc_sff_update, grid, 256, 0, st, w, x, u0, r->s1, r->acc, out, g, upd, mode);
     }
     return cudaGetLastError();
   }

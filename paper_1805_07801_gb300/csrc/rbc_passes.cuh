@@ -105,6 +105,7 @@ struct RZCfg {
 template <int N>
 __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
     k_rbc_z(float2* w, RBCSlots sl, const float2* __restrict__ tw, const float2* __restrict__ t3, int* err) {
+  pdl_wait();
   constexpr long long HW = ns_row(N), MM = (long long)N * N * HW;
   using C = RZCfg<N>;
   constexpr int H = C::H, G = C::G, S = C::S, KC = C::KC, NB = C::NBUF;
@@ -267,6 +268,7 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
     k_rbc_fwdx(const float2* __restrict__ w, const float2* x, const float2* u0, const float2* s1, float2* acc,
                float2* out, int ktiles, RBCUpdate upd, float scale, const float2* __restrict__ tw,
                const float2* __restrict__ t3) {
+  pdl_wait();
   constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace
   constexpr int KD = (N - 1) / 3;
@@ -382,7 +384,7 @@ static cudaError_t rbc_invx_n(fftk_plan p, const float2* x, float2* w, cudaStrea
   if (e != cudaSuccess) return e;
   constexpr int KD = (N - 1) / 3, KT = (KD + I::T) / I::T;
   LaunchScope ls(p, KK_X_INV, st);
-  k_ns_invx<N, true><<<(2 * KD + 1) * KT, I::THREADS, I::SMEM, st>>>(x, w, KT, twiddles(p, 1 << Log2<N>::value),
+  launch_pdl(k_ns_invx<N, true>, (2 * KD + 1) * KT, I::THREADS, I::SMEM, st, x, w, KT, twiddles(p, 1 << Log2<N>::value),
                                                                   p->d_tw3);
   return cudaGetLastError();
 }
@@ -397,8 +399,8 @@ static cudaError_t rbc_z_n(fftk_plan p, float2* w, const RBCSlots& sl, cudaStrea
   if (e != cudaSuccess) return e;
   const long long lines = (long long)N * N;
   LaunchScope ls(p, KK_RBC_Z, st);
-  k_rbc_z<N><<<(unsigned)((lines + C::LPC - 1) / C::LPC), C::THREADS, C::SMEM, st>>>(
-      w, sl, twiddles(p, 1 << Log2<N>::value), p->d_tw3, p->d_err);
+  launch_pdl(k_rbc_z<N>, (unsigned)((lines + C::LPC - 1) / C::LPC), C::THREADS, C::SMEM, st, w, sl, twiddles(p,
+             1 << Log2<N>::value), p->d_tw3, p->d_err);
   return cudaGetLastError();
 }
 
@@ -412,7 +414,8 @@ static cudaError_t rbc_fwdx_nm(fftk_plan p, const RBCStage& s, cudaStream_t st) 
   if (e != cudaSuccess) return e;
   constexpr int KD = (N - 1) / 3, KT = (KD + U::T) / U::T;
   LaunchScope ls(p, KK_RBC_UPDATE, st);
-  k_rbc_fwdx<N, MODE><<<(2 * KD + 1) * KT, U::THREADS, U::SMEM, st>>>(s.w, s.x, s.u0, s.s1, s.acc, s.out, KT, s.upd,
+  launch_pdl(k_rbc_fwdx<N, MODE>, (2 * KD + 1) * KT, U::THREADS, U::SMEM, st, s.w, s.x, s.u0, s.s1, s.acc, s.out, KT,
+             s.upd,
                                                                    s.scale, twiddles(p, 1 << Log2<N>::value),
                                                                    p->d_tw3);
   return cudaGetLastError();
