@@ -374,6 +374,11 @@ struct LineX {
   __device__ __forceinline__ int at(int pos) const { return (kMap4 ? swz_line4(pos) : swz_line(pos)) ^ x; }
   __device__ __forceinline__ void st(int pos, float2 v) const { s[at(pos)] = v; }
   __device__ __forceinline__ float2 ld(int pos) const { return s[at(pos)]; }
+  // unpermuted, for a line that is stored in the natural pattern and read as
+  // its mirror H - k: both are runs of consecutive slots (the permuted mirror
+  // took two wavefronts for one)
+  __device__ __forceinline__ void st_run(int pos, float2 v) const { s[pos ^ x] = v; }
+  __device__ __forceinline__ float2 ld_run(int pos) const { return s[pos ^ x]; }
   __device__ __forceinline__ void sync() const {
     if constexpr (WARP_SYNC)
       __syncwarp();

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   for (int m = 0; m < G; ++m) v[m] = valid ? src[j + m * S] : make_float2(0.f, 0.f);
   fft_line<H, G, -1, LOGN>(v, j, xc, tw, t3);
 #pragma unroll
-  for (int m = 0; m < G; ++m) xc.st(j + m * S, v[m]);
+  for (int m = 0; m < G; ++m) xc.st_run(j + m * S, v[m]);
   xc.sync();
   if (valid) {
     float2* dst = out + line * (H + 1);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
       const float2 A = v[m];
-      const float2 Bc = cconj(xc.ld(mirror<H>(k)));
+      const float2 Bc = cconj(xc.ld_run(mirror<H>(k)));
       const float2 E = cscale(cadd(A, Bc), 0.5f);
       const float2 D = csub(A, Bc);
       const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);  // D / (2i)
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
 #pragma unroll
   for (int m = 0; m < G; ++m) {
     v[m] = valid ? src[j + m * S] : make_float2(0.f, 0.f);
-    xc.st(j + m * S, v[m]);
+    xc.st_run(j + m * S, v[m]);
   }
   const float2 XH = valid ? src[H] : make_float2(0.f, 0.f);
   // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   for (int m = 0; m < G; ++m) {
     const int k = j + m * S;
     float2 A = v[m];
-    float2 B = k == 0 ? XH : xc.ld(H - k);
+    float2 B = k == 0 ? XH : xc.ld_run(H - k);
     if (k == 0) {
       A.y = 0.f;
       B.y = 0.f;

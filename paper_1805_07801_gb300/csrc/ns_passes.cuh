@@ -334,14 +334,14 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
   auto r2c = [&](int f, float2 (&U)[G]) {
     fft_line<H, G, -1, LOGN>(U, j, xc, tw, t3);
 #pragma unroll
-    for (int m = 0; m < G; ++m) xc.st(j + m * S, U[m]);
+    for (int m = 0; m < G; ++m) xc.st_run(j + m * S, U[m]);
     xc.sync();
     float2* dst = wo + f * MM + line * H1;
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
       const float2 A = U[m];
-      const float2 Bc = cconj(xc.ld(mirror<H>(k)));
+      const float2 Bc = cconj(xc.ld_run(mirror<H>(k)));
       const float2 E = cscale(cadd(A, Bc), 0.5f);
       const float2 D = csub(A, Bc);
       const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);

@@ -166,13 +166,13 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, SZCfg3<N>::MINB)
     }
     fft_line<H, G, -1, LOGN>(acc, j, xc, tw);
 #pragma unroll
-    for (int m = 0; m < G; ++m) xc.st(j + m * S, acc[m]);
+    for (int m = 0; m < G; ++m) xc.st_run(j + m * S, acc[m]);
     xc.sync();
     float2* dst = a + i * MW + line * HW;
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
-      const float2 Bc = cconj(xc.ld(mirror<H>(k)));
+      const float2 Bc = cconj(xc.ld_run(mirror<H>(k)));
       const float2 E = cscale(cadd(acc[m], Bc), 0.5f);
       const float2 D = csub(acc[m], Bc);
       const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);
