@@ -140,9 +140,11 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
 // ------------------------------------------------------- strided c2c pass --
 // Tile = T adjacent columns (contiguous index q) x the full line (L rows of
 // stride Q).  Loads and stores are T-wide row segments, coalesced along q.
-// Tile width T per line length: 32 warps per SM at <= 64 registers per
-// thread (2 CTAs of 512 threads up to L = 512, one of 1024 beyond), and row
-// segments of 128 bytes (T = 16) where the 227 KB of shared memory allows.
+// Tile width T per line length: 16 columns (128-byte rows) where the 227 KB of
+// shared memory allows and at least 64 threads come together; 32 warps per SM at
+// <= 64 registers per thread.  (256 threads per CTA with up to 256 columns, two
+// CTAs per SM: y passes of short rows left most columns empty.  Pairs: 64 fields
+// of 32^3 39 -> 25 us, 64 of 64^3 186 -> 149 us, 8 of 128^3 174 -> 140 us.)
 // Lines of 3 * 2^m points hold 24 values per thread at <= 128 registers, 512
 // threads per SM.
 template <int L>
@@ -150,9 +152,9 @@ struct CCfg {
   static constexpr int G = elems_per_thread(L);
   static constexpr int S = L / G;
   static constexpr int MAXT = L % 3 == 0 ? 512 : 1024;
-  static constexpr int T = S <= 16 ? (L % 3 == 0 ? 16 : 256 / S) : (16 * S <= MAXT ? 16 : MAXT / S);
+  static constexpr int T = S <= 16 ? (L % 3 == 0 ? 16 : (S >= 4 ? 16 : 64 / S)) : (16 * S <= MAXT ? 16 : MAXT / S);
   static constexpr int THREADS = T * S;
-  static constexpr int MINB = L % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1)) : (THREADS <= 512 ? 2 : 1);
+  static constexpr int MINB = L % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1)) : (1024 / THREADS < 16 ? 1024 / THREADS : 16);
   static constexpr size_t SMEM = sizeof(float2) * (size_t)L * T;
 };
 

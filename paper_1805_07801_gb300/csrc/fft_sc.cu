@@ -32,9 +32,9 @@ template <int L>
 struct SCfg {
   static constexpr int G = elems_per_thread(L);
   static constexpr int S = L / G;
-  static constexpr int T = S <= 16 ? 256 / S : (S <= 64 ? 16 : 1024 / S);
+  static constexpr int T = S <= 16 ? (S >= 4 ? 16 : 64 / S) : (S <= 64 ? 16 : 1024 / S);
   static constexpr int THREADS = T * S;
-  static constexpr int MINB = THREADS <= 512 ? 2 : 1;
+  static constexpr int MINB = 1024 / THREADS < 16 ? 1024 / THREADS : 16;
   static constexpr size_t SMEM = sizeof(float2) * (size_t)L * T;
 };
 
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(SCfg<L>::THREADS, SCfg<L>::MINB)
       }
     }
   } else {
-// the mirror coefficient C_{L-k} is a second read of another thread's row
+    // the mirror coefficient C_{L-k} is a second read of another thread's row
     // (an exchange through shared memory instead: 57 us per launch at 256^3, so
     // 54 us)
     float2 w[G];
