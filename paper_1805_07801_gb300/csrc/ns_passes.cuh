@@ -86,13 +86,14 @@ struct NICfg {
 //    omega_z = D_y - i k_y U_x   (five transforms instead of six).
 //    Output field order: u_x, u_y, u_z, omega_x, omega_y, omega_z.
 //    THETA (convection): field 3 of u, the temperature, goes to field 6 of w.
-template <int N, bool THETA = false>
+//    PADDED: u has the padded rows of the stage states.
+template <int N, bool THETA = false, bool PADDED = false>
 __global__ void __launch_bounds__(NICfg<N>::THREADS, NICfg<N>::MINB)
     k_ns_invx(const float2* __restrict__ u, float2* __restrict__ w, int ktiles, const float2* __restrict__ tw,
               const float2* __restrict__ t3) {
   pdl_wait();
-  constexpr long long H1 = N / 2 + 1, MM = (long long)N * N * H1;  // geometry of the n^3 grid
   constexpr long long HW = ns_row(N), MW = (long long)N * N * HW;  // the padded workspace
+  constexpr long long H1 = PADDED ? HW : N / 2 + 1, MM = (long long)N * N * H1;  // u
   constexpr int KD = (N - 1) / 3;                                  // largest kept |k| (2/3 rule)
   using C = NICfg<N>;
   constexpr int G = C::G, S = C::S, T = C::T;

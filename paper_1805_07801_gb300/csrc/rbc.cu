@@ -50,11 +50,12 @@ static fftk_status rbc_ensure(fftk_plan p) {
   const int kxs = (2 * g.n - 1) / 3;
   r->tab_len = kxs * kxs + 2 * g.kd * g.kd + 1;
   const size_t fw = sizeof(float2) * (size_t)g.n * g.n * (size_t)ns_row(g.n);  // padded rows
+  const size_t fs = fw > fb ? fw : fb;  // the periodic cube pads the stage state's and the accumulator's rows too
   cudaError_t e = cudaMalloc(&r->w7, 7 * fw);
-  if (e == cudaSuccess) e = cudaMalloc(&r->s1, 4 * fb);
-  if (e == cudaSuccess) e = cudaMemset(r->s1, 0, 4 * fb);
-  if (e == cudaSuccess) e = cudaMalloc(&r->acc, 4 * fb);
-  if (e == cudaSuccess) e = cudaMemset(r->acc, 0, 4 * fb);
+  if (e == cudaSuccess) e = cudaMalloc(&r->s1, 4 * fs);
+  if (e == cudaSuccess) e = cudaMemset(r->s1, 0, 4 * fs);
+  if (e == cudaSuccess) e = cudaMalloc(&r->acc, 4 * fs);
+  if (e == cudaSuccess) e = cudaMemset(r->acc, 0, 4 * fs);
   if (e == cudaSuccess) e = cudaMalloc(&r->tab, sizeof(float2) * 4 * (size_t)r->tab_len);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -256,7 +257,7 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
     return cudaGetLastError();
   }
   // w7 = [u_x, u_y, u_z, omega_x, omega_y, omega_z, theta] -> [n_x, n_y, n_z, u_x theta, ...]
-  e = rbc_invx(p, x, w, st);
+  e = rbc_invx(p, x, x == r->s1, w, st);
   if (e == cudaSuccess) e = ns_ypass(p, w, w, 7, +1, KK_Y_INV, st);
   const RBCSlots sl{{0, 1, 2, 3, 4, 5, 6}, {0, 1, 2, 3, 4, 5}};
   if (e == cudaSuccess) e = rbc_z(p, w, sl, st);

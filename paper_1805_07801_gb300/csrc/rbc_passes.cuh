@@ -21,9 +21,10 @@ __device__ __forceinline__ float2 mul_pair(float2 v, float2 E) {  // v * (hi + l
 }
 
 // the update of entry i of one field in mode MODE (the modes of
-// ns_mode_update): N = n, a = u0, b = the stage state or the accumulator
+// ns_mode_update): N = n, a = u0, b = the stage state or the accumulator; i is
+// the entry of out, ia that of the accumulator
 template <int MODE>
-__device__ __forceinline__ void rbc_entry_store(long long i, float2 n, float2 a, float2 b, float2 E, float2 H, float dt,
+__device__ __forceinline__ void rbc_entry_store(long long i, long long ia, float2 n, float2 a, float2 b, float2 E, float2 H, float dt,
                                                 float2* acc, float2* out) {
   if constexpr (MODE == NS_RHS) {
     out[i] = n;
@@ -36,11 +37,11 @@ __device__ __forceinline__ void rbc_entry_store(long long i, float2 n, float2 a,
     out[i] = make_float2(fmaf(dt / 6.f, n.x, b.x), fmaf(dt / 6.f, n.y, b.y));
   } else if constexpr (MODE == NS_RK4_1) {
     const float2 ea = mul_pair(a, E), en = mul_pair(n, E);
-    acc[i] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
+    acc[ia] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
     out[i] = mul_pair(make_float2(a.x + 0.5f * dt * n.x, a.y + 0.5f * dt * n.y), H);
   } else {
     const float2 hn = mul_pair(n, H);
-    acc[i] = make_float2(fmaf(dt / 3.f, hn.x, b.x), fmaf(dt / 3.f, hn.y, b.y));
+    acc[ia] = make_float2(fmaf(dt / 3.f, hn.x, b.x), fmaf(dt / 3.f, hn.y, b.y));
     if constexpr (MODE == NS_RK4_2) {
       const float2 ha = mul_pair(a, H);
       out[i] = make_float2(fmaf(0.5f * dt, n.x, ha.x), fmaf(0.5f * dt, n.y, ha.y));
@@ -61,10 +62,10 @@ struct RBCSlots {
 // What the launchers of one stage need besides the plan.
 struct RBCStage {
   float2* w;          // 7 fields, padded rows
-  const float2* x;    // the stage's input state
+  const float2* x;    // the stage's input state (the stage state from the second stage on)
   const float2* u0;   // the step's state
-  const float2* s1;   // stage state
-  float2* acc;        // RK4 accumulator
+  const float2* s1;   // stage state, padded rows
+  float2* acc;        // RK4 accumulator, padded rows
   float2* out;
   RBCUpdate upd;
   int mode;
@@ -76,8 +77,9 @@ cudaError_t rbc_z(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
 cudaError_t rbc_z3(fftk_plan p, float2* w, const RBCSlots& sl, cudaStream_t st);
 // periodic cube: the inverse x pass with the curl (state -> 7 fields), and the
 // forward x pass with the update (6 fields -> out)
-cudaError_t rbc_invx(fftk_plan p, const float2* x, float2* w, cudaStream_t st);
-cudaError_t rbc_invx3(fftk_plan p, const float2* x, float2* w, cudaStream_t st);
+// (padded: x is the stage state)
+cudaError_t rbc_invx(fftk_plan p, const float2* x, bool padded, float2* w, cudaStream_t st);
+cudaError_t rbc_invx3(fftk_plan p, const float2* x, bool padded, float2* w, cudaStream_t st);
 cudaError_t rbc_fwdx(fftk_plan p, const RBCStage& s, cudaStream_t st);
 cudaError_t rbc_fwdx3(fftk_plan p, const RBCStage& s, cudaStream_t st);
 
@@ -288,6 +290,11 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
   C::X::init(smn, tw, t3);
   const int ky = kwav(ay, N);
   const float2* bsrc = MODE == NS_STAGE2 ? s1 : acc;
+  // the caller's state has rows of n/2 + 1, the stage state and the accumulator
+  // padded ones: entry (row pos, this column) of a field
+  constexpr bool XP = MODE == NS_STAGE2 || MODE >= NS_RK4_2;                        // x
+  constexpr bool OP = MODE == NS_STAGE1 || (MODE >= NS_RK4_1 && MODE != NS_RK4_4);  // out
+  constexpr long long XM = XP ? MW : MM, OM = OP ? MW : MM;
   float2 V[G];
 #pragma unroll 1
   for (int i = 0; i < 6; ++i) {
@@ -302,15 +309,15 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
       }
       if (i == 4 || i == 5)
         for (int r = threadIdx.x; r < 2 * KD + 1; r += C::THREADS) {
-          const long long o = dense_to_a(r, N, KD) * rs + q - c;
+          const long long o = dense_to_a(r, N, KD) * rs + q - c, ow = dense_to_a(r, N, KD) * rw + qw - c;
           if (i == 4) {
-            prefetch_l2(x + 2 * MM + o);
-            prefetch_l2(x + 3 * MM + o);
+            prefetch_l2(x + 2 * XM + (XP ? ow : o));
+            prefetch_l2(x + 3 * XM + (XP ? ow : o));
           }
 #pragma unroll
           for (int f2 = 0; f2 < 4; ++f2) {
             if (A0 && i == 4) prefetch_l2(u0 + f2 * MM + o);
-            if (B0 && i == 5) prefetch_l2(bsrc + f2 * MM + o);
+            if (B0 && i == 5) prefetch_l2(bsrc + f2 * MW + ow);
           }
         }
     }
@@ -336,14 +343,14 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
   for (int m = 0; m < G; ++m) {
     const int pos = j + m * S;
     if (!C::parked(m) || !kept_xy(pos, N, KD)) continue;
-    const long long idx = pos * rs + q;
+    const long long idx = pos * rs + q, idw = pos * rw + qw;
     const int kx = kwav(pos, N), k2 = kx * kx + ky * ky + kz * kz;
     float2 a[4], b[4];
-    const float2 uz = x[idx + 2 * MM], th = x[idx + 3 * MM];
+    const float2 uz = x[(XP ? idw : idx) + 2 * XM], th = x[(XP ? idw : idx) + 3 * XM];
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       if (A0) a[f] = u0[idx + f * MM];
-      if (B0) b[f] = bsrc[idx + f * MM];
+      if (B0) b[f] = bsrc[idw + f * MW];
     }
     float2 E[2], H[2];
 #pragma unroll
@@ -369,24 +376,30 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
     }
 #pragma unroll
     for (int f = 0; f < 4; ++f)
-      rbc_entry_store<MODE>(idx + f * MM, nv[f], a[f], b[f], E[f == 3 ? 1 : 0], H[f == 3 ? 1 : 0], dt, acc, out);
+      rbc_entry_store<MODE>((OP ? idw : idx) + f * OM, idw + f * MW, nv[f], a[f], b[f], E[f == 3 ? 1 : 0],
+                            H[f == 3 ? 1 : 0], dt, acc, out);
   }
 }
 
 // ------------------------------------------------------------ launchers ----
-template <int N>
-static cudaError_t rbc_invx_n(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
+template <int N, bool PADDED>
+static cudaError_t rbc_invx_np(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
   using I = NICfg<N>;
   static PerDevice once;
   const cudaError_t e = once.run([](int) {
-    return cudaFuncSetAttribute(k_ns_invx<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I::SMEM);
+    return cudaFuncSetAttribute(k_ns_invx<N, true, PADDED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)I::SMEM);
   });
   if (e != cudaSuccess) return e;
   constexpr int KD = (N - 1) / 3, KT = (KD + I::T) / I::T;
   LaunchScope ls(p, KK_X_INV, st);
-  launch_pdl(k_ns_invx<N, true>, (2 * KD + 1) * KT, I::THREADS, I::SMEM, st, x, w, KT, twiddles(p, 1 << Log2<N>::value),
-                                                                  p->d_tw3);
+  launch_pdl(k_ns_invx<N, true, PADDED>, (2 * KD + 1) * KT, I::THREADS, I::SMEM, st, x, w, KT,
+             twiddles(p, 1 << Log2<N>::value), p->d_tw3);
   return cudaGetLastError();
+}
+
+template <int N>
+static cudaError_t rbc_invx_n(fftk_plan p, const float2* x, bool padded, float2* w, cudaStream_t st) {
+  return padded ? rbc_invx_np<N, true>(p, x, w, st) : rbc_invx_np<N, false>(p, x, w, st);
 }
 
 template <int N>

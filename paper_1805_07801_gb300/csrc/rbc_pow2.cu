@@ -3,15 +3,15 @@
 
 namespace fftk {
 
-cudaError_t rbc_invx(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
+cudaError_t rbc_invx(fftk_plan p, const float2* x, bool padded, float2* w, cudaStream_t st) {
   switch (p->nx) {
 #define CASE(n) \
   case n:       \
-    return rbc_invx_n<n>(p, x, w, st);
+    return rbc_invx_n<n>(p, x, padded, w, st);
     CASE(8) CASE(16) CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024)
 #undef CASE
     default:
-      return rbc_invx3(p, x, w, st);
+      return rbc_invx3(p, x, padded, w, st);
   }
 }
 

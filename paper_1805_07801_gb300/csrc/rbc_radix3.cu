@@ -3,11 +3,11 @@
 
 namespace fftk {
 
-cudaError_t rbc_invx3(fftk_plan p, const float2* x, float2* w, cudaStream_t st) {
+cudaError_t rbc_invx3(fftk_plan p, const float2* x, bool padded, float2* w, cudaStream_t st) {
   switch (p->nx) {
 #define CASE(n) \
   case n:       \
-    return rbc_invx_n<n>(p, x, w, st);
+    return rbc_invx_n<n>(p, x, padded, w, st);
     CASE(12) CASE(24) CASE(48) CASE(96) CASE(192) CASE(384) CASE(768)
 #undef CASE
   }
