@@ -246,7 +246,10 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
 // transformed, then n_x and n_y.  512^3, per launch: forward x pass 528 us and
 // update 922 us as kernels of their own, 1135 us fused (1607 us with all its L2
 // prefetches at the start instead of one field ahead, 1351 us with radices 8, 8,
-// 8 on 1024 threads instead of 32, 16 on 256).
+// 8 on 1024 threads instead of 32, 16 on 256), 1088 us with padded rows for the
+// stage state and the accumulator, 1052 us with the loads of four modes in
+// flight in the update.  Its six fields and eighteen kept arrays would take 632
+// us: eight warps do not cover the loads of each field and the exchanges.
 template <int N>
 struct RUCfg {
   static constexpr bool TWO = N == 512;  // radix 32, then 16
@@ -261,6 +264,9 @@ struct RUCfg {
   using X = XTransform<N, G, -1, T, TWO>;
   static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 3 * (size_t)SLOTS * THREADS);
   static constexpr int MINB = THREADS >= 512 ? 1 : (THREADS == 256 ? (N == 768 || TWO ? 1 : 2) : 4);
+  // modes whose loads are in flight together (1024 has no registers for two;
+  // four at 3 * 2^m spill, 384^3 422 us against 388 with two and 405 with one)
+  static constexpr int GROUP = N == 1024 ? 1 : (N % 3 == 0 ? 2 : 4);
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };
@@ -339,25 +345,40 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
   }
   if (!valid) return;
   const float fky = (float)ky, fkz = (float)kz, dt = upd.dt;
+  // out may be x or u0, which orders loads after stores: the loads of GROUP
+  // modes come before their first store
+  constexpr int NG = C::GROUP;
+  static_assert(G % NG == 0, "groups of modes");
+  float2 ga[NG][4], gb[NG][4], gx[NG][2], gE[NG][2], gH[NG][2];
 #pragma unroll
   for (int m = 0; m < G; ++m) {
-    const int pos = j + m * S;
+    if (m % NG == 0) {
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        const int pos = j + (m + i) * S;
+        if (!C::parked(m + i) || !kept_xy(pos, N, KD)) continue;
+        const long long idx = pos * rs + q, idw = pos * rw + qw;
+        const int kx = kwav(pos, N), k2 = kx * kx + ky * ky + kz * kz;
+        gx[i][0] = x[(XP ? idw : idx) + 2 * XM];
+        gx[i][1] = x[(XP ? idw : idx) + 3 * XM];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          if (A0) ga[i][f] = u0[idx + f * MM];
+          if (B0) gb[i][f] = bsrc[idw + f * MW];
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          if (MODE != NS_RHS && MODE != NS_RK4_4) gE[i][t] = __ldg(&upd.tab[t * upd.tab_len + k2]);
+          if (MODE >= NS_RK4_1 && MODE != NS_RK4_4) gH[i][t] = __ldg(&upd.tab[(2 + t) * upd.tab_len + k2]);
+        }
+      }
+    }
+    const int pos = j + m * S, gi = m % NG;
     if (!C::parked(m) || !kept_xy(pos, N, KD)) continue;
     const long long idx = pos * rs + q, idw = pos * rw + qw;
     const int kx = kwav(pos, N), k2 = kx * kx + ky * ky + kz * kz;
-    float2 a[4], b[4];
-    const float2 uz = x[(XP ? idw : idx) + 2 * XM], th = x[(XP ? idw : idx) + 3 * XM];
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      if (A0) a[f] = u0[idx + f * MM];
-      if (B0) b[f] = bsrc[idw + f * MW];
-    }
-    float2 E[2], H[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      if (MODE != NS_RHS && MODE != NS_RK4_4) E[t] = __ldg(&upd.tab[t * upd.tab_len + k2]);
-      if (MODE >= NS_RK4_1 && MODE != NS_RK4_4) H[t] = __ldg(&upd.tab[(2 + t) * upd.tab_len + k2]);
-    }
+    const float2 uz = gx[gi][0], th = gx[gi][1];
+    const float2 *a = ga[gi], *b = gb[gi], *E = gE[gi], *H = gH[gi];
     const float2 dv = park[C::slot(m) * C::THREADS];
     float2 px = cscale(park[(C::SLOTS + C::slot(m)) * C::THREADS], scale);
     float2 py = cscale(park[(2 * C::SLOTS + C::slot(m)) * C::THREADS], scale);
