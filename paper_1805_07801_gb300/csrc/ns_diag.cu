@@ -15,8 +15,8 @@ namespace fftk {
 
 // nint(|k|) for integer |k|^2, exact: an FP32 square root corrected by
 // integer comparisons; |k| >= K + 1/2 exactly when k2 >= K^2 + K + 1.
-__device__ __forceinline__ long long shell_index(long long k2) {
-  long long K = (long long)floorf(sqrtf((float)k2));
+__device__ __forceinline__ int shell_index(int k2) {
+  int K = (int)floorf(sqrtf((float)k2));
   while (K * K > k2) --K;
   while ((K + 1) * (K + 1) <= k2) ++K;
   if (k2 >= K * K + K + 1) ++K;
@@ -89,6 +89,8 @@ __device__ __forceinline__ float scale2(float v, int k) {
 // left to one histogram update per run.  Items are assigned to warps by a
 // fixed grid stride over diag_blocks(width) blocks; partials per block are
 // summed in block order by k_diag_final.
+// Items, modes and k^2 are 32-bit numbers (cubes to 1024: 5.1 million items);
+// only the element offset needs 64 bits.
 // With nh == nullptr the per-mode value is the energy 1/2 w |u|^2 (slots:
 // E, eps, E(K)); otherwise it is the transfer w Re(conj(u) . nh) (slots:
 // sum_K T(K), 0, T(K)).  Slot 0 is the sum of the shells.  nf: the number
@@ -105,18 +107,17 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
   __syncthreads();
   double* h = hist + warp * nb;
   const int nchunk = (g.kc + 31) / 32;
-  const long long items = (long long)g.nk * g.nk * nchunk;
+  const int items = g.nk * g.nk * nchunk;
   const bool dissip = !nh;
   double accD = 0.0;
   // the next item's loads are in flight while this one is reduced
-  auto fetch = [&](long long it, float (&a)[6], float (&b)[6], int& kz, long long& k2) {
-    const long long line = it / nchunk;
-    const int chunk = (int)(it - line * nchunk);
-    const int ax = dense_to_a((int)(line / g.nk), g.n, g.kd);
-    const int ay = dense_to_a((int)(line % g.nk), g.n, g.kd);
+  auto fetch = [&](int it, float (&a)[6], float (&b)[6], int& kz, int& k2) {
+    const int line = it / nchunk, chunk = it - line * nchunk;
+    const int ax = dense_to_a(line / g.nk, g.n, g.kd);
+    const int ay = dense_to_a(line % g.nk, g.n, g.kd);
     kz = chunk * 32 + lane;
-    const long long kx = kwav(ax, g.n), ky = kwav(ay, g.n);
-    k2 = kx * kx + ky * ky + (long long)kz * kz;
+    const int kx = kwav(ax, g.n), ky = kwav(ay, g.n);
+    k2 = kx * kx + ky * ky + kz * kz;
     const long long idx = ((long long)ax * g.n + ay) * g.h1 + kz;
 #pragma unroll
     for (int f = 0; f < 3; ++f) {
@@ -131,11 +132,11 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
       b[2 * f + 1] = q.y;
     }
   };
-  const long long stride = (long long)gridDim.x * DIAG_WARPS;
-  long long it = (long long)blockIdx.x * DIAG_WARPS + warp;
+  const int stride = gridDim.x * DIAG_WARPS;
+  int it = blockIdx.x * DIAG_WARPS + warp;
   float an[6], bn[6];
   int kzn = 0;
-  long long k2n = 0;
+  int k2n = 0;
   if (it < items) fetch(it, an, bn, kzn, k2n);
   for (; it < items; it += stride) {
     float a[6], b[6];
@@ -145,13 +146,13 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
       b[i] = bn[i];
     }
     const int kz = kzn;
-    const long long k2 = k2n;
+    const int k2 = k2n;
     if (it + stride < items) fetch(it + stride, an, bn, kzn, k2n);
     const bool valid = kz < g.kc;
     int shell = kmax + 1;
     if (valid) {
-      const long long K = shell_index(k2);
-      shell = K <= kmax ? (int)K : kmax + 1;
+      const int K = shell_index(k2);
+      shell = K <= kmax ? K : kmax + 1;
     }
     float amax = 0.f, bmax = 0.f;
 #pragma unroll
@@ -209,15 +210,22 @@ __global__ void __launch_bounds__(DIAG_WARPS * 32)
   if (lane == 0) wd[warp] = accD;
   __syncthreads();
   double* out = part + (long long)blockIdx.x * (2 + nb);
+  // the sum of the shells: by thread, by warp, then in warp order
+  __shared__ double ws[DIAG_WARPS];
+  double all = 0.0;
   for (int s = threadIdx.x; s < nb; s += blockDim.x) {
     double t = 0.0;
     for (int w2 = 0; w2 < DIAG_WARPS; ++w2) t += hist[w2 * nb + s];
     out[2 + s] = t;
+    all += t;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) all += __shfl_down_sync(0xffffffffu, all, o);
+  if (lane == 0) ws[warp] = all;
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;
-    for (int s = 0; s < nb; ++s) a += out[2 + s];
+    for (int w2 = 0; w2 < DIAG_WARPS; ++w2) a += ws[w2];
     for (int w2 = 0; w2 < DIAG_WARPS; ++w2) b += wd[w2];
     out[0] = a;
     out[1] = 2.0 * nu * b;
