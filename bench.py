@@ -108,9 +108,12 @@ def fft_pass_bytes(n):
 
 # --------------------------------------------------- measured DRAM traffic ---
 KERNEL_SOURCES = {
-    "ns": ["ns.cu", "ns_passes.cuh", "ns_radix3.cu", "ns_common.cuh", "fft_engine.cuh", "internal.h", "tcgen05.cuh"],
-    "fft": ["fft_passes.cu", "fft_engine.cuh", "internal.h", "abi.cu"],
-    "fft16": ["fft_tc.cu", "tcgen05.cuh", "fft_passes.cu", "fft_engine.cuh", "internal.h", "abi.cu"],
+    "ns": ["ns.cu", "ns_passes.cuh", "ns_update.cuh", "ns_fwdx.cuh", "ns_fwdx.cu", "ns_fwdx3.cu", "ns_ypass.cu",
+           "ns_radix3.cu", "ns_common.cuh", "fft_pipe.cuh", "fft_engine.cuh", "internal.h", "tcgen05.cuh"],
+    "fft": ["fft_passes.cu", "fft_stream.cu", "fft_pass_kernels.cuh", "fft_pipe.cuh", "fft_engine.cuh",
+            "sc_algebra.cuh", "tcgen05.cuh", "internal.h", "abi.cu"],
+    "fft16": ["fft_tc.cu", "tcgen05.cuh", "fft_passes.cu", "fft_pass_kernels.cuh", "fft_engine.cuh", "internal.h",
+              "abi.cu"],
 }
 
 
@@ -862,7 +865,7 @@ def run_schemes(n: int, steps: int):
     fk.fftk_plan_destroy(plan)
     import oracle
 
-    no = 128 if fused else 96
+    no = 128 if n & (n - 1) == 0 else 96
     uo = _oracle_state(no)
     out["oracle_cpu"] = oracle_beside("oracle RK4 step", no, lambda: oracle.ns_step_rk4(uo, NU, DT, 1), "steps/s")
     print(json.dumps({"workload": f"{n}^3 decaying turbulence, nu={NU}, dt={DT}, seed {SEED}",

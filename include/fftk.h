@@ -162,8 +162,7 @@ fftk_status fftk_inverse(fftk_plan p, const int *basis, const void *in, float *o
  * a six-field workspace (rows of n/2 + 1 complex values rounded up to a
  * multiple of 16), the three-field stage state, and for FP32 plans a second
  * six-field workspace that the fused passes alternate with the first (about
- * 8.5 GB at 512^3); 3 * 2^m cubes add six real fields.  Out of memory is
- * FFTK_ERR_OOM. */
+ * 8.5 GB at 512^3).  Out of memory is FFTK_ERR_OOM. */
 /* Learned subgrid-stress model (not in the paper; see tarang_mlp_*): the
  * network maps the 5 invariants of the resolved velocity gradient A
  * (tr S^2, tr R^2, tr S^3, tr R^2 S, tr R^2 S^2 with S, R the symmetric and
@@ -243,11 +242,10 @@ fftk_status tarang_ns_step(fftk_plan p, void *uhat, const tarang_params *prm, in
  * the z pass; between plates the x passes are sine/cosine passes.  FP32 in
  * both plan dtypes.  Cubes: n a power of two in [8, 1024] for both bases;
  * the periodic cube also takes n = 3 * 2^m in [12, 768] (the paper's XC40
- * convection sizes, Sec. 7), where the right-hand side runs through the
- * plan's full transforms (radix-3 passes) with the products formed in real
- * space (7 more real fields).  Other sizes: FFTK_ERR_UNSUPPORTED_SIZE.
- * Device memory: 15 more complex fields (allocated on first use, kept by
- * the plan). */
+ * convection sizes, Sec. 7), through the same fused passes.  Other sizes:
+ * FFTK_ERR_UNSUPPORTED_SIZE.
+ * Device memory: 15 more complex fields, seven of them with rows of n/2 + 1
+ * rounded up to a multiple of 16 (allocated on first use, kept by the plan). */
 enum { TARANG_RBC_FFF = 0, TARANG_RBC_SFF = 1 };
 
 typedef struct {
@@ -316,15 +314,16 @@ fftk_status tarang_transfer(fftk_plan p, const void *uhat, const tarang_params *
  * shell g through advection by the whole field.  T is antisymmetric, the
  * givers of a receiver add up to its share of tarang_transfer's T(K), and
  * the flux through a bound b is the sum of T(r <- g) over r >= b > g.
- * Evaluated pseudo-spectrally with the plan's transforms: u to real space
- * once, then per giver shell the gradient of its modes (nine c2r), the
- * product u_j d_j u_g,i (real space), three r2c and an FP64 reduction over
- * receivers in a fixed order (bitwise reproducible).  Givers beyond the
+ * Evaluated pseudo-spectrally: u to real space once, then per giver shell the
+ * inverse x and y passes of its modes, one z pass that forms the gradient and
+ * the product u_j d_j u_g,i in real space, the forward y and x passes and an
+ * FP64 reduction over receivers in a fixed order (bitwise reproducible).  Givers beyond the
  * dealiased radius are skipped (zero columns).
  * nshells: 1 .. kmax + 1; bounds: host array of nshells + 1 strictly
  * increasing integers in [0, kmax + 1] (kmax of tarang_diag_kmax); out_host:
- * nshells * nshells doubles, row-major by receiver.  Device memory: nine more
- * real fields (allocated on first use and kept by the plan).  Uses the plan's
+ * nshells * nshells doubles, row-major by receiver.  Device memory: three more
+ * real fields and the solver's second six-field workspace (allocated on first
+ * use and kept by the plan).  Uses the plan's
  * solver workspace (do not overlap with tarang_ns_step on the same plan);
  * synchronises cuda_stream.  INVALID_ARG for bad bounds, NONFINITE if any
  * entry is not finite. */

@@ -10,7 +10,11 @@
 // accumulators per thread (8 x 4), whose operands come from shared memory as
 // 16-byte loads (three per 32 multiply-adds), and the gradient of the two
 // 64 x 64 layers stays in registers from chunk to chunk.  Two CTAs share an
-// SM, so one fills the other's barriers.
+// SM, so one fills the other's barriers.  Batch of 65536: gradient 1019 -> 127
+// us (one sample per thread, weights by broadcast loads, before; the FP32 pipes
+// alone would take 45 us), with the sliced reduction and Adam 1121 -> 137 us.
+// Shared-memory loads are what bounds it: a 16-byte load takes four wavefronts
+// however many lanes share an address.
 #include <cuda_bf16.h>
 
 #include "internal.h"

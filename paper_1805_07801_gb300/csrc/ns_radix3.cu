@@ -2,7 +2,9 @@
 // runs use 768^3, Sec. 6): the kernels of ns_passes.cuh on lines whose last
 // stage takes the factor 3.  768^3 RK2 step: 64.8 ms through the plan's full
 // transforms with the products in real space, 30.2 ms fused (384^3: 8.07 and
-// 3.24 ms, 96^3: 0.26 and 0.12 ms).
+// 3.24 ms, 96^3: 0.26 and 0.12 ms), 22.1 ms with the y and forward x passes in
+// two long-radix stages (ns_ypass.cu, ns_fwdx3.cu) and 24 values per thread in
+// the z lines.
 #include <mutex>
 
 #include "ns_passes.cuh"
