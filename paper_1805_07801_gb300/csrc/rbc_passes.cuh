@@ -242,13 +242,15 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
 
 // ---- forward x pass with the update (periodic cube) ------------------------
 // As the Navier-Stokes forward x pass (ns_fwdx.cuh), with six fields and three
-// parked arrays: the divergence k . F(u theta), summed as its three fields are
-// transformed, then n_x and n_y.  512^3, per launch: forward x pass 528 us and
+// parked arrays: the divergence k . F(u theta), then n_x and n_y.  k_y and k_z
+// are constant along a line, so k_y u_y theta + k_z u_z theta is formed before
+// its transform: five transforms for six fields.  512^3, per launch: forward x pass 528 us and
 // update 922 us as kernels of their own, 1135 us fused (1607 us with all its L2
 // prefetches at the start instead of one field ahead, 1351 us with radices 8, 8,
 // 8 on 1024 threads instead of 32, 16 on 256), 1088 us with padded rows for the
 // stage state and the accumulator, 1052 us with the loads of four modes in
-// flight in the update.  Its six fields and eighteen kept arrays would take 632
+// flight in the update, 1014 us with five transforms (256^3 126 -> 119 us, 384^3
+// 388 -> 363 us).  Its six fields and eighteen kept arrays would take 632
 // us: eight warps do not cover the loads of each field and the exchanges.
 template <int N>
 struct RUCfg {
@@ -303,44 +305,54 @@ __global__ void __launch_bounds__(RUCfg<N>::THREADS, RUCfg<N>::MINB)
   constexpr long long XM = XP ? MW : MM, OM = OP ? MW : MM;
   float2 V[G];
 #pragma unroll 1
-  for (int i = 0; i < 6; ++i) {
-    const int f = i < 3 ? 3 + i : i - 3;  // u theta first, then n
+  for (int i = 0; i < 5; ++i) {
+    // u_x theta, k_y u_y theta + k_z u_z theta, then n
+    const int f = i < 2 ? 3 + i : i - 2;
 #pragma unroll
     for (int m = 0; m < G; ++m)
       V[m] = valid ? w[f * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
-    if constexpr (N >= 256) {  // the next field, and at last the update's reads, go to L2 meanwhile (see k_ns_fwdx)
-      if (i < 5) {
-        const int nf = i < 2 ? 4 + i : i - 2;
-        for (int r = threadIdx.x; r < N; r += C::THREADS) prefetch_l2(w + nf * MW + r * rw + qw - c);
+    if (i == 1) {
+#pragma unroll
+      for (int m = 0; m < G; ++m) {
+        const float2 t = valid ? w[5 * MW + (j + m * S) * rw + qw] : make_float2(0.f, 0.f);
+        V[m] = make_float2(fmaf((float)kz, t.x, (float)ky * V[m].x), fmaf((float)kz, t.y, (float)ky * V[m].y));
       }
-      if (i == 4 || i == 5)
+    }
+    if constexpr (N >= 256) {  // the next field, and at last the update's reads, go to L2 meanwhile (see k_ns_fwdx)
+      if (i < 4) {
+        const int nf = i == 0 ? 4 : i - 1;
+        for (int r = threadIdx.x; r < N; r += C::THREADS) {
+          prefetch_l2(w + nf * MW + r * rw + qw - c);
+          if (i == 0) prefetch_l2(w + 5 * MW + r * rw + qw - c);
+        }
+      }
+      if (i == 3 || i == 4)
         for (int r = threadIdx.x; r < 2 * KD + 1; r += C::THREADS) {
           const long long o = dense_to_a(r, N, KD) * rs + q - c, ow = dense_to_a(r, N, KD) * rw + qw - c;
-          if (i == 4) {
+          if (i == 3) {
             prefetch_l2(x + 2 * XM + (XP ? ow : o));
             prefetch_l2(x + 3 * XM + (XP ? ow : o));
           }
 #pragma unroll
           for (int f2 = 0; f2 < 4; ++f2) {
-            if (A0 && i == 4) prefetch_l2(u0 + f2 * MM + o);
-            if (B0 && i == 5) prefetch_l2(bsrc + f2 * MW + ow);
+            if (A0 && i == 3) prefetch_l2(u0 + f2 * MM + o);
+            if (B0 && i == 4) prefetch_l2(bsrc + f2 * MW + ow);
           }
         }
     }
     C::X::run(V, j, c, smn, tw, t3);
-    if (i < 3) {
+    if (i < 2) {
 #pragma unroll
       for (int m = 0; m < G; ++m)
         if (C::parked(m)) {
-          const float kf = i == 0 ? (float)kwav(j + m * S, N) : (i == 1 ? (float)ky : (float)kz);
           float2& d = park[C::slot(m) * C::THREADS];
           const float2 v = cscale(V[m], scale);
-          d = i == 0 ? make_float2(kf * v.x, kf * v.y) : make_float2(fmaf(kf, v.x, d.x), fmaf(kf, v.y, d.y));
+          d = i == 0 ? cscale(v, (float)kwav(j + m * S, N)) : cadd(d, v);
         }
-    } else if (i < 5) {
+    } else if (i < 4) {
 #pragma unroll
       for (int m = 0; m < G; ++m)
-        if (C::parked(m)) park[((i - 2) * C::SLOTS + C::slot(m)) * C::THREADS] = V[m];
+        if (C::parked(m)) park[((i - 1) * C::SLOTS + C::slot(m)) * C::THREADS] = V[m];
     }
   }
   if (!valid) return;
