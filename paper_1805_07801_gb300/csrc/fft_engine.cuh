@@ -27,14 +27,19 @@
 // the issue-bound kernels (the fused Navier-Stokes passes); a translation
 // unit whose kernels are bound by their global accesses instead (the plain
 // strided passes, measured slower with them) defines FFTK_PAIRED_FP32 as 0
-// before including this header.  The engine lives in an inline namespace
-// named after the choice, so the two forms never meet at link time.
+// before including this header.  2: the rotations by constants take one too
+// (the fused passes of powers of two: without it the 512-point inverse x pass
+// spills 8 bytes; the sine/cosine passes and the shell transfer run 1 to 7 %
+// slower with it).  The engine lives in an inline namespace named after the
+// choice, so the forms never meet at link time.
 #ifndef FFTK_PAIRED_FP32
 #define FFTK_PAIRED_FP32 1
 #endif
 
 namespace fftk {
-#if FFTK_PAIRED_FP32
+#if FFTK_PAIRED_FP32 == 2
+inline namespace paired_rot_fp32 {
+#elif FFTK_PAIRED_FP32
 inline namespace paired_fp32 {
 #else
 inline namespace scalar_fp32 {
@@ -57,8 +62,11 @@ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
 }
 #if FFTK_PAIRED_FP32
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
+// a s + b
+__device__ __forceinline__ float2 cscale_add(float2 a, float s, float2 b) { return __ffma2_rn(a, make_float2(s, s), b); }
 #else
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+__device__ __forceinline__ float2 cscale_add(float2 a, float s, float2 b) { return make_float2(fmaf(a.x, s, b.x), fmaf(a.y, s, b.y)); }
 #endif
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 // a * (SIGN * i)
@@ -76,22 +84,40 @@ struct Log2<1> {
   static constexpr int value = 0;
 };
 
-// Mathematical constants of the 8- and 16-point DFTs.
-#define FFTK_C8 0.70710678118654752440f   // cos(pi/4)
-#define FFTK_C16 0.92387953251128675613f  // cos(pi/8)
-#define FFTK_S16 0.38268343236508977173f  // sin(pi/8)
+// Mathematical constants of the 8- and 16-point DFTs (in FP64: rot rounds them).
+#define FFTK_C8 0.70710678118654752440   // cos(pi/4)
+#define FFTK_C16 0.92387953251128675613  // cos(pi/8)
+#define FFTK_S16 0.38268343236508977173  // sin(pi/8)
 
-// a * exp(SIGN i theta) with (cos, sin) = (c, s)
+// a * exp(SIGN i theta) with (cos, sin) = (c, s), constants after inlining.  The
+// larger of the two is applied as 1 + (c - 1), a multiply-add in place of the
+// product: rounded to FP32, the cosines of pi/16, pi/8 and pi/4 are all below the
+// true ones, by 3.0e-8, 3.1e-8 and 1.7e-8, so that every factor shrinks its value
+// and the losses add up over a transform and its inverse; the rounding of c - 1
+// weighs a third of that at most.  Round-trip error of a line, rounded -> so: 1024
+// points (32 x 32) 1.65e-7 -> 1.46e-7, 512 (32 x 16) 1.50e-7 -> 1.37e-7, 256
+// (16 x 16) 1.38e-7 -> 1.28e-7, in the same number of operations.  (pi/4, where
+// both components are the larger one, gains nothing and is left.)
 template <int SIGN>
-__device__ __forceinline__ float2 rot(float2 a, float c, float s) {
-  return cmul(a, make_float2(c, SIGN * s));
+__device__ __forceinline__ float2 rot(float2 a, double c, double s) {
+  const double t = SIGN * s, ac = c < 0. ? -c : c, at = t < 0. ? -t : t;
+  const float fc = (float)c, ft = (float)t;
+  if (ac == at) return cmul(a, make_float2(fc, ft));
+  const float m = (float)((ac > at ? ac : at) - 1.);
+#if FFTK_PAIRED_FP32 == 2
+  const float2 z = cscale_add(a, m, a);
+#else
+  const float2 z = make_float2(fmaf(a.x, m, a.x), fmaf(a.y, m, a.y));
+#endif
+  if (ac > at) return make_float2(fmaf(-a.y, ft, c < 0. ? -z.x : z.x), fmaf(a.x, ft, c < 0. ? -z.y : z.y));
+  return make_float2(fmaf(a.x, fc, t < 0. ? z.y : -z.y), fmaf(a.y, fc, t < 0. ? -z.x : z.x));
 }
 
 // cos and sin of pi/16 and 3 pi/16
-#define FFTK_C32A 0.98078528040323044913f
-#define FFTK_S32A 0.19509032201612826785f
-#define FFTK_C32B 0.83146961230254523708f
-#define FFTK_S32B 0.55557023301960222474f
+#define FFTK_C32A 0.98078528040323044913
+#define FFTK_S32A 0.19509032201612826785
+#define FFTK_C32B 0.83146961230254523708
+#define FFTK_S32B 0.55557023301960222474
 
 // a * exp(-2 pi i q / 32) for a q (0 <= q < 32) known at compile time after
 // unrolling: the eighth-turn remainder by its (cos, sin) constants, then the
@@ -115,13 +141,13 @@ __device__ __forceinline__ float2 mul_root32(float2 a, int q) {
 }
 
 // cos and sin of pi/24, 2 pi/24 and 5 pi/24
-#define FFTK_C48A 0.99144486137381041114f
-#define FFTK_S48A 0.13052619222005159155f
-#define FFTK_C48B 0.96592582628906828675f
-#define FFTK_S48B 0.25881904510252076235f
-#define FFTK_C48E 0.79335334029123516458f
-#define FFTK_S48E 0.60876142900872063942f
-#define FFTK_C6 0.86602540378443864676f  // cos(pi/6) = sin(pi/3)
+#define FFTK_C48A 0.99144486137381041114
+#define FFTK_S48A 0.13052619222005159155
+#define FFTK_C48B 0.96592582628906828675
+#define FFTK_S48B 0.25881904510252076235
+#define FFTK_C48E 0.79335334029123516458
+#define FFTK_S48E 0.60876142900872063942
+#define FFTK_C6 0.86602540378443864676  // cos(pi/6) = sin(pi/3)
 
 // a * exp(-2 pi i m / NR) for m in [0, NR/2) known at compile time, NR a power
 // of two up to 32 (mul_root32), 12, 24 or 48 (the same split for lines of
@@ -138,11 +164,11 @@ __device__ __forceinline__ float2 mul_root(float2 a, int m) {
       case 1: r = rot<-1>(a, FFTK_C48A, FFTK_S48A); break;
       case 2: r = rot<-1>(a, FFTK_C48B, FFTK_S48B); break;
       case 3: r = rot<-1>(a, FFTK_C16, FFTK_S16); break;
-      case 4: r = rot<-1>(a, FFTK_C6, 0.5f); break;
+      case 4: r = rot<-1>(a, FFTK_C6, 0.5); break;
       case 5: r = rot<-1>(a, FFTK_C48E, FFTK_S48E); break;
       case 6: r = rot<-1>(a, FFTK_C8, FFTK_C8); break;
       case 7: r = rot<-1>(a, FFTK_S48E, FFTK_C48E); break;
-      case 8: r = rot<-1>(a, 0.5f, FFTK_C6); break;
+      case 8: r = rot<-1>(a, 0.5, FFTK_C6); break;
       case 9: r = rot<-1>(a, FFTK_S16, FFTK_C16); break;
       case 10: r = rot<-1>(a, FFTK_S48B, FFTK_C48B); break;
       default: r = rot<-1>(a, FFTK_S48A, FFTK_C48A); break;
@@ -150,6 +176,29 @@ __device__ __forceinline__ float2 mul_root(float2 a, int m) {
     return q >= 12 ? mul_si<-1>(r) : r;
   }
 }
+
+// The Hermitian-split factors exp(-2 pi i k / N), k = j + m S, of a thread with G
+// values of a packed line (N = 2 G S points; t: the size-N table).  With four
+// values one correctly rounded load for each; else W_j times the roots of order
+// 2 G, whose product adds a rounding of its own.  (At 16 values per thread in
+// k_ns_z one load per value and use instead: 1.190 against 1.126 ms per launch at
+// 512^3.)
+template <int N, int G, bool TABLE = G == 4>
+struct SplitFactors {
+  static constexpr int S = N / (2 * G), LOADS = TABLE ? G : 1;
+  float2 w[LOADS];
+  __device__ __forceinline__ SplitFactors(const float2* __restrict__ t, int j) {
+#pragma unroll
+    for (int m = 0; m < LOADS; ++m) w[m] = __ldg(&t[j + m * S]);
+  }
+  __device__ __forceinline__ float2 operator()(int m) const {
+    if constexpr (TABLE) {
+      return w[m];
+    } else {
+      return mul_root<2 * G>(w[0], m);
+    }
+  }
+};
 
 // index of the mirror H - k of entry k of a packed line of H values (k = 0: itself)
 template <int H>
@@ -251,17 +300,24 @@ __device__ __forceinline__ void dft32(float2 (&x)[32]) {
   for (int k = 0; k < 32; ++k) x[k] = o[k];
 }
 
-// X1,2 = a - (b + c)/2 +- SIGN i sin(pi/3) (b - c)
-template <int SIGN>
+// X1,2 = a - (b + c)/2 +- SIGN i sin(pi/3) (b - c).  FUSED: the last product and
+// sum as one multiply-add each, a rounding less.
+template <int SIGN, bool FUSED>
 __device__ __forceinline__ void dft3(float2& a, float2& b, float2& c) {
-  const float2 s = cadd(b, c), d = cscale(mul_si<SIGN>(csub(b, c)), FFTK_C6);
+  const float2 s = cadd(b, c), d = mul_si<SIGN>(csub(b, c));
   const float2 t = make_float2(fmaf(-0.5f, s.x, a.x), fmaf(-0.5f, s.y, a.y));
   a = cadd(a, s);
-  b = cadd(t, d);
-  c = csub(t, d);
+  if constexpr (FUSED) {
+    b = cscale_add(d, (float)FFTK_C6, t);
+    c = cscale_add(make_float2(-d.x, -d.y), (float)FFTK_C6, t);
+  } else {
+    const float2 h = cscale_add(d, (float)(FFTK_C6 - 1.), d);  // as in rot
+    b = cadd(t, h);
+    c = csub(t, h);
+  }
 }
 
-template <int R, int SIGN>
+template <int R, int SIGN, bool FUSED = true>
 __device__ __forceinline__ void dftR(float2 (&a)[R]) {
   if constexpr (R % 3 == 0) {
     // R = 3 P, P = 1, 2, 4, 8 or 16: 3 and P have no common factor, so the DFT is
@@ -270,7 +326,7 @@ __device__ __forceinline__ void dftR(float2 (&a)[R]) {
     constexpr int P = R / 3;
     constexpr int E1 = P == 1 ? 1 : (P >= 8 ? 16 : 4), E2 = P == 1 ? 0 : (P == 2 ? 3 : (P == 16 ? 33 : 9));
 #pragma unroll
-    for (int n2 = 0; n2 < P; ++n2) dft3<SIGN>(a[3 * n2], a[(P + 3 * n2) % R], a[(2 * P + 3 * n2) % R]);
+    for (int n2 = 0; n2 < P; ++n2) dft3<SIGN, FUSED>(a[3 * n2], a[(P + 3 * n2) % R], a[(2 * P + 3 * n2) % R]);
     float2 o[R];
 #pragma unroll
     for (int k1 = 0; k1 < 3; ++k1) {
@@ -320,6 +376,7 @@ __device__ __forceinline__ int swz(int pos) {
 // Exchange buffer for a column tile: element (pos, c) of a [L][T] tile.
 template <int T>
 struct ColX {
+  static constexpr bool kTight = false;
   static constexpr bool kStageTables = false;  // a warp spans 32/T butterflies: gathers are near-broadcasts
   float2* s;
   int c;
@@ -364,9 +421,11 @@ __device__ __forceinline__ int line_xor(int li) {
 }
 
 // Exchange buffer for one contiguous line of S threads with G values each;
-// WARP_SYNC when a line's threads live in one warp.
-template <bool WARP_SYNC, int S = 32, int G = 16>
+// WARP_SYNC when a line's threads live in one warp.  TIGHT: a kernel without
+// registers to spare (see dft3).
+template <bool WARP_SYNC, int S = 32, int G = 16, bool TIGHT = false>
 struct LineX {
+  static constexpr bool kTight = TIGHT;
   static constexpr bool kStageTables = true;  // a warp spans 32 consecutive butterflies
   static constexpr bool kMap4 = G != 16 && (S < 16 || G % 8 != 0);
   float2* s;
@@ -473,7 +532,7 @@ struct Stage {
             a[r] = SIGN < 0 ? cmul(a[r], w) : cmulc(a[r], w);
           }
         }
-        dftR<R, SIGN>(a);
+        dftR<R, SIGN, !X::kTight>(a);
         if constexpr (LAST) {
 #pragma unroll
           for (int r = 0; r < R; ++r) v[t + r * B] = a[r];

@@ -23,7 +23,7 @@ namespace fftk {
 // slower with 8 (two 512^3 fields 2277 against 2190 us).
 __host__ __device__ constexpr int z_elems(int H) {
   if (H % 3 == 0) return H >= 192 ? 24 : (H >= 48 ? 12 : 6);
-  if (H <= 16) return H < 2 ? H : 2;
+  if (H < 16) return H < 2 ? H : 2;
   return H <= 64 ? 4 : (H <= 128 ? 8 : 16);
 }
 
@@ -37,6 +37,9 @@ struct ZCfg {
   static constexpr int LPC = S >= MAXT ? 1 : MAXT / S;  // lines per CTA
   static constexpr int THREADS = LPC * S;
   static constexpr bool WARP = S <= 32;
+  // split factors from the table: lines of 24 points have 3 % less error so (and
+  // those of 48 would take 4 % longer for half a percent)
+  static constexpr bool TABLE = G == 4 || (G == 6 && S <= 2);
   static constexpr int MINB = 4;  // 32 warps per SM at <= 64 registers (3 * 2^m: 16 at <= 128)
 };
 
@@ -67,8 +70,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
   xc.sync();
   if (valid) {
     float2* dst = out + line * (H + 1);
-    // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
-    const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
+    const SplitFactors<N, G, C::TABLE> split(N % 3 == 0 ? t3 + N : tw, j);
 #pragma unroll
     for (int m = 0; m < G; ++m) {
       const int k = j + m * S;
@@ -77,7 +79,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
       const float2 E = cscale(cadd(A, Bc), 0.5f);
       const float2 D = csub(A, Bc);
       const float2 O = make_float2(0.5f * D.y, -0.5f * D.x);  // D / (2i)
-      dst[k] = cscale(cadd(E, cmul(mul_root<2 * G>(Wj, m), O)), scale);
+      dst[k] = cscale(cadd(E, cmul(split(m), O)), scale);
     }
     if (j == 0) dst[H] = make_float2((v[0].x - v[0].y) * scale, 0.f);
   }
@@ -111,8 +113,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     xc.st_run(j + m * S, v[m]);
   }
   const float2 XH = valid ? src[H] : make_float2(0.f, 0.f);
-  // exp(-2 pi i k / N) = W_j exp(-2 pi i m / 2G), k = j + m S
-  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
+  const SplitFactors<N, G, C::TABLE> split(N % 3 == 0 ? t3 + N : tw, j);
   xc.sync();
 #pragma unroll
   for (int m = 0; m < G; ++m) {
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(ZCfg<N>::THREADS, ZCfg<N>::MINB)
     }
     const float2 Bc = cconj(B);
     const float2 E = cadd(A, Bc);
-    const float2 O = cmulc(csub(A, Bc), mul_root<2 * G>(Wj, m));
+    const float2 O = cmulc(csub(A, Bc), split(m));
     v[m] = make_float2(E.x - O.y, E.y + O.x);
   }
   xc.sync();  // every mirror has been read before the transform's exchanges

@@ -22,6 +22,7 @@
 #include <new>
 #include <vector>
 
+#define FFTK_PAIRED_FP32 2  // see fft_engine.cuh
 #include "ns_passes.cuh"
 
 namespace fftk {

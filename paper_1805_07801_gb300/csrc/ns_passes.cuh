@@ -254,7 +254,8 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
   const int li = threadIdx.x / S, j = threadIdx.x % S;
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < (long long)N * N;
-  const LineX<C::WARP, S, G> xc{smz + li * C::HB, line_xor<S>(li)};
+  // (dft3 with multiply-adds would spill 24 bytes at 96 points: step 64.7 -> 67.5 us)
+  const LineX<C::WARP, S, G, (N % 3 == 0 && G == 12)> xc{smz + li * C::HB, line_xor<S>(li)};
   float2* park = smz + C::LPC * C::HB + li * 3 * H + j;  // [3][G][S] per line, this thread's column
   constexpr int NB = C::NBUF;
   float2* stage = smz + C::FIELDS / sizeof(float2) + li * NB * C::KCP;  // this line's buffers
@@ -289,12 +290,7 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, NZCfg<N>::MINB)
     for (int b = 0; b < NB; ++b) issue(b);
   }
   xc.sync();  // the barriers are initialised before anyone polls them
-  // exp(-2 pi i k / N) at k = j + m S is Wj exp(-2 pi i m / (2G)) (N = 2 G S):
-  // one table load per thread instead of one per value
-  // (measured against one table load per value at 16 values per thread:
-  // 1.126 against 1.190 ms per launch at 512^3)
-  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
-  auto twk = [&](int m) { return mul_root<2 * G>(Wj, m); };
+  const SplitFactors<N, G> twk(N % 3 == 0 ? t3 + N : tw, j);
 
   // inverse z transform of field f (half-complex -> N real points, two per slot)
   auto c2r = [&](int f, float2 (&U)[G]) {

@@ -122,8 +122,7 @@ __global__ void __launch_bounds__(NZCfg<N>::THREADS, SZCfg3<N>::MINB)
   const long long line = (long long)blockIdx.x * C::LPC + li;
   const bool valid = line < (long long)N * N;
   const LineX<C::WARP, S, G> xc{sms + li * C::HB, line_xor<S>(li)};
-  const float2 Wj = __ldg(&tw[j]);
-  auto twk = [&](int m) { return mul_root<2 * G>(Wj, m); };
+  const SplitFactors<N, G> twk(tw, j);
   float2* park = sms + C::LPC * C::HB + li * 3 * H + j;  // u, [3][G][S], two real points per slot
 #pragma unroll
   for (int q = 0; q < 3; ++q) {

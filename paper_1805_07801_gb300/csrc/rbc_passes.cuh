@@ -146,8 +146,7 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
     for (int b = 0; b < NB; ++b) issue(b);
   }
   xc.sync();  // the barriers are initialised before anyone polls them
-  const float2 Wj = __ldg(N % 3 == 0 ? &t3[N + j] : &tw[j]);
-  auto twk = [&](int m) { return mul_root<2 * G>(Wj, m); };
+  const SplitFactors<N, G> twk(N % 3 == 0 ? t3 + N : tw, j);
 
   auto c2r = [&](int f, float2(&U)[G]) {
     const float2* src = stage + (f % NB) * C::KCP;
