@@ -417,7 +417,8 @@ fftk_status tarang_les_stress(fftk_plan p, const float *ubar, const float *tau, 
  * FP32 values W1[64][5], b1[64], W2[64][64], b2[64], W3[64][64], b3[64],
  * W4[6][64], b4[6].  Each layer's input (x, h1, h2, h3) is rounded to
  * bfloat16; products and sums are FP32.  x: [B][5], y and targets t: [B][6].
- * A context owns the per-block gradient partials for up to max_batch samples;
+ * A context owns the per-block gradient partials for up to max_batch samples
+ * (36 KB per block: 11 MB at 65536 samples, 44 MB at 2^20);
  * gradients are reduced in a fixed order (bitwise reproducible). */
 typedef struct tarang_mlp_s *tarang_mlp;
 fftk_status tarang_mlp_create(int max_batch, tarang_mlp *out);
@@ -445,8 +446,9 @@ fftk_status tarang_sgs_train(tarang_mlp m, float *params, float *adam_m, float *
  * context's inference expired since the last call (the flag is cleared). */
 fftk_status tarang_mlp_sync(tarang_mlp m, void *cuda_stream);
 /* Mean-squared-error loss (1/(6B)) sum (y - t)^2 (device double, may be NULL)
- * and its gradient grad[9094] (device), on the CUDA cores (128 samples per
- * block, per-block partials summed in a fixed order). */
+ * and its gradient grad[9094] (device), on the CUDA cores: FP32 sums over 64
+ * samples and up to 14 such chunks per block, the blocks' sums added in FP64 in
+ * a fixed order. */
 fftk_status tarang_mlp_loss_grad(tarang_mlp m, const float *params, const float *x, const float *t,
                                  int B, float *grad, double *loss, void *cuda_stream);
 /* Layer-input precision of the CUDA-core training kernels: BF16 (the

@@ -4,17 +4,23 @@
 // W4[6][64] b4.  Each layer's input (x, h1, h2, h3) is rounded to bfloat16
 // (or left as it is in the FP32 test mode); products and sums are FP32.
 //
-// The work is 26 k multiply-adds per sample against 44 bytes of input, so the
-// kernel is bound by the FP32 pipes.  A CTA of 128 threads takes chunks of 64
-// samples; every product of the chunk is a small matrix product with 32
-// accumulators per thread (8 x 4), whose operands come from shared memory as
-// 16-byte loads (three per 32 multiply-adds), and the gradient of the two
-// 64 x 64 layers stays in registers from chunk to chunk.  Two CTAs share an
-// SM, so one fills the other's barriers.  Batch of 65536: gradient 1019 -> 127
-// us (one sample per thread, weights by broadcast loads, before; the FP32 pipes
-// alone would take 45 us), with the sliced reduction and Adam 1121 -> 137 us.
-// Shared-memory loads are what bounds it: a 16-byte load takes four wavefronts
-// however many lanes share an address.
+// The work is 26 k multiply-adds per sample against 44 bytes of input.  A CTA of
+// 128 threads takes chunks of 64 samples; every product of the chunk is a small
+// matrix product with 32 accumulators per thread (8 x 4), whose operands come
+// from shared memory as 16-byte loads (three per 32 multiply-adds), and the
+// gradient of the two 64 x 64 layers stays in registers from chunk to chunk.
+// Two CTAs share an SM, so one fills the other's barriers.  Batch of 65536:
+// gradient 1019 -> 127 us (one sample per thread, weights by broadcast loads,
+// before; the FP32 pipes alone would take 45 us), with the sliced reduction and
+// Adam 1121 -> 137 us.  Shared-memory loads are what bounds it: a 16-byte load
+// takes four wavefronts however many lanes share an address.
+//
+// FP32 sums are short whatever the batch: 64 samples of a chunk, then at most
+// kRun chunks of a CTA, whose totals are added in FP64; no term passes through
+// more than 78 additions, and the rounding of a sum of equal terms (the worst
+// case) is that of 128 terms in a row.  (One running sum per resident CTA has no
+// such bound: of 2^21 equal samples, 108 chunks per CTA, it was off by 26 units
+// of 2^-24.)  The further CTAs cost 2 % at a batch of 2^20: 1.68 -> 1.71 ms.
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -28,7 +34,8 @@ constexpr int kChunk = 64;      // samples per chunk
 constexpr int kThreads = 128;
 constexpr int kLd = kChunk + 4;  // row length of [feature][sample] and [out][in] tiles: 16-byte rows, 4 banks apart
 constexpr int kPerSm = 2;        // CTAs per SM (shared memory)
-constexpr int kMaxBlocks = 152 * kPerSm;
+constexpr int kWave = 152 * kPerSm;
+constexpr int kRun = 14;         // chunks of one CTA at most
 // offsets in the parameter vector
 constexpr int oW1 = 0, oB1 = 320, oW2 = 384, oB2 = 4480, oW3 = 4544, oB3 = 8640, oW4 = 8704, oB4 = 9088;
 
@@ -371,7 +378,8 @@ __device__ __forceinline__ void adam_update(const AdamStep& a, int i, float gi) 
 
 // Sums of the per-CTA partials in a fixed order, FP64: 32 parameters per
 // block, eight threads each for every eighth partial, their sums in order.
-// Bound by the read of the partials (11 MB at most, which L2 holds).
+// Bound by the read of the partials (11 MB up to 272384 samples, 36 KB per 896
+// more; L2 holds those of 3 million).
 constexpr int kRedCols = 32, kRedRows = 8;
 template <bool ADAM>
 __global__ void __launch_bounds__(kRedCols* kRedRows)
@@ -414,9 +422,11 @@ __global__ void k_adam(AdamStep a, const float* __restrict__ g, int n) {
 // ------------------------------------------------------------ host side ----
 static int mlp_chunks(long long B) { return (int)((B + mlpcc::kChunk - 1) / mlpcc::kChunk); }
 
+// whole waves of CTAs from the first one on, as many as keep each to kRun chunks
 int mlp_grad_blocks(long long B) {
+  using namespace mlpcc;
   const int c = mlp_chunks(B);
-  return c < mlpcc::kMaxBlocks ? c : mlpcc::kMaxBlocks;
+  return c < kWave ? c : kWave * ((c + kWave * kRun - 1) / (kWave * kRun));
 }
 
 static cudaError_t mlp_cc_attrs() {
@@ -463,7 +473,7 @@ cudaError_t launch_mlp_reduce(int B, const float* part, const double* loss_part,
 cudaError_t launch_mlp_forward_cc(bool bf16, const float* params, const float* x, float* y, int B, cudaStream_t st) {
   const cudaError_t e = mlp_cc_attrs();
   if (e != cudaSuccess) return e;
-  const int blocks = mlp_grad_blocks(B), chunks = mlp_chunks(B);
+  const int chunks = mlp_chunks(B), blocks = chunks < mlpcc::kWave ? chunks : mlpcc::kWave;
   if (bf16)
     k_mlp_forward_cc<true><<<blocks, mlpcc::kThreads, sizeof(mlpcc::Smem), st>>>(params, x, y, B, chunks);
   else

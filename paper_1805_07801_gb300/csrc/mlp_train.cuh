@@ -9,7 +9,7 @@ namespace fftk {
 constexpr int kNP = 9094;  // parameters of the 5-64-64-64-6 network
 
 // blocks (and so gradient partials of kNP floats and loss partials) of a
-// gradient over at most B samples; grows with B up to a fixed bound
+// gradient over at most B samples; never falls as B grows
 int mlp_grad_blocks(long long B);
 
 // Adam's constants for one step: c1, c2 the bias corrections
