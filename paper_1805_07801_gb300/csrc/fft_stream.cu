@@ -313,18 +313,37 @@ static bool pipe_maps(CUtensorMap* m, CUtensorMap* mo, const float2* in, long lo
   return encode_f32_map(mo, in + Q - 1, 3, dims_odd, strides, box_odd);
 }
 
+// 256-point lines in a sine or cosine basis take the pipelined pass only in the
+// inverse with even rows: forward, the mirror exchange spills 120 bytes at the 64
+// registers of four CTAs per SM, and odd rows gain nothing (against k_scpass, with
+// which these run now: 256^3 cosine-cosine-sine forward 92.7 -> 70.7 us, two such
+// axes and Fourier 92.5 -> 68.5 us, its inverse 81.5 -> 75.9 us; the inverse x
+// pass of four fields of 256^3, even rows, takes 263.5 us there and 256.7 us here).
+constexpr bool pipe_built(int L, int sign, bool pair, int basis) {
+  return basis == 0 || L != 256 || (sign > 0 && !pair);
+}
+
+template <int L, int SIGN, bool PAIR, int BASIS>
+static bool pipe_run(fftk_plan p, const float2* in, float2* out, long long P, long long Q, float scale, int kind,
+                     cudaStream_t st, cudaError_t* e) {
+  if constexpr (!pipe_built(L, SIGN, PAIR, BASIS)) {
+    return false;
+  } else {
+    CUtensorMap m{}, mo{};
+    if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
+    *e = cpass_pipe<L, SIGN, PAIR, BASIS>(p, m, PAIR ? mo : m, out, P, Q, scale, kind, st);
+    return true;
+  }
+}
+
 template <int L, int BASIS>
 static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long long P, long long Q, float scale,
                    int kind, cudaStream_t st, cudaError_t* e) {
-  CUtensorMap m{}, mo{};
-  if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
   if (Q % 2 == 0)
-    *e = sign < 0 ? cpass_pipe<L, -1, false, BASIS>(p, m, m, out, P, Q, scale, kind, st)
-                  : cpass_pipe<L, +1, false, BASIS>(p, m, m, out, P, Q, scale, kind, st);
-  else
-    *e = sign < 0 ? cpass_pipe<L, -1, true, BASIS>(p, m, mo, out, P, Q, scale, kind, st)
-                  : cpass_pipe<L, +1, true, BASIS>(p, m, mo, out, P, Q, scale, kind, st);
-  return true;
+    return sign < 0 ? pipe_run<L, -1, false, BASIS>(p, in, out, P, Q, scale, kind, st, e)
+                    : pipe_run<L, +1, false, BASIS>(p, in, out, P, Q, scale, kind, st, e);
+  return sign < 0 ? pipe_run<L, -1, true, BASIS>(p, in, out, P, Q, scale, kind, st, e)
+                  : pipe_run<L, +1, true, BASIS>(p, in, out, P, Q, scale, kind, st, e);
 }
 
 // Arrays narrower than a tile, bases off 16 bytes and (below 768 points, where
