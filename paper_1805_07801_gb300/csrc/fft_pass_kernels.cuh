@@ -161,8 +161,7 @@ struct CCfg {
 
 // AHEAD > 0: while it transforms, the CTA asks for the rows of the tile AHEAD
 // places on (the one that comes next on some SM) in L2.  For lines that leave
-// room for one CTA per SM, whose loads nothing else covers: 768^3 pair 4.87 ->
-// 4.41 ms before fft_stream.cu had a pipelined pass for them.
+// room for one CTA per SM, whose loads nothing else covers.
 template <int L, int SIGN, int AHEAD>
 __global__ void __launch_bounds__(CCfg<L>::THREADS, CCfg<L>::MINB)
     k_cpass(const float2* in, float2* out, long long Q, long long qtiles,
@@ -239,10 +238,12 @@ template <int L, int SIGN>
 static cudaError_t cpass_l(fftk_plan p, const float2* in, float2* out, long long P, long long Q, float scale,
                            int kind, cudaStream_t st) {
   // rows further apart than a few pages (the x pass) only where 24 values per
-  // thread leave 16 warps on the SM (1024^3: y 2.07 -> 1.95 ms, but x, with 32
-  // warps, 2.01 against 2.12 ms); 1024 itself has a pipelined pass for all but
-  // narrow or unaligned arrays, and would spill here
-  if constexpr (L >= 768 && L != 1024)
+  // thread leave 16 warps on the SM (1024^3, before its pipelined pass: y 2.07 ->
+  // 1.95 ms, but x, with 32 warps, 2.01 against 2.12 ms).  Of the lines that
+  // fft_stream.cu takes unless the array is narrow or small, 768 points keep it
+  // (1000 planes of 9 columns, inverse 65.3 -> 62.4 us), 1536 do not (21.8 against
+  // 23.0 us, 57.2 against 60.0, 192 against 188), and 1024 would spill.
+  if constexpr (L == 768 || L >= 2048)
     if (Q <= 4096 || L % 3 == 0) return cpass_la<L, SIGN, 152>(p, in, out, P, Q, scale, kind, st);
   return cpass_la<L, SIGN, 0>(p, in, out, P, Q, scale, kind, st);
 }

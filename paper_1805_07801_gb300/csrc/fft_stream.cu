@@ -268,23 +268,30 @@ bool encode_f32_map(CUtensorMap* m, const void* base, int rank, const uint64_t* 
   return r == CUDA_SUCCESS;
 }
 
+// SMs of the current device
+static cudaError_t sm_count(int* n) {
+  static PerDevice once;
+  static int nsm[kMaxDevices];
+  int dev = 0;
+  const cudaError_t e =
+      once.run([](int d) { return cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d); }, &dev);
+  if (e == cudaSuccess) *n = nsm[dev];
+  return e;
+}
+
 template <int L, int SIGN, bool PAIR, int BASIS>
 static cudaError_t cpass_pipe(fftk_plan p, const CUtensorMap& m, const CUtensorMap& mo, float2* out, long long P,
                               long long Q, float scale, int kind, cudaStream_t st) {
   using C = PipeCfg<L, PAIR>;
   static PerDevice once;
-  static int nsm[kMaxDevices];
-  int dev = 0;
-  const cudaError_t e = once.run(
-      [](int d) {
-        cudaError_t err = cudaFuncSetAttribute(k_cpass_pipe<L, SIGN, PAIR, BASIS>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
-        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&nsm[d], cudaDevAttrMultiProcessorCount, d);
-        return err;
-      },
-      &dev);
+  cudaError_t e = once.run([](int) {
+    return cudaFuncSetAttribute(k_cpass_pipe<L, SIGN, PAIR, BASIS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)C::SMEM);
+  });
+  int nsm = 0;
+  if (e == cudaSuccess) e = sm_count(&nsm);
   if (e != cudaSuccess) return e;
-  const long long qtiles = (Q + C::T - 1) / C::T, ntiles = P * qtiles, cap = (long long)nsm[dev] * C::MINB;
+  const long long qtiles = (Q + C::T - 1) / C::T, ntiles = P * qtiles, cap = (long long)nsm * C::MINB;
   const unsigned grid = (unsigned)(ntiles < cap ? ntiles : cap);
   LaunchScope ls(p, kind, st);
   launch_pdl(k_cpass_pipe<L, SIGN, PAIR, BASIS>, grid, C::THREADS, C::SMEM, st, m, mo, out, Q, (int)qtiles,
@@ -313,11 +320,32 @@ static bool pipe_maps(CUtensorMap* m, CUtensorMap* mo, const float2* in, long lo
   return encode_f32_map(mo, in + Q - 1, 3, dims_odd, strides, box_odd);
 }
 
+// Arrays narrower than 16 columns, bases off 16 bytes and small passes keep the
+// general pass (false, nothing launched).  Staging the next tile pays from a CTA's
+// second tile on where one CTA fills an SM, and the later the more CTAs share it
+// and cover each other's loads: more than one tile per resident CTA for lines of
+// 768 points and more, two for 384 and 512, three for 256.  Transforms of batches
+// of planes, the y and z or x and z passes, general pass -> here:
+//   1024 points   152 tiles 15.6 -> 16.7 us   228 tiles 26.2 -> 25.5   912 tiles 87.1 -> 77.7
+//    768          152       12.3 -> 13.3      228       20.7 -> 19.9   912       67.1 -> 59.5
+//    512          400       19.8 -> 22.3      608       27.1 -> 26.5   912       39.4 -> 36.1
+//    384          400       15.9 -> 15.6      608       20.9 -> 21.1   912       30.1 -> 30.0
+//    256          912       18.2 -> 20.3     1824 (x)   90.3 -> 89.2  2432 (x)  117.5 -> 115.6
+template <int L>
+static bool pipe_applies(const float2* in, long long P, long long Q) {
+  if (P <= 0 || Q < 16 || reinterpret_cast<uintptr_t>(in) % 16 != 0) return false;
+  using C = PipeCfg<L, false>;
+  constexpr int TURNS = C::MINB == 4 ? 3 : C::MINB;
+  const long long tiles = P * ((Q + C::T - 1) / C::T);
+  int nsm = 0;
+  return tiles < (1LL << 31) && sm_count(&nsm) == cudaSuccess && tiles > (long long)TURNS * C::MINB * nsm;
+}
+
 // 256-point lines in a sine or cosine basis take the pipelined pass only in the
 // inverse with even rows: forward, the mirror exchange spills 120 bytes at the 64
 // registers of four CTAs per SM, and odd rows gain nothing (against k_scpass, with
 // which these run now: 256^3 cosine-cosine-sine forward 92.7 -> 70.7 us, two such
-// axes and Fourier 92.5 -> 68.5 us, its inverse 81.5 -> 75.9 us; the inverse x
+// axes and Fourier 92.5 -> 68.9 us, its inverse 81.5 -> 73.1 us; the inverse x
 // pass of four fields of 256^3, even rows, takes 263.5 us there and 256.7 us here).
 constexpr bool pipe_built(int L, int sign, bool pair, int basis) {
   return basis == 0 || L != 256 || (sign > 0 && !pair);
@@ -330,7 +358,7 @@ static bool pipe_run(fftk_plan p, const float2* in, float2* out, long long P, lo
     return false;
   } else {
     CUtensorMap m{}, mo{};
-    if (!pipe_maps<L>(&m, &mo, in, P, Q)) return false;
+    if (!pipe_applies<L>(in, P, Q) || !pipe_maps<L>(&m, &mo, in, P, Q)) return false;
     *e = cpass_pipe<L, SIGN, PAIR, BASIS>(p, m, PAIR ? mo : m, out, P, Q, scale, kind, st);
     return true;
   }
@@ -346,19 +374,8 @@ static bool pipe_l(fftk_plan p, int sign, const float2* in, float2* out, long lo
                   : pipe_run<L, +1, true, BASIS>(p, in, out, P, Q, scale, kind, st, e);
 }
 
-// Arrays narrower than a tile, bases off 16 bytes and (below 768 points, where
-// the general pass has several CTAs per SM) passes of less than two tiles per
-// SM keep the general pass: false, nothing launched.  (64 fields of 512 x 32:
-// 37 us a pair through k_cpass, 42 us here; 450 tiles of 256 x 16: the same.)
-static bool pipe_applies(int L, const float2* in, long long P, long long Q) {
-  if (P <= 0 || Q < 16 || reinterpret_cast<uintptr_t>(in) % 16 != 0) return false;
-  const long long tiles = P * ((Q + 7) / 8);  // of eight columns
-  return tiles < (1LL << 31) && (L >= 768 || tiles >= 4 * 152);
-}
-
 bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
                       float scale, int kind, cudaStream_t st, cudaError_t* e) {
-  if (!pipe_applies(L, in, P, Q)) return false;
   switch (L) {
 #define CASE(n) \
   case n:       \
@@ -371,7 +388,6 @@ bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* ou
 
 bool launch_scpass_tma(fftk_plan p, int L, bool sine, int dir, const float2* in, float2* out, long long P, long long Q,
                        float scale, int kind, cudaStream_t st, cudaError_t* e) {
-  if (!pipe_applies(L, in, P, Q)) return false;
   switch (L) {
 #define CASE(n) \
   case n:       \

@@ -184,12 +184,13 @@ cudaError_t launch_cpass(fftk_plan p, int L, int sign, const float2* in, float2*
 
 // split-FP16 tensor-core strided pass (FFTK_R32_SPLIT16), L in {256, 512, 1024, 2048}
 bool cpass_tc_supported(int L);
-// pipelined strided c2c pass with TMA tile loads for lines of 256, 512 and 1024
-// points: false (nothing launched) where it does not apply (fewer columns than
-// a tile, base not 16-byte aligned), else true with the launch status in *e
+// pipelined strided c2c pass with TMA tile loads for lines of 256, 384, 512, 768,
+// 1024 and 1536 points: false (nothing launched) where it does not apply (fewer
+// than 16 columns, base not 16-byte aligned, too few tiles for its persistent
+// CTAs), else true with the launch status in *e
 bool launch_cpass_tma(fftk_plan p, int L, int sign, const float2* in, float2* out, long long P, long long Q,
                       float scale, int kind, cudaStream_t st, cudaError_t* e);
-// the same for sine/cosine lines of 256, 512 and 1024 points
+// the same for sine/cosine lines of 256 (inverse with Q even only), 512 and 1024 points
 bool launch_scpass_tma(fftk_plan p, int L, bool sine, int dir, const float2* in, float2* out, long long P, long long Q,
                        float scale, int kind, cudaStream_t st, cudaError_t* e);
 // the split-FP16 pass restricted to the 2/3-rule set of an n^3 spectrum
