@@ -19,18 +19,21 @@ namespace fftk {
 // instead of three; 64^3: 12.6 -> 8.3 us; 768^3: 2.87 -> 2.26 ms, with radix 48
 // and 16 instead of 8, 8, 12 1.76 ms.
 //
-// One field is in registers and two are parked.  n = 512 and 768: two stages
-// with the half-size exchange (XTransform), 256 threads, 16 columns per tile;
-// other 3 * 2^m: 24 values per thread, 16 columns; other powers of two: 8
-// values per thread, 16 columns (8 at n = 1024).  At 512 and for 3 * 2^m only
-// the slots m whose rows j + m S can be kept by the 2/3 rule are parked, the
+// One field is in registers and two are parked.  From n = 256 on, two stages with
+// the half-size exchange (XTransform) on 256 threads, 16 columns per tile (8 at n =
+// 1024, whose parked fields fill the shared memory); below, and at 384, whose 24
+// values hold no whole number of radix-16 butterflies, the line engine with 24
+// (3 * 2^m) or 8 values per thread and 16 columns.  RK2 / RK4 step with 8 values
+// and so: 256^3 833 / 1706 -> 820 / 1682 us, 1024^3 62.6 / 128.8 -> 61.6 / 127.0 ms
+// (64 registers spilled up to 64 bytes there).  With two stages and for 3 * 2^m
+// only the slots m whose rows j + m S can be kept by the 2/3 rule are parked, the
 // first LOW and those from HIGH on.
 template <int N>
 struct NUCfg {
-  static constexpr bool TWO = N == 768 || N == 512;  // radix 48 or 32, then 16
-  static constexpr int G = N == 768 ? 48 : TWO ? 32 : (N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G);
+  static constexpr bool TWO = N >= 256 && N != 384;  // radix 48, 32 or 16, then 16 (32 at 1024)
+  static constexpr int G = N == 768 ? 48 : N == 256 ? 16 : TWO ? 32 : (N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G);
   static constexpr int S = N / G;
-  static constexpr int T = N % 3 == 0 || N == 512 ? 16 : (N == 1024 ? 8 : NFCfg<N>::T);
+  static constexpr int T = N == 1024 ? 8 : 16;
   static constexpr int THREADS = T * S;
   static constexpr int KD = (N - 1) / 3;
   static constexpr int LOW = N % 3 != 0 && !TWO ? G : KD / S + 1;
@@ -38,11 +41,10 @@ struct NUCfg {
   static constexpr int SLOTS = LOW + G - HIGH;
   using X = XTransform<N, G, -1, T, TWO>;
   static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 2 * (size_t)SLOTS * THREADS);
-  static constexpr int MINB = TWO ? 1
-                                  : N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
-                                  : N >= 512   ? 1024 / THREADS  // 64 registers; below 512 points 128
-                                               : (512 / THREADS < 8 ? 512 / THREADS : 8);
-  static constexpr int GROUP = N % 3 != 0 && N >= 512 && !TWO ? 2 : 4;  // modes whose loads are in flight together
+  static constexpr int MINB = TWO          ? (N == 256 ? 2 : 1)
+                              : N % 3 == 0 ? (THREADS <= 128 ? 4 : (THREADS <= 256 ? 2 : 1))
+                                           : (512 / THREADS < 8 ? 512 / THREADS : 8);
+  static constexpr int GROUP = 4;  // modes whose loads are in flight together
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };

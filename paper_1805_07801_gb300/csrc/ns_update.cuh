@@ -135,8 +135,8 @@ __device__ __forceinline__ void ns_mode_update(const NSModeIn& in, float2 nx, fl
 }
 
 // Transform of an x pass with its tile's buffers at `sm`: the line engine with
-// an exchange buffer of the tile's size, or (TWO, 768 points) two stages of
-// radix 48 and 16 with a half-size buffer and the twiddles behind it.
+// an exchange buffer of the tile's size, or (TWO) two long-radix stages with a
+// half-size buffer and the twiddles behind it.
 template <int N, int G, int SIGN, int T, bool TWO>
 struct XTransform {
   static constexpr size_t WORDS = TWO ? (size_t)N * T / 2 + N : (size_t)N * T;  // float2 at sm

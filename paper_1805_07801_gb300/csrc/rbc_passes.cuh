@@ -251,9 +251,13 @@ __global__ void __launch_bounds__(RZCfg<N>::THREADS, RZCfg<N>::MINB)
 // flight in the update, 1014 us with five transforms (256^3 126 -> 119 us, 384^3
 // 388 -> 363 us).  Its six fields and eighteen kept arrays would take 632
 // us: eight warps do not cover the loads of each field and the exchanges.
+// Two stages at n = 512 and 1024 (step at 1024^3, RK2 / RK4: 97.8 / 205.3 ->
+// 91.7 / 192.2 ms).  Not at 256, where 16 values on 128 registers spill up to 268
+// bytes (RK4 2345 -> 2403 us), nor at 768, where three parked fields leave room
+// for eight columns and so for four warps (74.9 -> 74.3 ms, below 1 %).
 template <int N>
 struct RUCfg {
-  static constexpr bool TWO = N == 512;  // radix 32, then 16
+  static constexpr bool TWO = N == 512 || N == 1024;  // radix 32, then 16 or 32
   static constexpr int G = TWO ? 32 : (N % 3 == 0 ? elems_per_thread(N) : NFCfg<N>::G);
   static constexpr int S = N / G;
   static constexpr int T = N == 512 ? 16 : (N >= 768 ? 8 : (N % 3 == 0 ? 16 : NFCfg<N>::T));
@@ -265,9 +269,9 @@ struct RUCfg {
   using X = XTransform<N, G, -1, T, TWO>;
   static constexpr size_t SMEM = sizeof(float2) * (X::WORDS + 3 * (size_t)SLOTS * THREADS);
   static constexpr int MINB = THREADS >= 512 ? 1 : (THREADS == 256 ? (N == 768 || TWO ? 1 : 2) : 4);
-  // modes whose loads are in flight together (1024 has no registers for two;
-  // four at 3 * 2^m spill, 384^3 422 us against 388 with two and 405 with one)
-  static constexpr int GROUP = N == 1024 ? 1 : (N % 3 == 0 ? 2 : 4);
+  // modes whose loads are in flight together (four at 3 * 2^m spill, 384^3 422 us
+  // against 388 with two and 405 with one)
+  static constexpr int GROUP = N % 3 == 0 ? 2 : 4;
   __host__ __device__ static constexpr bool parked(int m) { return m < LOW || m >= HIGH; }
   __host__ __device__ static constexpr int slot(int m) { return m < LOW ? m : m - HIGH + LOW; }
 };
