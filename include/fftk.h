@@ -244,8 +244,8 @@ fftk_status tarang_ns_step(fftk_plan p, void *uhat, const tarang_params *prm, in
  * the periodic cube also takes n = 3 * 2^m in [12, 768] (the paper's XC40
  * convection sizes, Sec. 7), through the same fused passes.  Other sizes:
  * FFTK_ERR_UNSUPPORTED_SIZE.
- * Device memory: 15 more complex fields, seven of them with rows of n/2 + 1
- * rounded up to a multiple of 16 (allocated on first use, kept by the plan). */
+ * Device memory: 15 more complex fields with rows of n/2 + 1 rounded up to a
+ * multiple of 16, for either basis (allocated on first use, kept by the plan). */
 enum { TARANG_RBC_FFF = 0, TARANG_RBC_SFF = 1 };
 
 typedef struct {

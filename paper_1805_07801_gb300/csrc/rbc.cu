@@ -50,7 +50,10 @@ static fftk_status rbc_ensure(fftk_plan p) {
   const int kxs = (2 * g.n - 1) / 3;
   r->tab_len = kxs * kxs + 2 * g.kd * g.kd + 1;
   const size_t fw = sizeof(float2) * (size_t)g.n * g.n * (size_t)ns_row(g.n);  // padded rows
-  const size_t fs = fw > fb ? fw : fb;  // the periodic cube pads the stage state's and the accumulator's rows too
+  // the periodic cube pads the rows of the stage state and of the accumulator too;
+  // plates leave them at n/2 + 1 in the same arrays (a plan serves both bases, and
+  // the second one may come up under stream capture, where nothing is allocated)
+  const size_t fs = fw > fb ? fw : fb;
   cudaError_t e = cudaMalloc(&r->w7, 7 * fw);
   if (e == cudaSuccess) e = cudaMalloc(&r->s1, 4 * fs);
   if (e == cudaSuccess) e = cudaMemset(r->s1, 0, 4 * fs);
@@ -131,41 +134,12 @@ __global__ void k_rbc_sff_prep(const float2* __restrict__ x, float2* __restrict_
   }
 }
 
-// the stage update of one field entry i (the modes of ns_mode_update)
-__device__ __forceinline__ void rbc_entry_update(long long i, float2 n, float2 E, float2 H, float dt, int mode,
-                                                 const float2* u0, const float2* s1, float2* acc, float2* out) {
-  if (mode == NS_RHS) {
-    out[i] = n;
-  } else if (mode == NS_STAGE1) {
-    const float2 v = u0[i];
-    out[i] = mul_pair(make_float2(v.x + dt * n.x, v.y + dt * n.y), E);
-  } else if (mode == NS_STAGE2) {
-    const float2 ea = mul_pair(u0[i], E), b1 = s1[i];
-    out[i] = make_float2(0.5f * (ea.x + (b1.x + dt * n.x)), 0.5f * (ea.y + (b1.y + dt * n.y)));
-  } else if (mode == NS_RK4_4) {
-    const float2 ac = acc[i];
-    out[i] = make_float2(fmaf(dt / 6.f, n.x, ac.x), fmaf(dt / 6.f, n.y, ac.y));
-  } else {
-    const float2 v = u0[i];
-    const float2 ea = mul_pair(v, E), ha = mul_pair(v, H), hn = mul_pair(n, H);
-    if (mode == NS_RK4_1) {
-      const float2 en = mul_pair(n, E);
-      acc[i] = make_float2(fmaf(dt / 6.f, en.x, ea.x), fmaf(dt / 6.f, en.y, ea.y));
-      out[i] = mul_pair(make_float2(v.x + 0.5f * dt * n.x, v.y + 0.5f * dt * n.y), H);
-    } else {
-      const float2 ac = acc[i];
-      acc[i] = make_float2(fmaf(dt / 3.f, hn.x, ac.x), fmaf(dt / 3.f, hn.y, ac.y));
-      out[i] = (mode == NS_RK4_2) ? make_float2(fmaf(0.5f * dt, n.x, ha.x), fmaf(0.5f * dt, n.y, ha.y))
-                                  : make_float2(fmaf(dt, hn.x, ea.x), fmaf(dt, hn.y, ea.y));
-    }
-  }
-}
-
 // w7 (spectra): [(u x omega)_x, (u_y theta), (u_z theta) in sine | (u x omega)_y,
 // (u x omega)_z, (u_x theta) in cosine].  v = u x omega + theta x, minus the
 // gradient of the cosine pressure p = -div v / k^2; N_theta = -div(u theta) + u_x.
-__global__ void k_rbc_sff_update(const float2* __restrict__ w7, const float2* x, const float2* u0, float2* s1,
-                                 float2* acc, float2* out, NSGeom g, RBCUpdate upd, int mode) {
+template <int MODE>
+__global__ void k_rbc_sff_update(const float2* __restrict__ w7, const float2* x, const float2* u0, const float2* s1,
+                                 float2* acc, float2* out, NSGeom g, RBCUpdate upd) {
   pdl_wait();
   const long long M = g.M, rowa = (long long)g.n * g.h1;
   const long long HW = ns_row(g.n), MW = (long long)g.n * g.n * HW, roww = (long long)g.n * HW;  // of w7
@@ -206,14 +180,20 @@ __global__ void k_rbc_sff_update(const float2* __restrict__ w7, const float2* x,
       const float2 d = csub(cadd(mul_i(sy, fky), mul_i(sz, fkz)), cscale(cx, fkx));
       nt = cadd(make_float2(-d.x, -d.y), ux);
     }
-    const float dt = upd.dt;
-    const float2 Eu = __ldg(&upd.tab[k2]), Et = __ldg(&upd.tab[upd.tab_len + k2]);
-    const float2 Hu = __ldg(&upd.tab[2 * upd.tab_len + k2]), Ht = __ldg(&upd.tab[3 * upd.tab_len + k2]);
-    rbc_entry_update(idx + M, vy, Eu, Hu, dt, mode, u0, s1, acc, out);
-    rbc_entry_update(idx + 2 * M, vz, Eu, Hu, dt, mode, u0, s1, acc, out);
+    // entry e of one field, its factors at offset t of each pair
+    auto update = [&](long long e, float2 n, int t) {
+      const float2 z = make_float2(0.f, 0.f);
+      const float2 a = MODE != NS_RHS && MODE != NS_RK4_4 ? u0[e] : z;
+      const float2 b = MODE == NS_STAGE2 ? s1[e] : (MODE >= NS_RK4_2 ? acc[e] : z);
+      const float2 E = MODE != NS_RHS && MODE != NS_RK4_4 ? __ldg(&upd.tab[t * upd.tab_len + k2]) : z;
+      const float2 H = MODE >= NS_RK4_1 && MODE != NS_RK4_4 ? __ldg(&upd.tab[(2 + t) * upd.tab_len + k2]) : z;
+      rbc_entry_store<MODE>(e, e, n, a, b, E, H, upd.dt, acc, out);
+    };
+    update(idx + M, vy, 0);
+    update(idx + 2 * M, vz, 0);
     if (has_s) {
-      rbc_entry_update(sidx, vx, Eu, Hu, dt, mode, u0, s1, acc, out);
-      rbc_entry_update(sidx + 3 * M, nt, Et, Ht, dt, mode, u0, s1, acc, out);
+      update(sidx, vx, 0);
+      update(sidx + 3 * M, nt, 1);
     }
   }
 }
@@ -252,7 +232,16 @@ static cudaError_t rbc_stage(fftk_plan p, const float2* x, const float2* u0, flo
     if (e != cudaSuccess) return e;
     {
       LaunchScope ls(p, KK_RBC_UPDATE, st);
-      launch_pdl(k_rbc_sff_update, grid, 256, 0, st, w, x, u0, r->s1, r->acc, out, g, upd, mode);
+      switch (mode) {
+#define MODE(m)                                                                                            \
+  case m:                                                                                                  \
+    launch_pdl(k_rbc_sff_update<m>, grid, 256, 0, st, w, x, u0, r->s1, r->acc, out, g, upd);               \
+    break;
+        MODE(NS_RHS) MODE(NS_STAGE1) MODE(NS_STAGE2) MODE(NS_RK4_1) MODE(NS_RK4_2) MODE(NS_RK4_3) MODE(NS_RK4_4)
+#undef MODE
+        default:
+          return cudaErrorInvalidValue;
+      }
     }
     return cudaGetLastError();
   }
