@@ -18,9 +18,9 @@ const char* const kKernelNames[KK_COUNT] = {
 bool is_pow2(long long v) { return v >= 1 && (v & (v - 1)) == 0; }
 bool is_pow2_or_3x(long long v) { return is_pow2(v) || (v % 3 == 0 && is_pow2(v / 3)); }
 
-// A transform length the passes support: a power of two up to 4096, or
-// 3 * 2^m (a radix-3 step over power-of-two sub-lines of at least 2 points)
-// up to 3072; along z (halved by the real packing) at least 12.
+// A transform length the passes support: a power of two up to 4096, or 3 * 2^m
+// (the last stage of a line takes the factor 3) from 6 up to 3072; along z (halved
+// by the real packing) from 12.
 static bool dim_ok(int n, bool z) {
   if (is_pow2(n)) return n <= 4096 && (!z || n >= 2);
   if (n % 3 != 0 || !is_pow2(n / 3)) return false;

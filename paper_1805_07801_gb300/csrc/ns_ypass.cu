@@ -14,12 +14,12 @@
 
 namespace fftk {
 
-template <int N, int SIGN>
+template <int N, int SIGN>  // N >= 384
 struct YPipeCfg {
   static constexpr bool ENGINE = N % 3 == 0 && N != 768;  // else two long-radix stages
-  static constexpr int G = ENGINE ? elems_per_thread(N) : (N == 768 ? 48 : (N >= 512 ? 32 : 16));
+  static constexpr int G = ENGINE ? elems_per_thread(N) : (N == 768 ? 48 : 32);
   static constexpr int S = N / G, T = 16, THREADS = S * T;
-  static constexpr int MINB = N >= 768 ? 1 : (N >= 384 ? 2 : 4);
+  static constexpr int MINB = N >= 768 ? 1 : 2;
   static constexpr int KD = (N - 1) / 3;
   // boxes: the inverse pass takes rows 0 .. KD and N - KD - 1 .. N - 1 (the first
   // of these is not used) in halves of at most 256 rows
